@@ -178,15 +178,18 @@ int fz_build_memo_into(const int32_t *tail, int k, int32_t top,
                        uint64_t rows_capacity, uint64_t *rows_needed,
                        void *stream);
 
-/* Launch schedules of the memo build (Section 2.2 names the two kinds of
- * parallelism of the dynamic pass; Section 2.4 gives the factorizationwise
- * algorithm).  All give the same memo.
+/* Launch schedules of the dynamic pass (Section 2.2 names the two kinds of
+ * parallelism; Section 2.4 gives the factorizationwise algorithm).  All give
+ * the same memo.  The calls without a schedule build it generator by
+ * generator instead (Lemma "disjlex" taken one coordinate at a time: Z(r,
+ * (t_i..)) is the concatenation over a_i, greatest first, of Z(r - a_i t_i,
+ * (t_{i+1}..)), one contiguous range of the level before when that is kept
+ * by residue class of t_i), which has no dependent batches; they fall back
+ * to FZ_MEMO_BATCHED for depths above 8 or when the levels' scratch cannot
+ * be allocated.
  *   FZ_MEMO_BATCHED    elementwise batches of min(tail) elements, each batch
  *                      factorizationwise parallel, all in ONE launch (batches
- *                      separated by a cluster or bounded grid barrier); the
- *                      schedule every other call uses, except that plans
- *                      fill memos of depth 1 and 2 from their closed forms
- *                      (the same rows, with no dependent batches).
+ *                      separated by a cluster or bounded grid barrier).
  *   FZ_MEMO_PER_BATCH  the same batches, one kernel launch per batch ("both"
  *                      parallelism, ordered by the stream).
  *   FZ_MEMO_PER_COPY   the factorizationwise parallel algorithm of Section

@@ -15,7 +15,7 @@
 #include <thread>
 #include <vector>
 
-#include "fz_internal.cuh"
+#include "fz_walk.cuh"
 
 namespace fz {
 
@@ -133,10 +133,11 @@ struct fz_plan_s {
     uint64_t slice_rows = 0;
     int64_t tmp_words = 0;
     DevBuf base;   // C, tmp, O, status, bar, counter
-    DevBuf memo;   // map + rows
+    DevBuf memo;   // memo in element order (rows, and the map of the dynamic pass)
     DevBuf runs;   // runs table for work-balanced slicing
-    DevBuf runm;   // memo in run order + class starts (full memo, k <= 3)
-    int4 *run_memo = nullptr;
+    DevBuf lvbuf;  // run-order tables of the memo's levels
+    RunLevels lv;
+    int4 *run_memo = nullptr;      // the memo in run order (full memo, k <= 3)
     uint64_t *cls_beg = nullptr;
     uint64_t *RT = nullptr;
     int lam_r = 0;
@@ -214,14 +215,21 @@ bool run_memo_enabled() {
 
 namespace {
 
-// Enqueue the memo of plan p (offsets scan, gather map, fill, run order).
+// Enqueue the memo of plan p: the run-order levels alone when the memo is
+// kept in run order; else the offsets scan and the memo in element order
+// (closed form for depth 1 and 2, levels up to CSR_MAX_K, the dynamic pass
+// beyond).
 int plan_enqueue_memo(fz_plan_s *p, cudaStream_t s) {
     if (p->K < 1 || p->top < 1) return FZ_OK;
+    if (p->run_memo) return launch_run_levels(p->lv, p->status, s);
     const int64_t cs = (int64_t)p->n + 1;
     const uint64_t *crow = p->C + (int64_t)(p->d - p->K) * cs;
     int rc = launch_exclusive_scan_tmp(crow, p->O, p->top, p->tmp, s);
     if (rc != FZ_OK) return rc;
     if (p->memo_rows == 0) return FZ_OK;
+    const int32_t *tail = p->g + (p->d - p->K);
+    if (p->K <= 2) return launch_memo_closed(tail, p->K, p->top, p->O, p->rows, p->status, s);
+    if (p->lv.n > 0) return launch_run_levels(p->lv, p->status, s);
     MemoBuffers mb;
     mb.Ct = crow;
     mb.cs = cs;
@@ -232,16 +240,7 @@ int plan_enqueue_memo(fz_plan_s *p, cudaStream_t s) {
     mb.bar = p->bar;
     // an enumeration capped below full occupancy leaves room for a small build
     mb.small_ctas = p->ctas_per_sm > 0 && p->ctas_per_sm <= 3;
-    // depth 1 and 2: the closed form of the tail sets (same rows as the
-    // dynamic pass, no dependent batches); deeper memos: the dynamic pass
-    if (p->K <= 2)
-        rc = launch_memo_closed(p->g + (p->d - p->K), p->K, p->top, p->O, p->rows, p->status, s);
-    else
-        rc = launch_memo_build(p->g + (p->d - p->K), p->K, p->top, p->memo_rows, mb, s);
-    if (rc != FZ_OK || !p->run_memo) return rc;
-    const int lam = p->d - p->K - 1;
-    return launch_run_memo(p->C, cs, lam, p->n, p->g[lam], p->O, p->rows, p->K, p->memo_rows,
-                           p->cls_beg, p->run_memo, p->status, s);
+    return launch_memo_build(tail, p->K, p->top, p->memo_rows, mb, s);
 }
 
 int read_status(int *status_dev, cudaStream_t s) {
@@ -255,23 +254,11 @@ int read_status(int *status_dev, cudaStream_t s) {
     return status_to_fz(h);
 }
 
-// Memo rows of depth k with full top = n + 1, from row d - k of the table
-// (exclusive scan into p->O, then one 8-byte read).  Synchronises.
-int memo_rows_for(fz_plan_s *p, int k, int32_t top, uint64_t *rows, cudaStream_t s) {
-    const int64_t cs = (int64_t)p->n + 1;
-    const uint64_t *crow = p->C + (int64_t)(p->d - k) * cs;
-    int rc = launch_exclusive_scan_tmp(crow, p->O, top, p->tmp, s);
-    if (rc != FZ_OK) return rc;
-    FZ_CUDA_TRY(cudaMemcpyAsync(rows, p->O + top, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    FZ_CUDA_TRY(cudaStreamSynchronize(s));
-    return FZ_OK;
-}
-
 // Memo depth chosen automatically: the deepest k in 2..min(d-1, 4) whose full
 // memo stays small next to the output and needs a bounded number of
-// elementwise batches; k = 0 (plain walk) when none qualifies.
-int choose_k(fz_plan_s *p, cudaStream_t s, int *k_out) {
-    *k_out = 0;
+// elementwise batches; k = 0 (plain walk) when none qualifies.  sums[j]: the
+// rows of all Z(r, (g_j..)), r <= n, exact below 2^32.
+int choose_k(const fz_plan_s *p, const uint64_t *sums) {
     const uint64_t out_bytes = p->count * (uint64_t)p->d * 4ull;
     const uint64_t budget = std::max<uint64_t>(8ull << 20, out_bytes / 8);
     for (int k = std::min(p->d - 1, 4); k >= 2; --k) {
@@ -279,16 +266,13 @@ int choose_k(fz_plan_s *p, cudaStream_t s, int *k_out) {
         for (int i = p->d - k; i < p->d; ++i) tmin = std::min(tmin, p->g[i]);
         const int64_t batches = ((int64_t)p->n + 1 + tmin - 1) / tmin;
         if (batches > 4096) continue;
-        uint64_t rows = 0;
-        int rc = memo_rows_for(p, k, p->n + 1, &rows, s);
-        if (rc != FZ_OK) return rc;
-        if (rows == ~0ull || rows > MEMO_MAX_ROWS) continue;
+        const uint64_t rows = sums[p->d - k];
+        if (rows > MEMO_MAX_ROWS) continue;
         const uint64_t bytes = rows * (uint64_t)(4 * k + 8);
         if (bytes > budget) continue;
-        *k_out = k;
-        return FZ_OK;
+        return k;
     }
-    return FZ_OK;
+    return 0;
 }
 
 // Measured options by (device, g, n), filled by fz_autotune.
@@ -310,6 +294,59 @@ bool autotune_lookup(const int32_t *g, int d, int32_t n, fz_opts_t *out) {
     if (it == g_tune.end()) return false;
     *out = it->second;
     return true;
+}
+
+// sums[j] (host) = rows of Z(r, ·) over r < top for the rows j = 0..nrows-1 of
+// a count table; exact below 2^32.  Synchronises.
+int row_sums(const uint64_t *C, int64_t cs, int nrows, int64_t top, uint64_t *dev, uint64_t *sums,
+             cudaStream_t s) {
+    int rc = launch_row_sums(C, cs, nrows, top, dev, s);
+    if (rc != FZ_OK) return rc;
+    FZ_CUDA_TRY(cudaMemcpyAsync(sums, dev, (size_t)nrows * 8, cudaMemcpyDeviceToHost, s));
+    FZ_CUDA_TRY(cudaStreamSynchronize(s));
+    return FZ_OK;
+}
+
+// Buffers of the memo of plan p (depth K, top and memo_rows set): in run
+// order for a full memo of depth <= 3 under a walked coordinate, else in
+// element order, by levels when their scratch fits, else with the gather map
+// of the dynamic pass.  sums[j]: the rows of all Z(r, (g_j..)), r < top.
+int plan_alloc_memo(fz_plan_s *p, const uint64_t *sums, cudaStream_t s) {
+    const int d = p->d, k = p->K;
+    const int64_t cs = (int64_t)p->n + 1;
+    const int lam = d - k - 1;
+    if (p->top > p->n && k <= 3 && lam >= 0 && run_memo_enabled()) {
+        if (p->lvbuf.alloc(run_levels_bytes(p->g + lam, k + 1, p->n, sums + lam, false)) ==
+            FZ_OK) {
+            const int rc = run_levels_init(p->g + lam, k + 1, p->n, sums + lam, false,
+                                           p->C + (int64_t)lam * cs, cs, nullptr, nullptr,
+                                           p->lvbuf.p, &p->lv, s);
+            if (rc != FZ_OK) return rc;
+            p->run_memo = reinterpret_cast<int4 *>(p->lv.rows);
+            p->cls_beg = p->lv.cls;
+            return FZ_OK;
+        }
+        cudaGetLastError();  // optional: without it the leaf-by-leaf copy runs
+    }
+    const bool csr = k >= 3 && k <= CSR_MAX_K && !memo_fill_forced();
+    const size_t rows_bytes = align256(p->memo_rows * (size_t)k * 4 + 16);
+    if (csr && p->memo_rows > 0) {
+        const size_t b = run_levels_bytes(p->g + (d - k), k, p->top - 1, sums + (d - k), true);
+        if (p->lvbuf.alloc(b) == FZ_OK && p->memo.alloc(rows_bytes) == FZ_OK) {
+            p->rows = p->memo.as<int32_t>();
+            return run_levels_init(p->g + (d - k), k, p->top - 1, sums + (d - k), true,
+                                   p->C + (int64_t)(d - k) * cs, cs, p->O, p->rows, p->lvbuf.p,
+                                   &p->lv, s);
+        }
+        cudaGetLastError();
+        p->lvbuf.release();
+    }
+    const size_t off_rows = k <= 2 ? 0 : align256(p->memo_rows * 8);
+    int rc = p->memo.alloc(off_rows + rows_bytes);
+    if (rc != FZ_OK) return rc;
+    p->map = k <= 2 ? nullptr : p->memo.as<uint64_t>();
+    p->rows = reinterpret_cast<int32_t *>(p->memo.as<char>() + off_rows);
+    return FZ_OK;
 }
 
 int plan_create_impl(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, fz_plan_s *p,
@@ -351,9 +388,17 @@ int plan_create_impl(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, f
 
     rc = launch_count_table_tmp(g, d, n, p->C, p->tmp, s);
     if (rc != FZ_OK) return rc;
+    // the count, and the memo rows of every depth (one read)
+    uint64_t sums[FZ_MAX_D + 1] = {};
+    uint64_t *sums_dev = reinterpret_cast<uint64_t *>(p->status + 16);
     FZ_CUDA_TRY(cudaMemcpyAsync(&p->count, p->C + n, sizeof(uint64_t), cudaMemcpyDeviceToHost,
                                 s));
-    FZ_CUDA_TRY(cudaStreamSynchronize(s));
+    if (!opt || opt->k != 0) {
+        rc = row_sums(p->C, cs, d + 1, cs, sums_dev, sums, s);
+        if (rc != FZ_OK) return rc;
+    } else {
+        FZ_CUDA_TRY(cudaStreamSynchronize(s));
+    }
     if (p->count == ~0ull) return set_error(FZ_EOVERFLOW, "|Z(n)| does not fit in 64 bits");
 
     // memo depth and top: the caller's, else a measured choice cached by
@@ -366,8 +411,7 @@ int plan_create_impl(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, f
             k = cached.k;
             tuned_slice = cached.slice_rows;
         } else {
-            rc = choose_k(p, s, &k);
-            if (rc != FZ_OK) return rc;
+            k = choose_k(p, sums);
         }
     }
     int64_t top = (opt && opt->top != FZ_AUTO) ? opt->top : (int64_t)n + 1;
@@ -376,29 +420,15 @@ int plan_create_impl(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, f
     p->K = k;
     p->top = (int32_t)top;
     if (k >= 1 && top >= 1) {
-        rc = memo_rows_for(p, k, p->top, &p->memo_rows, s);
-        if (rc != FZ_OK) return rc;
-        if (p->memo_rows == ~0ull || p->memo_rows > MEMO_MAX_ROWS)
-            return set_error(FZ_EINVAL, "memo too large (more than 2^30 rows); lower k or top");
-        const size_t off_rows = align256(p->memo_rows * 8);
-        rc = p->memo.alloc(off_rows + p->memo_rows * (size_t)k * 4 + 16);
-        if (rc != FZ_OK) return rc;
-        p->map = p->memo.as<uint64_t>();
-        p->rows = reinterpret_cast<int32_t *>(p->memo.as<char>() + off_rows);
-        // full memo of depth <= 3: also keep it in run order (16 bytes per
-        // row), which lets the enumeration copy whole subtrees of the last
-        // walked coordinate as one contiguous range
-        if (p->top > n && k <= 3 && k <= d - 1 && run_memo_enabled()) {
-            const int32_t glam = p->g[d - k - 1];
-            const int64_t G = glam < (int64_t)n + 1 ? glam : (int64_t)n + 1;
-            const size_t rm_bytes = align256(p->memo_rows * 16);
-            if (p->runm.alloc(rm_bytes + (size_t)(G + 1) * 8) == FZ_OK) {
-                p->run_memo = p->runm.as<int4>();
-                p->cls_beg = reinterpret_cast<uint64_t *>(p->runm.as<char>() + rm_bytes);
-            } else {
-                cudaGetLastError();  // optional: without it the leaf-by-leaf copy runs
-            }
+        if (p->top <= n) {
+            rc = row_sums(p->C, cs, d + 1, p->top, sums_dev, sums, s);
+            if (rc != FZ_OK) return rc;
         }
+        p->memo_rows = sums[d - k];
+        if (p->memo_rows > MEMO_MAX_ROWS)
+            return set_error(FZ_EINVAL, "memo too large (more than 2^30 rows); lower k or top");
+        rc = plan_alloc_memo(p, sums, s);
+        if (rc != FZ_OK) return rc;
         rc = plan_enqueue_memo(p, s);
         if (rc != FZ_OK) return rc;
         rc = read_status(p->status, s);
@@ -877,7 +907,7 @@ int fz_memo_rows(const int32_t *tail, int k, int32_t top, uint64_t *rows, void *
 
 static int build_memo_to(const int32_t *tail, int k, int32_t top, uint64_t *O, int32_t **R,
                          uint64_t rows_capacity, uint64_t *rows_needed, DevBuf *own_rows,
-                         cudaStream_t s, int schedule = FZ_MEMO_BATCHED) {
+                         cudaStream_t s, int schedule = MEMO_LEVELS) {
     DevBuf table, work;
     uint64_t *C = nullptr;
     int64_t tmpw = 0;
@@ -900,6 +930,39 @@ static int build_memo_to(const int32_t *tail, int k, int32_t top, uint64_t *O, i
         return set_error(FZ_ENOSPC, "memo rows exceed rows_capacity");
     }
     if (rows == 0) return FZ_OK;
+    if (schedule == MEMO_LEVELS) {
+        // depth 1 and 2: the closed form; deeper: the run-order levels while
+        // they apply and their scratch fits; else the dynamic pass
+        schedule = FZ_MEMO_BATCHED;
+        if (!memo_fill_forced() && k <= CSR_MAX_K) {
+            uint64_t sums[FZ_MAX_D + 1];
+            size_t bytes = 256;
+            bool fits = true;
+            uint64_t *small = C + (k + 1) * cs + tmpw;  // 64 words past the scan scratch
+            if (k > 2) {
+                rc = row_sums(C, cs, k, top, small, sums, s);
+                if (rc != FZ_OK) return rc;
+                sums[0] = rows;
+                fits = sums[1] < (1ull << 32) && rows / 256 < (1ull << 31);
+                if (fits) bytes += run_levels_bytes(tail, k, top - 1, sums, true);
+            }
+            if (fits && work.alloc(bytes) == FZ_OK) {
+                int *status = work.as<int>();
+                FZ_CUDA_TRY(cudaMemsetAsync(status, 0, 256, s));
+                if (k <= 2) {
+                    rc = launch_memo_closed(tail, k, top, O, *R, status, s);
+                } else {
+                    RunLevels lv;
+                    rc = run_levels_init(tail, k, top - 1, sums, true, C, cs, O, *R,
+                                         work.as<char>() + 256, &lv, s);
+                    if (rc == FZ_OK) rc = launch_run_levels(lv, status, s);
+                }
+                if (rc != FZ_OK) return rc;
+                return read_status(status, s);
+            }
+            cudaGetLastError();
+        }
+    }
     // gather map + status + barrier words
     const size_t map_bytes = align256(rows * 8);
     rc = work.alloc(map_bytes + 512);
@@ -918,11 +981,29 @@ static int build_memo_to(const int32_t *tail, int k, int32_t top, uint64_t *O, i
     return read_status(mb.status, s);
 }
 
+static int build_memo_caller(const int32_t *tail, int k, int32_t top, int schedule,
+                             uint64_t *offsets_dev, int32_t *rows_dev, uint64_t rows_capacity,
+                             uint64_t *rows_needed, cudaStream_t s) {
+    if (!offsets_dev || (!rows_dev && rows_capacity > 0))
+        return set_error(FZ_EINVAL, "memo buffers: null pointer");
+    if (top == 0) {
+        int rc = validate_gens(tail, k);
+        if (rc != FZ_OK) return rc;
+        if (rows_needed) *rows_needed = 0;
+        FZ_CUDA_TRY(cudaMemsetAsync(offsets_dev, 0, 8, s));
+        FZ_CUDA_TRY(cudaStreamSynchronize(s));
+        return FZ_OK;
+    }
+    int32_t *R = rows_dev;
+    return build_memo_to(tail, k, top, offsets_dev, &R, rows_capacity, rows_needed, nullptr, s,
+                         schedule);
+}
+
 int fz_build_memo_into(const int32_t *tail, int k, int32_t top, uint64_t *offsets_dev,
                        int32_t *rows_dev, uint64_t rows_capacity, uint64_t *rows_needed,
                        void *stream) {
-    return fz_build_memo_schedule(tail, k, top, FZ_MEMO_BATCHED, offsets_dev, rows_dev,
-                                  rows_capacity, rows_needed, stream);
+    return build_memo_caller(tail, k, top, MEMO_LEVELS, offsets_dev, rows_dev, rows_capacity,
+                             rows_needed, as_stream(stream));
 }
 
 int fz_build_memo_schedule(const int32_t *tail, int k, int32_t top, int schedule,
@@ -931,19 +1012,8 @@ int fz_build_memo_schedule(const int32_t *tail, int k, int32_t top, int schedule
     if (schedule != FZ_MEMO_BATCHED && schedule != FZ_MEMO_PER_BATCH &&
         schedule != FZ_MEMO_PER_COPY)
         return set_error(FZ_EINVAL, "unknown memo schedule");
-    if (!offsets_dev || (!rows_dev && rows_capacity > 0))
-        return set_error(FZ_EINVAL, "memo buffers: null pointer");
-    if (top == 0) {
-        int rc = validate_gens(tail, k);
-        if (rc != FZ_OK) return rc;
-        if (rows_needed) *rows_needed = 0;
-        FZ_CUDA_TRY(cudaMemsetAsync(offsets_dev, 0, 8, as_stream(stream)));
-        FZ_CUDA_TRY(cudaStreamSynchronize(as_stream(stream)));
-        return FZ_OK;
-    }
-    int32_t *R = rows_dev;
-    return build_memo_to(tail, k, top, offsets_dev, &R, rows_capacity, rows_needed, nullptr,
-                         as_stream(stream), schedule);
+    return build_memo_caller(tail, k, top, schedule, offsets_dev, rows_dev, rows_capacity,
+                             rows_needed, as_stream(stream));
 }
 
 int fz_build_memo(const int32_t *tail, int k, int32_t top, fz_memo_t *memo, void *stream) {
@@ -1159,7 +1229,7 @@ int fz_plan_info(fz_plan_t p, fz_plan_info_t *info) {
     info->k = p->K;
     info->top = p->top;
     info->memo_rows = p->memo_rows;
-    info->device_bytes = p->base.bytes + p->memo.bytes + p->runs.bytes;
+    info->device_bytes = p->base.bytes + p->memo.bytes + p->runs.bytes + p->lvbuf.bytes;
     info->slice_rows = (int32_t)p->slice_rows;
     info->run_order = p->run_memo ? 1 : 0;
     return FZ_OK;

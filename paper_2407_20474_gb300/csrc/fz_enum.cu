@@ -33,7 +33,7 @@
 
 #include <cstdlib>
 
-#include "fz_internal.cuh"
+#include "fz_walk.cuh"
 
 namespace fz {
 
@@ -41,24 +41,6 @@ constexpr int ENUM_WARPS = 8;
 constexpr int ENUM_THREADS = ENUM_WARPS * 32;
 constexpr int RING_BYTES_PER_WARP = 6 * 1024;  // two halves; 4 CTAs of 8 warps per SM
 constexpr uint32_t CAP32 = 0xffffffffu;
-
-// Division and remainder of a 32-bit value by a fixed divisor via one
-// precomputed 64-bit multiplier (Lemire, Kaser and Kurz, "Faster remainder by
-// direct computation", 2019): M = floor((2^64 - 1) / g) + 1, a / g =
-// hi64(M * a), a % g = hi64(lo64(M * a) * g), exact for all a, g < 2^32, g > 1.
-struct FastDiv {
-    uint64_t M;
-    uint32_t g;
-};
-__host__ __device__ inline FastDiv make_fastdiv(uint32_t g) {
-    FastDiv f;
-    f.g = g;
-    f.M = g > 1 ? ~0ull / g + 1 : 0ull;
-    return f;
-}
-__device__ __forceinline__ uint32_t fd_div(uint32_t a, FastDiv f) {
-    return f.g > 1 ? (uint32_t)__umul64hi(f.M, a) : a;
-}
 
 struct EnumParams {
     const uint64_t *C;     // count table rows 0..d, stride cs
@@ -101,10 +83,6 @@ struct EnumParams {
     int pair_memo;
     FastDiv fd_e, fd_h1, fd_g2;  // division by e, h1 and g_{d-2}
 };
-
-__device__ __forceinline__ uint32_t fd_mod(uint32_t a, FastDiv f) {
-    return a - fd_div(a, f) * f.g;
-}
 
 // First a_{d-2} of pair-memo leaf p (meaningful when the leaf is not empty):
 // 32-bit divisions by precomputed multipliers; the product (p/e mod h1) inv
@@ -419,34 +397,7 @@ __device__ __forceinline__ int item_rows(const EnumParams &P, uint64_t s, uint64
 __device__ __forceinline__ void flush_rows(const EnumParams &P, const int32_t *src,
                                            uint64_t out_row, uint32_t nrows, int d, int lane,
                                            uint64_t pol) {
-    int32_t *gdst = P.out + out_row * (uint64_t)d;
-    const uint32_t words = nrows * (uint32_t)d;
-    if (P.aligned) {
-        const uint32_t bytes = words * 4u;
-        const uint32_t bulk = bytes & ~15u;
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0 && bulk) {
-            bulk_store(gdst, src, bulk, pol);
-            bulk_commit();
-        }
-        const uint32_t rem_words = (bytes - bulk) >> 2;
-        if ((uint32_t)lane < rem_words) gdst[(bulk >> 2) + lane] = src[(bulk >> 2) + lane];
-    } else {
-        // plain stores (unaligned output, or host memory over the host link):
-        // 16-byte vectors when both sides allow it
-        __syncwarp();
-        uint32_t w0 = 0;
-        if ((((uintptr_t)gdst | (uintptr_t)src) & 15u) == 0) {
-            const uint32_t nv = words >> 2;
-            const int4 *s4 = reinterpret_cast<const int4 *>(src);
-            int4 *g4 = reinterpret_cast<int4 *>(gdst);
-            for (uint32_t v = lane; v < nv; v += 32) g4[v] = s4[v];
-            w0 = nv << 2;
-        }
-        for (uint32_t w = w0 + lane; w < words; w += 32) gdst[w] = src[w];
-        __syncwarp();
-    }
+    flush_words(P.out + out_row * (uint64_t)d, P.aligned, src, nrows * (uint32_t)d, lane, pol);
 }
 
 // 4-byte global -> shared copy that does not hold a register (cp.async).
@@ -1354,6 +1305,34 @@ __global__ void __launch_bounds__(ENUM_THREADS)
     const uint64_t nw = (uint64_t)gridDim.x * ENUM_WARPS;
     for (uint64_t i = (uint64_t)blockIdx.x * ENUM_WARPS + wid; i < m; i += nw) {
         const uint64_t R = ranks[i];
+        if (P.run_memo) {
+            // the leading coordinates by search, the rest is one table row
+            const int lamf = D - P.K - 1;
+            int rem = P.n, mine = 0;
+            uint64_t left = R;
+            bool good = R < __ldg(P.C + P.n);
+            for (int c = 0; good && c < lamf; ++c) {
+                int v;
+                uint64_t before;
+                find_child(P, c, rem, left, lane, v, before);
+                if (lane == c) mine = v;
+                left -= before;
+                rem -= v * P.g[c];
+            }
+            const int gl = P.g[lamf], vmax = rem / gl;
+            const uint64_t row = good ? __ldg(P.cls_beg + (rem - vmax * gl)) + left : 0ull;
+            good = good && row < P.memo_rows;
+            if (!good && lane == 0) atomicExch(P.status, (int)DEV_INTERNAL);
+            if (lane < D) {
+                if (good && lane >= lamf) {
+                    const int32_t *m = reinterpret_cast<const int32_t *>(P.run_memo) +
+                                       (size_t)row * run_stride(P.K + 1);
+                    mine = lane == lamf ? vmax - __ldg(m) : __ldg(m + (lane - lamf));
+                }
+                P.out[i * D + lane] = good ? mine : -1;
+            }
+            continue;
+        }
         RunState st;
         bool ok;
         const uint64_t off = unrank_to_leaf(P, wp, R, lane, st, &ok);
@@ -1599,8 +1578,9 @@ static EnumParams make_params(const EnumLaunch &L) {
 int launch_enumerate(const EnumLaunch &L, uint64_t rank_begin, uint64_t nrows, int32_t *out,
                      uint64_t slice_rows, cudaStream_t s) {
     if (nrows == 0) return FZ_OK;
-    if (!out || !L.C || !L.status || !L.slice_counter || (L.K >= 1 && L.top > 0 && !L.O) ||
-        (L.K >= 1 && L.top > 0 && L.memo_rows > 0 && !L.memo))
+    if (!out || !L.C || !L.status || !L.slice_counter ||
+        (L.K >= 1 && L.top > 0 && !L.run_memo &&
+         (!L.O || (L.memo_rows > 0 && !L.memo))))
         return set_error(FZ_EINTERNAL, "enumerate: missing device buffer");
     EnumParams P = make_params(L);
     P.out = out;
@@ -1640,7 +1620,7 @@ int launch_enumerate(const EnumLaunch &L, uint64_t rank_begin, uint64_t nrows, i
 int launch_unrank(const EnumLaunch &L, const uint64_t *ranks, uint64_t m, int32_t *out,
                   cudaStream_t s) {
     if (m == 0) return FZ_OK;
-    if (!out || !ranks || !L.C || !L.status || (L.K >= 1 && L.top > 0 && !L.O))
+    if (!out || !ranks || !L.C || !L.status || (L.K >= 1 && L.top > 0 && !L.O && !L.run_memo))
         return set_error(FZ_EINTERNAL, "unrank: missing device buffer");
     EnumParams P = make_params(L);
     P.out = out;

@@ -114,6 +114,12 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+__device__ __forceinline__ uint64_t policy_evict_normal() {
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+    return pol;
+}
+
 __device__ __forceinline__ uint64_t policy_evict_first() {
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
@@ -332,6 +338,12 @@ int launch_memo_closed(const int32_t *tail, int k, int32_t top, const uint64_t *
 // schedule: FZ_MEMO_BATCHED (one launch), FZ_MEMO_PER_BATCH or FZ_MEMO_PER_COPY.
 int launch_memo_build(const int32_t *tail, int k, int32_t top, uint64_t rows,
                       const MemoBuffers &mb, cudaStream_t s, int schedule = FZ_MEMO_BATCHED);
+// FZ_MEMO_FILL names a fill of the dynamic pass (tuning and testing): memos
+// in element order of depth >= 3 are then built by it.
+bool memo_fill_forced();
+// Build memos by the run-order levels (fz_runs.cu) where they apply; the
+// public schedules name the paper's dynamic pass.
+constexpr int MEMO_LEVELS = -1;
 // Many small memos, one CTA each (fz_memo.cu).
 struct MemoJob {
     const uint64_t *Ct;  // tail count table rows 0..k, stride cs (row 0: |Z(r, tail)|)
@@ -344,16 +356,6 @@ struct MemoJob {
 };
 int launch_memo_sizes(const MemoJob *jobs, int njobs, uint64_t *rows_out, cudaStream_t s);
 
-// The memo of a full plan (tail = g_{lam+1}..g_{d-1}, every element 0..n) in
-// run order: the rows of the elements p = c, c + g_lam, c + 2 g_lam, ... of
-// each residue class c mod g_lam, classes in increasing order, each row as
-// int4 (p div g_lam, its k <= 3 memo words, zero padding).  For a prefix
-// with remainder r at level lam, the rows of its whole subtree over a_lam are
-// then the contiguous range [cls_beg[r mod g_lam], + C[lam][r]), and a_lam =
-// r div g_lam - (first word).  cls_beg: G = min(g_lam, n + 1) class starts.
-int launch_run_memo(const uint64_t *C, int64_t cs, int lam, int32_t n, int32_t g_lam,
-                    const uint64_t *O, const int32_t *rows, int k, uint64_t memo_rows,
-                    uint64_t *cls_beg, int4 *run_memo, int *status, cudaStream_t s);
 // The memos of a batch, one per job (jobs sorted longest first): the first
 // ncoop jobs each by a thread-block cluster, the rest one per CTA (claim: a
 // device counter the launch zeroes).  memo_coop_count picks ncoop (0: the
@@ -362,7 +364,7 @@ int memo_coop_count(const MemoJob *sorted, int njobs);
 int launch_memo_cta_build(const MemoJob *jobs, int njobs, int ncoop, unsigned *claim,
                           int *status, cudaStream_t s);
 
-// One run-order memo of a batch (the layout of launch_run_memo) for the
+// One run-order memo of a batch (the run-order layout of fz_runs.cu) for the
 // elements 0..n: its rows come from an element-order memo of depth k <= 3
 // (O, rows), or, with O null, from the closed form of the tail: k = 1, the
 // one row p / ta when ta divides p (ta = g_{d-1}); k = 2, the pair (t0, t1)
@@ -429,7 +431,7 @@ struct EnumLaunch {
     // at most this many CTAs of the enumeration kernel per SM (0 = as many as
     // fit), leaving room for other kernels to run beside it
     int ctas_per_sm = 0;
-    // full memo of depth K <= 3 in run order (see launch_run_memo), or null
+    // full memo of depth K <= 3 in run order (fz_runs.cu), or null
     const int4 *run_memo = nullptr;
     const uint64_t *cls_beg = nullptr;
     // K == 2, full: the memo is the closed form of Z(p, (g_{d-2}, g_{d-1}))

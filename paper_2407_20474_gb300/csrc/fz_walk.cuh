@@ -1,0 +1,476 @@
+// fz_walk.cuh -- device pieces shared by the enumeration (fz_enum.cu), the
+// run-order tables and the memo build (fz_runs.cu): invariant division, the
+// staged row writer and the flat leaf walk.
+#pragma once
+
+#include "fz_internal.cuh"
+
+namespace fz {
+
+// Division and remainder of a 32-bit value by a fixed divisor via one
+// precomputed 64-bit multiplier (Lemire, Kaser and Kurz, "Faster remainder by
+// direct computation", 2019): M = floor((2^64 - 1) / g) + 1, a / g =
+// hi64(M * a), a % g = hi64(lo64(M * a) * g), exact for all a, g < 2^32, g > 1.
+struct FastDiv {
+    uint64_t M;
+    uint32_t g;
+};
+__host__ __device__ inline FastDiv make_fastdiv(uint32_t g) {
+    FastDiv f;
+    f.g = g;
+    f.M = g > 1 ? ~0ull / g + 1 : 0ull;
+    return f;
+}
+__device__ __forceinline__ uint32_t fd_div(uint32_t a, FastDiv f) {
+    return f.g > 1 ? (uint32_t)__umul64hi(f.M, a) : a;
+}
+__device__ __forceinline__ uint32_t fd_mod(uint32_t a, FastDiv f) {
+    return a - fd_div(a, f) * f.g;
+}
+
+// The pair (g, h) of the last two generators as a closed form: with e =
+// gcd(g, h), h1 = h / e, g1 = g / e, inv = g1^-1 mod h1, row o of
+// Z(p, (g, h)) is (a_top - o h1, b_0 + o g1), a_top the largest valid first
+// coordinate and b_0 = (p - a_top g) / h.
+struct PairForm {
+    FastDiv fe, fh1, fg, fh;
+    uint32_t inv, h1, g1, g;
+};
+
+__host__ inline PairForm make_pair_form(int32_t g, int32_t h) {
+    int64_t e, h1, g1, inv;
+    pair_params(g, h, &e, &h1, &g1, &inv);
+    PairForm F;
+    F.fe = make_fastdiv((uint32_t)e);
+    F.fh1 = make_fastdiv((uint32_t)h1);
+    F.fg = make_fastdiv((uint32_t)g);
+    F.fh = make_fastdiv((uint32_t)h);
+    F.inv = (uint32_t)inv;
+    F.h1 = (uint32_t)h1;
+    F.g1 = (uint32_t)g1;
+    F.g = (uint32_t)g;
+    return F;
+}
+
+// a_top of element p (meaningful when Z(p, (g, h)) is not empty): the
+// product (p / e mod h1) inv fits 32 bits when h1 < 2^16, else it takes a
+// 64-bit remainder.
+__device__ __forceinline__ uint32_t pair_form_top(const PairForm &F, uint32_t p) {
+    const uint32_t xr = fd_mod(fd_div(p, F.fe), F.fh1);
+    const uint32_t astar = F.h1 < 65536u ? fd_mod(xr * F.inv, F.fh1)
+                                         : (uint32_t)((uint64_t)xr * F.inv % F.h1);
+    const uint32_t q = fd_div(p, F.fg);
+    return q >= astar ? q - fd_mod(q - astar, F.fh1) : 0u;
+}
+
+// ---------------------------------------------------------------------------
+// Staged rows.  A warp assembles rows in a shared-memory ring of two halves
+// of B rows and sends every full half to global memory with one bulk (TMA)
+// store, or with plain stores when the output is not 16-byte aligned (or is
+// host memory reached over the host link).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void flush_words(int32_t *gdst, bool aligned, const int32_t *src,
+                                            uint32_t words, int lane, uint64_t pol) {
+    if (aligned) {
+        const uint32_t bytes = words * 4u;
+        const uint32_t bulk = bytes & ~15u;
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0 && bulk) {
+            bulk_store(gdst, src, bulk, pol);
+            bulk_commit();
+        }
+        const uint32_t rem_words = (bytes - bulk) >> 2;
+        if ((uint32_t)lane < rem_words) gdst[(bulk >> 2) + lane] = src[(bulk >> 2) + lane];
+    } else {
+        // plain stores (unaligned output, or host memory over the host link):
+        // 16-byte vectors when both sides allow it
+        __syncwarp();
+        uint32_t w0 = 0;
+        if ((((uintptr_t)gdst | (uintptr_t)src) & 15u) == 0) {
+            const uint32_t nv = words >> 2;
+            const int4 *s4 = reinterpret_cast<const int4 *>(src);
+            int4 *g4 = reinterpret_cast<int4 *>(gdst);
+            for (uint32_t v = lane; v < nv; v += 32) g4[v] = s4[v];
+            w0 = nv << 2;
+        }
+        for (uint32_t w = w0 + lane; w < words; w += 32) gdst[w] = src[w];
+        __syncwarp();
+    }
+}
+
+// One row of DS words to shared memory, in the widest stores its alignment
+// allows (row starts are multiples of DS words from a 128-byte boundary).
+// DS = 8: lanes 4-7 of each eight store their upper half first, so the eight
+// 16-byte stores of a phase fall on different banks.
+template <int DS>
+__device__ __forceinline__ void store_row(int32_t *dst, const int (&w)[DS], int lane) {
+    if constexpr (DS == 8) {
+        const bool hi = (lane & 4) != 0;
+        const int4 lo4 = make_int4(w[0], w[1], w[2], w[3]), hi4 = make_int4(w[4], w[5], w[6], w[7]);
+        int4 *d4 = reinterpret_cast<int4 *>(dst);
+        d4[hi ? 1 : 0] = hi ? hi4 : lo4;
+        d4[hi ? 0 : 1] = hi ? lo4 : hi4;
+    } else if constexpr (DS % 4 == 0) {
+#pragma unroll
+        for (int c = 0; c < DS; c += 4)
+            *reinterpret_cast<int4 *>(dst + c) = make_int4(w[c], w[c + 1], w[c + 2], w[c + 3]);
+    } else if constexpr (DS % 2 == 0) {
+#pragma unroll
+        for (int c = 0; c < DS; c += 2)
+            *reinterpret_cast<int2 *>(dst + c) = make_int2(w[c], w[c + 1]);
+    } else {
+#pragma unroll
+        for (int c = 0; c < DS; ++c) dst[c] = w[c];
+    }
+}
+
+// Words between the rows of a run-order table whose rows hold W words (the
+// quotient and W - 1 coordinates): whole 16-byte vectors.
+__host__ __device__ constexpr int run_stride(int W) { return (W + 3) & ~3; }
+
+// Where the rows of a leaf (an element p) come from.
+//   SRC_RUN:  the run-order table of (gen; tail): the rows of Z(p, (gen,
+//             tail)) are the contiguous range [cls[p mod gen], + count) of
+//             `rows`, each row (quotient, tail words), and the coordinate of
+//             gen is p div gen - quotient.
+//   SRC_PAIR: the closed form of the last two generators; nothing is read.
+enum : int { SRC_RUN = 0, SRC_PAIR = 1 };
+struct LeafSource {
+    const int32_t *rows;
+    const uint64_t *cls;
+    uint64_t nrows;
+    FastDiv fg;
+    PairForm pair;
+};
+
+// One table (or memo in element order) to be written by run_build_kernel
+// (fz_runs.cu).  Jobs of a launch own consecutive block ranges from blk0 on.
+struct RunBuild {
+    LeafSource src;       // depth 1: src.fg holds the tail's one generator
+    const uint64_t *F;    // row ends: element p of class c ends at cls[c] + F[p]
+    const uint64_t *cls;  // class starts of this table (G + 1), null in element order
+    int32_t *dst;
+    uint64_t rows;
+    int32_t n;            // elements 0..n
+    int32_t g, G;         // class generator, G = min(g, n + 1)
+    uint32_t qn, rr;      // n div g, n mod g
+    uint32_t per_warp;    // rows a warp writes
+    uint32_t blk0;
+    FastDiv fq1, fq;      // division by qn + 1 and qn
+};
+
+// The levels of one chain (fz_runs.cu): tables[, the memo in element order].
+struct RunLevels {
+    RunBuild *jobs_dev = nullptr;
+    int n = 0, tables = 0;
+    bool csr = false;
+    int K[FZ_MAX_D] = {};
+    uint32_t blocks[FZ_MAX_D] = {};
+    int32_t *rows = nullptr;       // the last table: rows and class starts
+    uint64_t *cls = nullptr;
+};
+
+// Deepest memo the levels build (rows of a table: quotient and coordinates).
+constexpr int RUN_MAX_K = 7;   // run-order tables
+constexpr int CSR_MAX_K = 8;   // memos in element order (from depth 3 on)
+
+// sums[j] (device) = sum over r < top of row j of C, exact when below 2^32.
+int launch_row_sums(const uint64_t *C, int64_t cs, int rows, int64_t top, uint64_t *sums,
+                    cudaStream_t s);
+// Chain over the generators t_0..t_{k-1} and elements 0..n: the run-order
+// table keyed by t_0 of the rows of Z(p, (t_1..)) (csr false, 2 <= k <= 8), or the
+// memo Z(p, (t_0..)) in element order (csr true, 3 <= k <= 8; O: its
+// offsets, csr_rows: its rows).  sums[j] = rows of all Z(p, (t_j..)), p <= n,
+// below 2^32 from j = 1 on; Ct: count table rows 0..k of t.  `mem` has
+// run_levels_bytes bytes and holds tables, scratch and jobs.
+size_t run_levels_bytes(const int32_t *t, int k, int32_t n, const uint64_t *sums, bool csr);
+int run_levels_init(const int32_t *t, int k, int32_t n, const uint64_t *sums, bool csr,
+                    const uint64_t *Ct, int64_t cs, const uint64_t *O, int32_t *csr_rows,
+                    void *mem, RunLevels *L, cudaStream_t s);
+int launch_run_levels(const RunLevels &L, int *status, cudaStream_t s);
+// The pieces, for many chains at once (batches).
+void fill_run_build(const int32_t *t, int k, int32_t n, int j, bool csr, int sms, RunBuild *out);
+uint32_t run_build_blocks(const RunBuild &R, int K);
+int launch_run_classes(const RunBuild *jobs_dev, int njobs, int *status, cudaStream_t s);
+int launch_run_build(const RunBuild *jobs_dev, int njobs, int K, bool csr, uint32_t blocks,
+                     int *status, cudaStream_t s);
+
+// Descriptors of a warp's 32 leaves, as 16-byte vectors [DV][32].
+template <int NP, int SRC>
+__host__ __device__ constexpr int leaf_vecs() {
+    return ((SRC == SRC_RUN ? 2 : 3) + NP + 3) / 4;
+}
+template <int NP, int SRC>
+__host__ __device__ constexpr int leaf_bytes() {
+    return leaf_vecs<NP, SRC>() * 32 * 16;
+}
+// Rows per ring half when a warp has `bytes` of shared memory for both its
+// leaf descriptors and its ring of DS-word rows.
+template <int NP, int SRC, int DS>
+__host__ __device__ constexpr uint32_t flat_half_rows(int bytes) {
+    const int b = (bytes - ((SRC == SRC_RUN ? 2 : 3) + NP + 3) / 4 * 512) / (8 * DS) / 32 * 32;
+    return b < 32 ? 32u : (uint32_t)b;
+}
+
+// ---------------------------------------------------------------------------
+// The flat leaf walk.  The output of an enumeration, of a run-order table and
+// of a memo in element order are all the concatenation, over a sequence of
+// leaves (elements p with a few prefix words), of rows copied from a
+// LeafSource.  A warp writes rows [row0, row0 + left) of such an output:
+// lane l holds leaf f + l of the sequence and reads its cumulative row end
+// from a count row, so 32 leaves cost one round of loads whatever they hold;
+// their descriptors go to shared memory (empty leaves dropped), and rounds of
+// 32 RPL output rows then find their leaves by counting the leaf ends that
+// lie inside the round (one ballot and one OR-reduction of end bits).  So a
+// leaf of a few rows costs no round of its own, and a long leaf's rounds are
+// plain copies.  The table rows of the next round are loaded before this
+// round's rows are stored.
+//
+// What bounds it: instruction issue.  A copy with one leaf a warp at a time
+// needs about 12 warp instructions a row where leaves hold a row or two.
+//
+// Walk: leaf(p, end, pre) gives lane's element, cumulative row end and
+// prefix words and returns false past the last leaf (a suffix of the
+// lanes); next() moves every lane 32 leaves on.  `base` is the row at which
+// leaf 0 starts (same origin as the ends) and `skip` its rows already behind.
+// Returns false, with the status recorded, if the tables disagree.
+// ---------------------------------------------------------------------------
+template <int NP, int W, int DS, int SRC, class Walk>
+__device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip,
+                                          const LeafSource &S, int32_t *out, bool aligned,
+                                          uint64_t row0, uint32_t left, int4 *desc,
+                                          int32_t *ring, uint32_t B, int *status, uint64_t pol,
+                                          int lane) {
+    static_assert(NP + W <= DS, "row words");
+    constexpr int RPL = SRC == SRC_PAIR || W <= 4 ? 2 : 1;  // rows a lane per round
+    constexpr int DV = leaf_vecs<NP, SRC>();
+    constexpr int SS = SRC == SRC_RUN ? run_stride(W) : 4;
+    constexpr uint32_t RR = 32u * RPL;
+    const uint32_t le = 0xffffffffu >> (31 - lane);
+    uint32_t hpos = 0, half = 0, nfull = 0;
+    bool ok = true;
+
+    struct Frag {
+        int4 v[RPL][SRC == SRC_RUN ? SS / 4 : 1];
+        int l[RPL];
+    };
+
+    while (left > 0) {
+        // ---- 32 leaves
+        uint32_t p = 0;
+        uint64_t E = 0;
+        int pre[NP > 0 ? NP : 1];
+        const bool live = wk.leaf(p, E, pre);
+        const int nlive = __popc(__ballot_sync(FULL, live));
+        if (nlive == 0) {  // past the last leaf with rows still owed
+            if (lane == 0) atomicExch(status, (int)DEV_INTERNAL);
+            ok = false;
+            break;
+        }
+        const uint64_t Elast = shfl_u64(E, nlive - 1);
+        if (!live) E = Elast;
+        uint64_t Eprev = __shfl_up_sync(FULL, E, 1);
+        if (lane == 0) Eprev = base;
+        const uint64_t size = E - Eprev;
+        const uint32_t e = E - base < 0xffffffffull ? (uint32_t)(E - base) : 0xffffffffu;
+        const uint32_t s = Eprev - base < 0xffffffffull ? (uint32_t)(Eprev - base) : 0xffffffffu;
+        const uint32_t e_all = __shfl_sync(FULL, e, 31);
+        // the end of this batch's rows (skip lies in leaf 0, so only an
+        // inconsistent table has e_all below it)
+        const uint32_t q_end = e_all <= skip ? skip : e_all - skip < left ? e_all : skip + left;
+        // leaves with rows in the window, in order
+        const bool used = live && e > s && e > skip && s < q_end;
+        const uint32_t rank = __popc(__ballot_sync(FULL, used) & (le >> 1));
+        bool bad = E < Eprev || e_all < skip;
+        __syncwarp();  // the previous batch's descriptors have been read
+        if (used) {
+            int d[DV * 4];
+#pragma unroll
+            for (int c = 0; c < DV * 4; ++c) d[c] = 0;
+            constexpr int H = SRC == SRC_RUN ? 2 : 3;
+            if constexpr (SRC == SRC_RUN) {
+                const uint32_t qt = fd_div(p, S.fg);
+                const uint64_t src = __ldg(S.cls + (p - qt * S.fg.g));
+                bad = bad || src + size > S.nrows;  // bounds guard: the leaf lies in the table
+                d[0] = (int)((uint32_t)src - s);
+                d[1] = (int)qt;
+            } else {
+                const uint32_t at = pair_form_top(S.pair, p);
+                d[0] = (int)s;
+                d[1] = (int)at;
+                d[2] = (int)fd_div(p - at * S.pair.g, S.pair.fh);
+            }
+#pragma unroll
+            for (int c = 0; c < NP; ++c) d[H + c] = pre[c];
+#pragma unroll
+            for (int v = 0; v < DV; ++v)
+                desc[v * 32 + rank] = make_int4(d[4 * v], d[4 * v + 1], d[4 * v + 2], d[4 * v + 3]);
+        }
+        if (__any_sync(FULL, bad)) {
+            if (lane == 0) atomicExch(status, (int)DEV_INTERNAL);
+            ok = false;
+            break;
+        }
+        __syncwarp();
+
+        // ---- rounds
+        auto fetch = [&](Frag &F, uint32_t q0, uint32_t cnt) {
+#pragma unroll
+            for (int u = 0; u < RPL; ++u) {
+                const uint32_t qh = q0 + 32u * u;
+                const uint32_t done = __popc(__ballot_sync(FULL, used && e <= qh));
+                const uint32_t b = e - qh;
+                const unsigned bits =
+                    __reduce_or_sync(FULL, used && b - 1u < 31u ? 1u << b : 0u);
+                F.l[u] = (int)(done + __popc(bits & le));
+                if constexpr (SRC == SRC_RUN) {
+                    if ((uint32_t)lane + 32u * u < cnt) {
+                        const uint32_t row =
+                            reinterpret_cast<const uint32_t *>(desc + F.l[u])[0] + qh + lane;
+                        const int4 *src =
+                            reinterpret_cast<const int4 *>(S.rows) + (size_t)row * (SS / 4);
+#pragma unroll
+                        for (int v = 0; v < SS / 4; ++v) F.v[u][v] = __ldg(src + v);
+                    }
+                }
+            }
+        };
+        auto emit = [&](const Frag &F, uint32_t q0, uint32_t cnt) {
+            if (hpos == 0 && nfull >= 2) {
+                // re-entering a half: the bulk store issued from it two
+                // flushes ago must have finished reading it
+                if (lane == 0) bulk_wait_read<1>();
+                __syncwarp();
+            }
+            int32_t *dst = ring + (size_t)(half * B + hpos + lane) * DS;
+#pragma unroll
+            for (int u = 0; u < RPL; ++u) {
+                if ((uint32_t)lane + 32u * u < cnt) {
+                    int d[DV * 4];
+#pragma unroll
+                    for (int v = 0; v < DV; ++v) {
+                        const int4 x = desc[v * 32 + F.l[u]];
+                        d[4 * v] = x.x;
+                        d[4 * v + 1] = x.y;
+                        d[4 * v + 2] = x.z;
+                        d[4 * v + 3] = x.w;
+                    }
+                    constexpr int H = SRC == SRC_RUN ? 2 : 3;
+                    int w[DS];
+#pragma unroll
+                    for (int c = 0; c < DS; ++c) w[c] = 0;
+#pragma unroll
+                    for (int c = 0; c < NP; ++c) w[c] = d[H + c];
+                    if constexpr (SRC == SRC_RUN) {
+                        int x[SS];
+#pragma unroll
+                        for (int v = 0; v < SS / 4; ++v) {
+                            x[4 * v] = F.v[u][v].x;
+                            x[4 * v + 1] = F.v[u][v].y;
+                            x[4 * v + 2] = F.v[u][v].z;
+                            x[4 * v + 3] = F.v[u][v].w;
+                        }
+                        w[NP] = d[1] - x[0];
+#pragma unroll
+                        for (int c = 1; c < W; ++c) w[NP + c] = x[c];
+                    } else {
+                        const uint32_t o = q0 + 32u * u + lane - (uint32_t)d[0];
+                        w[NP] = d[1] - (int)(o * S.pair.h1);
+                        w[NP + 1] = d[2] + (int)(o * S.pair.g1);
+                    }
+                    store_row<DS>(dst + u * 32 * DS, w, lane);
+                }
+            }
+            hpos += cnt;
+            if (hpos == B) {
+                flush_words(out + (row0 + (uint64_t)nfull * B) * DS, aligned,
+                            ring + (size_t)half * B * DS, B * DS, lane, pol);
+                ++nfull;
+                half ^= 1u;
+                hpos = 0;
+            }
+        };
+        // rows of the round at q0 with `at` rows already in the ring half
+        // (rounds never cross a half)
+        auto rows_at = [&](uint32_t q0, uint32_t at) {
+            uint32_t c = q_end - q0;
+            if (c > RR) c = RR;
+            return c < B - at ? c : B - at;
+        };
+        uint32_t q0 = skip;
+        if (q0 < q_end) {
+            if constexpr (SRC == SRC_RUN) {
+                Frag x, y;
+                uint32_t c0 = rows_at(q0, hpos);
+                fetch(x, q0, c0);
+                for (;;) {
+                    uint32_t c1 = 0;
+                    if (q0 + c0 < q_end) {
+                        c1 = rows_at(q0 + c0, hpos + c0 == B ? 0u : hpos + c0);
+                        fetch(y, q0 + c0, c1);
+                    }
+                    emit(x, q0, c0);
+                    q0 += c0;
+                    if (c1 == 0) break;
+                    c0 = 0;
+                    if (q0 + c1 < q_end) {
+                        c0 = rows_at(q0 + c1, hpos + c1 == B ? 0u : hpos + c1);
+                        fetch(x, q0 + c1, c0);
+                    }
+                    emit(y, q0, c1);
+                    q0 += c1;
+                    if (c0 == 0) break;
+                }
+            } else {
+                Frag x;
+                while (q0 < q_end) {
+                    const uint32_t c = rows_at(q0, hpos);
+                    fetch(x, q0, c);
+                    emit(x, q0, c);
+                    q0 += c;
+                }
+            }
+            left -= q_end - skip;
+        }
+        skip = 0;
+        base = Elast;
+        if (left > 0) wk.next();
+    }
+    if (hpos > 0)
+        flush_words(out + (row0 + (uint64_t)nfull * B) * DS, aligned,
+                    ring + (size_t)half * B * DS, hpos * DS, lane, pol);
+    if (lane == 0) bulk_wait_read_all();
+    __syncwarp();
+    return ok;
+}
+
+// Largest u in [0, n) with f(u) <= R (f non-decreasing, f(0) <= R), searched
+// 32 probes at a time by a warp; *val = f(u).
+template <class Fn>
+__device__ __forceinline__ uint32_t warp_last_le(uint32_t n, uint64_t R, int lane, uint64_t *val,
+                                                 Fn f) {
+    uint32_t lo = 0, hi = n;  // f(lo) <= R; f(hi) > R or hi == n
+    uint64_t flo = f(0u);
+    while (hi - lo > 1) {
+        const uint32_t step = (hi - lo + 31) >> 5;
+        const uint64_t u = (uint64_t)lo + (uint64_t)(lane + 1) * step;
+        bool okp = false;
+        uint64_t fu = 0;
+        if (u < hi) {
+            fu = f((uint32_t)u);
+            okp = fu <= R;
+        }
+        const int cnt = __popc(__ballot_sync(FULL, okp));
+        const uint64_t fsel = shfl_u64(fu, cnt > 0 ? cnt - 1 : 0);
+        if (cnt > 0) {
+            flo = fsel;
+            lo += (uint32_t)cnt * step;
+        }
+        if (lo + step < hi) hi = lo + step;
+    }
+    *val = flo;
+    return lo;
+}
+
+}  // namespace fz

@@ -1,0 +1,72 @@
+"""Memos and run-order tables built by levels against the oracle, and plans
+that read them (enumeration and random access)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2407_20474_gb300 import workloads
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+CANARY = -7
+
+
+@pytest.fixture(scope="module")
+def fz():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2407_20474_gb300 as m
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    torch.cuda.set_device(0)
+    return m
+
+
+# depths 1..9 (9: past the levels), every order, repeats, common factors, a 1,
+# generators above the last element, one element, ring and warp-window
+# remainders
+TAILS = [((5,), 40), ((11, 14), 501), ((14, 11), 501), ((4, 9, 10), 300), ((10, 4, 9), 301), ((2, 2, 3), 130),
+         ((6, 10, 15), 400), ((5, 1, 4), 200), ((900, 3, 4, 5), 310), ((3, 900, 4, 5), 310), ((3, 5, 7, 8), 260),
+         ((7, 5, 6, 4, 9), 150), ((4, 6, 8, 10, 12, 14), 170), ((3, 4, 5, 6, 7, 8, 9), 75),
+         ((3, 4, 5, 6, 7, 8, 9, 10), 60), ((3, 4, 5, 6, 7, 8, 9, 10, 11), 45), ((4, 9, 10), 1), ((7, 3, 5, 2), 2),
+         ((33, 2, 3, 5), 700)]
+
+
+@pytest.mark.parametrize("tail,top", TAILS)
+@pytest.mark.parametrize("shift", [0, 1])
+def test_memo_by_levels(fz, tail, top, shift):
+    """shift: rows at an address that is 4-byte aligned only."""
+    ref_off, ref_rows = oracle.memo_csr(tail, top)
+    rows, k = int(ref_off[-1]), len(tail)
+    off = torch.zeros(top + 1, dtype=torch.int64, device="cuda")
+    buf = torch.full((shift + (rows + 4) * k,), CANARY, dtype=torch.int32, device="cuda")
+    assert fz.fz_build_memo_into(tail, top, off, buf[shift:], rows) == rows
+    torch.cuda.synchronize()
+    host = buf.cpu().numpy()
+    assert (host[:shift] == CANARY).all() and (host[shift + rows * k:] == CANARY).all()
+    assert np.array_equal(off.cpu().numpy().view(np.uint64), ref_off)
+    assert np.array_equal(host[shift:shift + rows * k].reshape(rows, k), ref_rows)
+
+
+@pytest.mark.parametrize("g,target", [((5, 8, 11, 14), 4000), ((14, 5, 11, 8, 9), 9000), ((2, 2, 3, 3), 5000),
+                                      ((9, 6, 12, 15, 21, 10), 20000), ((400, 7, 3, 5), 3000),
+                                      ((3, 5, 7, 9, 11, 13, 4), 30000), ((13, 37, 38, 40, 41, 42, 43, 44, 45), 20000)])
+def test_plans_on_levels(fz, g, target):
+    """Every memo depth: enumeration after two rebuilds, and the tuple of every
+    rank by random access."""
+    n = workloads.find_n(oracle.count_upto, g, target, 64)
+    ref = oracle.enumerate_desc(g, n)
+    total, d = ref.shape
+    ranks = torch.randperm(total, device="cuda")
+    for k in range(1, d):
+        with fz.Plan(g, n, k=k) as plan:
+            for _ in range(2):
+                plan.rebuild()
+            out = torch.full((total + 3, d), CANARY, dtype=torch.int32, device="cuda")
+            assert plan.enumerate(out[:total]) == total
+            pick = torch.full((total + 3, d), CANARY, dtype=torch.int32, device="cuda")
+            plan.unrank(ranks, pick[:total])
+            plan.sync()
+            assert np.array_equal(out[:total].cpu().numpy(), ref), k
+            assert np.array_equal(pick[:total].cpu().numpy(), ref[ranks.cpu().numpy()]), k
+            assert bool((out[total:] == CANARY).all()) and bool((pick[total:] == CANARY).all())

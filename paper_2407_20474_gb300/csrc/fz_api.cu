@@ -137,7 +137,7 @@ struct fz_plan_s {
     DevBuf runs;   // runs table for work-balanced slicing
     DevBuf lvbuf;  // run-order tables of the memo's levels
     RunLevels lv;
-    int4 *run_memo = nullptr;      // the memo in run order (full memo, k <= 3)
+    int4 *run_memo = nullptr;      // the memo in run order (full memo)
     uint64_t *cls_beg = nullptr;
     uint64_t *RT = nullptr;
     int lam_r = 0;
@@ -170,8 +170,8 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 }  // namespace
 
 // FZ_RUN_COST overrides W (tuning only).
-void balance_level(int d, int K, int top, int n, bool run_order, int *lam_r, uint64_t *W,
-                   int *clamp_row) {
+void balance_level(int d, int K, int top, int n, bool run_order, bool pair, int *lam_r,
+                   uint64_t *W, int *clamp_row) {
     static const long long forced = [] {
         const char *e = getenv("FZ_RUN_COST");
         return e ? atoll(e) : 0ll;
@@ -182,11 +182,11 @@ void balance_level(int d, int K, int top, int n, bool run_order, int *lam_r, uin
         // the run-order walk visits every prefix of the leading d - K - 1
         // coordinates (empty or not) and copies its run
         *lam_r = d - K - 1;
-        *W = 64;
+        *W = flat_serves(d, d - K - 1, SRC_RUN) ? FLAT_LEAF_COST : 64;
     } else if (memo && top > n) {
         // full memo: the leaves are the memo leaves, evaluated 32 at a time
         *lam_r = d - K;
-        *W = 16;
+        *W = pair && flat_serves(d, d - 2, SRC_PAIR) ? FLAT_LEAF_COST : 16;
     } else if (K == 1 || !walk_progression_enabled()) {
         // walk leaves evaluated candidate by candidate: count the candidates
         *lam_r = d - 1;
@@ -196,7 +196,7 @@ void balance_level(int d, int K, int top, int n, bool run_order, int *lam_r, uin
         // prefix plus a progression; a memo leaf (a prefix of length d - K
         // with remainder below top) is one unit whatever lies under it
         *lam_r = d - 2;
-        *W = 64;
+        *W = !memo && flat_serves(d, d - 2, SRC_PAIR) ? FLAT_LEAF_COST : 64;
         if (memo && K > 2) *clamp_row = d - K;
     }
     if (*lam_r < 0) *lam_r = 0;
@@ -254,11 +254,57 @@ int read_status(int *status_dev, cudaStream_t s) {
     return status_to_fz(h);
 }
 
-// Memo depth chosen automatically: the deepest k in 2..min(d-1, 4) whose full
-// memo stays small next to the output and needs a bounded number of
-// elementwise batches; k = 0 (plain walk) when none qualifies.  sums[j]: the
-// rows of all Z(r, (g_j..)), r <= n, exact below 2^32.
+// Prefixes (a_0..a_{lam-1}) of Z(n, g): the volume n'^lam / (lam! prod g), n' = n
+// plus half the generators.
+double prefix_volume(const fz_plan_s *p, int lam) {
+    double x = (double)p->n, v = 1.0;
+    for (int i = 0; i < lam; ++i) x += 0.5 * p->g[i];
+    for (int i = 0; i < lam; ++i) v *= x / (double)(i + 1) / (double)p->g[i];
+    return v < 1.0 ? 1.0 : v;
+}
+
+// Memo depth chosen automatically for the flat walk: the least estimated time
+// of walk and memo in ns.  A leaf costs about 3.5 warp instructions of 7e11 a
+// second (5 with the pair's closed form, which needs no memo: k = 0), a table
+// row 1.6 and its bytes, an element of a table as much as a leaf, and every
+// level a launch (3 us; an output of 1e4 rows takes k = 0 or 2, 1.4e7 rows of
+// width 9 take k = 5).  Tables stay within an eighth of the output (or 8 MB),
+// so their rows stay in L2.  k = 0 only up to width 6: the prefixes of d - 2
+// coordinates of wider tuples are mostly empty leaves.  -1 when neither
+// applies.  sums[j]: the rows of all Z(r, (g_j..)), r <= n, exact below 2^32.
+int choose_k_flat(const fz_plan_s *p, const uint64_t *sums) {
+    const int d = p->d;
+    const uint64_t out_bytes = p->count * (uint64_t)d * 4ull;
+    const uint64_t budget = std::max<uint64_t>(8ull << 20, out_bytes / 8);
+    int best = d <= 6 ? 0 : -1;
+    double best_ns = d <= 6 ? prefix_volume(p, d - 2) * 0.007 : 1e300;
+    double build = 3000.0;  // class starts
+    for (int k = 2; k <= d - 2 && k <= RUN_MAX_K; ++k) {
+        const uint64_t rows = sums[d - k];
+        const uint64_t bytes = rows * 4ull * run_stride(k + 1);
+        if (rows > MEMO_MAX_ROWS || bytes > budget) break;
+        build += 3000.0 + (double)rows * 0.0025 + (double)bytes * 0.0002 + (double)p->n * 0.005;
+        const int lam = d - 1 - k;
+        if (!flat_serves(d, lam, SRC_RUN)) continue;
+        const double ns = build + prefix_volume(p, lam) * 0.005;
+        if (ns < best_ns) {
+            best_ns = ns;
+            best = k;
+        }
+    }
+    return best;
+}
+
+// Memo depth chosen automatically: the flat walk's where it applies, else the
+// deepest k in 2..min(d-1, 4) whose full memo stays small next to the
+// output and needs a bounded number of elementwise batches; k = 0 (plain
+// walk) when none qualifies.
 int choose_k(const fz_plan_s *p, const uint64_t *sums) {
+    if (walk_progression_enabled() && run_memo_enabled() &&
+        flat_serves(p->d, p->d - 2, SRC_PAIR)) {
+        const int k = choose_k_flat(p, sums);
+        if (k >= 0) return k;
+    }
     const uint64_t out_bytes = p->count * (uint64_t)p->d * 4ull;
     const uint64_t budget = std::max<uint64_t>(8ull << 20, out_bytes / 8);
     for (int k = std::min(p->d - 1, 4); k >= 2; --k) {
@@ -308,14 +354,15 @@ int row_sums(const uint64_t *C, int64_t cs, int nrows, int64_t top, uint64_t *de
 }
 
 // Buffers of the memo of plan p (depth K, top and memo_rows set): in run
-// order for a full memo of depth <= 3 under a walked coordinate, else in
+// order for a full memo that an enumeration kernel reads so, else in
 // element order, by levels when their scratch fits, else with the gather map
 // of the dynamic pass.  sums[j]: the rows of all Z(r, (g_j..)), r < top.
 int plan_alloc_memo(fz_plan_s *p, const uint64_t *sums, cudaStream_t s) {
     const int d = p->d, k = p->K;
     const int64_t cs = (int64_t)p->n + 1;
     const int lam = d - k - 1;
-    if (p->top > p->n && k <= 3 && lam >= 0 && run_memo_enabled()) {
+    if (p->top > p->n && lam >= 0 && (k <= 3 || flat_serves(d, lam, SRC_RUN)) &&
+        run_memo_enabled()) {
         if (p->lvbuf.alloc(run_levels_bytes(p->g + lam, k + 1, p->n, sums + lam, false)) ==
             FZ_OK) {
             const int rc = run_levels_init(p->g + lam, k + 1, p->n, sums + lam, false,
@@ -438,7 +485,7 @@ int plan_create_impl(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, f
     // single block: d == 1 or k == d with a full memo)
     const bool single_block = d == 1 || (p->K == d && p->top > n);
     if (!single_block && p->count > 0) {
-        balance_level(d, p->K, p->top, n, p->run_memo != nullptr, &p->lam_r, &p->W,
+        balance_level(d, p->K, p->top, n, p->run_memo != nullptr, false, &p->lam_r, &p->W,
                       &p->clamp_row);
         rc = p->runs.alloc((size_t)(p->lam_r + 1) * cs * 8);
         if (rc != FZ_OK) return rc;

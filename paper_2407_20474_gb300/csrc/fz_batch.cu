@@ -18,7 +18,7 @@
 #include <mutex>
 #include <vector>
 
-#include "fz_internal.cuh"
+#include "fz_walk.cuh"
 
 namespace fz {
 namespace {
@@ -533,7 +533,7 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
         words += (size_t)(I.d + 1) * len;
         I.off_RT = (size_t)-1;
         if (I.d >= 2) {
-            balance_level(I.d, I.K, I.top, I.n, I.run, &I.lam_r, &I.W, &I.clamp_row);
+            balance_level(I.d, I.K, I.top, I.n, I.run, I.pair, &I.lam_r, &I.W, &I.clamp_row);
             I.off_RT = words;
             words += (size_t)(I.lam_r + 1) * len;
         } else {

@@ -33,372 +33,9 @@
 
 #include <cstdlib>
 
-#include "fz_walk.cuh"
+#include "fz_enum.cuh"
 
 namespace fz {
-
-constexpr int ENUM_WARPS = 8;
-constexpr int ENUM_THREADS = ENUM_WARPS * 32;
-constexpr int RING_BYTES_PER_WARP = 6 * 1024;  // two halves; 4 CTAs of 8 warps per SM
-constexpr uint32_t CAP32 = 0xffffffffu;
-
-struct EnumParams {
-    const uint64_t *C;     // count table rows 0..d, stride cs
-    int64_t cs;
-    const uint64_t *O;     // memo CSR offsets (top + 1), or null
-    const int32_t *memo;   // memo rows, K int32 each, or null
-    uint64_t memo_rows;    // rows in memo (bounds guard)
-    int32_t *out;          // row 0 = rank rank_begin
-    int *status;
-    unsigned long long *slice_counter;
-    uint64_t rank_begin;   // absolute rank of out row 0
-    uint64_t nrows;        // rows to write
-    uint64_t slice_rows;   // S (multiple of 4), used when RT is null
-    uint64_t nslices;
-    const uint64_t *RT;    // candidates table rows 0..lam_r (stride cs), or null
-    uint64_t W;            // cost of one unit of walk work (a prefix of length lam_r), in rows
-    uint64_t slice_cost;   // cost units per work item when RT is set
-    int lam_r;             // one past the leaf coordinate (RT[lam_r] = 1)
-    int n, d, K, top;
-    int lam_m;             // coordinate whose children are memo leaves (d-K-1), or -1
-    int lam_w;             // coordinate whose children are walk leaves (d-2)
-    int half_rows;         // B: rows per ring half (multiple of 32)
-    int aligned;           // out is 16-byte aligned
-    int ctas_per_sm;       // occupancy cap of the launch (0 = none)
-    int dense_min;         // memo batches with >= dense_min rows per leaf go leaf by leaf
-    const int4 *run_memo;  // full memo in run order (k <= 3), or null
-    const uint64_t *cls_beg;
-    int g[FZ_MAX_D];
-    FastDiv glast;         // division by g_{d-1} (walk leaves)
-    // Walk leaves as a progression: with e = gcd(g_{d-2}, g_{d-1}), the
-    // candidates a_{d-2} = v of remainder r with g_{d-1} | r - v g_{d-2} are
-    // v = v* (mod h1), h1 = g_{d-1}/e, v* = (r/e) inv (mod h1), inv the inverse
-    // of g1 = g_{d-2}/e mod h1 (0 when h1 = 1); e must divide r.  Along the
-    // progression a_{d-1} grows by g1.  wl_h1 = 0: candidate by candidate.
-    int wl_e, wl_h1, wl_g1, wl_inv;
-    // Pair memo: a full memo of depth 2 kept as a formula, no table.  Memo
-    // leaf p (remainder at depth d-2) holds Z(p, (g_{d-2}, g_{d-1})): row o
-    // is a_{d-2} = a_top - o h1, a_{d-1} = (p - a_{d-2} g_{d-2}) / g_{d-1},
-    // with a_top the largest valid a_{d-2} (the progression above).
-    int pair_memo;
-    FastDiv fd_e, fd_h1, fd_g2;  // division by e, h1 and g_{d-2}
-};
-
-// First a_{d-2} of pair-memo leaf p (meaningful when the leaf is not empty):
-// 32-bit divisions by precomputed multipliers; the product (p/e mod h1) inv
-// fits 32 bits when h1 < 2^16, else it takes a 64-bit remainder.
-__device__ __forceinline__ uint32_t pair_top(const EnumParams &P, int p) {
-    const uint32_t up = (uint32_t)p;
-    const uint32_t h1 = (uint32_t)P.wl_h1;
-    const uint32_t xr = fd_mod(fd_div(up, P.fd_e), P.fd_h1);
-    const uint32_t astar = h1 < 65536u
-                               ? fd_mod(xr * (uint32_t)P.wl_inv, P.fd_h1)
-                               : (uint32_t)((uint64_t)xr * (uint32_t)P.wl_inv % h1);
-    const uint32_t q = fd_div(up, P.fd_g2);
-    return q >= astar ? q - fd_mod(q - astar, P.fd_h1) : 0u;
-}
-
-struct WarpPath {
-    int a[FZ_MAX_D];      // a_0..a_{lam-1}
-    int r[FZ_MAX_D + 1];  // r[0] = n, r[c+1] = r[c] - a[c] g[c]
-};
-
-enum LeafType : int { T_NONE = 0, T_MEMO = 1, T_WALK = 2, T_INTERNAL = 3 };
-
-// Largest u in [0, umax] with F(u) <= R, F(u) = C[c][rem - (umax + 1 - u) g_c]
-// (rows in the children with a_c > umax - u), searched 32 probes at a time.
-// Returns the child a_c = umax - u holding relative rank R and the rows
-// before it.  Requires R < C[c][rem].
-__device__ __forceinline__ void find_child(const EnumParams &P, int c, int rem, uint64_t R,
-                                           int lane, int &v_out, uint64_t &before_out) {
-    const long long g = P.g[c];
-    const long long umax = rem / g;
-    const long long base = (long long)rem - (umax + 1) * g;
-    const uint64_t *row = P.C + (long long)c * P.cs;
-    long long lo = 0, hi = umax + 1;
-    uint64_t flo = 0;
-    while (hi - lo > 1) {
-        const long long step = (hi - lo + 31) >> 5;
-        const long long u = lo + (long long)(lane + 1) * step;
-        bool ok = false;
-        uint64_t fu = 0;
-        if (u < hi) {
-            const long long idx = base + u * g;
-            fu = idx >= 0 ? __ldg(row + idx) : 0ull;
-            ok = fu <= R;
-        }
-        const unsigned m = __ballot_sync(FULL, ok);
-        const int cnt = __popc(m);
-        const uint64_t fsel = shfl_u64(fu, cnt > 0 ? cnt - 1 : 0);
-        if (cnt > 0) {
-            flo = fsel;
-            lo += (long long)cnt * step;
-        }
-        const long long nh = lo + step;
-        if (nh < hi) hi = nh;
-    }
-    v_out = (int)(umax - lo);
-    before_out = flo;
-}
-
-// Walk state of one warp (warp-uniform).
-struct RunState {
-    int lam;          // coordinate of the current run of sibling leaves
-    int inwalk;       // inside the subtree of a memo-level child with p >= top
-    long long vcur;   // next candidate value of a_lam (descending)
-    uint64_t base;    // rows in the siblings before vcur
-};
-
-// Choose the first live child at depths c_from..c_to-1 (path stored by lane 0).
-__device__ __forceinline__ void descend(const EnumParams &P, WarpPath *wp, int c_from,
-                                        int c_to, int lane) {
-    int rem = wp->r[c_from];
-    for (int c = c_from; c < c_to; ++c) {
-        int v = rem / P.g[c];
-        // usually the largest child is live (one load); else search
-        if (__ldg(P.C + (long long)(c + 1) * P.cs + (rem - v * P.g[c])) == 0ull) {
-            uint64_t before;
-            find_child(P, c, rem, 0ull, lane, v, before);
-        }
-        rem -= v * P.g[c];
-        if (lane == 0) {
-            wp->a[c] = v;
-            wp->r[c + 1] = rem;
-        }
-    }
-    __syncwarp();
-}
-
-// Position the warp on the leaf holding absolute rank R.  Returns the offset
-// of R inside that leaf.  Sets *ok = false if the table is inconsistent.
-__device__ uint64_t unrank_to_leaf(const EnumParams &P, WarpPath *wp, uint64_t R, int lane,
-                                   RunState &st, bool *ok) {
-    int rem = P.n;
-    if (lane == 0) wp->r[0] = rem;
-    int inwalk = 0;
-    const bool memo = P.lam_m >= 0;
-    *ok = true;
-    for (int c = 0; c < P.d; ++c) {
-        const int runlev = (memo && !inwalk) ? P.lam_m : P.lam_w;
-        const uint64_t total = __ldg(P.C + (long long)c * P.cs + rem);
-        if (R >= total) {
-            *ok = false;
-            break;
-        }
-        int v;
-        uint64_t before;
-        find_child(P, c, rem, R, lane, v, before);
-        R -= before;
-        const int p = rem - v * P.g[c];
-        if (c == runlev) {
-            if (memo && !inwalk && p >= P.top && P.lam_m < P.lam_w) {
-                // memo-level child beyond the memo: walk its subtree
-                if (lane == 0) {
-                    wp->a[c] = v;
-                    wp->r[c + 1] = p;
-                }
-                rem = p;
-                inwalk = 1;
-                continue;
-            }
-            st.lam = c;
-            st.inwalk = inwalk;
-            st.vcur = v;
-            st.base = before;
-            __syncwarp();
-            return R;
-        }
-        if (lane == 0) {
-            wp->a[c] = v;
-            wp->r[c + 1] = p;
-        }
-        rem = p;
-    }
-    __syncwarp();
-    *ok = false;
-    return 0;
-}
-
-// Move to the next run after the current one is exhausted.  Returns false at
-// the end of the stream.
-__device__ bool advance(const EnumParams &P, WarpPath *wp, int lane, RunState &st) {
-    const bool memo = P.lam_m >= 0;
-    for (int j = st.lam - 1; j >= 0; --j) {
-        const int rem = wp->r[j];
-        const int aj = wp->a[j];
-        const uint64_t *row = P.C + (long long)j * P.cs;
-        const uint64_t R = __ldg(row + (rem - aj * P.g[j]));  // rows in children >= aj
-        const uint64_t total = __ldg(row + rem);
-        if (R >= total) continue;
-        // usually the next smaller value is live (one load); else search
-        int v = aj - 1;
-        if (__ldg(P.C + (long long)(j + 1) * P.cs + (rem - v * P.g[j])) == 0ull) {
-            uint64_t before;
-            find_child(P, j, rem, R, lane, v, before);
-        }
-        const int p = rem - v * P.g[j];
-        if (lane == 0) {
-            wp->a[j] = v;
-            wp->r[j + 1] = p;
-        }
-        __syncwarp();
-        int nw;
-        if (memo && j < P.lam_m)
-            nw = 0;
-        else if (memo)
-            nw = 1;  // at or below the memo level: inside a walked subtree
-        else
-            nw = 0;
-        const int newlam = (memo && !nw) ? P.lam_m : P.lam_w;
-        descend(P, wp, j + 1, newlam, lane);
-        st.lam = newlam;
-        st.inwalk = nw;
-        st.vcur = wp->r[newlam] / P.g[newlam];
-        st.base = 0;
-        return true;
-    }
-    return false;
-}
-
-// ---------------------------------------------------------------------------
-// Work-balanced slicing.  The cost of a subtree is its rows plus W for every
-// unit of walk work in it -- a leaf candidate, a walk run or a run-order run,
-// i.e. a prefix of length lam_r the walk evaluates, live or not (balance_level
-// picks lam_r and W); RT[j][x] counts those prefixes (RT[lam_r] = 1, and row j
-// is row j+1 strided-summed with stride g_j, like the count table; a memo
-// leaf above level lam_r is clamped to one unit), so the cost of the
-// children a_j >= v of a node is
-// C[j][x] + W RT[j][x] with x = rem - v g_j.  Work items are equal cost ranges, located by the same
-// 32-probe search as ranks, then snapped to ranks that are multiples of 32
-// from rank_begin: 32 rows are 128 d bytes, so every bulk store of a slice
-// starts on a 128-byte line when the output is 128-byte aligned.
-// ---------------------------------------------------------------------------
-// A memo leaf above the counted level (a partial memo of depth K > 2 whose
-// runs table counts walk runs): the node at depth j is one unit of cost.
-__device__ __forceinline__ bool is_memo_unit(const EnumParams &P, int j, int rem) {
-    return P.lam_m >= 0 && j == P.lam_m + 1 && j < P.lam_r && rem < P.top;
-}
-
-__device__ __forceinline__ uint64_t cost_at(const EnumParams &P, int j, long long idx) {
-    if (idx < 0) return 0ull;
-    return __ldg(P.C + (long long)j * P.cs + idx) + P.W * __ldg(P.RT + (long long)j * P.cs + idx);
-}
-
-// Rank of the first row whose cumulative cost reaches `target` (clamped to
-// the total row count).
-__device__ uint64_t cost_to_rank(const EnumParams &P, uint64_t target, int lane) {
-    int rem = P.n;
-    uint64_t rank = 0;
-    if (target >= cost_at(P, 0, rem)) return __ldg(P.C + rem);
-    int lev = P.lam_r;
-    for (int j = 0; j < P.lam_r; ++j) {
-        if (is_memo_unit(P, j, rem)) {
-            lev = j;
-            break;
-        }
-        const long long g = P.g[j];
-        const long long umax = rem / g;
-        const long long base = (long long)rem - (umax + 1) * g;
-        long long lo = 0, hi = umax + 1;
-        uint64_t flo = 0;
-        while (hi - lo > 1) {
-            const long long step = (hi - lo + 31) >> 5;
-            const long long u = lo + (long long)(lane + 1) * step;
-            bool ok = false;
-            uint64_t fu = 0;
-            if (u < hi) {
-                fu = cost_at(P, j, base + u * g);
-                ok = fu <= target;
-            }
-            const int cnt = __popc(__ballot_sync(FULL, ok));
-            const uint64_t fsel = shfl_u64(fu, cnt > 0 ? cnt - 1 : 0);
-            if (cnt > 0) {
-                flo = fsel;
-                lo += (long long)cnt * step;
-            }
-            const long long nh = lo + step;
-            if (nh < hi) hi = nh;
-        }
-        const long long idx = base + lo * g;
-        rank += idx >= 0 ? __ldg(P.C + (long long)j * P.cs + idx) : 0ull;
-        target -= flo;
-        rem = (int)(rem - (umax - lo) * g);
-    }
-    const uint64_t rows = __ldg(P.C + (long long)lev * P.cs + rem);
-    const uint64_t t = target > P.W ? target - P.W : 0ull;
-    return rank + (t < rows ? t : rows);
-}
-
-// Cumulative cost of everything before rank R.
-__device__ uint64_t rank_to_cost(const EnumParams &P, uint64_t R, int lane) {
-    int rem = P.n;
-    if (R >= __ldg(P.C + rem)) return cost_at(P, 0, rem);
-    uint64_t cost = 0;
-    for (int j = 0; j < P.lam_r; ++j) {
-        if (is_memo_unit(P, j, rem)) break;
-        int v;
-        uint64_t before;
-        find_child(P, j, rem, R, lane, v, before);
-        cost += before + P.W * (rem - (long long)(v + 1) * P.g[j] >= 0
-                                    ? __ldg(P.RT + (long long)j * P.cs +
-                                            (rem - (long long)(v + 1) * P.g[j]))
-                                    : 0ull);
-        R -= before;
-        rem -= v * P.g[j];
-    }
-    return cost + P.W + R;
-}
-
-// Rows [row0, row1) (relative to out) of work item s.  With a candidates
-// table the items are cost ranges of [cost_lo, cost_hi) snapped to multiples
-// of 32 rows: the first four fifths of the cost in items of slice_cost, the
-// rest in items of an eighth of that, so the warps that take the last items
-// finish close together.  Otherwise equal-row ranges.  Returns 0 when s is
-// past the last item, 1 when the item is empty, 2 otherwise.
-__device__ __forceinline__ int item_rows(const EnumParams &P, uint64_t s, uint64_t cost_lo,
-                                         uint64_t cost_hi, int lane, uint64_t &row0,
-                                         uint64_t &row1) {
-    if (P.RT) {
-        const uint64_t sc = P.slice_cost;
-        const uint64_t n1 = (cost_hi - cost_lo) / sc * 4 / 5;  // large items
-        const uint64_t sc_t = sc / 8 > 64 ? sc / 8 : 64;
-        uint64_t c0, c1;
-        if (s < n1) {
-            c0 = cost_lo + s * sc;
-            c1 = c0 + sc;
-        } else {
-            const uint64_t t = s - n1;
-            const uint64_t base = cost_lo + n1 * sc;
-            if (t >= (cost_hi - base + sc_t - 1) / sc_t) return 0;
-            c0 = base + t * sc_t;
-            c1 = c0 + sc_t;
-        }
-        if (c0 >= cost_hi) return 0;
-        row0 = 0;
-        if (s > 0) {
-            const uint64_t r = cost_to_rank(P, c0, lane);
-            row0 = r > P.rank_begin ? ((r - P.rank_begin) & ~31ull) : 0ull;
-            if (row0 > P.nrows) row0 = P.nrows;
-        }
-        row1 = P.nrows;
-        if (c1 < cost_hi) {
-            const uint64_t r = cost_to_rank(P, c1, lane);
-            row1 = r > P.rank_begin ? ((r - P.rank_begin) & ~31ull) : 0ull;
-            if (row1 > P.nrows) row1 = P.nrows;
-        }
-        return row1 > row0 ? 2 : 1;
-    }
-    if (s >= P.nslices) return 0;
-    row0 = s * P.slice_rows;
-    row1 = row0 + P.slice_rows < P.nrows ? row0 + P.slice_rows : P.nrows;
-    return 2;
-}
-
-__device__ __forceinline__ void flush_rows(const EnumParams &P, const int32_t *src,
-                                           uint64_t out_row, uint32_t nrows, int d, int lane,
-                                           uint64_t pol) {
-    flush_words(P.out + out_row * (uint64_t)d, P.aligned, src, nrows * (uint32_t)d, lane, pol);
-}
 
 // 4-byte global -> shared copy that does not hold a register (cp.async).
 // No memory clobber: the source (memo) is read-only, the destination word is
@@ -491,7 +128,7 @@ __device__ __forceinline__ bool enum_slice(const EnumParams &P, WarpPath *wp, in
         const int glam = P.g[lam];
         const bool memo_run =
             LAMF >= 0 ? true : ((P.lam_m >= 0) && !st.inwalk && lam == P.lam_m);
-        if (LAMF < 0 && !memo_run && lam == P.lam_w && P.wl_h1 > 0) {
+        if (LAMF < 0 && !memo_run && lam == P.lam_w && P.progression) {
             // A run of walk leaves (the ordinary step at the last two
             // coordinates): only the candidates a_{d-2} = v whose remainder
             // g_{d-1} divides hold a row, and they form a progression, so
@@ -499,12 +136,12 @@ __device__ __forceinline__ bool enum_slice(const EnumParams &P, WarpPath *wp, in
             // <= st.vcur down by h1, a_{d-1} up by g1 -- with no candidate
             // that holds no row evaluated.
             long long vtop = -1;
-            if (rem % P.wl_e == 0) {
-                const long long h1 = P.wl_h1;
-                const long long vstar = (long long)((rem / P.wl_e) % h1) * P.wl_inv % h1;
+            if (rem % (int)P.leaf.pair.fe.g == 0) {
+                const long long h1 = (int)P.leaf.pair.h1;
+                const long long vstar = (long long)((rem / (int)P.leaf.pair.fe.g) % h1) * (int)P.leaf.pair.inv % h1;
                 if (st.vcur >= vstar) vtop = st.vcur - (st.vcur - vstar) % h1;
             }
-            const uint32_t nrun = vtop >= 0 ? (uint32_t)(vtop / P.wl_h1) + 1u : 0u;
+            const uint32_t nrun = vtop >= 0 ? (uint32_t)(vtop / (int)P.leaf.pair.h1) + 1u : 0u;
             const int wtop =
                 vtop >= 0 ? (int)(((long long)rem - vtop * glam) / P.g[d - 1]) : 0;
             uint64_t qe = skip + rows_left;
@@ -523,8 +160,8 @@ __device__ __forceinline__ bool enum_slice(const EnumParams &P, WarpPath *wp, in
                         if (c >= d - 2) break;
                         dst[c] = pre[c];
                     }
-                    dst[d - 2] = (int)(vtop - (long long)q * P.wl_h1);
-                    dst[d - 1] = wtop + q * P.wl_g1;
+                    dst[d - 2] = (int)(vtop - (long long)q * (int)P.leaf.pair.h1);
+                    dst[d - 1] = wtop + q * (int)P.leaf.pair.g1;
                 }
                 q0 += cnt;
                 after_round(cnt);
@@ -560,8 +197,8 @@ __device__ __forceinline__ bool enum_slice(const EnumParams &P, WarpPath *wp, in
                 p = 0;
             }
             if (walk_run) {
-                wq = fd_div((uint32_t)p, P.glast);
-                wvalid = (uint32_t)p - wq * P.glast.g == 0u;
+                wq = fd_div((uint32_t)p, P.leaf.pair.fh);
+                wvalid = (uint32_t)p - wq * P.leaf.pair.fh.g == 0u;
             } else {
                 incl = __ldg(P.C + (long long)lam * P.cs + p);
             }
@@ -590,9 +227,9 @@ __device__ __forceinline__ bool enum_slice(const EnumParams &P, WarpPath *wp, in
             const uint64_t e = incl - st.base;
             E32 = e < (uint64_t)CAP32 ? (uint32_t)e : CAP32;
             if (type == T_MEMO)
-                X32 = (LAMF < 0 && P.pair_memo) ? pair_top(P, p) : (uint32_t)__ldg(P.O + p);
+                X32 = (LAMF < 0 && P.pair_memo) ? pair_form_top(P.leaf.pair, (uint32_t)p) : (uint32_t)__ldg(P.O + p);
             else if (type == T_WALK)
-                X32 = walk_run ? wq : fd_div((uint32_t)p, P.glast);
+                X32 = walk_run ? wq : fd_div((uint32_t)p, P.leaf.pair.fh);
         }
         uint64_t q_end64 = skip + rows_left;
         if (q_end64 > batch_rows) q_end64 = batch_rows;
@@ -634,7 +271,7 @@ __device__ __forceinline__ bool enum_slice(const EnumParams &P, WarpPath *wp, in
                             if (pair) {
                                 // pair memo: the row from the progression
                                 const int o = (int)(q0 + lane - sj);
-                                const int av = (int)xj - o * P.wl_h1;
+                                const int av = (int)xj - o * (int)P.leaf.pair.h1;
 #pragma unroll
                                 for (int c = 0; c < DM; ++c) {
                                     if (c >= lam) break;
@@ -643,7 +280,7 @@ __device__ __forceinline__ bool enum_slice(const EnumParams &P, WarpPath *wp, in
                                 dst[lam] = vj;
                                 dst[lam + 1] = av;
                                 dst[lam + 2] = (int)fd_div(
-                                    (uint32_t)(pj - av * P.g[d - 2]), P.glast);
+                                    (uint32_t)(pj - av * P.g[d - 2]), P.leaf.pair.fh);
                             } else if constexpr (LAMF >= 0) {
 #pragma unroll
                                 for (int c = 0; c < LAMF; ++c) dst[c] = pre[c];
@@ -725,7 +362,7 @@ __device__ __forceinline__ bool enum_slice(const EnumParams &P, WarpPath *wp, in
                     }
                 } else if (pair) {
                     // pair memo: the row from the progression
-                    const int av = (int)xl - (int)o * P.wl_h1;
+                    const int av = (int)xl - (int)o * (int)P.leaf.pair.h1;
 #pragma unroll
                     for (int c = 0; c < DM; ++c) {
                         if (c >= lam) break;
@@ -733,7 +370,7 @@ __device__ __forceinline__ bool enum_slice(const EnumParams &P, WarpPath *wp, in
                     }
                     dst[lam] = vrow;
                     dst[lam + 1] = av;
-                    dst[lam + 2] = (int)fd_div((uint32_t)(pl - av * P.g[d - 2]), P.glast);
+                    dst[lam + 2] = (int)fd_div((uint32_t)(pl - av * P.g[d - 2]), P.leaf.pair.fh);
                 } else {
                     const int32_t *mrow =
                         mleaf ? P.memo + (size_t)(xl + o) * (size_t)P.K : nullptr;
@@ -1176,6 +813,46 @@ __device__ __noinline__ bool runs_slice_rt(const EnumParams &P, int32_t *ring, u
     return ok;
 }
 
+// The flat walk inside the batch kernel, one routine per shape (not inlined,
+// so no shape's registers weigh on another's).  Items are numbered by shape,
+// so the warps of an SM mostly run the same one.
+template <int D, int NP, int SRC>
+__device__ __noinline__ bool flat_batch_one(const EnumParams &P, unsigned char *mem,
+                                            uint64_t row0, uint64_t row1, uint64_t pol,
+                                            int lane) {
+    constexpr uint32_t B = flat_half_rows<NP, SRC, D>(RING_BYTES_PER_WARP);
+    static_assert(leaf_bytes<NP, SRC>() + 2 * (int)B * D * 4 <= RING_BYTES_PER_WARP, "ring");
+    return flat_slice<D, NP, SRC>(P, mem, B, row0, row1, pol, lane);
+}
+
+template <int D>
+__device__ __forceinline__ bool flat_batch_d(const EnumParams &P, unsigned char *mem,
+                                             uint64_t row0, uint64_t row1, uint64_t pol,
+                                             int lane) {
+    if (P.flat_src == SRC_PAIR)
+        return flat_batch_one<D, D - 2, SRC_PAIR>(P, mem, row0, row1, pol, lane);
+    if (P.flat_np == 1) return flat_batch_one<D, 1, SRC_RUN>(P, mem, row0, row1, pol, lane);
+    if constexpr (D >= 4)
+        if (P.flat_np == 2) return flat_batch_one<D, 2, SRC_RUN>(P, mem, row0, row1, pol, lane);
+    if constexpr (D >= 5)
+        if (P.flat_np == 3) return flat_batch_one<D, 3, SRC_RUN>(P, mem, row0, row1, pol, lane);
+    if (lane == 0) atomicExch(P.status, (int)DEV_INTERNAL);  // shapes the host never sends here
+    return false;
+}
+
+__device__ __forceinline__ bool flat_batch_slice(const EnumParams &P, unsigned char *mem,
+                                                 uint64_t row0, uint64_t row1, uint64_t pol,
+                                                 int lane) {
+    switch (P.d) {
+        case 3: return flat_batch_d<3>(P, mem, row0, row1, pol, lane);
+        case 4: return flat_batch_d<4>(P, mem, row0, row1, pol, lane);
+        case 5: return flat_batch_d<5>(P, mem, row0, row1, pol, lane);
+        case 6: return flat_batch_d<6>(P, mem, row0, row1, pol, lane);
+        case 7: return flat_batch_d<7>(P, mem, row0, row1, pol, lane);
+        default: return flat_batch_d<8>(P, mem, row0, row1, pol, lane);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Many instances in one persistent launch.  Work items (instance, slice) are
 // numbered consecutively, instance i owning items [item0[i], item0[i+1]); a
@@ -1270,12 +947,14 @@ __global__ void __launch_bounds__(ENUM_THREADS, 4)
             }
             continue;
         }
-        // full memos in run order take the run copy; otherwise one walk for
-        // every width up to 8 (row loops unrolled to 8), the 16-wide one
-        // beyond: three code paths at most, so warps of different instances
-        // share the instruction cache
+        // the flat walk where it has a kernel for the shape; else full memos
+        // in run order take the run copy, and the rest one walk for every
+        // width up to 8 (row loops unrolled to 8), the 16-wide one beyond
         bool ok;
-        if (P.run_memo)
+        if (P.flat_np)
+            ok = flat_batch_slice(P, smem_raw + (size_t)wid * BATCH_RING_BYTES, row0, row1, pol,
+                                  lane);
+        else if (P.run_memo)
             ok = runs_slice_rt(P, ring, (uint32_t)P.half_rows, row0, row1, pol, lane);
         else if (P.d <= 8)
             ok = enum_slice<0, -1, 8>(P, wp, ring, (uint32_t)P.half_rows, row0, row1, pol, lane);
@@ -1358,7 +1037,7 @@ __global__ void __launch_bounds__(ENUM_THREADS)
             else if (mleaf)
                 x = __ldg(P.memo + (size_t)(__ldg(P.O + p) + off) * P.K + (lane - lam - 1));
             else
-                x = (int)fd_div((uint32_t)p, P.glast);
+                x = (int)fd_div((uint32_t)p, P.leaf.pair.fh);
             P.out[i * D + lane] = x;
         }
         __syncwarp();
@@ -1407,34 +1086,13 @@ static int ring_bytes_for(int ctas_per_sm) {
     return b > 16 * 1024 ? 16 * 1024 : (b / 1024) * 1024;
 }
 
-constexpr int ENUM_MAX_SMEM = 200 * 1024;
-
 template <typename Kern>
 static int launch_enum_kernel(Kern kern, const EnumParams &P, int D, cudaStream_t s, int sms,
                               DeviceOnce &attr_set) {
-    const size_t smem = (size_t)ENUM_WARPS * 2 * P.half_rows * D * 4 +
-                        (size_t)ENUM_WARPS * sizeof(WarpPath);
-    if (smem > (size_t)ENUM_MAX_SMEM) return set_error(FZ_EINTERNAL, "enumerate: ring too large");
-    int dev = 0;
-    FZ_CUDA_TRY(cudaGetDevice(&dev));
-    if (!attr_set.is_set(dev)) {
-        FZ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         ENUM_MAX_SMEM));
-        attr_set.set(dev);
-    }
-    int per_sm = 0;
-    FZ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, ENUM_THREADS, smem));
-    if (P.ctas_per_sm > 0 && per_sm > P.ctas_per_sm) per_sm = P.ctas_per_sm;
-    if (per_sm < 1) per_sm = 1;
-    uint64_t want = (P.nslices + ENUM_WARPS - 1) / ENUM_WARPS;
-    uint64_t grid = (uint64_t)per_sm * sms;
-    if (want < grid) grid = want;
-    if (grid < 1) grid = 1;
-    FZ_CUDA_TRY(cudaMemsetAsync(P.slice_counter, 0, sizeof(unsigned long long), s));
-    kern<<<(unsigned)grid, ENUM_THREADS, smem, s>>>(P);
-    note_launch();
-    FZ_CUDA_TRY(cudaGetLastError());
-    return FZ_OK;
+    return launch_enum_grid(kern, P,
+                            (size_t)ENUM_WARPS * 2 * P.half_rows * D * 4 +
+                                (size_t)ENUM_WARPS * sizeof(WarpPath),
+                            s, sms, attr_set);
 }
 
 template <int D, int LAMF>
@@ -1521,21 +1179,13 @@ static EnumParams make_params(const EnumLaunch &L) {
     P.K = L.K;
     P.top = L.top;
     for (int i = 0; i < L.d; ++i) P.g[i] = L.g[i];
-    P.glast = make_fastdiv((uint32_t)L.g[L.d - 1]);
-    P.wl_e = 1;
-    P.wl_h1 = P.wl_g1 = P.wl_inv = 0;
-    P.fd_e = P.fd_h1 = P.fd_g2 = make_fastdiv(1u);
     P.pair_memo = L.pair_memo && L.K == 2 && L.d >= 3 && L.top > L.n;
-    if (L.d >= 2 && (walk_progression_enabled() || P.pair_memo)) {
-        int64_t e, h1, g1, inv;
-        pair_params(L.g[L.d - 2], L.g[L.d - 1], &e, &h1, &g1, &inv);
-        P.wl_e = (int)e;
-        P.wl_h1 = (int)h1;
-        P.wl_g1 = (int)g1;
-        P.wl_inv = (int)inv;
-        P.fd_e = make_fastdiv((uint32_t)e);
-        P.fd_h1 = make_fastdiv((uint32_t)h1);
-        P.fd_g2 = make_fastdiv((uint32_t)L.g[L.d - 2]);
+    P.leaf = LeafSource{};
+    if (L.d >= 2) {
+        P.leaf.pair = make_pair_form(L.g[L.d - 2], L.g[L.d - 1]);
+        P.progression = walk_progression_enabled() || P.pair_memo;
+    } else {
+        P.leaf.pair.fh = make_fastdiv((uint32_t)L.g[0]);
     }
     const bool memo = L.K >= 1 && L.K <= L.d - 1 && L.top > 0;
     P.lam_m = memo ? L.d - L.K - 1 : -1;
@@ -1544,10 +1194,24 @@ static EnumParams make_params(const EnumLaunch &L) {
         P.K = 0;
         P.top = 0;
     }
-    // the run-order memo serves full memos of depth 1..3
-    const bool runs = memo && L.top > L.n && L.K <= 3 && L.run_memo && L.cls_beg;
+    // the run-order memo serves full memos
+    const bool runs = memo && L.top > L.n && L.run_memo && L.cls_beg;
     P.run_memo = runs ? L.run_memo : nullptr;
     P.cls_beg = runs ? L.cls_beg : nullptr;
+    for (int j = 0; j < FLAT_MAX_NP && j < L.d; ++j) P.fdg[j] = make_fastdiv((uint32_t)L.g[j]);
+    if (runs) {
+        P.leaf.rows = reinterpret_cast<const int32_t *>(L.run_memo);
+        P.leaf.cls = L.cls_beg;
+        P.leaf.nrows = L.memo_rows;
+        P.leaf.fg = make_fastdiv((uint32_t)L.g[L.d - L.K - 1]);
+        P.flat_np = L.d - L.K - 1;
+        P.flat_src = SRC_RUN;
+    } else if (P.pair_memo || (!memo && P.progression)) {
+        // no memo table: leaves are the prefixes above the last two generators
+        P.flat_np = L.d - 2;
+        P.flat_src = SRC_PAIR;
+    }
+    if (!flat_serves(L.d, P.flat_np, P.flat_src)) P.flat_np = 0;
     // the run walk's candidates are the prefixes of its LAMF = d - K - 1
     // leading coordinates; a table counted at another level cannot balance it
     if (runs && P.lam_r != L.d - L.K - 1) P.RT = nullptr;
@@ -1613,6 +1277,7 @@ int launch_enumerate(const EnumLaunch &L, uint64_t rank_begin, uint64_t nrows, i
         uint64_t sc = (uint64_t)((double)slice_rows * per_row);
         P.slice_cost = sc < 64 ? 64 : sc;
     }
+    if (P.flat_np > 0) return launch_enum_flat(P, ring_bytes_for(L.ctas_per_sm), s, dp.sms);
     P.half_rows = half_rows_for(L.d, ring_bytes_for(L.ctas_per_sm));
     FZ_DISPATCH_D(L.d, launch_enum_d, P, s, dp.sms);
 }
@@ -1643,6 +1308,7 @@ void fill_batch_params(const EnumLaunch &L, int32_t *out, uint64_t count, uint64
     P.slice_rows = slice_rows < 4 ? 4 : ((slice_rows + 3) & ~3ull);
     P.nslices = (count + P.slice_rows - 1) / P.slice_rows;
     P.half_rows = half_rows_for(L.d);
+    if (L.d > 8) P.flat_np = 0;  // the batch kernel's flat walk: widths 3..8
     P.slice_cost = slice_cost < 64 ? 64 : slice_cost;
     memcpy(dst, &P, sizeof(P));
 }

@@ -400,14 +400,16 @@ bool walk_progression_enabled();
 // Work balancing: the level lam_r whose prefixes the candidates table counts
 // and the cost W of one such prefix in rows, for an instance of d generators
 // with memo depth K and top (top > n: full memo); run_order: the memo is kept
-// in run order.  Walk runs (the last two coordinates as a progression) and
-// run-order runs cost a chain of dependent loads each (W = 64); memo leaves
-// and candidates evaluated 32 at a time cost W = 16.
+// in run order; pair: it is the closed form of the last two generators.  Walk
+// runs (the last two coordinates as a progression) and run-order runs walked
+// one at a time cost a chain of dependent loads each (W = 64); memo leaves
+// and candidates evaluated 32 at a time cost W = 16, leaves of the flat walk
+// FLAT_LEAF_COST.
 // *clamp_row >= 0: the table row whose entries below top are set to 1 (a
 // memo leaf is one unit, whatever lies under it), else -1.
 bool run_memo_enabled();
-void balance_level(int d, int K, int top, int n, bool run_order, int *lam_r, uint64_t *W,
-                   int *clamp_row);
+void balance_level(int d, int K, int top, int n, bool run_order, bool pair, int *lam_r,
+                   uint64_t *W, int *clamp_row);
 
 struct EnumLaunch {
     const uint64_t *C = nullptr;   // count table rows 0..d, stride cs = n + 1

@@ -35,7 +35,7 @@
 #include <unordered_map>
 #include <vector>
 
-#include "fz_internal.cuh"
+#include "fz_walk.cuh"
 
 struct fz_server_s;
 
@@ -273,11 +273,14 @@ uint64_t serve_direct_rows() {
     return v;
 }
 
-// Whether the batch kernel serves a launch of this shape (its run-order
-// copy takes widths up to 8 with at least one walked coordinate).
+// Whether the batch kernel serves a launch of this shape (run order: widths
+// up to 8 by the flat walk, or by the run copy with at least one walked
+// coordinate and depth up to 3).
 bool batch_kernel_serves(const EnumLaunch &L) {
     if (!L.run_memo) return true;
-    return L.d <= 8 && L.d - L.K - 1 >= 1 && L.K >= 1 && L.K <= 3;
+    if (L.d > 8) return false;
+    const int lam = L.d - L.K - 1;
+    return flat_serves(L.d, lam, SRC_RUN) || (lam >= 1 && L.K >= 1 && L.K <= 3);
 }
 
 // Enqueue a group of admitted requests (called by the server thread, lock

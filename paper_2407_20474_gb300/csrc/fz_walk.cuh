@@ -171,6 +171,13 @@ struct RunLevels {
     uint64_t *cls = nullptr;
 };
 
+// fz_flat.cu: true if the flat walk has a kernel for tuples of width d with
+// leaves of np prefix words.
+bool flat_serves(int d, int np, int src);
+// Cost of a leaf of the flat walk in rows (work-balanced slicing): 32 leaves
+// take about as many instructions as 100 rows.
+constexpr uint64_t FLAT_LEAF_COST = 4;
+
 // Deepest memo the levels build (rows of a table: quotient and coordinates).
 constexpr int RUN_MAX_K = 7;   // run-order tables
 constexpr int CSR_MAX_K = 8;   // memos in element order (from depth 3 on)
@@ -227,8 +234,9 @@ __host__ __device__ constexpr uint32_t flat_half_rows(int bytes) {
 // plain copies.  The table rows of the next round are loaded before this
 // round's rows are stored.
 //
-// What bounds it: instruction issue.  A copy with one leaf a warp at a time
-// needs about 12 warp instructions a row where leaves hold a row or two.
+// What bounds it: instruction issue while leaves are short (a copy with one
+// leaf a warp at a time needed about 12 warp instructions a row where leaves
+// hold a row or two), the output's bandwidth when they are long.
 //
 // Walk: leaf(p, end, pre) gives lane's element, cumulative row end and
 // prefix words and returns false past the last leaf (a suffix of the

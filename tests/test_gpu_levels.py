@@ -70,3 +70,60 @@ def test_plans_on_levels(fz, g, target):
             assert np.array_equal(out[:total].cpu().numpy(), ref), k
             assert np.array_equal(pick[:total].cpu().numpy(), ref[ranks.cpu().numpy()]), k
             assert bool((out[total:] == CANARY).all()) and bool((pick[total:] == CANARY).all())
+
+
+def _window(fz, g, n, k, begin, end, slice_rows, shift):
+    d = len(g)
+    out = torch.full((shift + (end - begin + 3) * d,), CANARY, dtype=torch.int32, device="cuda")
+    with fz.Plan(g, n, k=k, slice_rows=slice_rows) as plan:
+        assert plan.enumerate(out[shift:], begin, end) == end - begin
+        plan.sync()
+    host = out.cpu().numpy()
+    last = shift + (end - begin) * d
+    assert (host[:shift] == CANARY).all() and (host[last:] == CANARY).all()
+    return host[shift:last].reshape(-1, d)
+
+
+@pytest.mark.parametrize("d", [3, 4, 5, 6, 7, 8, 9])
+@pytest.mark.parametrize("lo,hi", [(2, 9), (20, 60)])
+def test_flat_walk(fz, d, lo, hi):
+    """Leaves of one to three prefix words over run-order tables and of d - 2
+    over the pair's closed form (k = 0): dense leaves (small generators) and
+    mostly empty ones (large generators), items that start inside a leaf,
+    ring remainders, rank windows, outputs aligned to 4 bytes only."""
+    rng = np.random.Generator(np.random.PCG64(1000 * d + lo))
+    g = tuple(int(x) for x in rng.integers(lo, hi, size=d))
+    n = workloads.find_n(oracle.count_upto, g, 12000)
+    ref = oracle.enumerate_desc(g, n)
+    total = ref.shape[0]
+    for k in {0, d - 2, max(0, d - 3), max(0, d - 4), -1}:
+        for slice_rows in (4, 100, 0):
+            assert np.array_equal(_window(fz, g, n, k, 0, total, slice_rows, 0), ref), (g, n, k)
+        for shift in (0, 1, 2):
+            a, b = sorted(int(x) for x in rng.integers(0, total, size=2))
+            got = _window(fz, g, n, k, a, b + 1, 40, shift)
+            assert np.array_equal(got, ref[a:b + 1]), (g, n, k, a, b, shift)
+
+
+def test_batch_flat_shapes(fz):
+    """Every shape of the batch kernel's flat walk in one batch, and each depth
+    on its own."""
+    rng = np.random.Generator(np.random.PCG64(77))
+    inst = []
+    for d in range(3, 9):
+        for lo, hi, target in ((2, 12, 6000), (15, 70, 3000), (40, 200, 300)):
+            g = tuple(int(x) for x in rng.integers(lo, hi, size=d))
+            inst.append((g, workloads.find_n(oracle.count_upto, g, target)))
+    refs = [oracle.enumerate_desc(g, n) for g, n in inst]
+    for k in (-1, 0, 1, 2, 3, 4, 5, 6):
+        sub = [i for i, (g, _) in enumerate(inst) if k <= len(g) - 1]
+        with fz.Batch([inst[i] for i in sub], k=k) as b:
+            out = torch.full((b.total_words + 8,), CANARY, dtype=torch.int32, device="cuda")
+            b.rebuild()
+            b.enumerate(out)
+            b.sync()
+            host = out.cpu().numpy()
+            assert (host[b.total_words:] == CANARY).all()
+            for j, i in enumerate(sub):
+                at, ref = int(b.word_offsets[j]), refs[i]
+                assert np.array_equal(host[at:at + ref.size].reshape(ref.shape), ref), (inst[i], k)

@@ -326,16 +326,16 @@ int fz_plan_destroy(fz_plan_t plan);
 /* ------------------------------------------------------------------------
  * Batches: many instances Z(n_i, g_i) of possibly different d_i in one set
  * of launches -- batched counting tables, one memo per distinct tail shared
- * by the instances that have it (each built by the elementwise dynamic pass,
- * Sections 2.2-2.4, cut to at most 512 element batches; larger
- * remainders take the ordinary next-candidate step, Section 3.1; a memo of
- * depth 2 over the last two generators is kept as its closed form, with no
- * table), and one persistent enumeration launch over (instance, slice) work
- * items.  Full memos of depth 1..3 (widths d <= 8 with at least one walked
- * coordinate above the memo) are also kept in run order, as in plans, so a
- * prefix's whole subtree is one contiguous copy; for the closed form that
- * table is computed from the formula when it stays small.  The memo depth
- * of each generator set is chosen by the library unless opts.k is given.
+ * by the instances that have it, and one persistent enumeration launch over
+ * (instance, slice) work items.  Full memos (widths 3..8 with at least one
+ * walked coordinate above the memo) are tables in run order, built generator
+ * by generator, so a prefix's whole subtree is one contiguous copy; a memo of
+ * depth 2 over the last two generators may be kept as its closed form, with
+ * no table.  Memos in element order (partial memos, or where the policy turns
+ * run order off) are built by the elementwise dynamic pass (Sections 2.2-2.4),
+ * cut to at most 512 element batches; larger remainders take the ordinary
+ * next-candidate step (Section 3.1).  The memo depth of each generator set is
+ * chosen by the library unless opts.k is given.
  * Output: instance i's rows (d_i int32 each, descending lexicographic order)
  * start at word word_offsets[i] of the output buffer (multiples of 32 words,
  * so 128-byte aligned when the buffer is); word_offsets[count] is the total.
@@ -356,9 +356,12 @@ typedef struct fz_batch_info {
     uint64_t work_items;   /* (instance, slice) items of one enumeration */
     int32_t run_order;     /* instances whose full memo is copied in run order */
     int32_t run_memos;     /* distinct run-order memos */
-    int32_t coop_memos;    /* memos built by a thread-block cluster (the
-                              longest, when one alone would outlast an even
-                              share of the build) */
+    int32_t coop_memos;    /* memos built by more than one thread block: by a
+                              thread-block cluster (the longest in element
+                              order, when one alone would outlast an even
+                              share of the build), or tables in run order,
+                              their intermediate levels included, that take
+                              several blocks */
     int32_t reserved;
 } fz_batch_info_t;
 
@@ -399,11 +402,13 @@ int fz_plan_batch(const fz_instance_t *inst, int count, const fz_opts_t *opt,
                   void *stream);
 
 /* Measured choice of memos for batches (the memo depth, Section 3.1's
- * memoDim, and the memo layout).  A batch chooses per generator set the
- * deepest full memo whose estimated rows stay within cap_rows times the
- * instance's estimated rows (else a partial depth-3 memo for d >= 5, else
- * the closed form of the last two generators), and keeps full memos of
- * depth <= 3 in run order when run_order is set; both are per tuple width.
+ * memoDim, and the memo layout).  With run_order set, a batch chooses per
+ * generator set the depth with the least estimated walk and build among the
+ * run-order memos whose estimated rows stay within cap_rows times the
+ * instance's estimated rows and the closed form of the last two generators;
+ * without it, the deepest full memo in element order within the same cap
+ * (else a partial depth-3 memo for d >= 5, else the closed form).  Both are
+ * per tuple width.
  * fz_batch_autotune times, on the device, the given instances of each width
  * >= 3 (up to 1024 of them, spread over the list) under cap_rows in
  * {0, 1/4, 1, 4, 16}

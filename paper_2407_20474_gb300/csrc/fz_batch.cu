@@ -4,10 +4,11 @@
 // work-balanced slicing) and, per distinct tail, one memo shared by the
 // instances with that tail.  A rebuild is: one initialisation launch and
 // three launches per table level for all instances' tables together (the
-// batched strided scans of fz_count.cu), then one launch that builds every
-// memo (one CTA per memo, the elementwise dynamic pass of Section 2).  The
-// enumeration is one persistent launch over (instance, slice) work items
-// (fz_enum.cu).  Everything after creation is asynchronous, so a rebuild plus
+// batched strided scans of fz_count.cu), then the run-order tables of every
+// tail, one launch per depth (fz_runs.cu), and one launch for the memos kept
+// in element order, if any (one CTA per memo, the elementwise dynamic pass of
+// Section 2).  The enumeration is one persistent launch over (instance, slice)
+// work items (fz_enum.cu).  Everything after creation is asynchronous, so a rebuild plus
 // an enumeration can be captured in a CUDA graph.
 #include <cuda_runtime.h>
 
@@ -62,7 +63,7 @@ constexpr double BATCH_MEMO_MAX_ROWS = 1 << 20;
 struct Inst {
     int d = 0, n = 0, K = 0, top = 0, lam_r = 0, clamp_row = -1;
     bool pair = false;  // K = 2 kept as the closed form (no memo table)
-    bool run = false;   // full memo copied in run order (RunJob run_job)
+    bool run = false;   // full memo in run order (table run_job)
     int run_job = -1;
     const int4 *run_memo = nullptr;
     const uint64_t *cls_beg = nullptr;
@@ -98,9 +99,18 @@ struct fz_batch_s {
     int memo_ncoop = 0;              // memos built by a cluster
     unsigned *memo_claim = nullptr;  // claim counter of the memo build
     std::vector<MemoJob> memo_jobs;
-    RunJob *run_jobs_dev = nullptr;
+    // run-order tables of every depth, in build order: jobs, and per depth
+    // (first job, jobs, blocks)
+    RunBuild *run_jobs_dev = nullptr;
     int nrun = 0, run_inst = 0;
-    uint64_t run_blocks = 0;  // blocks of the run-row kernel
+    struct RunLevel {
+        int K, first, jobs;
+        uint32_t blocks;
+    };
+    std::vector<RunLevel> run_levels;
+    int run_final = 0, run_deep = 0, run_wide = 0;  // tables instances read; of depth >= 3;
+                                                    // of all tables, built by several blocks
+    uint64_t run_table_rows = 0;
     int ctas_per_sm = 0;      // cap of the enumeration kernel (0: as many as fit)
     void *params_dev = nullptr;       // EnumParams images (out = word offset)
     uint64_t *item0_dev = nullptr;
@@ -159,7 +169,7 @@ int build_scan_plan(fz_batch_s *b, uint64_t *table_base, std::vector<ScanJob> &j
                 jp.h = I.g[I.d - 1];
                 // row d-1 is read by a memo build from this table, or as the
                 // leaf row of a candidates table counted at level d - 1
-                jp.ones_below = ((I.K > 0 && !I.pair) || I.lam_r >= I.d - 1) ? 1 : 0;
+                jp.ones_below = ((I.K > 0 && !I.pair && !I.run) || I.lam_r >= I.d - 1) ? 1 : 0;
                 pair_params(jp.g, jp.h, &jp.e, &jp.h1, &jp.g1, &jp.inv);
                 if (!jp.ones_below && (I.d == 2 || (I.d == 3 && I.pair))) chain_view(jp, I);
                 jobs.push_back(jp);
@@ -292,6 +302,18 @@ int build_scan_plan(fz_batch_s *b, uint64_t *table_base, std::vector<ScanJob> &j
     return FZ_OK;
 }
 
+// Class starts of every run-order table, then the tables depth by depth (a
+// depth reads the one before).
+int batch_enqueue_runs(fz_batch_s *b, cudaStream_t s) {
+    int rc = launch_run_classes(b->run_jobs_dev, b->nrun, b->status_dev, s);
+    for (const auto &L : b->run_levels) {
+        if (rc != FZ_OK) break;
+        rc = launch_run_build(b->run_jobs_dev + L.first, L.jobs, L.K, false, L.blocks,
+                              b->status_dev, s);
+    }
+    return rc;
+}
+
 int batch_enqueue_rebuild(fz_batch_s *b, cudaStream_t s) {
     for (const auto &L : b->scan_launches) {
         int rc = launch_scan_tasks(b->jobs_dev, b->tasks_dev + L.first, L.second, s);
@@ -300,7 +322,7 @@ int batch_enqueue_rebuild(fz_batch_s *b, cudaStream_t s) {
     int rc = launch_memo_cta_build(b->memo_jobs_dev, b->nmemo, b->memo_ncoop, b->memo_claim,
                                    b->status_dev, s);
     if (rc != FZ_OK) return rc;
-    return launch_run_memo_batch(b->run_jobs_dev, b->nrun, b->run_blocks, b->status_dev, s);
+    return batch_enqueue_runs(b, s);
 }
 
 __global__ void gather_kernel(const uint64_t *const *ptrs, uint64_t *out, int count) {
@@ -327,33 +349,15 @@ int gather(const std::vector<const uint64_t *> &ptrs, std::vector<uint64_t> &out
     return FZ_OK;
 }
 
-// Memo depth of a batch instance, chosen for the largest element n_set
-// asked of the same generators in the batch (so instances of one generator
-// set share one memo).  A memo's rows are estimated by the volume
-// top^K / (K! prod tail), with top = min(n_set + 1, batch_memo_batches()
-// elementwise batches of min(tail) elements).  Preferred: the deepest full
-// memo (top > n_set) of depth >= 3 within BATCH_MEMO_MAX_ROWS rows and
-// cap_rows times the instance's estimated rows (volume n^(d-1) / ((d-1)!
-// prod g)) -- the deeper the memo, the fewer prefixes the walk visits.  Otherwise, for
-// d >= 5, a partial memo of depth 3 within BATCH_MEMO_MAX_ROWS rows (the
-// pair memo's leaves, prefixes of length d - 2, would be mostly empty
-// there: the d = 5 instances of a 4096-instance batch took 11.3 ms with it,
-// 2 ms with depth
-// 3).  Otherwise the pair memo: depth 2, full, as the closed form of
-// Z(p, (g_{d-2}, g_{d-1})) -- no table to build, and its leaves are
-// evaluated 32 at a time.
-// Estimated |Z(n, g)|: the volume n^(d-1) / ((d-1)! prod g).
-double volume_rows(const Inst &I, int n) {
-    double count = 1.0 / (double)I.g[I.d - 1];
-    for (int i = 0; i < I.d - 1; ++i) count *= (double)n / (double)(i + 1) / (double)I.g[i];
-    return count;
+// Lattice points x_1 g_1 + .. + x_m g_m <= n (slack: with an unbounded unit
+// coordinate) or = n: about n'^e / (e! prod g), n' = n plus half the weights.
+double lattice_volume(const int32_t *g, int m, double n, bool slack) {
+    double x = n + (slack ? 0.5 : 0.0), v = 1.0;
+    for (int i = 0; i < m; ++i) x += 0.5 * g[i];
+    const int e = slack ? m : m - 1;
+    for (int i = 0; i < e; ++i) v *= x / (double)(i + 1) / (double)g[i];
+    return slack ? v : v / (double)g[m - 1];
 }
-
-// Run-order memos of the pair's closed form are kept within this many times
-// the instance's estimated rows: they cost 16 bytes a row, built in one
-// fully parallel pass, and replace memo leaves of one to three rows that
-// cost about 12 warp instructions per output row.
-constexpr double RUN_PAIR_CAP = 2.0;
 
 // FZ_BATCH_ORDER=0 numbers the work items in the caller's instance order
 // (tuning only; see the item numbering in batch_create_impl).
@@ -366,8 +370,8 @@ bool batch_item_order_enabled() {
 }
 
 // How a batch chooses memos, per tuple width d: the memo rows allowed per
-// estimated instance row (cap_rows, see choose_batch_memo) and whether full
-// memos of depth <= 3 are also kept in run order.  The defaults are the
+// estimated instance row (cap_rows, see choose_batch_memo) and whether memos
+// are kept in run order.  The defaults are the
 // hand-set rule; fz_batch_autotune replaces them per device by the fastest
 // measured candidates.
 struct BatchPolicy {
@@ -399,6 +403,47 @@ BatchPolicy current_policy() {
     return it == g_policy.end() ? default_policy() : it->second;
 }
 
+// Memo depth of a batch instance, chosen for the largest element n_set asked
+// of the same generators in the batch (so instances of one generator set
+// share one table).
+//
+// Run order (widths 3..8): the depth with the least estimated work in warp
+// instructions -- 3.5 per leaf (prefix of d - 1 - K coordinates), 1.6 per
+// 16 bytes of table row and 3.5 per element of every level -- or the closed
+// form of the last two generators with no table at all (5 per prefix of
+// d - 2 coordinates).  A table's rows stay within BATCH_MEMO_MAX_ROWS and
+// cap_rows times the instance's estimated rows.
+void choose_batch_run(Inst &I, int n_set, double cap_rows) {
+    const int d = I.d;
+    const double count = lattice_volume(I.g, d, n_set, false);
+    I.K = 2;
+    I.pair = true;
+    I.top = I.n + 1;
+    double best = 5.0 * lattice_volume(I.g, d - 2, n_set, true);
+    double build = 0;
+    for (int K = 2; K <= d - 2 && K <= RUN_MAX_K; ++K) {
+        const double rows = K == 2 ? (double)pair_rows_upto(n_set, I.g[d - 2], I.g[d - 1])
+                                   : lattice_volume(I.g + (d - K), K, n_set, true);
+        if (rows > BATCH_MEMO_MAX_ROWS || rows > cap_rows * count + 4096.0) break;
+        build += 0.4 * rows * run_stride(K + 1) + 3.5 * n_set;
+        const int lam = d - 1 - K;
+        if (!flat_serves(d, lam, SRC_RUN)) continue;
+        const double work = build + 3.5 * lattice_volume(I.g, lam, n_set, true);
+        if (work < best) {
+            best = work;
+            I.K = K;
+            I.pair = false;
+        }
+    }
+}
+
+// Element order: a memo's rows are estimated by the volume top^K / (K! prod
+// tail), with top = min(n_set + 1, batch_memo_batches() elementwise batches of
+// min(tail) elements).  Preferred: the deepest full memo (top > n_set) of
+// depth >= 3 within BATCH_MEMO_MAX_ROWS rows and cap_rows times the instance's
+// estimated rows.  Otherwise, for d >= 5, a partial memo of depth 3 within
+// BATCH_MEMO_MAX_ROWS rows.  Otherwise the pair memo: depth 2, full, as the
+// closed form of Z(p, (g_{d-2}, g_{d-1})), no table.
 void choose_batch_memo(Inst &I, int n_set, double cap_rows) {
     I.K = 0;
     I.top = 0;
@@ -461,6 +506,143 @@ int fz_batch_create(const fz_instance_t *inst, int count, const fz_opts_t *opt,
 namespace fz {
 namespace {
 
+// Run-order tables of the batch (4096 instances of widths 3..8, 4.2e8 rows:
+// 1.08 ms for every table against 3.81 ms for one CTA per element-order memo
+// and 1.02 ms for their copies in run order; 96 small instances 0.06 against
+// 0.52 ms, bound there by the launches).  For every instance in run order the chain
+// from depth 2 (or 1) up to its own depth, one table per distinct suffix of
+// generators, built for the largest element any instance asks of it.
+int batch_create_runs(fz_batch_s *b, uint64_t *tb, cudaStream_t s) {
+    struct Table {
+        int K, src, n;   // depth, source instance, last element
+        bool final = false;
+    };
+    std::map<std::vector<int32_t>, int> of;
+    std::vector<Table> tab;
+    std::vector<std::vector<int32_t>> gens;
+    for (int i = 0; i < (int)b->inst.size(); ++i) {
+        Inst &I = b->inst[i];
+        if (!I.run) continue;
+        ++b->run_inst;
+        const int lam = I.d - I.K - 1, last = I.K == 1 ? lam : I.d - 3;
+        for (int j = lam; j <= last; ++j) {
+            std::vector<int32_t> key(I.g + j, I.g + I.d);
+            auto it = of.emplace(key, (int)tab.size());
+            if (it.second) {
+                tab.push_back({I.d - 1 - j, i, I.n});
+                gens.push_back(key);
+            } else if (I.n > tab[it.first->second].n) {
+                tab[it.first->second].n = I.n;
+                tab[it.first->second].src = i;
+            }
+            if (j == lam) {
+                tab[it.first->second].final = true;
+                I.run_job = it.first->second;
+            }
+        }
+    }
+    const int m = (int)tab.size();
+    b->nrun = m;
+    if (m == 0) return FZ_OK;
+    // jobs in build order: by depth
+    std::vector<int> order(m), at(m);
+    for (int t = 0; t < m; ++t) order[t] = t;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return tab[x].K < tab[y].K; });
+    for (int p = 0; p < m; ++p) at[order[p]] = p;
+    std::vector<RunBuild> rj(m);
+    size_t cls_words = 0;
+    for (int p = 0; p < m; ++p) {
+        const Table &T = tab[order[p]];
+        const std::vector<int32_t> &g = gens[order[p]];
+        const Inst &S = b->inst[T.src];
+        fill_run_build(g.data(), (int)g.size(), T.n, 0, false, &rj[p]);
+        rj[p].F = tb + S.off_C + (size_t)(S.d - (int)g.size()) * ((size_t)S.n + 1);
+        cls_words += a256(((size_t)rj[p].G + 1) * 8) / 8;
+    }
+    // rows of every table, then memory and the build
+    DevArena sizes;
+    const size_t jb = a256((size_t)m * sizeof(RunBuild));
+    int rc = sizes.alloc(jb + (size_t)m * 8);
+    if (rc != FZ_OK) return rc;
+    RunBuild *tj = static_cast<RunBuild *>(sizes.p);
+    uint64_t *td = reinterpret_cast<uint64_t *>(static_cast<char *>(sizes.p) + jb);
+    std::vector<uint64_t> rows(m);
+    FZ_CUDA_TRY(cudaMemcpyAsync(tj, rj.data(), (size_t)m * sizeof(RunBuild),
+                                cudaMemcpyHostToDevice, s));
+    rc = launch_run_totals(tj, m, td, s);
+    if (rc != FZ_OK) return rc;
+    FZ_CUDA_TRY(cudaMemcpyAsync(rows.data(), td, (size_t)m * 8, cudaMemcpyDeviceToHost, s));
+    FZ_CUDA_TRY(cudaStreamSynchronize(s));
+    size_t bytes = jb + cls_words * 8;
+    for (int p = 0; p < m; ++p) {
+        if (rows[p] > MEMO_MAX_ROWS)
+            return set_error(FZ_EINVAL, "batch run-order memo too large");
+        rj[p].rows = rows[p];
+        bytes += a256((size_t)rows[p] * 4 * run_stride(tab[order[p]].K + 1) + 16);
+    }
+    rc = b->runs.alloc(bytes);
+    if (rc != FZ_OK) return rc;
+    char *base = static_cast<char *>(b->runs.p);
+    size_t off = jb;
+    for (int p = 0; p < m; ++p) {
+        rj[p].cls = reinterpret_cast<uint64_t *>(base + off);
+        off += a256(((size_t)rj[p].G + 1) * 8);
+    }
+    for (int p = 0; p < m; ++p) {
+        rj[p].dst = reinterpret_cast<int32_t *>(base + off);
+        off += a256((size_t)rows[p] * 4 * run_stride(tab[order[p]].K + 1) + 16);
+    }
+    DeviceProps dp;
+    rc = device_props(&dp);
+    if (rc != FZ_OK) return rc;
+    for (int p = 0; p < m;) {
+        const int K = tab[order[p]].K;
+        int e = p;
+        uint64_t cost = 0;
+        for (; e < m && tab[order[e]].K == K; ++e) cost += run_build_cost(rj[e], false);
+        const uint32_t share = run_build_share(cost, dp.sms);
+        uint64_t blocks = 0;
+        for (int q = p; q < e; ++q) {
+            RunBuild &R = rj[q];
+            if (K > 2) {
+                const std::vector<int32_t> &g = gens[order[q]];
+                const int src = at[of[std::vector<int32_t>(g.begin() + 1, g.end())]];
+                R.src.rows = rj[src].dst;
+                R.src.cls = rj[src].cls;
+                R.src.nrows = rows[src];
+            }
+            R.per_warp = share;
+            R.blk0 = (uint32_t)blocks;
+            const uint32_t nb = run_build_blocks(R, K, false);
+            blocks += nb;
+            if (nb > 1) ++b->run_wide;
+            if (tab[order[q]].final) {
+                ++b->run_final;
+                b->run_table_rows += R.rows;
+                if (K >= 3) ++b->run_deep;
+            }
+        }
+        if (blocks > 0x7fffffffull)
+            return set_error(FZ_EINVAL, "batch run-order memos too large");
+        b->run_levels.push_back({K, p, e - p, (uint32_t)blocks});
+        p = e;
+    }
+    b->run_jobs_dev = reinterpret_cast<RunBuild *>(base);
+    FZ_CUDA_TRY(cudaMemcpyAsync(b->run_jobs_dev, rj.data(), (size_t)m * sizeof(RunBuild),
+                                cudaMemcpyHostToDevice, s));
+    rc = batch_enqueue_runs(b, s);
+    if (rc != FZ_OK) return rc;
+    FZ_CUDA_TRY(cudaStreamSynchronize(s));  // rj is a host temporary
+    for (Inst &I : b->inst) {
+        if (!I.run) continue;
+        const RunBuild &R = rj[at[I.run_job]];
+        I.run_memo = reinterpret_cast<const int4 *>(R.dst);
+        I.cls_beg = R.cls;
+        I.run_rows = R.rows;
+    }
+    return FZ_OK;
+}
+
 int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt,
                       const BatchPolicy &pol, fz_batch_t *batch, cudaStream_t s) {
     if (!batch) return set_error(FZ_EINVAL, "batch: null pointer");
@@ -493,7 +675,13 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
         I.d = x.d;
         I.n = x.n;
         for (int j = 0; j < x.d; ++j) I.g[j] = x.g[j];
-        choose_batch_memo(I, n_set[std::vector<int32_t>(x.g, x.g + x.d)], pol.cap_rows[x.d]);
+        const int ns = n_set[std::vector<int32_t>(x.g, x.g + x.d)];
+        const bool runs = run_memo_enabled() && pol.run_order[I.d];
+        const bool part = opt && opt->top != FZ_AUTO && opt->top <= I.n;  // a partial memo
+        if (runs && !part && walk_progression_enabled() && I.d >= 3 && I.d <= 8)
+            choose_batch_run(I, ns, pol.cap_rows[x.d]);
+        else
+            choose_batch_memo(I, ns, pol.cap_rows[x.d]);
         if (opt && opt->k != FZ_AUTO) {
             if (opt->k < 0 || opt->k > x.d - 1)
                 return fail(set_error(FZ_EINVAL, "opts.k must be in 0..d-1 for every instance"));
@@ -509,25 +697,12 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
         }
         if (I.K > 0 && I.top <= 0) I.K = 0;
         if (I.K == 0) I.top = 0;
-        // run order: a full memo of depth 1..3 under at least one walked
-        // coordinate, width <= 8 (the batch walk's run copy); the pair's
-        // closed form gets a run-order table when that stays small
-        I.run = false;
-        if (run_memo_enabled() && pol.run_order[I.d] && I.K >= 1 && I.K <= 3 && I.top > I.n &&
-            I.d <= 8 &&
-            I.d - I.K - 1 >= 1) {
-            if (!I.pair) {
-                I.run = true;
-            } else {
-                const int ns = n_set[std::vector<int32_t>(x.g, x.g + x.d)];
-                const int64_t t0 = I.g[I.d - 2], t1 = I.g[I.d - 1];
-                if ((int64_t)ns / t0 < (int64_t)BATCH_MEMO_MAX_ROWS) {
-                    const double rows = (double)pair_rows_upto(ns, t0, t1);
-                    I.run = rows <= BATCH_MEMO_MAX_ROWS &&
-                            rows <= RUN_PAIR_CAP * volume_rows(I, ns) + 4096.0;
-                }
-            }
-        }
+        // run order also serves a caller's full memo under a walked
+        // coordinate (width <= 8): any depth where the flat walk has a kernel,
+        // depth 1..3 by the run copy
+        const int lam = I.d - I.K - 1;
+        I.run = runs && !I.pair && I.K >= 1 && I.top > I.n && I.d <= 8 && lam >= 1 &&
+                (flat_serves(I.d, lam, SRC_RUN) || I.K <= 3);
         const size_t len = (size_t)I.n + 1;
         I.off_C = words;
         words += (size_t)(I.d + 1) * len;
@@ -567,9 +742,7 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
     std::vector<int> memo_src;  // instance whose table rows feed the memo
     for (int i = 0; i < count; ++i) {
         Inst &I = b->inst[i];
-        // run-order instances of depth 1 and 2 take their rows from the
-        // tail's closed form: no element-order memo
-        if (I.K <= 0 || I.pair || (I.run && I.K <= 2)) continue;
+        if (I.K <= 0 || I.pair || I.run) continue;  // run-order tables: below
         std::vector<int32_t> key(I.g + (I.d - I.K), I.g + I.d);
         auto it = memo_of.find(key);
         int m;
@@ -685,105 +858,8 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
                                    b->status_dev, s);
         if (rc != FZ_OK) return fail(rc);
     }
-    // run-order memos, one per distinct (g_lam, tail) and source (memo or
-    // closed form), built for the largest element asked of it
-    {
-        std::map<std::vector<int32_t>, int> run_of;
-        std::vector<int> run_src;
-        for (int i = 0; i < count; ++i) {
-            Inst &I = b->inst[i];
-            if (!I.run) continue;
-            std::vector<int32_t> key(I.g + (I.d - I.K - 1), I.g + I.d);
-            key.push_back(I.pair ? -1 : I.K);
-            auto it = run_of.find(key);
-            if (it == run_of.end()) {
-                I.run_job = (int)run_src.size();
-                run_of[key] = I.run_job;
-                run_src.push_back(i);
-            } else {
-                I.run_job = it->second;
-                if (I.n > b->inst[run_src[I.run_job]].n) run_src[I.run_job] = i;
-            }
-            ++b->run_inst;
-        }
-        b->nrun = (int)run_src.size();
-        std::vector<RunJob> rj(b->nrun);
-        size_t bytes = a256((size_t)b->nrun * sizeof(RunJob));
-        for (int j = 0; j < b->nrun; ++j) {
-            const Inst &S = b->inst[run_src[j]];
-            RunJob &R = rj[j];
-            const int lam = S.d - S.K - 1;
-            const size_t len = (size_t)S.n + 1;
-            R.Clam = tb + S.off_C + (size_t)lam * len;
-            R.Cnext = tb + S.off_C + (size_t)(lam + 1) * len;
-            R.n = S.n;
-            R.g = S.g[lam];
-            R.G = (int32_t)std::min<int64_t>(R.g, (int64_t)S.n + 1);
-            R.k = S.K;
-            // depth 1 and 2: the tail's closed form (k = 1, one row when ta
-            // divides p; k = 2, the pair (t0, t1)); depth 3: rows copied from
-            // the element-order memo
-            if (S.K == 2) {
-                R.t0 = S.g[S.d - 2];
-                R.t1 = S.g[S.d - 1];
-                int64_t g1;
-                pair_params(R.t0, R.t1, &R.e, &R.h1, &g1, &R.inv);
-                R.expect_rows = pair_rows_upto(S.n, R.t0, R.t1);
-            } else if (S.K == 1) {
-                R.ta = S.g[S.d - 1];
-                R.expect_rows = (uint64_t)(S.n / R.ta) + 1;
-            } else if (S.K == 3) {
-                if (S.memo < 0 || b->memo_jobs[S.memo].top < S.n + 1)
-                    return fail(set_error(FZ_EINTERNAL, "run-order memo without its full memo"));
-                const MemoJob &M = b->memo_jobs[S.memo];
-                R.O = M.O;
-                R.rows = M.R;
-                R.expect_rows = M.rows;
-            } else {
-                return fail(set_error(FZ_EINTERNAL, "run-order memo of depth > 3"));
-            }
-            R.out_rows = R.expect_rows;
-            if (R.out_rows > MEMO_MAX_ROWS)
-                return fail(set_error(FZ_EINVAL, "batch run-order memo too large"));
-            bytes += a256((size_t)R.out_rows * 16 + 16) + a256(((size_t)R.G + 1) * 8);
-        }
-        if (b->nrun) {
-            rc = b->runs.alloc(bytes);
-            if (rc != FZ_OK) return fail(rc);
-            char *base = static_cast<char *>(b->runs.p);
-            size_t off = a256((size_t)b->nrun * sizeof(RunJob));
-            for (RunJob &R : rj) {
-                R.out = reinterpret_cast<int4 *>(base + off);
-                off += a256((size_t)R.out_rows * 16 + 16);
-                R.cls_beg = reinterpret_cast<uint64_t *>(base + off);
-                off += a256(((size_t)R.G + 1) * 8);
-            }
-            // block ranges of the row kernel (256 threads a block, a thread
-            // per element)
-            uint64_t bt = 0;
-            for (RunJob &R : rj) {
-                R.blk0 = bt;
-                bt += ((uint64_t)R.n + 256) / 256;
-            }
-            if (bt > 0x7fffffffull)
-                return fail(set_error(FZ_EINVAL, "batch run-order memos too large"));
-            b->run_blocks = bt;
-            b->run_jobs_dev = reinterpret_cast<RunJob *>(base);
-            FZ_CUDA_TRY(cudaMemcpyAsync(b->run_jobs_dev, rj.data(), rj.size() * sizeof(RunJob),
-                                        cudaMemcpyHostToDevice, s));
-            rc = launch_run_memo_batch(b->run_jobs_dev, b->nrun, b->run_blocks, b->status_dev, s);
-            if (rc != FZ_OK) return fail(rc);
-            FZ_CUDA_TRY(cudaStreamSynchronize(s));  // rj is a host temporary
-        }
-        for (int i = 0; i < count; ++i) {
-            Inst &I = b->inst[i];
-            if (!I.run) continue;
-            const RunJob &R = rj[I.run_job];
-            I.run_memo = R.out;
-            I.cls_beg = R.cls_beg;
-            I.run_rows = R.out_rows;
-        }
-    }
+    rc = batch_create_runs(b, tb, s);
+    if (rc != FZ_OK) return fail(rc);
     // counts and run totals
     std::vector<const uint64_t *> pc(count), pr(count);
     for (int i = 0; i < count; ++i) {
@@ -823,18 +899,21 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
     std::vector<uint64_t> item0(count + 1, 0);
     b->params_host.resize((size_t)count * pbytes);
     // Work items are numbered instance by instance in an order grouped by
-    // code path (run copy, walk up to width 8, wider walk) and then by width,
-    // so that warps taking consecutive items run the same code: warps of
-    // one SM mixing the paths evict each other's instructions.  The output
+    // width and then by code path (leaf length and source), so that warps
+    // taking consecutive items run the same code: warps of one SM mixing the
+    // paths evict each other's instructions.  The output
     // layout (word offsets) keeps the caller's order.
     std::vector<int> order(count);
     for (int i = 0; i < count; ++i) order[i] = i;
     if (batch_item_order_enabled()) {
-        auto path = [&](const Inst &I) { return I.run ? 0 : (I.d <= 8 ? 1 : 2); };
+        auto path = [&](const Inst &I) {
+            if (I.run) return I.d - I.K - 1;  // prefix words of its leaves
+            return I.pair ? 16 : I.d <= 8 ? 17 : 18;
+        };
         std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
             const Inst &A = b->inst[x], &B = b->inst[y];
-            if (path(A) != path(B)) return path(A) < path(B);
-            return A.d < B.d;
+            if (A.d != B.d) return A.d < B.d;
+            return path(A) < path(B);
         });
     }
     for (int pos = 0; pos < count; ++pos) {
@@ -896,15 +975,15 @@ extern "C" {
 int fz_batch_info(fz_batch_t b, fz_batch_info_t *info) {
     if (!b || !info) return set_error(FZ_EINVAL, "null pointer");
     info->count = b->count;
-    info->memos = b->nmemo;
+    info->memos = b->nmemo + b->run_deep;
     info->total_rows = b->total_rows;
     info->total_words = b->total_words;
     info->device_bytes =
         b->tables.bytes + b->scratch.bytes + b->memos.bytes + b->meta.bytes + b->runs.bytes;
     info->work_items = b->nitems;
     info->run_order = b->run_inst;
-    info->run_memos = b->nrun;
-    info->coop_memos = b->memo_ncoop;
+    info->run_memos = b->run_final;
+    info->coop_memos = b->memo_ncoop + b->run_wide;
     info->reserved = 0;
     return FZ_OK;
 }
@@ -1118,10 +1197,10 @@ int fz_batch_autotune(const fz_instance_t *inst, int count, fz_batch_tune_entry_
                     E.d = d;
                     E.run_order = cand.second ? 1 : 0;
                     E.instances = (int32_t)sub.size();
-                    E.memos = b->nmemo;
+                    E.memos = b->nmemo + b->run_final;
                     E.cap_rows = cand.first;
                     E.rows = b->total_rows;
-                    uint64_t mr = 0;
+                    uint64_t mr = b->run_table_rows;
                     for (const MemoJob &J : b->memo_jobs) mr += J.rows;
                     E.memo_rows = mr;
                     E.build_ms = b_ms;
@@ -1169,10 +1248,10 @@ int fz_batch_autotune(const fz_instance_t *inst, int count, fz_batch_tune_entry_
                 E.d = 0;            // the whole batch
                 E.run_order = tag;  // 0: the starting policy; w: after trying width w
                 E.instances = count;
-                E.memos = b->nmemo;
+                E.memos = b->nmemo + b->run_final;
                 E.cap_rows = -1.0;
                 E.rows = b->total_rows;
-                uint64_t mr = 0;
+                uint64_t mr = b->run_table_rows;
                 for (const MemoJob &J : b->memo_jobs) mr += J.rows;
                 E.memo_rows = mr;
                 E.build_ms = b_ms;

@@ -1048,163 +1048,7 @@ __global__ void __launch_bounds__(T, 1024 / T) memo_cluster_build_kernel(
     }
 }
 
-// ---------------------------------------------------------------------------
-// The memo in run order (declared in fz_internal.cuh).  The element p of
-// class c = p mod g_lam, q = p div g_lam, starts at
-//   cls_beg[c] + sum_{p' = c mod g, p' < p} |Z(p', tail)|
-//             = cls_beg[c] + C[lam][p] - C[lam+1][p]
-// because the rows of a class up to p are exactly Z(p, (g_lam, tail)).
-// ---------------------------------------------------------------------------
-constexpr int RUN_CB_THREADS = 1024;
-
-// Batches: one CTA per run job for its class starts.  The total must be the
-// memo's rows up to n (O[n + 1]), or the closed form's count.
-__global__ void __launch_bounds__(RUN_CB_THREADS) run_class_begin_batch_kernel(
-    const RunJob *__restrict__ jobs, int *status) {
-    __shared__ uint64_t sums[33];
-    const RunJob &J = jobs[blockIdx.x];
-    const uint64_t *Clam = J.Clam;
-    const int32_t n = J.n, g = J.g, G = J.G;
-    uint64_t carry = 0;
-    for (int base = 0; base < G; base += blockDim.x) {
-        const int c = base + (int)threadIdx.x;
-        uint64_t v = 0;
-        if (c < G) {
-            const int64_t last = c + (int64_t)((n - c) / g) * g;
-            v = __ldg(Clam + last);
-        }
-        uint64_t total;
-        const uint64_t ex = block_exclusive_scan(v, sums, &total);
-        if (c < G) J.cls_beg[c] = carry + ex;
-        carry += total;
-    }
-    if (threadIdx.x == 0) {
-        J.cls_beg[G] = carry;
-        const uint64_t want = J.O ? __ldg(J.O + (int64_t)n + 1) : J.expect_rows;
-        if (carry != want || carry > J.out_rows) atomicExch(status, (int)DEV_INTERNAL);
-    }
-}
-
-// Batches: a thread per element (these elements hold a few rows each), each
-// job owning the blocks [blk0, blk0 + ceil((n + 1) / 256)) of the launch.
-// Rows come from the element-order memo (O, rows), or from the closed form:
-// k = 1, the one row p / ta when ta divides p; k = 2, the progression of the
-// pair (t0, t1).
-__device__ __forceinline__ uint32_t pair_first(const RunJob &J, int64_t r, int64_t *atop) {
-    // rows of Z(r, (t0, t1)): a_{d-2} = atop, atop - h1, ..., >= 0 (none if
-    // atop < 0); r, t0 and h1 fit in 32 bits
-    *atop = -1;
-    if (r < 0) return 0;
-    const uint32_t ru = (uint32_t)r, e = (uint32_t)J.e, h1 = (uint32_t)J.h1;
-    const uint32_t re = ru / e;
-    if (re * e != ru) return 0;
-    const uint32_t astar = (uint32_t)((uint64_t)(re % h1) * (uint64_t)J.inv % h1);
-    const uint32_t q0 = ru / (uint32_t)J.t0;
-    if (q0 < astar) return 0;
-    const uint32_t top = q0 - (q0 - astar) % h1;
-    *atop = top;
-    return top / h1 + 1u;
-}
-
-// The job of block `blk` for a kernel whose jobs own the consecutive block
-// ranges [blk0(j), blk0(j + 1)) (blk0 non-decreasing; jobs owning no block
-// have equal starts): the last job whose range starts at or before blk.
-template <class F>
-__device__ __forceinline__ int job_of_block(int njobs, uint64_t blk, F blk0) {
-    int lo = 0, hi = njobs;  // blk0(lo) <= blk < blk0(hi) (blk0(njobs) = total)
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (blk0(mid) <= blk)
-            lo = mid;
-        else
-            hi = mid;
-    }
-    return lo;
-}
-
-__global__ void __launch_bounds__(THREADS) run_rows_batch_kernel(const RunJob *__restrict__ jobs,
-                                                                 int njobs, int *status) {
-    __shared__ int s_job;
-    if (threadIdx.x == 0)
-        s_job = job_of_block(njobs, blockIdx.x, [&](int j) { return jobs[j].blk0; });
-    __syncthreads();
-    {
-        const RunJob &J = jobs[s_job];
-        const int64_t g = J.g;
-        const int64_t p = (int64_t)(blockIdx.x - J.blk0) * blockDim.x + threadIdx.x;
-        if (p <= J.n) {
-            const int64_t q = p / g, c = p - q * g;
-            const uint64_t tail_rows = __ldg(J.Cnext + p);
-            const uint64_t dst = __ldg(J.cls_beg + c) + __ldg(J.Clam + p) - tail_rows;
-            if (dst + tail_rows > J.out_rows) {
-                atomicExch(status, (int)DEV_INTERNAL);
-                return;
-            }
-            int4 *o = J.out + dst;
-            if (J.O) {
-                const uint64_t o0 = __ldg(J.O + p), len = __ldg(J.O + p + 1) - o0;
-                if (len != tail_rows) {
-                    atomicExch(status, (int)DEV_INTERNAL);
-                    return;
-                }
-                const int k = J.k;
-                const int32_t *s = J.rows + o0 * (uint64_t)k;
-                // four rows' loads before their stores
-                uint64_t r = 0;
-                for (; r + 4 <= len; r += 4, s += 4 * k) {
-                    int4 v[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        v[u] = make_int4((int)q, __ldg(s + u * k), k > 1 ? __ldg(s + u * k + 1) : 0,
-                                         k > 2 ? __ldg(s + u * k + 2) : 0);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) o[r + u] = v[u];
-                }
-                for (; r < len; ++r, s += k)
-                    o[r] = make_int4((int)q, __ldg(s), k > 1 ? __ldg(s + 1) : 0,
-                                     k > 2 ? __ldg(s + 2) : 0);
-            } else if (J.k == 1) {
-                const uint64_t want = p % J.ta == 0 ? 1u : 0u;
-                if (want != tail_rows) {
-                    atomicExch(status, (int)DEV_INTERNAL);
-                    return;
-                }
-                if (want) o[0] = make_int4((int)q, (int)(p / J.ta), 0, 0);
-            } else {
-                int64_t atop;
-                const uint64_t want = pair_first(J, p, &atop);
-                if (want != tail_rows) {
-                    atomicExch(status, (int)DEV_INTERNAL);
-                    return;
-                }
-                // a0 falls by h1 = t1 / e a row, so the last coordinate
-                // (p - a0 t0) / t1 rises by t0 / e: one division an element
-                if (want > 0) {
-                    int64_t a0 = atop, b0 = (p - atop * J.t0) / J.t1;
-                    const int64_t bstep = J.t0 / J.e;
-                    for (uint64_t r = 0; r < want; ++r, a0 -= J.h1, b0 += bstep)
-                        o[r] = make_int4((int)q, (int)a0, (int)b0, 0);
-                }
-            }
-        }
-    }
-}
-
 }  // namespace
-
-int launch_run_memo_batch(const RunJob *jobs, int njobs, uint64_t blocks, int *status,
-                          cudaStream_t s) {
-    if (njobs <= 0) return FZ_OK;
-    if (!jobs || !status) return set_error(FZ_EINTERNAL, "run memo batch: missing device buffer");
-    run_class_begin_batch_kernel<<<njobs, RUN_CB_THREADS, 0, s>>>(jobs, status);
-    note_launch();
-    if (blocks > 0) {
-        run_rows_batch_kernel<<<(unsigned)blocks, THREADS, 0, s>>>(jobs, njobs, status);
-        note_launch();
-    }
-    FZ_CUDA_TRY(cudaGetLastError());
-    return FZ_OK;
-}
 
 int launch_memo_sizes(const MemoJob *jobs, int njobs, uint64_t *rows_out, cudaStream_t s) {
     if (njobs <= 0) return FZ_OK;

@@ -75,24 +75,16 @@ struct ElementWalk {
     __device__ __forceinline__ void next() { f = f <= 0x7fffffffu ? f + 32u : f; }
 };
 
-// The job that block `blk` belongs to: jobs own consecutive block ranges from
-// blk0 on (jobs owning no block have equal starts).
-__device__ __forceinline__ int build_job_of(const RunBuild *jobs, int njobs, uint32_t blk) {
-    int lo = 0, hi = njobs;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (jobs[mid].blk0 <= blk)
-            lo = mid;
-        else
-            hi = mid;
-    }
-    return lo;
-}
-
-// The job of this block into shared memory.
+// The job of this block into shared memory: jobs own consecutive block ranges
+// from blk0 on (jobs owning no block have equal starts).
 __device__ __forceinline__ void load_job(const RunBuild *jobs, int njobs, RunBuild &sj) {
     __shared__ int s_id;
-    if (threadIdx.x == 0) s_id = build_job_of(jobs, njobs, blockIdx.x);
+    if (threadIdx.x < 32) {
+        uint64_t first;
+        const uint32_t id = warp_last_le((uint32_t)njobs, blockIdx.x, (int)threadIdx.x, &first,
+                                         [&](uint32_t u) { return (uint64_t)jobs[u].blk0; });
+        if (threadIdx.x == 0) s_id = (int)id;
+    }
     __syncthreads();
     const uint32_t *src = reinterpret_cast<const uint32_t *>(jobs + s_id);
     uint32_t *dst = reinterpret_cast<uint32_t *>(&sj);
@@ -100,8 +92,41 @@ __device__ __forceinline__ void load_job(const RunBuild *jobs, int njobs, RunBui
     __syncthreads();
 }
 
-// Rows of one level: a warp writes the rows [item, + 1) x per_warp of its
-// job.  K: coordinates a row; CSR: the memo in element order (K packed
+// A place in a table: leaf f, which starts at row `base`, and a row of it.
+struct TablePlace {
+    uint32_t f;
+    uint64_t base, row;
+};
+
+// The row that cost x of a table falls on.  An element costs FLAT_LEAF_COST
+// and a row 1, so tables of far more elements than rows (short tails of long
+// ranges: 324 rows of 1106 elements) still spread over many warps.
+__device__ __forceinline__ TablePlace table_place(const RunBuild &J, uint64_t x, int lane) {
+    const uint32_t q1 = J.qn + 1u;
+    auto first = [&](uint32_t c) {  // flat index of class c's first element
+        return c <= J.rr ? c * q1 : (J.rr + 1u) * q1 + (c - J.rr - 1u) * J.qn;
+    };
+    uint64_t cc, ct;
+    const uint32_t c = warp_last_le((uint32_t)J.G, x, lane, &cc, [&](uint32_t u) {
+        return __ldg(J.cls + u) + FLAT_LEAF_COST * first(u);
+    });
+    const uint64_t *F = J.F + c;
+    const uint32_t g = (uint32_t)J.g, cnt = J.qn + (c <= J.rr ? 1u : 0u);
+    auto before = [&](uint32_t u) { return u == 0 ? 0ull : __ldg(F + (uint64_t)(u - 1) * g); };
+    const uint32_t t = warp_last_le(cnt, x - cc, lane, &ct, [&](uint32_t u) {
+        return before(u) + FLAT_LEAF_COST * u;
+    });
+    const uint64_t in = x - cc - ct, b = before(t);
+    const uint64_t size = __ldg(F + (uint64_t)t * g) - b;
+    const uint64_t o = in > FLAT_LEAF_COST ? in - FLAT_LEAF_COST : 0ull;
+    TablePlace pl;
+    pl.f = first(c) + t;
+    pl.base = cc - FLAT_LEAF_COST * first(c) + b;
+    pl.row = pl.base + (o < size ? o : size);
+    return pl;
+}
+
+// Rows of one level: a warp writes an even share (per_warp) of its job.  K: coordinates a row; CSR: the memo in element order (K packed
 // words a row), else a run-order table (quotient first).
 template <int K, int SRC, bool CSR>
 __global__ void __launch_bounds__(BT, 4)
@@ -112,10 +137,6 @@ __global__ void __launch_bounds__(BT, 4)
     const RunBuild &J = sj;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint64_t item = (uint64_t)(blockIdx.x - J.blk0) * BW + wid;
-    const uint64_t row0 = item * J.per_warp;
-    if (row0 >= J.rows) return;
-    const uint64_t rest = J.rows - row0;
-    const uint32_t left = rest < J.per_warp ? (uint32_t)rest : J.per_warp;
     constexpr int NP = CSR ? 0 : 1;
     constexpr int W = K;
     constexpr int DS = CSR ? K : run_stride(K + 1);
@@ -127,6 +148,11 @@ __global__ void __launch_bounds__(BT, 4)
     const bool aligned = ((uintptr_t)J.dst & 15u) == 0;
     uint64_t base = 0;
     if constexpr (CSR) {
+        // equal rows, in multiples of 32 (16-byte aligned bulk stores)
+        const uint64_t row0 = item * J.per_warp;
+        if (row0 >= J.rows) return;
+        const uint64_t rest = J.rows - row0;
+        const uint32_t left = rest < J.per_warp ? (uint32_t)rest : J.per_warp;
         const uint64_t *F = J.F;
         const uint32_t f = warp_last_le((uint32_t)J.n + 1u, row0, lane, &base, [&](uint32_t u) {
             return u == 0 ? 0ull : __ldg(F + u - 1);
@@ -135,21 +161,26 @@ __global__ void __launch_bounds__(BT, 4)
         flat_rows<NP, W, DS, SRC>(wk, base, (uint32_t)(row0 - base), J.src, J.dst, aligned, row0,
                                   left, desc, ring, B, status, pol, lane);
     } else {
-        uint64_t cb = 0;
-        const uint32_t c = warp_last_le((uint32_t)J.G, row0, lane, &cb,
-                                        [&](uint32_t u) { return __ldg(J.cls + u); });
-        const uint32_t cnt = J.qn + (c <= J.rr ? 1u : 0u);
-        const uint64_t *F = J.F + c;
-        const uint32_t g = (uint32_t)J.g;
-        const uint32_t t = warp_last_le(cnt, row0 - cb, lane, &base, [&](uint32_t u) {
-            return u == 0 ? 0ull : __ldg(F + (uint64_t)(u - 1) * g);
-        });
-        base += cb;
-        const uint32_t lim = (J.rr + 1u) * (J.qn + 1u);
-        const uint32_t f = c <= J.rr ? c * (J.qn + 1u) + t : lim + (c - J.rr - 1u) * J.qn + t;
-        ClassWalk wk{J, f + (uint32_t)lane};
-        flat_rows<NP, W, DS, SRC>(wk, base, (uint32_t)(row0 - base), J.src, J.dst, aligned, row0,
-                                  left, desc, ring, B, status, pol, lane);
+        // equal cost; a table's rows are whole 16-byte vectors, so a warp may
+        // start at any row
+        __shared__ uint64_t s_row[BW + 1];
+        const uint64_t total = J.rows + FLAT_LEAF_COST * ((uint64_t)J.n + 1u);
+        const uint64_t x = item * J.per_warp;
+        TablePlace pl{0, 0, J.rows};
+        if (x < total) pl = table_place(J, x, lane);
+        if (lane == 0) s_row[wid] = pl.row;
+        if (wid == 0) {
+            const uint64_t xe = (item + BW) * J.per_warp;
+            const uint64_t re = xe < total ? table_place(J, xe, lane).row : J.rows;
+            if (lane == 0) s_row[BW] = re;
+        }
+        __syncthreads();
+        const uint64_t end = s_row[wid + 1];
+        if (end <= pl.row) return;
+        ClassWalk wk{J, pl.f + (uint32_t)lane};
+        flat_rows<NP, W, DS, SRC>(wk, pl.base, (uint32_t)(pl.row - pl.base), J.src, J.dst, aligned,
+                                  pl.row, (uint32_t)(end - pl.row), desc, ring, B, status, pol,
+                                  lane);
     }
     if (lane == 0) bulk_wait_all();
     __syncwarp();
@@ -210,6 +241,27 @@ __global__ void __launch_bounds__(BT)
     }
 }
 
+// totals[i] = rows of job i's table (its classes' last count entries).
+__global__ void __launch_bounds__(BT)
+    run_totals_kernel(const RunBuild *__restrict__ jobs, uint64_t *__restrict__ totals) {
+    __shared__ uint64_t warp_sum[BW];
+    const RunBuild &J = jobs[blockIdx.x];
+    const int32_t n = J.n, g = J.g, G = J.G;
+    uint64_t acc = 0;
+    for (int c = threadIdx.x; c < G; c += BT) {
+        const uint64_t v = __ldg(J.F + (c + (int64_t)((n - c) / g) * g));
+        acc += v < (1ull << 32) ? v : (1ull << 32);  // as row_sums_kernel
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+    if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < BW; ++w) acc += warp_sum[w];
+        totals[blockIdx.x] = acc;
+    }
+}
+
 // sums[j] += the first `top` entries of row j (j = blockIdx.y) of a count
 // table, each entry clamped to 2^32: a sum below 2^32 is exact, and at most
 // 2^31 entries cannot wrap.
@@ -250,6 +302,14 @@ int launch_run_classes(const RunBuild *jobs_dev, int njobs, int *status, cudaStr
     return FZ_OK;
 }
 
+int launch_run_totals(const RunBuild *jobs_dev, int njobs, uint64_t *totals, cudaStream_t s) {
+    if (njobs <= 0) return FZ_OK;
+    run_totals_kernel<<<njobs, BT, 0, s>>>(jobs_dev, totals);
+    note_launch();
+    FZ_CUDA_TRY(cudaGetLastError());
+    return FZ_OK;
+}
+
 int launch_run_build(const RunBuild *jobs_dev, int njobs, int K, bool csr, uint32_t blocks,
                      int *status, cudaStream_t s) {
     if (njobs <= 0 || blocks == 0) return FZ_OK;
@@ -280,7 +340,7 @@ int launch_run_build(const RunBuild *jobs_dev, int njobs, int K, bool csr, uint3
     }
 }
 
-void fill_run_build(const int32_t *t, int k, int32_t n, int j, bool csr, int sms, RunBuild *out) {
+void fill_run_build(const int32_t *t, int k, int32_t n, int j, bool csr, RunBuild *out) {
     RunBuild &R = *out;
     R.n = n;
     const int K = csr ? k - j : k - 1 - j;  // coordinates of a row
@@ -297,17 +357,24 @@ void fill_run_build(const int32_t *t, int k, int32_t n, int j, bool csr, int sms
         R.src.pair = make_pair_form(t[leaf], t[leaf + 1]);
     else
         R.src.fg = make_fastdiv((uint32_t)t[leaf]);
-    // about four items a resident warp, of 256 to 8192 rows (multiples of 32
-    // rows: every bulk store of an aligned table starts on a 128-byte line)
-    uint64_t per = R.rows / ((uint64_t)sms * 32 * 4 + 1);
-    per = per < 256 ? 256 : per > 8192 ? 8192 : per;
-    R.per_warp = (uint32_t)((per + 31) & ~31ull);
 }
 
-uint32_t run_build_blocks(const RunBuild &R, int K) {
+uint64_t run_build_cost(const RunBuild &R, bool csr) {
+    return csr ? R.rows : R.rows + FLAT_LEAF_COST * ((uint64_t)R.n + 1u);
+}
+
+// A warp's share of a launch of `total` cost: about four shares a resident
+// warp, 256 to 8192 (a multiple of 32 rows).
+uint32_t run_build_share(uint64_t total, int sms) {
+    uint64_t per = total / ((uint64_t)sms * 32 * 4 + 1);
+    per = per < 256 ? 256 : per > 8192 ? 8192 : per;
+    return (uint32_t)((per + 31) & ~31ull);
+}
+
+uint32_t run_build_blocks(const RunBuild &R, int K, bool csr) {
     if (R.rows == 0) return 0;
     if (K == 1) return (uint32_t)(((uint64_t)R.n / R.src.fg.g + 1 + BT - 1) / BT);
-    const uint64_t items = (R.rows + R.per_warp - 1) / R.per_warp;
+    const uint64_t items = (run_build_cost(R, csr) + R.per_warp - 1) / R.per_warp;
     return (uint32_t)((items + BW - 1) / BW);
 }
 
@@ -380,14 +447,15 @@ int run_levels_init(const int32_t *t, int k, int32_t n, const uint64_t *sums, bo
         R.F = Ct + (int64_t)j * cs;
         R.cls = cls[j];
         R.dst = rows[j];
-        fill_run_build(t, k, n, j, false, dp.sms, &R);
+        fill_run_build(t, k, n, j, false, &R);
+        R.per_warp = run_build_share(run_build_cost(R, false), dp.sms);
         L->K[L->n] = k - 1 - j;
         if (j < last) {
             R.src.rows = rows[j + 1];
             R.src.cls = cls[j + 1];
             R.src.nrows = sums[j + 2];
         }
-        L->blocks[L->n] = run_build_blocks(R, L->K[L->n]);
+        L->blocks[L->n] = run_build_blocks(R, L->K[L->n], false);
         ++L->n;
     }
     L->tables = L->n;
@@ -400,12 +468,13 @@ int run_levels_init(const int32_t *t, int k, int32_t n, const uint64_t *sums, bo
         R.F = O + 1;
         R.cls = nullptr;
         R.dst = csr_rows;
-        fill_run_build(t, k, n, 0, true, dp.sms, &R);
+        fill_run_build(t, k, n, 0, true, &R);
+        R.per_warp = run_build_share(R.rows, dp.sms);
         R.src.rows = rows[0];
         R.src.cls = cls[0];
         R.src.nrows = sums[1];
         L->K[L->n] = k;
-        L->blocks[L->n] = run_build_blocks(R, k);
+        L->blocks[L->n] = run_build_blocks(R, k, true);
         ++L->n;
     }
     // the jobs are a host temporary: the copy from pageable memory returns

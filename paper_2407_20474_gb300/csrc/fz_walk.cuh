@@ -155,7 +155,7 @@ struct RunBuild {
     int32_t n;            // elements 0..n
     int32_t g, G;         // class generator, G = min(g, n + 1)
     uint32_t qn, rr;      // n div g, n mod g
-    uint32_t per_warp;    // rows a warp writes
+    uint32_t per_warp;    // a warp's share: rows (element order) or cost (tables)
     uint32_t blk0;
     FastDiv fq1, fq;      // division by qn + 1 and qn
 };
@@ -197,8 +197,11 @@ int run_levels_init(const int32_t *t, int k, int32_t n, const uint64_t *sums, bo
                     void *mem, RunLevels *L, cudaStream_t s);
 int launch_run_levels(const RunLevels &L, int *status, cudaStream_t s);
 // The pieces, for many chains at once (batches).
-void fill_run_build(const int32_t *t, int k, int32_t n, int j, bool csr, int sms, RunBuild *out);
-uint32_t run_build_blocks(const RunBuild &R, int K);
+void fill_run_build(const int32_t *t, int k, int32_t n, int j, bool csr, RunBuild *out);
+uint64_t run_build_cost(const RunBuild &R, bool csr);
+uint32_t run_build_share(uint64_t total, int sms);
+uint32_t run_build_blocks(const RunBuild &R, int K, bool csr);
+int launch_run_totals(const RunBuild *jobs_dev, int njobs, uint64_t *totals, cudaStream_t s);
 int launch_run_classes(const RunBuild *jobs_dev, int njobs, int *status, cudaStream_t s);
 int launch_run_build(const RunBuild *jobs_dev, int njobs, int K, bool csr, uint32_t blocks,
                      int *status, cudaStream_t s);

@@ -74,7 +74,6 @@ struct Inst {
     uint64_t count = 0, runs = 0;
     uint64_t W = 16;  // cost of one prefix counted by the runs table, in rows
     uint64_t word_off = 0;
-    uint64_t items = 0, slice_cost = 0, slice_rows = 0;
 };
 
 }  // namespace
@@ -114,7 +113,8 @@ struct fz_batch_s {
     int ctas_per_sm = 0;      // cap of the enumeration kernel (0: as many as fit)
     void *params_dev = nullptr;       // EnumParams images (out = word offset)
     uint64_t *item0_dev = nullptr;
-    unsigned long long *counter_dev = nullptr;
+    std::vector<BatchGroup> groups;   // instances by enumeration kernel
+    unsigned long long *counter_dev = nullptr;  // a work-item counter per group
     int *status_dev = nullptr;
     uint64_t nitems = 0;
     uint64_t total_rows = 0, total_words = 0;
@@ -357,16 +357,6 @@ double lattice_volume(const int32_t *g, int m, double n, bool slack) {
     const int e = slack ? m : m - 1;
     for (int i = 0; i < e; ++i) v *= x / (double)(i + 1) / (double)g[i];
     return slack ? v : v / (double)g[m - 1];
-}
-
-// FZ_BATCH_ORDER=0 numbers the work items in the caller's instance order
-// (tuning only; see the item numbering in batch_create_impl).
-bool batch_item_order_enabled() {
-    static const bool on = [] {
-        const char *e = getenv("FZ_BATCH_ORDER");
-        return !(e && e[0] == '0');
-    }();
-    return on;
 }
 
 // How a batch chooses memos, per tuple width d: the memo rows allowed per
@@ -785,7 +775,8 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
     const size_t o_params = a256(o_mjobs + (size_t)b->nmemo * sizeof(MemoJob));
     const size_t o_item0 = a256(o_params + (size_t)count * pbytes);
     const size_t o_misc = a256(o_item0 + ((size_t)count + 1) * 8);
-    const size_t o_mrows = a256(o_misc + 256);
+    const size_t o_count = a256(o_misc + 256);
+    const size_t o_mrows = a256(o_count + BATCH_MAX_GROUPS * sizeof(unsigned long long));
     rc = b->meta.alloc(a256(o_mrows + (size_t)b->nmemo * 8) + 256);
     if (rc != FZ_OK) return fail(rc);
     char *mb = static_cast<char *>(b->meta.p);
@@ -794,7 +785,7 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
     b->memo_jobs_dev = reinterpret_cast<MemoJob *>(mb + o_mjobs);
     b->params_dev = mb + o_params;
     b->item0_dev = reinterpret_cast<uint64_t *>(mb + o_item0);
-    b->counter_dev = reinterpret_cast<unsigned long long *>(mb + o_misc);
+    b->counter_dev = reinterpret_cast<unsigned long long *>(mb + o_count);
     b->status_dev = reinterpret_cast<int *>(mb + o_misc + 64);
     b->memo_claim = reinterpret_cast<unsigned *>(mb + o_misc + 128);
     uint64_t *mrows_dev = reinterpret_cast<uint64_t *>(mb + o_mrows);
@@ -880,7 +871,6 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
     DeviceProps dp;
     rc = device_props(&dp);
     if (rc != FZ_OK) return fail(rc);
-    uint64_t total_cost = 0;
     uint64_t word = 0;
     for (int i = 0; i < count; ++i) {
         Inst &I = b->inst[i];
@@ -891,39 +881,16 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
         I.word_off = word;
         word += I.count * (uint64_t)I.d;
         b->total_rows += I.count;
-        total_cost += I.count + I.W * I.runs;
     }
     b->total_words = word;
-    const uint64_t warps = (uint64_t)dp.sms * 16;
-    const uint64_t target = std::max<uint64_t>(4096, total_cost / (warps * 8 + 1));
-    std::vector<uint64_t> item0(count + 1, 0);
-    b->params_host.resize((size_t)count * pbytes);
-    // Work items are numbered instance by instance in an order grouped by
-    // width and then by code path (leaf length and source), so that warps
-    // taking consecutive items run the same code: warps of one SM mixing the
-    // paths evict each other's instructions.  The output
-    // layout (word offsets) keeps the caller's order.
-    std::vector<int> order(count);
-    for (int i = 0; i < count; ++i) order[i] = i;
-    if (batch_item_order_enabled()) {
-        auto path = [&](const Inst &I) {
-            if (I.run) return I.d - I.K - 1;  // prefix words of its leaves
-            return I.pair ? 16 : I.d <= 8 ? 17 : 18;
-        };
-        std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-            const Inst &A = b->inst[x], &B = b->inst[y];
-            if (A.d != B.d) return A.d < B.d;
-            return path(A) < path(B);
-        });
-    }
-    for (int pos = 0; pos < count; ++pos) {
-        const int i = order[pos];
+    // Parameter images in the caller's order, then grouped by enumeration
+    // kernel: the work items of a group are numbered instance by instance.
+    // The output layout (word offsets) keeps the caller's order.
+    std::vector<unsigned char> images((size_t)count * pbytes);
+    std::vector<uint64_t> costs((size_t)count);
+    for (int i = 0; i < count; ++i) {
         Inst &I = b->inst[i];
-        const uint64_t cost = I.count + I.W * I.runs;
-        I.items = I.count == 0 ? 0 : std::max<uint64_t>(1, (cost + target - 1) / target);
-        I.slice_cost = I.items ? (cost + I.items - 1) / I.items : 64;
-        I.slice_rows = I.items ? std::max<uint64_t>(4, (I.count + I.items - 1) / I.items) : 4;
-        item0[pos + 1] = item0[pos] + I.items;
+        costs[i] = I.count + I.W * I.runs;
         EnumLaunch L;
         L.C = tb + I.off_C;
         L.cs = (int64_t)I.n + 1;
@@ -952,9 +919,18 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
             L.lam_r = I.lam_r;
         }
         // out holds the word offset; the kernel adds the output base
-        fill_batch_params(L, reinterpret_cast<int32_t *>(I.word_off * 4), I.count, I.slice_rows,
-                          I.slice_cost, b->params_host.data() + (size_t)pos * pbytes);
+        fill_batch_params(L, reinterpret_cast<int32_t *>(I.word_off * 4), I.count,
+                          images.data() + (size_t)i * pbytes);
     }
+    std::vector<int> order;
+    batch_order(images.data(), pbytes, costs.data(), count, &order, &b->groups);
+    std::vector<uint64_t> item0((size_t)count + 1, 0);
+    b->params_host.resize((size_t)count * pbytes);
+    for (int pos = 0; pos < count; ++pos)
+        memcpy(b->params_host.data() + (size_t)pos * pbytes,
+               images.data() + (size_t)order[pos] * pbytes, pbytes);
+    batch_items(b->params_host.data(), pbytes, costs.data(), order.data(), &b->groups, dp.sms,
+                item0.data());
     b->nitems = item0[count];
     if (count) {
         FZ_CUDA_TRY(cudaMemcpyAsync(b->params_dev, b->params_host.data(), b->params_host.size(),
@@ -1020,9 +996,9 @@ int fz_batch_enumerate(fz_batch_t b, int32_t *out_dev, uint64_t out_capacity_wor
     if (!out_dev) return set_error(FZ_EINVAL, "out: null pointer");
     if (((uintptr_t)out_dev & 3u) != 0) return set_error(FZ_EINVAL, "out must be 4-byte aligned");
     if (out_capacity_words < b->total_words) return set_error(FZ_ENOSPC, "output capacity too small");
-    return launch_enumerate_batch(b->params_dev, b->item0_dev, b->count, b->nitems,
-                                  b->counter_dev, out_dev, static_cast<cudaStream_t>(stream),
-                                  b->ctas_per_sm);
+    return launch_enumerate_batch(b->params_dev, b->item0_dev, b->groups.data(),
+                                  (int)b->groups.size(), b->counter_dev, out_dev,
+                                  static_cast<cudaStream_t>(stream), b->ctas_per_sm);
 }
 
 int fz_batch_sync(fz_batch_t b, void *stream) {

@@ -29,7 +29,9 @@
 // ring of two halves and each full half is written to HBM with one bulk
 // (TMA) store, so the stream is written with 16-byte aligned, fully
 // coalesced transactions while the warp generates the next half.
+#include <algorithm>
 #include <cstring>
+#include <map>
 
 #include <cstdlib>
 
@@ -813,63 +815,11 @@ __device__ __noinline__ bool runs_slice_rt(const EnumParams &P, int32_t *ring, u
     return ok;
 }
 
-// The flat walk inside the batch kernel, one routine per shape (not inlined,
-// so no shape's registers weigh on another's).  Items are numbered by shape,
-// so the warps of an SM mostly run the same one.
-template <int D, int NP, int SRC>
-__device__ __noinline__ bool flat_batch_one(const EnumParams &P, unsigned char *mem,
-                                            uint64_t row0, uint64_t row1, uint64_t pol,
-                                            int lane) {
-    constexpr uint32_t B = flat_half_rows<NP, SRC, D>(RING_BYTES_PER_WARP);
-    static_assert(leaf_bytes<NP, SRC>() + 2 * (int)B * D * 4 <= RING_BYTES_PER_WARP, "ring");
-    return flat_slice<D, NP, SRC>(P, mem, B, row0, row1, pol, lane);
-}
-
-template <int D>
-__device__ __forceinline__ bool flat_batch_d(const EnumParams &P, unsigned char *mem,
-                                             uint64_t row0, uint64_t row1, uint64_t pol,
-                                             int lane) {
-    if (P.flat_src == SRC_PAIR)
-        return flat_batch_one<D, D - 2, SRC_PAIR>(P, mem, row0, row1, pol, lane);
-    if (P.flat_np == 1) return flat_batch_one<D, 1, SRC_RUN>(P, mem, row0, row1, pol, lane);
-    if constexpr (D >= 4)
-        if (P.flat_np == 2) return flat_batch_one<D, 2, SRC_RUN>(P, mem, row0, row1, pol, lane);
-    if constexpr (D >= 5)
-        if (P.flat_np == 3) return flat_batch_one<D, 3, SRC_RUN>(P, mem, row0, row1, pol, lane);
-    if (lane == 0) atomicExch(P.status, (int)DEV_INTERNAL);  // shapes the host never sends here
-    return false;
-}
-
-__device__ __forceinline__ bool flat_batch_slice(const EnumParams &P, unsigned char *mem,
-                                                 uint64_t row0, uint64_t row1, uint64_t pol,
-                                                 int lane) {
-    switch (P.d) {
-        case 3: return flat_batch_d<3>(P, mem, row0, row1, pol, lane);
-        case 4: return flat_batch_d<4>(P, mem, row0, row1, pol, lane);
-        case 5: return flat_batch_d<5>(P, mem, row0, row1, pol, lane);
-        case 6: return flat_batch_d<6>(P, mem, row0, row1, pol, lane);
-        case 7: return flat_batch_d<7>(P, mem, row0, row1, pol, lane);
-        default: return flat_batch_d<8>(P, mem, row0, row1, pol, lane);
-    }
-}
-
 // ---------------------------------------------------------------------------
-// Many instances in one persistent launch.  Work items (instance, slice) are
-// numbered consecutively, instance i owning items [item0[i], item0[i+1]); a
-// warp takes the next item from an atomic counter, finds its instance by a
-// binary search over item0, copies that instance's parameters into its own
-// shared-memory slot (when it changes) and runs the same slice routine as the
-// single-instance kernel with the tuple width read at run time.
+// Batches: the instances the flat walk has no kernel for (partial memos,
+// memos in element order, widths above 8, single blocks), any mix of widths in
+// one persistent launch with the tuple width read at run time.
 // ---------------------------------------------------------------------------
-struct BatchEnumParams {
-    const EnumParams *inst;   // per-instance parameters; `out` holds a byte offset
-    int32_t *out_base;        // output base the offsets are added to
-    const uint64_t *item0;    // count + 1 prefix of work items
-    int count;
-    uint64_t nitems;
-    unsigned long long *item_counter;
-};
-
 constexpr size_t BATCH_RING_BYTES = RING_BYTES_PER_WARP;
 
 __global__ void __launch_bounds__(ENUM_THREADS, 4)
@@ -887,34 +837,11 @@ __global__ void __launch_bounds__(ENUM_THREADS, 4)
     int cur = -1;
     for (;;) {
         unsigned long long item = 0;
-        if (lane == 0) item = atomicAdd(BP.item_counter, 1ull);
+        if (lane == 0) item = BP.item_lo + atomicAdd(BP.item_counter, 1ull);
         item = __shfl_sync(FULL, item, 0);
-        if (item >= BP.nitems) break;
-        // largest i with item0[i] <= item
-        int lo = 0, hi = BP.count;  // item0[lo] <= item < item0[hi]
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (__ldg(BP.item0 + mid) <= item)
-                lo = mid;
-            else
-                hi = mid;
-        }
-        if (lo != cur) {
-            const uint32_t *src = reinterpret_cast<const uint32_t *>(BP.inst + lo);
-            uint32_t *dst = reinterpret_cast<uint32_t *>(ep);
-            for (int w = lane; w < (int)(sizeof(EnumParams) / 4); w += 32) dst[w] = __ldg(src + w);
-            __syncwarp();
-            if (lane == 0) {
-                int32_t *o = reinterpret_cast<int32_t *>(reinterpret_cast<char *>(BP.out_base) +
-                                                         reinterpret_cast<uintptr_t>(ep->out));
-                ep->out = o;
-                ep->aligned = ((uintptr_t)o & 15u) == 0;
-            }
-            __syncwarp();
-            cur = lo;
-        }
+        if (item >= BP.item_hi) break;
+        const uint64_t s = batch_locate(BP, ep, cur, item, lane);
         const EnumParams &P = *ep;
-        const uint64_t s = item - __ldg(BP.item0 + lo);
         uint64_t row0, row1;
         if (P.RT) {
             const uint64_t cost_hi = cost_at(P, 0, P.n);
@@ -947,14 +874,10 @@ __global__ void __launch_bounds__(ENUM_THREADS, 4)
             }
             continue;
         }
-        // the flat walk where it has a kernel for the shape; else full memos
-        // in run order take the run copy, and the rest one walk for every
-        // width up to 8 (row loops unrolled to 8), the 16-wide one beyond
+        // full memos in run order take the run copy, the rest one walk for
+        // every width up to 8 (row loops unrolled to 8), the 16-wide one beyond
         bool ok;
-        if (P.flat_np)
-            ok = flat_batch_slice(P, smem_raw + (size_t)wid * BATCH_RING_BYTES, row0, row1, pol,
-                                  lane);
-        else if (P.run_memo)
+        if (P.run_memo)
             ok = runs_slice_rt(P, ring, (uint32_t)P.half_rows, row0, row1, pol, lane);
         else if (P.d <= 8)
             ok = enum_slice<0, -1, 8>(P, wp, ring, (uint32_t)P.half_rows, row0, row1, pol, lane);
@@ -1297,55 +1220,134 @@ int launch_unrank(const EnumLaunch &L, const uint64_t *ranks, uint64_t m, int32_
 size_t enum_params_bytes() { return sizeof(EnumParams); }
 
 // EnumParams of one batch instance (host-side image, copied to the device).
-void fill_batch_params(const EnumLaunch &L, int32_t *out, uint64_t count, uint64_t slice_rows,
-                       uint64_t slice_cost, void *dst) {
+// (its work items: batch_items)
+void fill_batch_params(const EnumLaunch &L, int32_t *out, uint64_t count, void *dst) {
     EnumParams P = make_params(L);
     P.dense_min = dense_min_for(true);
     P.out = out;
     P.rank_begin = 0;
     P.nrows = count;
     P.aligned = ((uintptr_t)out & 15u) == 0;
-    P.slice_rows = slice_rows < 4 ? 4 : ((slice_rows + 3) & ~3ull);
-    P.nslices = (count + P.slice_rows - 1) / P.slice_rows;
     P.half_rows = half_rows_for(L.d);
     if (L.d > 8) P.flat_np = 0;  // the batch kernel's flat walk: widths 3..8
-    P.slice_cost = slice_cost < 64 ? 64 : slice_cost;
     memcpy(dst, &P, sizeof(P));
 }
 
-int launch_enumerate_batch(const void *params_dev, const uint64_t *item0_dev, int count,
-                           uint64_t nitems, unsigned long long *item_counter, int32_t *out_base,
-                           cudaStream_t s, int ctas_per_sm) {
-    if (nitems == 0) return FZ_OK;
+uint32_t enum_params_shape(const void *image) {
+    EnumParams P;
+    memcpy(&P, image, sizeof(P));
+    return P.flat_np ? (uint32_t)(P.d << 8 | P.flat_np << 1 | P.flat_src) : 0u;
+}
+
+void batch_order(const unsigned char *images, size_t pb, const uint64_t *cost, int count,
+                 std::vector<int> *order, std::vector<BatchGroup> *groups) {
+    std::vector<uint32_t> shape((size_t)count);
+    std::map<uint32_t, uint64_t> total;
+    for (int i = 0; i < count; ++i) {
+        shape[(size_t)i] = enum_params_shape(images + (size_t)i * pb);
+        total[shape[(size_t)i]] += cost[i];
+    }
+    order->resize((size_t)count);
+    for (int i = 0; i < count; ++i) (*order)[(size_t)i] = i;
+    // the general kernel last: it is not one of the overlapped launches
+    std::stable_sort(order->begin(), order->end(), [&](int x, int y) {
+        const uint32_t a = shape[(size_t)x], b = shape[(size_t)y];
+        if (a == b) return false;
+        if (!a || !b) return !b;
+        return total[a] != total[b] ? total[a] > total[b] : a < b;
+    });
+    groups->clear();
+    for (int p = 0; p < count; ++p) {
+        const uint32_t k = shape[(size_t)(*order)[(size_t)p]];
+        if (groups->empty() || groups->back().shape != k)
+            groups->push_back({k, p, p, 0, 0});
+        groups->back().last = p + 1;
+    }
+}
+
+// Work items: 1/8 of a resident warp's share of the whole call, 512 to 2048 of
+// cost.  Small items keep the instances being written at any time few, so
+// that their tables stay in L2 (4096 instances of 1e2..1e6 rows, 4.3e8 in
+// all: 4.5 ms with items of 15400, 3.5 with 7700, 3.2 with 3900, 3.0 with
+// 1900), although an item starts with a dozen dependent loads (about 10 us).
+void batch_items(unsigned char *params, size_t pb, const uint64_t *cost, const int *order,
+                 std::vector<BatchGroup> *groups, int sms, uint64_t *item0) {
+    uint64_t total = 0;
+    for (const BatchGroup &G : *groups)
+        for (int p = G.first; p < G.last; ++p) total += cost[order[p]];
+    uint64_t target = total / ((uint64_t)sms * 24 * 8 + 1);
+    target = target < 512 ? 512 : target > 2048 ? 2048 : target;
+    item0[0] = 0;
+    for (BatchGroup &G : *groups) {
+        G.item_lo = item0[G.first];
+        for (int p = G.first; p < G.last; ++p) {
+            EnumParams P;
+            memcpy(&P, params + (size_t)p * pb, sizeof(P));
+            const uint64_t c = cost[order[p]];
+            const uint64_t items = P.nrows == 0 || c == 0 ? 0 : (c + target - 1) / target;
+            if (items) {
+                P.slice_cost = (c + items - 1) / items;
+                P.slice_rows = (P.nrows + items - 1) / items;
+                if (P.slice_cost < 64) P.slice_cost = 64;
+                P.slice_rows = P.slice_rows < 4 ? 4 : (P.slice_rows + 3) & ~3ull;
+                memcpy(params + (size_t)p * pb, &P, sizeof(P));
+            }
+            item0[p + 1] = item0[p] + items;
+        }
+        G.item_hi = item0[G.last];
+    }
+}
+
+int launch_enumerate_batch(const void *params_dev, const uint64_t *item0_dev,
+                           const BatchGroup *groups, int ngroups, unsigned long long *counters,
+                           int32_t *out_base, cudaStream_t s, int ctas_per_sm) {
+    if (ngroups <= 0) return FZ_OK;
+    if (ngroups > BATCH_MAX_GROUPS) return set_error(FZ_EINTERNAL, "batch: too many groups");
     DeviceProps dp;
     int rc = device_props(&dp);
     if (rc != FZ_OK) return rc;
-    const size_t smem = enum_batch_smem_bytes();
-    static DeviceOnce attr_set;
-    if (!attr_set.is_set(dp.device)) {
-        FZ_CUDA_TRY(cudaFuncSetAttribute(fz_enum_batch_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr_set.set(dp.device);
+    FZ_CUDA_TRY(cudaMemsetAsync(counters, 0, (size_t)ngroups * sizeof(unsigned long long), s));
+    bool chained = false;
+    for (int i = 0; i < ngroups; ++i) {
+        const BatchGroup &G = groups[i];
+        BatchEnumParams BP;
+        BP.inst = static_cast<const EnumParams *>(params_dev);
+        BP.out_base = out_base;
+        BP.item0 = item0_dev;
+        BP.first = G.first;
+        BP.last = G.last;
+        BP.item_lo = G.item_lo;
+        BP.item_hi = G.item_hi;
+        BP.item_counter = counters + i;
+        BP.chained = chained ? 1 : 0;
+        if (G.shape) {
+            rc = launch_flat_batch(BP, (int)(G.shape >> 8), (int)(G.shape >> 1 & 127),
+                                   (int)(G.shape & 1), s, dp.sms, ctas_per_sm);
+            if (rc != FZ_OK) return rc;
+            chained = true;
+            continue;
+        }
+        chained = false;
+        const size_t smem = (size_t)ENUM_WARPS *
+                            (BATCH_RING_BYTES + sizeof(EnumParams) + sizeof(WarpPath));
+        static DeviceOnce attr_set;
+        if (!attr_set.is_set(dp.device)) {
+            FZ_CUDA_TRY(cudaFuncSetAttribute(
+                fz_enum_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            attr_set.set(dp.device);
+        }
+        int per_sm = 0;
+        FZ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fz_enum_batch_kernel,
+                                                                  ENUM_THREADS, smem));
+        if (per_sm < 1) per_sm = 1;
+        if (ctas_per_sm > 0 && ctas_per_sm < per_sm) per_sm = ctas_per_sm;
+        uint64_t grid = (uint64_t)per_sm * dp.sms;
+        const uint64_t want = (G.item_hi - G.item_lo + ENUM_WARPS - 1) / ENUM_WARPS;
+        if (want < grid) grid = want;
+        fz_enum_batch_kernel<<<(unsigned)grid, ENUM_THREADS, smem, s>>>(BP);
+        note_launch();
+        FZ_CUDA_TRY(cudaGetLastError());
     }
-    int per_sm = 0;
-    FZ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fz_enum_batch_kernel,
-                                                              ENUM_THREADS, smem));
-    if (per_sm < 1) per_sm = 1;
-    if (ctas_per_sm > 0 && ctas_per_sm < per_sm) per_sm = ctas_per_sm;
-    uint64_t grid = (uint64_t)per_sm * dp.sms;
-    const uint64_t want = (nitems + ENUM_WARPS - 1) / ENUM_WARPS;
-    if (want < grid) grid = want;
-    BatchEnumParams BP;
-    BP.inst = static_cast<const EnumParams *>(params_dev);
-    BP.out_base = out_base;
-    BP.item0 = item0_dev;
-    BP.count = count;
-    BP.nitems = nitems;
-    BP.item_counter = item_counter;
-    FZ_CUDA_TRY(cudaMemsetAsync(item_counter, 0, sizeof(unsigned long long), s));
-    fz_enum_batch_kernel<<<(unsigned)grid, ENUM_THREADS, smem, s>>>(BP);
-    note_launch();
-    FZ_CUDA_TRY(cudaGetLastError());
     return FZ_OK;
 }
 

@@ -339,20 +339,46 @@ __device__ __forceinline__ void flush_rows(const EnumParams &P, const int32_t *s
     flush_words(P.out + out_row * (uint64_t)d, P.aligned, src, nrows * (uint32_t)d, lane, pol);
 }
 
+// Parameters of a launch as a walk and a sink read them: in constant memory
+// (a kernel parameter), or in the warp's shared memory, whose address is
+// hidden at every use so that nothing is kept in registers between uses.
+struct ConstParams {
+    const EnumParams &p;
+    __device__ __forceinline__ const EnumParams &operator()() const { return p; }
+};
+extern __shared__ __align__(128) unsigned char enum_smem[];
+struct SharedParams {
+    uint32_t off;  // from the start of the block's dynamic shared memory
+    __device__ __forceinline__ const EnumParams &operator()() const {
+        uint32_t o = off;
+        asm volatile("" : "+r"(o));
+        return *reinterpret_cast<const EnumParams *>(enum_smem + o);
+    }
+};
+template <class PA>
+struct EnumSink {
+    PA params;
+    __device__ __forceinline__ const LeafSource &src() const { return params().leaf; }
+    __device__ __forceinline__ int32_t *out() const { return params().out; }
+    __device__ __forceinline__ bool aligned() const { return params().aligned != 0; }
+    __device__ __forceinline__ int *status() const { return params().status; }
+};
+
 // The flat walk's leaves of an enumeration: the prefixes (a_0..a_{NP-1}) in
 // descending order, each lane at its own, 32 apart from one batch to the
 // next.  Row ends are absolute ranks: the rows of the greater prefixes of
 // every level (pb, read again when the parent changes) plus the count row of
 // the last prefix coordinate.
-template <int NP>
+template <int NP, class PA>
 struct PrefixWalk {
-    const EnumParams &P;
+    PA params;
     int a[NP], r[NP];  // r[j]: remainder before a_j
     uint64_t pb = 0;
     bool dead = false;
-    __device__ __forceinline__ explicit PrefixWalk(const EnumParams &p) : P(p) {}
+    __device__ __forceinline__ explicit PrefixWalk(const PA &pa) : params(pa) {}
 
     __device__ __forceinline__ void parents() {
+        const EnumParams &P = params();
         pb = 0;
 #pragma unroll
         for (int j = 0; j < NP - 1; ++j) {
@@ -368,6 +394,7 @@ struct PrefixWalk {
                 dead = true;
                 return;
             } else {
+                const EnumParams &P = params();
                 do {
                     const int owe = -x - 1;  // prefixes past the next parent's first
                     // the next parent: decrement its deepest positive
@@ -395,12 +422,12 @@ struct PrefixWalk {
         }
         a[NP - 1] = x;
     }
-    __device__ __forceinline__ bool leaf(uint32_t &p, uint64_t &E, int (&pre)[NP]) const {
+    __device__ __forceinline__ int word(int c) const { return a[c]; }
+    __device__ __forceinline__ bool leaf(uint32_t &p, uint64_t &E) const {
         if (dead) return false;
+        const EnumParams &P = params();
         p = (uint32_t)(r[NP - 1] - a[NP - 1] * P.g[NP - 1]);
         E = pb + __ldg(P.C + (int64_t)(NP - 1) * P.cs + p);
-#pragma unroll
-        for (int c = 0; c < NP; ++c) pre[c] = a[c];
         return true;
     }
     __device__ __forceinline__ void next() { step(32); }
@@ -408,11 +435,12 @@ struct PrefixWalk {
 
 // Rows [row0, row1) of an enumeration by the flat walk.  `mem`: the warp's
 // shared memory (leaf descriptors, then a ring of two halves of B rows).
-template <int D, int NP, int SRC>
-__device__ __forceinline__ bool flat_slice(const EnumParams &P, unsigned char *mem, uint32_t B,
+template <int D, int NP, int SRC, class PA>
+__device__ __forceinline__ bool flat_slice(const PA &pa, unsigned char *mem, uint32_t B,
                                            uint64_t row0, uint64_t row1, uint64_t pol, int lane) {
+    const EnumParams &P = pa();
     const uint64_t R = P.rank_begin + row0;
-    PrefixWalk<NP> wk(P);
+    PrefixWalk<NP, PA> wk(pa);
     uint64_t off = R;
     int rem = P.n;
 #pragma unroll
@@ -427,13 +455,124 @@ __device__ __forceinline__ bool flat_slice(const EnumParams &P, unsigned char *m
     wk.step(lane);
     int4 *desc = reinterpret_cast<int4 *>(mem);
     int32_t *ring = reinterpret_cast<int32_t *>(mem + leaf_bytes<NP, SRC>());
-    return flat_rows<NP, D - NP, D, SRC>(wk, R - off, (uint32_t)off, P.leaf, P.out, P.aligned != 0,
-                                         row0, (uint32_t)(row1 - row0), desc, ring, B, P.status,
-                                         pol, lane);
+    return flat_rows<NP, D - NP, D, SRC>(wk, R - off, (uint32_t)off, EnumSink<PA>{pa}, row0,
+                                         (uint32_t)(row1 - row0), desc, ring, B, pol, lane);
+}
+
+// Ranks at which the cumulative costs t0 <= t1 are reached (cost_to_rank for a
+// candidates table counted at level NP), both searches' loads in flight
+// together.
+template <int NP>
+__device__ __forceinline__ void flat_cost_to_ranks(const EnumParams &P, uint64_t t0, uint64_t t1,
+                                                   int lane, uint64_t &rank0, uint64_t &rank1) {
+    uint64_t tgt[2] = {t0, t1}, rank[2] = {0, 0};
+    uint32_t rem[2] = {(uint32_t)P.n, (uint32_t)P.n};
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+        const uint32_t g = (uint32_t)P.g[j];
+        const uint64_t *C = P.C + (int64_t)j * P.cs, *T = P.RT + (int64_t)j * P.cs;
+        uint32_t lo[2] = {0, 0}, hi[2], um[2];
+        uint64_t flo[2] = {0, 0}, clo[2] = {0, 0};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            um[k] = fd_div(rem[k], P.fdg[j]);
+            hi[k] = um[k] + 1u;
+        }
+        while (hi[0] - lo[0] > 1u || hi[1] - lo[1] > 1u) {
+            uint64_t cu[2] = {0, 0}, fu[2] = {0, 0};
+            uint32_t step[2];
+            bool in[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                step[k] = (hi[k] - lo[k] + 31) >> 5;
+                const uint64_t u = (uint64_t)lo[k] + (uint64_t)(lane + 1) * step[k];
+                in[k] = u < hi[k];
+                if (in[k]) {
+                    const uint32_t x = rem[k] - (um[k] + 1u - (uint32_t)u) * g;
+                    cu[k] = __ldg(C + x);
+                    fu[k] = __ldg(T + x);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                fu[k] = cu[k] + P.W * fu[k];
+                const int cnt = __popc(__ballot_sync(FULL, in[k] && fu[k] <= tgt[k]));
+                const int src = cnt > 0 ? cnt - 1 : 0;
+                const uint64_t fs = shfl_u64(fu[k], src), cs = shfl_u64(cu[k], src);
+                if (hi[k] - lo[k] > 1u) {
+                    if (cnt > 0) {
+                        flo[k] = fs;
+                        clo[k] = cs;
+                        lo[k] += (uint32_t)cnt * step[k];
+                    }
+                    if (lo[k] + step[k] < hi[k]) hi[k] = lo[k] + step[k];
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            rank[k] += clo[k];
+            tgt[k] -= flo[k];
+            rem[k] -= (um[k] - lo[k]) * g;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const uint64_t rows = __ldg(P.C + (int64_t)NP * P.cs + rem[k]);
+        const uint64_t t = tgt[k] > P.W ? tgt[k] - P.W : 0ull;
+        rank[k] += t < rows ? t : rows;
+    }
+    rank0 = rank[0];
+    rank1 = rank[1];
+}
+
+// ---------------------------------------------------------------------------
+// Many instances.  Work items (instance, slice) are numbered consecutively,
+// instance i owning items [item0[i], item0[i+1]); a launch covers the
+// instances [first, last) -- those of one shape, or all the general kernel
+// takes -- and its warps take items from an atomic counter, copying the
+// instance's parameters into their own shared-memory slot when it changes.
+// ---------------------------------------------------------------------------
+struct BatchEnumParams {
+    const EnumParams *inst;   // per-instance parameters; `out` holds a byte offset
+    int32_t *out_base;        // output base the offsets are added to
+    const uint64_t *item0;    // prefix of work items over all instances
+    int first, last;
+    uint64_t item_lo, item_hi;  // items of this launch
+    unsigned long long *item_counter;
+    int chained;              // launched to overlap the launch before it
+};
+
+// Instance of `item`, its parameters in *ep.
+__device__ __forceinline__ uint64_t batch_locate(const BatchEnumParams &BP, EnumParams *ep,
+                                                 int &cur, uint64_t item, int lane) {
+    uint64_t start;
+    const int id = BP.first + (int)warp_last_le((uint32_t)(BP.last - BP.first), item, lane, &start,
+                                                [&](uint32_t u) {
+                                                    return __ldg(BP.item0 + BP.first + u);
+                                                });
+    if (id != cur) {
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(BP.inst + id);
+        uint32_t *dst = reinterpret_cast<uint32_t *>(ep);
+        __syncwarp();
+        for (int w = lane; w < (int)(sizeof(EnumParams) / 4); w += 32) dst[w] = __ldg(src + w);
+        __syncwarp();
+        if (lane == 0) {
+            int32_t *o = reinterpret_cast<int32_t *>(reinterpret_cast<char *>(BP.out_base) +
+                                                     reinterpret_cast<uintptr_t>(ep->out));
+            ep->out = o;
+            ep->aligned = ((uintptr_t)o & 15u) == 0;
+        }
+        __syncwarp();
+        cur = id;
+    }
+    return item - start;
 }
 
 // fz_flat.cu
 int launch_enum_flat(const EnumParams &P, int warp_bytes, cudaStream_t s, int sms);
+int launch_flat_batch(const BatchEnumParams &BP, int d, int np, int src, cudaStream_t s, int sms,
+                      int ctas_per_sm);
 // fz_enum.cu: grid and launch of a persistent enumeration kernel.
 constexpr int ENUM_MAX_SMEM = 200 * 1024;
 template <typename Kern, typename... Args>

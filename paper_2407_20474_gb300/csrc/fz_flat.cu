@@ -19,10 +19,9 @@ namespace {
 template <int D, int NP, int SRC>
 __global__ void __launch_bounds__(ENUM_THREADS, 4)
     fz_enum_flat_kernel(const __grid_constant__ EnumParams P, int warp_bytes) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
-    unsigned char *mem = smem_raw + (size_t)wid * warp_bytes;
+    unsigned char *mem = enum_smem + (size_t)wid * warp_bytes;
     const uint64_t pol = policy_evict_first();
     uint64_t cost_lo = 0, cost_hi = 0;
     if (P.RT) {
@@ -37,7 +36,9 @@ __global__ void __launch_bounds__(ENUM_THREADS, 4)
         const int it = item_rows(P, s, cost_lo, cost_hi, lane, row0, row1);
         if (it == 0) break;
         if (it == 1) continue;
-        if (!flat_slice<D, NP, SRC>(P, mem, (uint32_t)P.half_rows, row0, row1, pol, lane)) break;
+        if (!flat_slice<D, NP, SRC>(ConstParams{P}, mem, (uint32_t)P.half_rows, row0, row1, pol,
+                                    lane))
+            break;
     }
     if (lane == 0) bulk_wait_all();
     __syncwarp();
@@ -51,6 +52,107 @@ int launch_one(EnumParams P, int warp_bytes, cudaStream_t s, int sms) {
     const int bytes = (need > warp_bytes ? need : warp_bytes + 127) & ~127;
     auto kern = fz_enum_flat_kernel<D, NP, SRC>;
     return launch_enum_grid(kern, P, (size_t)ENUM_WARPS * bytes, s, sms, attr_set, bytes);
+}
+
+// The flat walk of a batch's instances of one shape.  A launch may start while
+// the one before it drains (chained): it reads nothing that one writes, and
+// waits for its completion only before it ends, so the last launch's end is
+// the end of all.  Three blocks an SM: at 64 registers the loops spill (see
+// flat_rows), 4 blocks of them are no faster.
+template <int D, int NP, int SRC>
+__global__ void __launch_bounds__(ENUM_THREADS, 3)
+    fz_flat_batch_kernel(const __grid_constant__ BatchEnumParams BP) {
+    const int lane = threadIdx.x & 31;
+    const int wid = threadIdx.x >> 5;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    unsigned char *mem = enum_smem + (size_t)wid * RING_BYTES_PER_WARP;
+    const SharedParams params{(uint32_t)(ENUM_WARPS * RING_BYTES_PER_WARP + wid * sizeof(EnumParams))};
+    EnumParams *ep = reinterpret_cast<EnumParams *>(enum_smem + params.off);
+    constexpr uint32_t B = flat_half_rows<NP, SRC, D>(RING_BYTES_PER_WARP);
+    static_assert(leaf_bytes<NP, SRC>() + 2 * (int)B * D * 4 <= RING_BYTES_PER_WARP, "ring");
+    const uint64_t pol = policy_evict_first();
+    int cur = -1;
+    unsigned long long next = 0;
+    if (lane == 0) next = atomicAdd(BP.item_counter, 1ull);
+    for (;;) {
+        const uint64_t item = BP.item_lo + __shfl_sync(FULL, next, 0);
+        if (item >= BP.item_hi) break;
+        if (lane == 0) next = atomicAdd(BP.item_counter, 1ull);  // read after this item
+        const uint64_t s = batch_locate(BP, ep, cur, item, lane);
+        const EnumParams &P = params();
+        uint64_t row0, row1;
+        if (P.RT) {
+            const uint64_t cost_hi = cost_at(P, 0, P.n);
+            const uint64_t c0 = s * P.slice_cost, c1 = c0 + P.slice_cost;
+            if (c0 >= cost_hi) continue;
+            row0 = 0;
+            row1 = P.nrows;
+            if (s > 0 || c1 < cost_hi) {
+                uint64_t r0, r1;
+                flat_cost_to_ranks<NP>(P, c0, c1 < cost_hi ? c1 : c0, lane, r0, r1);
+                if (s > 0) row0 = r0 & ~31ull;
+                if (c1 < cost_hi) row1 = r1 & ~31ull;
+                if (row0 > P.nrows) row0 = P.nrows;
+                if (row1 > P.nrows) row1 = P.nrows;
+            }
+        } else {
+            row0 = s * P.slice_rows;
+            row1 = row0 + P.slice_rows < P.nrows ? row0 + P.slice_rows : P.nrows;
+        }
+        if (row1 <= row0) continue;
+        if (!flat_slice<D, NP, SRC>(params, mem, B, row0, row1, pol, lane)) break;
+    }
+    if (lane == 0) bulk_wait_all();
+    __syncwarp();
+    if (BP.chained) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <int D, int NP, int SRC>
+int launch_batch_one(const BatchEnumParams &BP, cudaStream_t s, int sms, int ctas_per_sm) {
+    auto kern = fz_flat_batch_kernel<D, NP, SRC>;
+    constexpr size_t smem = (size_t)ENUM_WARPS * (RING_BYTES_PER_WARP + sizeof(EnumParams));
+    static DeviceOnce attr_set;
+    static int occupancy[64];
+    int dev = 0;
+    FZ_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return set_error(FZ_EINVAL, "device ordinal out of range");
+    if (!attr_set.is_set(dev)) {
+        FZ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem));
+        FZ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occupancy[dev], kern,
+                                                                  ENUM_THREADS, smem));
+        attr_set.set(dev);
+    }
+    int per_sm = occupancy[dev] < 1 ? 1 : occupancy[dev];
+    if (ctas_per_sm > 0 && ctas_per_sm < per_sm) per_sm = ctas_per_sm;
+    uint64_t grid = (uint64_t)per_sm * sms;
+    const uint64_t want = (BP.item_hi - BP.item_lo + ENUM_WARPS - 1) / ENUM_WARPS;
+    if (want < grid) grid = want;
+    if (grid < 1) return FZ_OK;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(ENUM_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = BP.chained ? 1 : 0;
+    FZ_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, BP));
+    note_launch();
+    return FZ_OK;
+}
+
+template <int D>
+int launch_batch_d(const BatchEnumParams &BP, int np, int src, cudaStream_t s, int sms, int cap) {
+    if (src == SRC_PAIR) return launch_batch_one<D, D - 2, SRC_PAIR>(BP, s, sms, cap);
+    if (np == 1) return launch_batch_one<D, 1, SRC_RUN>(BP, s, sms, cap);
+    if constexpr (D >= 4)
+        if (np == 2) return launch_batch_one<D, 2, SRC_RUN>(BP, s, sms, cap);
+    if constexpr (D >= 5)
+        if (np == 3) return launch_batch_one<D, 3, SRC_RUN>(BP, s, sms, cap);
+    return set_error(FZ_EINTERNAL, "flat walk: no kernel for this shape");
 }
 
 template <int D>
@@ -86,6 +188,19 @@ int launch_enum_flat(const EnumParams &P, int warp_bytes, cudaStream_t s, int sm
         case 7: return launch_d<7>(P, warp_bytes, s, sms);
         case 8: return launch_d<8>(P, warp_bytes, s, sms);
         case 9: return launch_d<9>(P, warp_bytes, s, sms);
+        default: return set_error(FZ_EINTERNAL, "flat walk: no kernel for this shape");
+    }
+}
+
+int launch_flat_batch(const BatchEnumParams &BP, int d, int np, int src, cudaStream_t s, int sms,
+                      int ctas_per_sm) {
+    switch (d) {
+        case 3: return launch_batch_d<3>(BP, np, src, s, sms, ctas_per_sm);
+        case 4: return launch_batch_d<4>(BP, np, src, s, sms, ctas_per_sm);
+        case 5: return launch_batch_d<5>(BP, np, src, s, sms, ctas_per_sm);
+        case 6: return launch_batch_d<6>(BP, np, src, s, sms, ctas_per_sm);
+        case 7: return launch_batch_d<7>(BP, np, src, s, sms, ctas_per_sm);
+        case 8: return launch_batch_d<8>(BP, np, src, s, sms, ctas_per_sm);
         default: return set_error(FZ_EINTERNAL, "flat walk: no kernel for this shape");
     }
 }

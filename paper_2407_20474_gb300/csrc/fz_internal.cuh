@@ -426,13 +426,31 @@ int launch_unrank(const EnumLaunch &L, const uint64_t *ranks, uint64_t m, int32_
                   cudaStream_t s);
 uint64_t default_slice_rows(uint64_t nrows, int sms);
 // Batched enumeration (fz_enum.cu): per-instance parameter images, then one
-// persistent launch over all work items.
+// persistent launch per group of instances of one shape (the flat walk's
+// kernels are compiled per width, leaf length and source; shape 0: the
+// general kernel).  Launches of a call overlap: each starts while the one
+// before it drains.
 size_t enum_params_bytes();
-void fill_batch_params(const EnumLaunch &L, int32_t *out, uint64_t count, uint64_t slice_rows,
-                       uint64_t slice_cost, void *dst);
-int launch_enumerate_batch(const void *params_dev, const uint64_t *item0_dev, int count,
-                           uint64_t nitems, unsigned long long *item_counter, int32_t *out_base,
-                           cudaStream_t s, int ctas_per_sm = 0);
+void fill_batch_params(const EnumLaunch &L, int32_t *out, uint64_t count, void *dst);
+uint32_t enum_params_shape(const void *image);
+struct BatchGroup {
+    uint32_t shape;
+    int first, last;             // instances, by their place in the parameter images
+    uint64_t item_lo, item_hi;   // their work items
+};
+constexpr int BATCH_MAX_GROUPS = 32;  // 24 shapes and the general kernel
+// counters: BATCH_MAX_GROUPS words of device memory.
+int launch_enumerate_batch(const void *params_dev, const uint64_t *item0_dev,
+                           const BatchGroup *groups, int ngroups, unsigned long long *counters,
+                           int32_t *out_base, cudaStream_t s, int ctas_per_sm = 0);
+// Place of each of `count` parameter images (pb bytes apart) grouped by shape,
+// the shapes with the most cost first; their groups, without items.
+void batch_order(const unsigned char *images, size_t pb, const uint64_t *cost, int count,
+                 std::vector<int> *order, std::vector<BatchGroup> *groups);
+// Cuts the instances of `params` (images in `order`) into work items: their
+// slice fields, item0 (count + 1) and the groups' item ranges.
+void batch_items(unsigned char *params, size_t pb, const uint64_t *cost, const int *order,
+                 std::vector<BatchGroup> *groups, int sms, uint64_t *item0);
 
 // Plans as seen by the batch and serve layers (fz_api.cu): the launch
 // description of a plan for an element n <= its n, and host copies of row 0

@@ -34,29 +34,45 @@ constexpr int BW = 8;                  // warps a block
 constexpr int BT = BW * 32;
 constexpr int WARP_BYTES = 5632;       // leaf descriptors + ring per warp (44 KB a block)
 
+extern __shared__ __align__(128) unsigned char build_smem[];
+
+// The block's job, kept after the warps' rings; its address is hidden at every
+// use (see flat_rows).
+struct JobRef {
+    __device__ __forceinline__ const RunBuild &operator()() const {
+        uint32_t o = BW * WARP_BYTES;
+        asm volatile("" : "+r"(o));
+        return *reinterpret_cast<const RunBuild *>(build_smem + o);
+    }
+    __device__ __forceinline__ const LeafSource &src() const { return (*this)().src; }
+    __device__ __forceinline__ int32_t *out() const { return (*this)().dst; }
+    __device__ __forceinline__ bool aligned() const { return ((uintptr_t)out() & 15u) == 0; }
+    int *st;
+    __device__ __forceinline__ int *status() const { return st; }
+};
+
 // The elements of a class-ordered table: flat index f -> (class c, step t),
 // element c + t g.  Classes 0..rr have qn + 1 elements, the rest qn.
 struct ClassWalk {
-    const RunBuild &J;
+    JobRef job;
     uint32_t f;
-    __device__ __forceinline__ void at(uint32_t x, uint32_t &c, uint32_t &t) const {
-        const uint32_t lim = (J.rr + 1u) * (J.qn + 1u);
-        if (x < lim) {
-            c = fd_div(x, J.fq1);
-            t = x - c * (J.qn + 1u);
-        } else {
-            const uint32_t y = fd_div(x - lim, J.fq);
-            c = J.rr + 1u + y;
-            t = x - lim - y * J.qn;
-        }
-    }
-    __device__ __forceinline__ bool leaf(uint32_t &p, uint64_t &E, int (&pre)[1]) const {
+    uint32_t t = 0;
+    __device__ __forceinline__ int word(int) const { return (int)t; }
+    __device__ __forceinline__ bool leaf(uint32_t &p, uint64_t &E) {
+        const RunBuild &J = job();
         if (f > (uint32_t)J.n) return false;
-        uint32_t c, t;
-        at(f, c, t);
+        const uint32_t q1 = J.qn + 1u, lim = (J.rr + 1u) * q1;
+        uint32_t c;
+        if (f < lim) {
+            c = fd_div(f, J.fq1);
+            t = f - c * q1;
+        } else {
+            const uint32_t y = fd_div(f - lim, J.fq);
+            c = J.rr + 1u + y;
+            t = f - lim - y * J.qn;
+        }
         p = c + t * (uint32_t)J.g;
         E = __ldg(J.cls + c) + __ldg(J.F + p);
-        pre[0] = (int)t;
         return true;
     }
     __device__ __forceinline__ void next() { f = f <= 0x7fffffffu ? f + 32u : f; }
@@ -64,9 +80,11 @@ struct ClassWalk {
 
 // Elements in increasing order.
 struct ElementWalk {
-    const RunBuild &J;
+    JobRef job;
     uint32_t f;
-    __device__ __forceinline__ bool leaf(uint32_t &p, uint64_t &E, int (&)[1]) const {
+    __device__ __forceinline__ int word(int) const { return 0; }
+    __device__ __forceinline__ bool leaf(uint32_t &p, uint64_t &E) const {
+        const RunBuild &J = job();
         if (f > (uint32_t)J.n) return false;
         p = f;
         E = __ldg(J.F + f);
@@ -131,21 +149,19 @@ __device__ __forceinline__ TablePlace table_place(const RunBuild &J, uint64_t x,
 template <int K, int SRC, bool CSR>
 __global__ void __launch_bounds__(BT, 4)
     run_build_kernel(const RunBuild *__restrict__ jobs, int njobs, int *status) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ RunBuild sj;
-    load_job(jobs, njobs, sj);
-    const RunBuild &J = sj;
+    load_job(jobs, njobs, *reinterpret_cast<RunBuild *>(build_smem + BW * WARP_BYTES));
+    const JobRef job{status};
+    const RunBuild &J = job();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint64_t item = (uint64_t)(blockIdx.x - J.blk0) * BW + wid;
     constexpr int NP = CSR ? 0 : 1;
     constexpr int W = K;
     constexpr int DS = CSR ? K : run_stride(K + 1);
     constexpr uint32_t B = flat_half_rows<NP, SRC, DS>(WARP_BYTES);
-    int4 *desc = reinterpret_cast<int4 *>(smem + (size_t)wid * WARP_BYTES);
-    int32_t *ring = reinterpret_cast<int32_t *>(smem + (size_t)wid * WARP_BYTES +
+    int4 *desc = reinterpret_cast<int4 *>(build_smem + (size_t)wid * WARP_BYTES);
+    int32_t *ring = reinterpret_cast<int32_t *>(build_smem + (size_t)wid * WARP_BYTES +
                                                 leaf_bytes<NP, SRC>());
     const uint64_t pol = policy_evict_normal();
-    const bool aligned = ((uintptr_t)J.dst & 15u) == 0;
     uint64_t base = 0;
     if constexpr (CSR) {
         // equal rows, in multiples of 32 (16-byte aligned bulk stores)
@@ -157,9 +173,9 @@ __global__ void __launch_bounds__(BT, 4)
         const uint32_t f = warp_last_le((uint32_t)J.n + 1u, row0, lane, &base, [&](uint32_t u) {
             return u == 0 ? 0ull : __ldg(F + u - 1);
         });
-        ElementWalk wk{J, f + (uint32_t)lane};
-        flat_rows<NP, W, DS, SRC>(wk, base, (uint32_t)(row0 - base), J.src, J.dst, aligned, row0,
-                                  left, desc, ring, B, status, pol, lane);
+        ElementWalk wk{job, f + (uint32_t)lane};
+        flat_rows<NP, W, DS, SRC>(wk, base, (uint32_t)(row0 - base), job, row0, left, desc, ring,
+                                  B, pol, lane);
     } else {
         // equal cost; a table's rows are whole 16-byte vectors, so a warp may
         // start at any row
@@ -177,10 +193,9 @@ __global__ void __launch_bounds__(BT, 4)
         __syncthreads();
         const uint64_t end = s_row[wid + 1];
         if (end <= pl.row) return;
-        ClassWalk wk{J, pl.f + (uint32_t)lane};
-        flat_rows<NP, W, DS, SRC>(wk, pl.base, (uint32_t)(pl.row - pl.base), J.src, J.dst, aligned,
-                                  pl.row, (uint32_t)(end - pl.row), desc, ring, B, status, pol,
-                                  lane);
+        ClassWalk wk{job, pl.f + (uint32_t)lane};
+        flat_rows<NP, W, DS, SRC>(wk, pl.base, (uint32_t)(pl.row - pl.base), job, pl.row,
+                                  (uint32_t)(end - pl.row), desc, ring, B, pol, lane);
     }
     if (lane == 0) bulk_wait_all();
     __syncwarp();
@@ -284,7 +299,8 @@ __global__ void __launch_bounds__(256)
 
 template <int K, int SRC, bool CSR>
 int launch_level(const RunBuild *jobs, int njobs, uint32_t blocks, int *status, cudaStream_t s) {
-    run_build_kernel<K, SRC, CSR><<<blocks, BT, BW * WARP_BYTES, s>>>(jobs, njobs, status);
+    run_build_kernel<K, SRC, CSR>
+        <<<blocks, BT, BW * WARP_BYTES + sizeof(RunBuild), s>>>(jobs, njobs, status);
     note_launch();
     FZ_CUDA_TRY(cudaGetLastError());
     return FZ_OK;

@@ -27,6 +27,7 @@
 #include <atomic>
 #include <chrono>
 #include <cstdlib>
+#include <cstring>
 #include <condition_variable>
 #include <deque>
 #include <map>
@@ -284,9 +285,9 @@ bool batch_kernel_serves(const EnumLaunch &L) {
 }
 
 // Enqueue a group of admitted requests (called by the server thread, lock
-// not held): one batch launch over all of them (request j's items follow
-// request j-1's, equal-cost items as in batches), requests the batch kernel
-// does not serve launched one by one after it, then the status words back
+// not held): one batch launch per shape over all of them (requests of a shape
+// next to each other, equal-cost items as in batches), requests the batch
+// kernels do not serve launched one by one after it, then the status words back
 // and the completion callback.
 int launch_group(fz_server_s *s, Group &G) {
     const size_t pb = enum_params_bytes();
@@ -297,7 +298,6 @@ int launch_group(fz_server_s *s, Group &G) {
     std::vector<EnumLaunch> Ls(m);
     std::vector<uint64_t> cost(m, 0);
     std::vector<char> direct(m, 0);
-    uint64_t total_cost = 0;
     for (int j = 0; j < m; ++j) {
         const Req *r = G.reqs[j];
         const SetRec &S = s->sets[r->set];
@@ -316,33 +316,36 @@ int launch_group(fz_server_s *s, Group &G) {
         // or run copy writes faster than the batch kernel's generic one);
         // so do those the batch kernel does not serve
         direct[j] = (!batch_kernel_serves(L) || r->count >= serve_direct_rows()) ? 1 : 0;
-        if (!direct[j]) total_cost += cost[j];
     }
-    const uint64_t warps = (uint64_t)dp.sms * 16;
-    const uint64_t target = std::max<uint64_t>(4096, total_cost / (warps * 8 + 1));
-    uint64_t *item0 = reinterpret_cast<uint64_t *>(G.stage + G.o_item0);
-    item0[0] = 0;
+    std::vector<unsigned char> images((size_t)m * pb);
     for (int j = 0; j < m; ++j) {
         const Req *r = G.reqs[j];
-        uint64_t items = 0, slice_cost = 64, slice_rows = 4;
-        if (!direct[j] && r->count > 0) {
-            items = std::max<uint64_t>(1, (cost[j] + target - 1) / target);
-            slice_cost = (cost[j] + items - 1) / items;
-            slice_rows = std::max<uint64_t>(4, (r->count + items - 1) / items);
-        }
         // out holds the byte offset of the request's rows in the arena
-        fill_batch_params(Ls[j], reinterpret_cast<int32_t *>((uintptr_t)r->off), r->count,
-                          slice_rows, slice_cost, G.stage + (size_t)j * pb);
-        item0[j + 1] = item0[j] + items;
+        fill_batch_params(Ls[j], reinterpret_cast<int32_t *>((uintptr_t)r->off),
+                          direct[j] ? 0 : r->count, images.data() + (size_t)j * pb);
+        if (direct[j]) cost[j] = 0;
         reinterpret_cast<int *>(G.stage + G.o_status)[j] = DEV_OK;
     }
+    // requests of one shape next to each other
+    std::vector<int> order;
+    std::vector<BatchGroup> groups;
+    batch_order(images.data(), pb, cost.data(), m, &order, &groups);
+    uint64_t *item0 = reinterpret_cast<uint64_t *>(G.stage + G.o_item0);
+    for (int p = 0; p < m; ++p)
+        memcpy(G.stage + (size_t)p * pb, images.data() + (size_t)order[p] * pb, pb);
+    batch_items(reinterpret_cast<unsigned char *>(G.stage), pb, cost.data(), order.data(), &groups,
+                dp.sms, item0);
+    int ng = 0;
+    for (const BatchGroup &B : groups)
+        if (B.item_hi > B.item_lo) groups[ng++] = B;
     // parameters, item prefix and zeroed status words: one transfer
     FZ_CUDA_TRY(cudaMemcpyAsync(G.dev, G.stage, G.o_status + (size_t)m * sizeof(int),
                                 cudaMemcpyHostToDevice, G.st));
     int32_t *base = static_cast<int32_t *>(s->arena_base);
-    rc = launch_enumerate_batch(G.dev, reinterpret_cast<const uint64_t *>(G.dev + G.o_item0), m,
-                                item0[m], reinterpret_cast<unsigned long long *>(G.dev + G.o_counter),
-                                base, G.st);
+    rc = launch_enumerate_batch(G.dev, reinterpret_cast<const uint64_t *>(G.dev + G.o_item0),
+                                groups.data(), ng,
+                                reinterpret_cast<unsigned long long *>(G.dev + G.o_counter), base,
+                                G.st);
     if (rc != FZ_OK) return rc;
     for (int j = 0; j < m; ++j) {
         if (!direct[j] || G.reqs[j]->count == 0) continue;
@@ -521,7 +524,7 @@ int fz_serve_create(const fz_serve_cfg_t *cfg, fz_server_t *srv) {
             G.o_item0 = ((size_t)s->max_group * pb + 255) & ~size_t(255);
             G.o_status = (G.o_item0 + ((size_t)s->max_group + 1) * 8 + 255) & ~size_t(255);
             G.o_counter = (G.o_status + (size_t)s->max_group * 4 + 255) & ~size_t(255);
-            G.bytes = G.o_counter + 256;
+            G.bytes = G.o_counter + BATCH_MAX_GROUPS * sizeof(unsigned long long);
             e = cudaMalloc((void **)&G.dev, G.bytes);
             if (e != cudaSuccess) return fail(cuda_error(e, "cudaMalloc (serve group)"));
             e = cudaHostAlloc((void **)&G.stage, G.o_counter, cudaHostAllocDefault);

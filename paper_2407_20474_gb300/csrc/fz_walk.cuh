@@ -241,18 +241,22 @@ __host__ __device__ constexpr uint32_t flat_half_rows(int bytes) {
 // leaf a warp at a time needed about 12 warp instructions a row where leaves
 // hold a row or two), the output's bandwidth when they are long.
 //
-// Walk: leaf(p, end, pre) gives lane's element, cumulative row end and
-// prefix words and returns false past the last leaf (a suffix of the
-// lanes); next() moves every lane 32 leaves on.  `base` is the row at which
+// Walk: leaf(p, end) gives lane's element and cumulative row end and returns
+// false past the last leaf (a suffix of the lanes), word(c) its prefix words;
+// next() moves every lane 32 leaves on.  `base` is the row at which
 // leaf 0 starts (same origin as the ends) and `skip` its rows already behind.
 // Returns false, with the status recorded, if the tables disagree.
 // ---------------------------------------------------------------------------
-template <int NP, int W, int DS, int SRC, class Walk>
-__device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip,
-                                          const LeafSource &S, int32_t *out, bool aligned,
+//
+// Sink: src(), out(), aligned() and status() of the rows written.  Parameters
+// kept in shared memory are read through a Sink (and a Walk) that hides their
+// address from the compiler at every use: hoisted into registers they cost
+// the kernel its 64 (spills of 100 to 300 bytes a thread that miss the small
+// L1 left beside 4 blocks' shared memory: 2.0 TB/s written instead of 4).
+template <int NP, int W, int DS, int SRC, class Walk, class Sink>
+__device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip, const Sink &K,
                                           uint64_t row0, uint32_t left, int4 *desc,
-                                          int32_t *ring, uint32_t B, int *status, uint64_t pol,
-                                          int lane) {
+                                          int32_t *ring, uint32_t B, uint64_t pol, int lane) {
     static_assert(NP + W <= DS, "row words");
     constexpr int RPL = SRC == SRC_PAIR || W <= 4 ? 2 : 1;  // rows a lane per round
     constexpr int DV = leaf_vecs<NP, SRC>();
@@ -267,15 +271,29 @@ __device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip
         int l[RPL];
     };
 
+    // lane's leaf of the next batch: its row end and where its rows start are
+    // loaded together, before the rounds of the batch in hand
+    uint32_t p = 0, qt = 0;
+    uint64_t nE = 0, nsrc = 0;
+    bool have = false;
+    auto load_leaf = [&] {
+        have = wk.leaf(p, nE);
+        if constexpr (SRC == SRC_RUN) {
+            if (have) {
+                const LeafSource &S = K.src();
+                qt = fd_div(p, S.fg);
+                nsrc = __ldg(S.cls + (p - qt * S.fg.g));
+            }
+        }
+    };
+    load_leaf();
     while (left > 0) {
         // ---- 32 leaves
-        uint32_t p = 0;
-        uint64_t E = 0;
-        int pre[NP > 0 ? NP : 1];
-        const bool live = wk.leaf(p, E, pre);
+        uint64_t E = nE;
+        const bool live = have;
         const int nlive = __popc(__ballot_sync(FULL, live));
         if (nlive == 0) {  // past the last leaf with rows still owed
-            if (lane == 0) atomicExch(status, (int)DEV_INTERNAL);
+            if (lane == 0) atomicExch(K.status(), (int)DEV_INTERNAL);
             ok = false;
             break;
         }
@@ -301,29 +319,33 @@ __device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip
             for (int c = 0; c < DV * 4; ++c) d[c] = 0;
             constexpr int H = SRC == SRC_RUN ? 2 : 3;
             if constexpr (SRC == SRC_RUN) {
-                const uint32_t qt = fd_div(p, S.fg);
-                const uint64_t src = __ldg(S.cls + (p - qt * S.fg.g));
-                bad = bad || src + size > S.nrows;  // bounds guard: the leaf lies in the table
-                d[0] = (int)((uint32_t)src - s);
+                bad = bad || nsrc + size > K.src().nrows;  // bounds guard: in the table
+                d[0] = (int)((uint32_t)nsrc - s);
                 d[1] = (int)qt;
             } else {
+                const LeafSource &S = K.src();
                 const uint32_t at = pair_form_top(S.pair, p);
                 d[0] = (int)s;
                 d[1] = (int)at;
                 d[2] = (int)fd_div(p - at * S.pair.g, S.pair.fh);
             }
 #pragma unroll
-            for (int c = 0; c < NP; ++c) d[H + c] = pre[c];
+            for (int c = 0; c < NP; ++c) d[H + c] = wk.word(c);
 #pragma unroll
             for (int v = 0; v < DV; ++v)
                 desc[v * 32 + rank] = make_int4(d[4 * v], d[4 * v + 1], d[4 * v + 2], d[4 * v + 3]);
         }
         if (__any_sync(FULL, bad)) {
-            if (lane == 0) atomicExch(status, (int)DEV_INTERNAL);
+            if (lane == 0) atomicExch(K.status(), (int)DEV_INTERNAL);
             ok = false;
             break;
         }
         __syncwarp();
+        const uint32_t rows = q_end - skip;
+        if (left > rows) {
+            wk.next();
+            load_leaf();
+        }
 
         // ---- rounds
         auto fetch = [&](Frag &F, uint32_t q0, uint32_t cnt) {
@@ -340,7 +362,7 @@ __device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip
                         const uint32_t row =
                             reinterpret_cast<const uint32_t *>(desc + F.l[u])[0] + qh + lane;
                         const int4 *src =
-                            reinterpret_cast<const int4 *>(S.rows) + (size_t)row * (SS / 4);
+                            reinterpret_cast<const int4 *>(K.src().rows) + (size_t)row * (SS / 4);
 #pragma unroll
                         for (int v = 0; v < SS / 4; ++v) F.v[u][v] = __ldg(src + v);
                     }
@@ -387,15 +409,15 @@ __device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip
                         for (int c = 1; c < W; ++c) w[NP + c] = x[c];
                     } else {
                         const uint32_t o = q0 + 32u * u + lane - (uint32_t)d[0];
-                        w[NP] = d[1] - (int)(o * S.pair.h1);
-                        w[NP + 1] = d[2] + (int)(o * S.pair.g1);
+                        w[NP] = d[1] - (int)(o * K.src().pair.h1);
+                        w[NP + 1] = d[2] + (int)(o * K.src().pair.g1);
                     }
                     store_row<DS>(dst + u * 32 * DS, w, lane);
                 }
             }
             hpos += cnt;
             if (hpos == B) {
-                flush_words(out + (row0 + (uint64_t)nfull * B) * DS, aligned,
+                flush_words(K.out() + (row0 + (uint64_t)nfull * B) * DS, K.aligned(),
                             ring + (size_t)half * B * DS, B * DS, lane, pol);
                 ++nfull;
                 half ^= 1u;
@@ -442,14 +464,13 @@ __device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip
                     q0 += c;
                 }
             }
-            left -= q_end - skip;
         }
+        left -= rows;
         skip = 0;
         base = Elast;
-        if (left > 0) wk.next();
     }
     if (hpos > 0)
-        flush_words(out + (row0 + (uint64_t)nfull * B) * DS, aligned,
+        flush_words(K.out() + (row0 + (uint64_t)nfull * B) * DS, K.aligned(),
                     ring + (size_t)half * B * DS, hpos * DS, lane, pol);
     if (lane == 0) bulk_wait_read_all();
     __syncwarp();

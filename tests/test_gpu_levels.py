@@ -127,3 +127,35 @@ def test_batch_flat_shapes(fz):
             for j, i in enumerate(sub):
                 at, ref = int(b.word_offsets[j]), refs[i]
                 assert np.array_equal(host[at:at + ref.size].reshape(ref.shape), ref), (inst[i], k)
+
+
+def test_batch_in_a_graph(fz):
+    """Rebuild and enumeration captured in a CUDA graph (the overlapped launches
+    of the shapes included) and replayed: the same bytes, twice."""
+    rng = np.random.Generator(np.random.PCG64(78))
+    inst = []
+    for d in (3, 4, 5, 6, 7, 8, 2, 9):
+        g = tuple(int(x) for x in rng.integers(5, 40, size=d))
+        inst.append((g, workloads.find_n(oracle.count_upto, g, 20000)))
+    with fz.Batch(inst) as b:
+        out = torch.full((b.total_words + 8,), CANARY, dtype=torch.int32, device="cuda")
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(side):
+            b.rebuild(stream=side)
+            b.enumerate(out, stream=side)
+            side.synchronize()
+            with torch.cuda.graph(graph, stream=side):
+                b.rebuild(stream=side)
+                b.enumerate(out, stream=side)
+        for _ in range(2):
+            out.fill_(CANARY)
+            graph.replay()
+            # the end of the graph is the end of every launch in it
+            host = out.cpu().numpy()
+            for j, (g, n) in enumerate(inst):
+                ref = oracle.enumerate_desc(g, n)
+                at = int(b.word_offsets[j])
+                assert np.array_equal(host[at:at + ref.size].reshape(ref.shape), ref), (g, n)
+        b.sync()

@@ -894,75 +894,80 @@ size_t enum_batch_smem_bytes() {
     return (size_t)ENUM_WARPS * (BATCH_RING_BYTES + sizeof(EnumParams) + sizeof(WarpPath));
 }
 
-// Tuples of given ranks (one warp per rank).
+// Tuples of given ranks, a thread per rank.  Each leading coordinate is a
+// search in one count row: the rows of the children a_j >= v number
+// C[j][rem - v g_j], which grows about as the (d - 1 - j)-th power of its
+// index, so the search starts at that power's estimate and gallops from it
+// (two to four dependent loads a coordinate where a binary search over 300 to
+// 600 children takes 9).  With the memo in run order the coordinates from
+// d - K - 1 on are one table row; otherwise the searches go down to a_{d-2}.
+// Rows are staged in shared memory and written coalesced.
+//
+// Bound by the latency of the dependent loads, all of them random: a million
+// ranks of a width-6 set of 1e8 rows with a depth-3 table took 418 us with a
+// warp per rank and 32-probe searches, 33 us with a thread per rank.
+constexpr int UNRANK_THREADS = 256;
+
 template <int D>
-__global__ void __launch_bounds__(ENUM_THREADS)
-    fz_unrank_kernel(const __grid_constant__ EnumParams P,
-                                                                 const uint64_t *ranks,
-                                                                 uint64_t m) {
-    __shared__ WarpPath paths[ENUM_WARPS];
+__global__ void __launch_bounds__(UNRANK_THREADS)
+    fz_unrank_kernel(const __grid_constant__ EnumParams P, const uint64_t *ranks, uint64_t m) {
+    __shared__ int32_t stage[UNRANK_THREADS * D];
     const int lane = threadIdx.x & 31;
-    const int wid = threadIdx.x >> 5;
-    WarpPath *wp = &paths[wid];
-    const uint64_t nw = (uint64_t)gridDim.x * ENUM_WARPS;
-    for (uint64_t i = (uint64_t)blockIdx.x * ENUM_WARPS + wid; i < m; i += nw) {
-        const uint64_t R = ranks[i];
-        if (P.run_memo) {
-            // the leading coordinates by search, the rest is one table row
-            const int lamf = D - P.K - 1;
-            int rem = P.n, mine = 0;
-            uint64_t left = R;
-            bool good = R < __ldg(P.C + P.n);
-            for (int c = 0; good && c < lamf; ++c) {
-                int v;
-                uint64_t before;
-                find_child(P, c, rem, left, lane, v, before);
-                if (lane == c) mine = v;
-                left -= before;
-                rem -= v * P.g[c];
+    int32_t *mine = stage + (size_t)(threadIdx.x & ~31) * D;
+    const int levels = P.run_memo ? D - P.K - 1 : D - 1;
+    const uint64_t total = __ldg(P.C + P.n);
+    const uint64_t stride = (uint64_t)gridDim.x * UNRANK_THREADS;
+    for (uint64_t base = (uint64_t)blockIdx.x * UNRANK_THREADS + (threadIdx.x & ~31); base < m;
+         base += stride) {
+        const uint64_t i = base + lane;
+        if (i < m) {
+            uint64_t R = __ldg(ranks + i);
+            bool good = R < total;
+            int a[D];
+#pragma unroll
+            for (int c = 0; c < D; ++c) a[c] = 0;
+            uint32_t rem = (uint32_t)P.n;
+            uint64_t all = total;  // rows under the current prefix
+#pragma unroll
+            for (int j = 0; j < D - 1; ++j) {
+                if (j >= levels || !good) break;
+                const uint32_t g = (uint32_t)P.g[j];
+                const uint64_t *row = P.C + (int64_t)j * P.cs;
+                const uint32_t vmax = rem / g;
+                uint64_t ahi;
+                const uint32_t hi = thread_child(row, rem, g, vmax, R, all, D - 1 - j, &ahi);
+                a[j] = (int)hi;
+                R -= ahi;
+                rem -= hi * g;
+                all = j + 1 < levels ? __ldg(row + P.cs + rem) : 0ull;
+                good = j + 1 >= levels || R < all;
             }
-            const int gl = P.g[lamf], vmax = rem / gl;
-            const uint64_t row = good ? __ldg(P.cls_beg + (rem - vmax * gl)) + left : 0ull;
-            good = good && row < P.memo_rows;
-            if (!good && lane == 0) atomicExch(P.status, (int)DEV_INTERNAL);
-            if (lane < D) {
-                if (good && lane >= lamf) {
-                    const int32_t *m = reinterpret_cast<const int32_t *>(P.run_memo) +
-                                       (size_t)row * run_stride(P.K + 1);
-                    mine = lane == lamf ? vmax - __ldg(m) : __ldg(m + (lane - lamf));
+            if (P.run_memo) {
+                const uint32_t gl = P.leaf.fg.g, q = fd_div(rem, P.leaf.fg);
+                const uint64_t at = good ? __ldg(P.cls_beg + (rem - q * gl)) + R : 0ull;
+                good = good && at < P.memo_rows;  // bounds guard
+                if (good) {
+                    const int32_t *t = reinterpret_cast<const int32_t *>(P.run_memo) +
+                                       (size_t)at * run_stride(P.K + 1);
+#pragma unroll
+                    for (int c = 0; c < D; ++c)
+                        if (c == levels)
+                            a[c] = (int)q - __ldg(t);
+                        else if (c > levels)
+                            a[c] = __ldg(t + (c - levels));
                 }
-                P.out[i * D + lane] = good ? mine : -1;
+            } else {
+                a[D - 1] = (int)fd_div(rem, P.leaf.pair.fh);
+                good = good && (uint32_t)a[D - 1] * P.leaf.pair.fh.g == rem;
             }
-            continue;
+            if (!good) atomicExch(P.status, (int)DEV_INTERNAL);
+#pragma unroll
+            for (int c = 0; c < D; ++c) mine[lane * D + c] = good ? a[c] : -1;
         }
-        RunState st;
-        bool ok;
-        const uint64_t off = unrank_to_leaf(P, wp, R, lane, st, &ok);
-        if (!ok) {
-            if (lane < D) P.out[i * D + lane] = -1;
-            if (lane == 0) atomicExch(P.status, (int)DEV_INTERNAL);
-            continue;
-        }
-        const int lam = st.lam;
-        const int v = (int)st.vcur;
-        const int p = wp->r[lam] - v * P.g[lam];
-        bool mleaf = (P.lam_m >= 0) && !st.inwalk && lam == P.lam_m && p < P.top;
-        if (mleaf && __ldg(P.O + p) + off >= P.memo_rows) {  // bounds guard
-            if (lane == 0) atomicExch(P.status, (int)DEV_INTERNAL);
-            mleaf = false;
-        }
-        if (lane < D) {
-            int x;
-            if (lane < lam)
-                x = wp->a[lane];
-            else if (lane == lam)
-                x = v;
-            else if (mleaf)
-                x = __ldg(P.memo + (size_t)(__ldg(P.O + p) + off) * P.K + (lane - lam - 1));
-            else
-                x = (int)fd_div((uint32_t)p, P.leaf.pair.fh);
-            P.out[i * D + lane] = x;
-        }
+        __syncwarp();
+        const uint64_t left = (m - base) * D;
+        const uint32_t words = left < 32u * D ? (uint32_t)left : 32u * D;
+        for (uint32_t w = lane; w < words; w += 32) P.out[base * D + w] = mine[w];
         __syncwarp();
     }
 }
@@ -1050,10 +1055,9 @@ static int launch_enum_d(const EnumParams &P, cudaStream_t s, int sms) {
 template <int D>
 static int launch_unrank_d(const EnumParams &P, const uint64_t *ranks, uint64_t m,
                            cudaStream_t s) {
-    uint64_t blocks = (m + ENUM_WARPS - 1) / ENUM_WARPS;
-    if (blocks > 4096) blocks = 4096;
-    if (blocks < 1) blocks = 1;
-    fz_unrank_kernel<D><<<(unsigned)blocks, ENUM_THREADS, 0, s>>>(P, ranks, m);
+    uint64_t blocks = (m + UNRANK_THREADS - 1) / UNRANK_THREADS;
+    if (blocks > 65536) blocks = 65536;
+    fz_unrank_kernel<D><<<(unsigned)blocks, UNRANK_THREADS, 0, s>>>(P, ranks, m);
     note_launch();
     FZ_CUDA_TRY(cudaGetLastError());
     return FZ_OK;
@@ -1200,6 +1204,10 @@ int launch_enumerate(const EnumLaunch &L, uint64_t rank_begin, uint64_t nrows, i
         uint64_t sc = (uint64_t)((double)slice_rows * per_row);
         P.slice_cost = sc < 64 ? 64 : sc;
     }
+    // more prefixes than rows: by rank (the flat walk visits every prefix)
+    if (P.flat_np > 0 && P.flat_src == SRC_PAIR && rank_walk_serves(L.d) && L.RT &&
+        L.total_cost > L.total_rows + L.W * L.total_rows)
+        return launch_rank_walk(P, ring_bytes_for(L.ctas_per_sm), s, dp.sms);
     if (P.flat_np > 0) return launch_enum_flat(P, ring_bytes_for(L.ctas_per_sm), s, dp.sms);
     P.half_rows = half_rows_for(L.d, ring_bytes_for(L.ctas_per_sm));
     FZ_DISPATCH_D(L.d, launch_enum_d, P, s, dp.sms);

@@ -80,6 +80,67 @@ __device__ __forceinline__ void find_child(const EnumParams &P, int c, int rem, 
     v_out = (int)(umax - u);
 }
 
+// find_child by one thread: the child a_j = v of a node with remainder rem that
+// holds relative rank R, i.e. the least v with at most R rows in the children
+// above it, C[j][rem - (v + 1) g] <= R; *before = those rows.  Gallops from v0.
+__device__ __forceinline__ uint32_t thread_child_from(const uint64_t *row, uint32_t rem,
+                                                      uint32_t g, uint32_t vmax, uint64_t R,
+                                                      uint32_t v0, uint64_t *before) {
+    auto above = [&](uint32_t v) {
+        return v >= vmax ? 0ull : __ldg(row + (rem - (v + 1u) * g));
+    };
+    // lo: above(lo) > R (or -1); hi: above(hi) <= R
+    int64_t lo, hi;
+    uint64_t ahi = above(v0);
+    int64_t st = 1;
+    if (ahi <= R) {
+        hi = v0;
+        for (;; st *= 2) {
+            lo = hi - st;
+            if (lo < 0) {
+                lo = -1;
+                break;
+            }
+            const uint64_t t = above((uint32_t)lo);
+            if (t > R) break;
+            hi = lo;
+            ahi = t;
+        }
+    } else {
+        lo = v0;
+        for (;; st *= 2) {
+            hi = lo + st;
+            if (hi > (int64_t)vmax) hi = vmax;
+            ahi = above((uint32_t)hi);
+            if (ahi <= R) break;
+            lo = hi;
+        }
+    }
+    while (hi - lo > 1) {
+        const int64_t mid = (lo + hi) >> 1;
+        const uint64_t t = above((uint32_t)mid);
+        if (t <= R) {
+            hi = mid;
+            ahi = t;
+        } else {
+            lo = mid;
+        }
+    }
+    *before = ahi;
+    return (uint32_t)hi;
+}
+
+// The same from an estimate: the rows above grow about as the `power`-th power
+// of the count row's index (all: rows under the node).
+__device__ __forceinline__ uint32_t thread_child(const uint64_t *row, uint32_t rem, uint32_t g,
+                                                 uint32_t vmax, uint64_t R, uint64_t all,
+                                                 int power, uint64_t *before) {
+    const float f = __log2f((float)R + 0.5f) - __log2f((float)all);
+    const float x = (float)rem * exp2f(f / (float)power);
+    uint32_t v = x < (float)rem ? (uint32_t)(((float)rem - x) / (float)g) : 0u;
+    return thread_child_from(row, rem, g, vmax, R, v < vmax ? v : vmax, before);
+}
+
 // Walk state of one warp (warp-uniform).
 struct RunState {
     int lam;          // coordinate of the current run of sibling leaves
@@ -571,6 +632,9 @@ __device__ __forceinline__ uint64_t batch_locate(const BatchEnumParams &BP, Enum
 
 // fz_flat.cu
 int launch_enum_flat(const EnumParams &P, int warp_bytes, cudaStream_t s, int sms);
+// The rank walk: sets whose prefixes of d - 2 coordinates are mostly empty.
+bool rank_walk_serves(int d);
+int launch_rank_walk(const EnumParams &P, int warp_bytes, cudaStream_t s, int sms);
 int launch_flat_batch(const BatchEnumParams &BP, int d, int np, int src, cudaStream_t s, int sms,
                       int ctas_per_sm);
 // fz_enum.cu: grid and launch of a persistent enumeration kernel.

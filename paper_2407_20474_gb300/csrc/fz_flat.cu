@@ -54,6 +54,131 @@ int launch_one(EnumParams P, int warp_bytes, cudaStream_t s, int sms) {
     return launch_enum_grid(kern, P, (size_t)ENUM_WARPS * bytes, s, sms, attr_set, bytes);
 }
 
+// ---------------------------------------------------------------------------
+// The rank walk: no memo, and most prefixes of d - 2 coordinates empty (a
+// width-6 set of 1e7 rows has 8.6e7 of them).  Instead of visiting them, a
+// lane goes from its row to the row 32 ranks on: each coordinate whose
+// subtree ends before that rank is searched again in its count row, from the
+// value it had (or, under a new parent, from the power-law estimate), so
+// lanes of a warp follow consecutive rows and mostly share the upper
+// coordinates' loads.  The last two coordinates are the pair's closed form.
+// The cost is per row, so items are equal row ranges.
+//
+// Bound by the latency of the searches' dependent loads.  The case above: 1054
+// us by the flat walk, 409 by the rank walk.
+// ---------------------------------------------------------------------------
+template <int D>
+__global__ void __launch_bounds__(ENUM_THREADS, 4)
+    fz_enum_rank_kernel(const __grid_constant__ EnumParams P, int warp_bytes) {
+    constexpr int NP = D - 2;
+    const int lane = threadIdx.x & 31;
+    const int wid = threadIdx.x >> 5;
+    int32_t *ring = reinterpret_cast<int32_t *>(enum_smem + (size_t)wid * warp_bytes);
+    const uint32_t B = (uint32_t)P.half_rows;
+    const uint64_t pol = policy_evict_first();
+    const PairForm &F = P.leaf.pair;
+    bool ok = true;
+    while (ok) {
+        unsigned long long s = 0;
+        if (lane == 0) s = atomicAdd(P.slice_counter, 1ull);
+        s = __shfl_sync(FULL, s, 0);
+        if (s >= P.nslices) break;
+        const uint64_t row0 = s * P.slice_rows;
+        const uint64_t rest = P.nrows - row0;
+        const uint32_t rows = rest < P.slice_rows ? (uint32_t)rest : (uint32_t)P.slice_rows;
+        // a[j], remainders, and the ranks where the subtree of (a_0..a_{j-1})
+        // begins and that of (a_0..a_j) ends
+        uint32_t a[NP], r[NP + 1];
+        uint64_t beg[NP + 1], end[NP];
+        r[0] = (uint32_t)P.n;
+        beg[0] = 0;
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+            a[j] = 0;
+            end[j] = 0;
+        }
+        uint32_t at = 0, b0 = 0, hpos = 0, half = 0, nfull = 0;
+        for (uint32_t q = 0; q < rows;) {
+            uint32_t cnt = rows - q;
+            if (cnt > 32u) cnt = 32u;
+            if (cnt > B - hpos) cnt = B - hpos;
+            const bool act = (uint32_t)lane < cnt;
+            const uint64_t R = P.rank_begin + row0 + q + lane;
+            if (act && R >= end[NP - 1]) {
+                bool fresh = false;  // the parent changed
+#pragma unroll
+                for (int j = 0; j < NP; ++j) {
+                    if (!fresh && R < end[j]) continue;
+                    const uint32_t g = (uint32_t)P.g[j];
+                    const uint64_t *row = P.C + (int64_t)j * P.cs;
+                    const uint32_t vmax = fd_div(r[j], P.fdg[j]);
+                    const bool again = !fresh && end[j] > 0;  // same parent, a later child
+                    const uint64_t all = again ? 0ull : __ldg(row + r[j]);
+                    uint64_t before;
+                    if (again)
+                        a[j] = thread_child_from(row, r[j], g, vmax, R - beg[j],
+                                                 a[j] > 0 ? a[j] - 1u : 0u, &before);
+                    else
+                        a[j] = thread_child(row, r[j], g, vmax, R - beg[j], all, D - 1 - j, &before);
+                    r[j + 1] = r[j] - a[j] * g;
+                    end[j] = beg[j] + __ldg(row + r[j + 1]);
+                    beg[j + 1] = beg[j] + before;
+                    fresh = true;
+                }
+                at = pair_form_top(F, r[NP]);
+                b0 = fd_div(r[NP] - at * F.g, F.fh);
+                if (R >= end[NP - 1]) ok = false;  // the tables disagree
+            }
+            if (hpos == 0 && nfull >= 2) {
+                if (lane == 0) bulk_wait_read<1>();
+                __syncwarp();
+            }
+            if (act) {
+                const uint32_t o = (uint32_t)(R - beg[NP]);
+                int w[D];
+#pragma unroll
+                for (int j = 0; j < NP; ++j) w[j] = (int)a[j];
+                w[NP] = (int)(at - o * F.h1);
+                w[NP + 1] = (int)(b0 + o * F.g1);
+                store_row<D>(ring + (size_t)(half * B + hpos + lane) * D, w, lane);
+            }
+            q += cnt;
+            hpos += cnt;
+            if (hpos == B) {
+                flush_words(P.out + (row0 + (uint64_t)nfull * B) * D, P.aligned != 0,
+                            ring + (size_t)half * B * D, B * D, lane, pol);
+                ++nfull;
+                half ^= 1u;
+                hpos = 0;
+            }
+        }
+        if (hpos > 0)
+            flush_words(P.out + (row0 + (uint64_t)nfull * B) * D, P.aligned != 0,
+                        ring + (size_t)half * B * D, hpos * D, lane, pol);
+        if (lane == 0) bulk_wait_read_all();
+        ok = __all_sync(FULL, ok);
+        if (!ok && lane == 0) atomicExch(P.status, (int)DEV_INTERNAL);
+    }
+    if (lane == 0) bulk_wait_all();
+    __syncwarp();
+}
+
+template <int D>
+int launch_rank_d(EnumParams P, int warp_bytes, cudaStream_t s, int sms) {
+    static DeviceOnce attr_set;
+    uint32_t b = (uint32_t)(warp_bytes / (8 * D)) / 32 * 32;
+    P.half_rows = (int)(b < 32 ? 32 : b);
+    const int bytes = (2 * P.half_rows * D * 4 + 127) & ~127;
+    // an item starts with a full search: 256 to 2048 rows, about eight a warp
+    uint64_t rows = P.nrows / ((uint64_t)sms * 32 * 8 + 1);
+    rows = rows < 256 ? 256 : rows > 2048 ? 2048 : rows;
+    if (P.slice_rows < rows) rows = P.slice_rows;
+    P.slice_rows = (rows + 31) & ~31ull;
+    P.nslices = (P.nrows + P.slice_rows - 1) / P.slice_rows;
+    return launch_enum_grid(fz_enum_rank_kernel<D>, P, (size_t)ENUM_WARPS * bytes, s, sms, attr_set,
+                            bytes);
+}
+
 // The flat walk of a batch's instances of one shape.  A launch may start while
 // the one before it drains (chained): it reads nothing that one writes, and
 // waits for its completion only before it ends, so the last launch's end is
@@ -202,6 +327,18 @@ int launch_flat_batch(const BatchEnumParams &BP, int d, int np, int src, cudaStr
         case 7: return launch_batch_d<7>(BP, np, src, s, sms, ctas_per_sm);
         case 8: return launch_batch_d<8>(BP, np, src, s, sms, ctas_per_sm);
         default: return set_error(FZ_EINTERNAL, "flat walk: no kernel for this shape");
+    }
+}
+
+bool rank_walk_serves(int d) { return d >= 4 && d <= 7; }
+
+int launch_rank_walk(const EnumParams &P, int warp_bytes, cudaStream_t s, int sms) {
+    switch (P.d) {
+        case 4: return launch_rank_d<4>(P, warp_bytes, s, sms);
+        case 5: return launch_rank_d<5>(P, warp_bytes, s, sms);
+        case 6: return launch_rank_d<6>(P, warp_bytes, s, sms);
+        case 7: return launch_rank_d<7>(P, warp_bytes, s, sms);
+        default: return set_error(FZ_EINTERNAL, "rank walk: no kernel for this width");
     }
 }
 

@@ -531,6 +531,7 @@ EnumLaunch launch_of(const fz_plan_s *p) {
     L.cls_beg = p->cls_beg;
     if (p->RT) {
         L.RT = p->RT;
+        L.by_cost = true;
         L.W = p->W;
         L.lam_r = p->lam_r;
         L.total_rows = p->count;

@@ -64,6 +64,7 @@ struct Inst {
     int d = 0, n = 0, K = 0, top = 0, lam_r = 0, clamp_row = -1;
     bool pair = false;  // K = 2 kept as the closed form (no memo table)
     bool run = false;   // full memo in run order (table run_job)
+    bool flat = false;  // enumerated by the flat walk
     int run_job = -1;
     const int4 *run_memo = nullptr;
     const uint64_t *cls_beg = nullptr;
@@ -127,8 +128,7 @@ namespace {
 // Row 0 of an instance's count and runs tables is only ever read along the
 // chain n, n - g_1, n - 2 g_1, ... (unranking, the walk at the first
 // coordinate, the costs and the totals): its jobs cover that chain alone,
-// as a strided view of n div g_1 + 1 entries.  For d = 3 with the pair memo
-// the same holds for row 1, which only feeds row 0's chain.
+// as a strided view of n div g_1 + 1 entries.
 void chain_view(ScanJob &J, const Inst &I) {
     J.off = I.n % I.g[0];
     J.es = I.g[0];
@@ -138,7 +138,6 @@ void chain_view(ScanJob &J, const Inst &I) {
 int build_scan_plan(fz_batch_s *b, uint64_t *table_base, std::vector<ScanJob> &jobs,
                     std::vector<ScanTask> &tasks, size_t *scratch_words) {
     const int64_t DIRECT = scan_direct_limit();
-    const int64_t LANE_LIMIT = scan_lane_limit();
     const int64_t BS_TASK = scan_blocks_per_task();
     const int RBk = scan_block_rows();
     int maxlev = 0;
@@ -160,24 +159,23 @@ int build_scan_plan(fz_batch_s *b, uint64_t *table_base, std::vector<ScanJob> &j
                 jobs.push_back(jd);
                 for (int64_t a = 0; a < len; a += 8192)
                     tasks.push_back({(int)jobs.size() - 1, TK_DELTA, a, std::min(len, a + 8192)});
-            } else {
-                // rows d-2 and d-1 in closed form (no scans)
+            } else if (!(I.d == 3 && I.pair && I.flat)) {
+                // rows d-2 and d-1 in closed form (no scans); a pair memo of
+                // width 3 reads row 0 only, whose scan computes row 1
                 ScanJob jp{};
                 jp.out = table_base + I.off_C + (size_t)(I.d - 2) * len;
                 jp.len = len;
-                jp.g = I.g[I.d - 2];
-                jp.h = I.g[I.d - 1];
+                jp.pair = make_pair_form(I.g[I.d - 2], I.g[I.d - 1]);
                 // row d-1 is read by a memo build from this table, or as the
                 // leaf row of a candidates table counted at level d - 1
                 jp.ones_below = ((I.K > 0 && !I.pair && !I.run) || I.lam_r >= I.d - 1) ? 1 : 0;
-                pair_params(jp.g, jp.h, &jp.e, &jp.h1, &jp.g1, &jp.inv);
-                if (!jp.ones_below && (I.d == 2 || (I.d == 3 && I.pair))) chain_view(jp, I);
+                if (!jp.ones_below && I.d == 2) chain_view(jp, I);
                 jobs.push_back(jp);
                 for (int64_t a = 0; a < jp.len; a += 8192)
                     tasks.push_back(
                         {(int)jobs.size() - 1, TK_PAIR, a, std::min(jp.len, a + 8192)});
             }
-            if (I.lam_r >= 0 && I.off_RT != (size_t)-1) {
+            if (I.lam_r >= 0 && I.off_RT != (size_t)-1 && !I.flat) {
                 if (I.lam_r == 0) {
                     ScanJob jo{};
                     jo.out = table_base + I.off_RT + (size_t)I.lam_r * len;
@@ -218,6 +216,10 @@ int build_scan_plan(fz_batch_s *b, uint64_t *table_base, std::vector<ScanJob> &j
                 J.out = table_base + I.off_C + (size_t)j * len;
                 J.len = len;
                 J.g = I.g[j];
+                if (I.d == 3 && I.pair && I.flat) {
+                    J.input = SCAN_PAIR;
+                    J.pair = make_pair_form(I.g[1], I.g[2]);
+                }
                 if (j == 0) {
                     chain_view(J, I);
                     J.g = 1;  // consecutive entries of the chain
@@ -234,6 +236,11 @@ int build_scan_plan(fz_batch_s *b, uint64_t *table_base, std::vector<ScanJob> &j
                 J.out = table_base + I.off_RT + (size_t)j * len;
                 J.len = len;
                 J.g = I.g[j];
+                if (I.flat && t == 0) {
+                    // the flat walk computes row lam_r - 1 where it needs it
+                    J.input = SCAN_LINEAR;
+                    J.lin = make_fastdiv((uint32_t)I.g[j + 1]);
+                }
                 if (j == I.clamp_row) J.ones_below = I.top;
                 if (j == 0) {
                     chain_view(J, I);
@@ -248,7 +255,7 @@ int build_scan_plan(fz_batch_s *b, uint64_t *table_base, std::vector<ScanJob> &j
         for (int ji : step_jobs) {
             ScanJob &J = jobs[ji];
             const int64_t T = (J.len + J.g - 1) / J.g;
-            if (T > DIRECT) {
+            if (scan_plan(std::min<int64_t>(J.g, J.len), T) < 0) {
                 // blocks of at least RBk entries, more for long chains, so
                 // that each chain of block sums is scanned directly
                 J.rb = std::max<int64_t>(RBk, (T + DIRECT - 1) / DIRECT);
@@ -260,20 +267,29 @@ int build_scan_plan(fz_batch_s *b, uint64_t *table_base, std::vector<ScanJob> &j
             }
         }
         max_scratch = std::max(max_scratch, sw);
+        auto plan = [&](const ScanJob &J) {
+            return scan_plan(std::min<int64_t>(J.g, J.len), (J.len + J.g - 1) / J.g);
+        };
         int first = (int)tasks.size();
-        for (int ji : step_jobs) {
+        for (int ji : step_jobs) {  // the longest tasks first
             const ScanJob &J = jobs[ji];
+            const int w = plan(J);
+            if (w <= 0) continue;
+            for (int64_t a = 0; a < std::min<int64_t>(J.g, J.len); a += w)
+                tasks.push_back({ji, TK_TILE, a, w});
+        }
+        std::stable_sort(tasks.begin() + first, tasks.end(),
+                         [&](const ScanTask &x, const ScanTask &y) {
+                             return jobs[x.job].len / jobs[x.job].g > jobs[y.job].len / jobs[y.job].g;
+                         });
+                for (int ji : step_jobs) {
+            const ScanJob &J = jobs[ji];
+            if (plan(J) > 0) continue;
             if (!J.slen) {
                 const int64_t chains = std::min<int64_t>(J.g, J.len);
-                const int64_t T = (J.len + J.g - 1) / J.g;
-                if (chains >= 32 && T <= LANE_LIMIT) {
-                    // 256 chains a task, one a lane
-                    for (int64_t a = 0; a < chains; a += 256)
-                        tasks.push_back({ji, TK_LANES, a, std::min(chains, a + 256)});
-                } else {
-                    for (int64_t a = 0; a < chains; a += 8)
-                        tasks.push_back({ji, TK_DIRECT, a, std::min(chains, a + 8)});
-                }
+                // 256 chains a task, one a lane
+                for (int64_t a = 0; a < chains; a += 256)
+                    tasks.push_back({ji, TK_LANES, a, std::min(chains, a + 256)});
             } else {
                 // one block sum a thread: a block is rb strided entries
                 for (int64_t a = 0; a < J.slen; a += BS_TASK)
@@ -314,12 +330,18 @@ int batch_enqueue_runs(fz_batch_s *b, cudaStream_t s) {
     return rc;
 }
 
-int batch_enqueue_rebuild(fz_batch_s *b, cudaStream_t s) {
+int batch_enqueue_scans(fz_batch_s *b, cudaStream_t s) {
     for (const auto &L : b->scan_launches) {
-        int rc = launch_scan_tasks(b->jobs_dev, b->tasks_dev + L.first, L.second, s);
+        const int rc = launch_scan_tasks(b->jobs_dev, b->tasks_dev + L.first, L.second, s);
         if (rc != FZ_OK) return rc;
     }
-    int rc = launch_memo_cta_build(b->memo_jobs_dev, b->nmemo, b->memo_ncoop, b->memo_claim,
+    return FZ_OK;
+}
+
+int batch_enqueue_rebuild(fz_batch_s *b, cudaStream_t s) {
+    int rc = batch_enqueue_scans(b, s);
+    if (rc != FZ_OK) return rc;
+    rc = launch_memo_cta_build(b->memo_jobs_dev, b->nmemo, b->memo_ncoop, b->memo_claim,
                                    b->status_dev, s);
     if (rc != FZ_OK) return rc;
     return batch_enqueue_runs(b, s);
@@ -399,32 +421,40 @@ BatchPolicy current_policy() {
 //
 // Run order (widths 3..8): the depth with the least estimated work in warp
 // instructions -- 3.5 per leaf (prefix of d - 1 - K coordinates), 1.6 per
-// 16 bytes of table row and 3.5 per element of every level -- or the closed
-// form of the last two generators with no table at all (5 per prefix of
-// d - 2 coordinates).  A table's rows stay within BATCH_MEMO_MAX_ROWS and
+// 16 bytes of table row and, from depth 3 on, 3.5 per element of every level
+// -- or the closed form of the last two generators with no table at all (5 per
+// prefix of d - 2 coordinates).  A table's rows stay within BATCH_MEMO_MAX_ROWS and
 // cap_rows times the instance's estimated rows.
-void choose_batch_run(Inst &I, int n_set, double cap_rows) {
+//
+// `few` (batches of under BATCH_FEW_ROWS rows, where every launch counts): one
+// shape per width -- two walked coordinates above the table from width 5 on,
+// no table below -- unless that costs BATCH_FEW_WORK more.
+constexpr double BATCH_FEW_ROWS = 4e6, BATCH_FEW_WORK = 2e5;
+void choose_batch_run(Inst &I, int n_set, double cap_rows, bool few) {
     const int d = I.d;
     const double count = lattice_volume(I.g, d, n_set, false);
-    I.K = 2;
-    I.pair = true;
-    I.top = I.n + 1;
-    double best = 5.0 * lattice_volume(I.g, d - 2, n_set, true);
-    double build = 0;
+    const double pair = 5.0 * lattice_volume(I.g, d - 2, n_set, true);
+    int best_k = 0;  // 0: the closed form
+    double best = pair, build = 0, two = d <= 4 ? pair : 1e300;
     for (int K = 2; K <= d - 2 && K <= RUN_MAX_K; ++K) {
         const double rows = K == 2 ? (double)pair_rows_upto(n_set, I.g[d - 2], I.g[d - 1])
                                    : lattice_volume(I.g + (d - K), K, n_set, true);
         if (rows > BATCH_MEMO_MAX_ROWS || rows > cap_rows * count + 4096.0) break;
-        build += 0.4 * rows * run_stride(K + 1) + 3.5 * n_set;
+        build += 0.4 * rows * run_stride(K + 1) +
+                 (K > 2 ? 3.5 * n_set : 4.0 * std::min(rows, (double)n_set));
         const int lam = d - 1 - K;
         if (!flat_serves(d, lam, SRC_RUN)) continue;
         const double work = build + 3.5 * lattice_volume(I.g, lam, n_set, true);
+        if (lam == 2 && d > 4) two = work;
         if (work < best) {
             best = work;
-            I.K = K;
-            I.pair = false;
+            best_k = K;
         }
     }
+    if (few && two <= best + BATCH_FEW_WORK) best_k = d <= 4 ? 0 : d - 3;
+    I.pair = best_k == 0;
+    I.K = I.pair ? 2 : best_k;
+    I.top = I.n + 1;
 }
 
 // Element order: a memo's rows are estimated by the volume top^K / (K! prod
@@ -506,6 +536,7 @@ int batch_create_runs(fz_batch_s *b, uint64_t *tb, cudaStream_t s) {
     struct Table {
         int K, src, n;   // depth, source instance, last element
         bool final = false;
+        int kind = 0;    // how it is built (run_build_kind)
     };
     std::map<std::vector<int32_t>, int> of;
     std::vector<Table> tab;
@@ -534,40 +565,49 @@ int batch_create_runs(fz_batch_s *b, uint64_t *tb, cudaStream_t s) {
     const int m = (int)tab.size();
     b->nrun = m;
     if (m == 0) return FZ_OK;
-    // jobs in build order: by depth
-    std::vector<int> order(m), at(m);
-    for (int t = 0; t < m; ++t) order[t] = t;
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return tab[x].K < tab[y].K; });
-    for (int p = 0; p < m; ++p) at[order[p]] = p;
-    std::vector<RunBuild> rj(m);
-    size_t cls_words = 0;
-    for (int p = 0; p < m; ++p) {
-        const Table &T = tab[order[p]];
-        const std::vector<int32_t> &g = gens[order[p]];
-        const Inst &S = b->inst[T.src];
-        fill_run_build(g.data(), (int)g.size(), T.n, 0, false, &rj[p]);
-        rj[p].F = tb + S.off_C + (size_t)(S.d - (int)g.size()) * ((size_t)S.n + 1);
-        cls_words += a256(((size_t)rj[p].G + 1) * 8) / 8;
-    }
-    // rows of every table, then memory and the build
+    // rows of every table
+    std::vector<uint64_t> rows(m);
     DevArena sizes;
     const size_t jb = a256((size_t)m * sizeof(RunBuild));
     int rc = sizes.alloc(jb + (size_t)m * 8);
     if (rc != FZ_OK) return rc;
     RunBuild *tj = static_cast<RunBuild *>(sizes.p);
     uint64_t *td = reinterpret_cast<uint64_t *>(static_cast<char *>(sizes.p) + jb);
-    std::vector<uint64_t> rows(m);
-    FZ_CUDA_TRY(cudaMemcpyAsync(tj, rj.data(), (size_t)m * sizeof(RunBuild),
+    std::vector<RunBuild> byt(m);
+    size_t cls_words = 0;
+    for (int t = 0; t < m; ++t) {
+        const std::vector<int32_t> &g = gens[t];
+        const Inst &S = b->inst[tab[t].src];
+        fill_run_build(g.data(), (int)g.size(), tab[t].n, 0, false, &byt[t]);
+        byt[t].F = tb + S.off_C + (size_t)(S.d - (int)g.size()) * ((size_t)S.n + 1);
+        cls_words += a256(((size_t)byt[t].G + 1) * 8) / 8;
+    }
+    FZ_CUDA_TRY(cudaMemcpyAsync(tj, byt.data(), (size_t)m * sizeof(RunBuild),
                                 cudaMemcpyHostToDevice, s));
     rc = launch_run_totals(tj, m, td, s);
     if (rc != FZ_OK) return rc;
     FZ_CUDA_TRY(cudaMemcpyAsync(rows.data(), td, (size_t)m * 8, cudaMemcpyDeviceToHost, s));
     FZ_CUDA_TRY(cudaStreamSynchronize(s));
+    for (int t = 0; t < m; ++t) {
+        byt[t].rows = rows[t];
+        tab[t].kind = run_build_kind(byt[t], tab[t].K);
+    }
+    // jobs in build order: by depth, then by kind
+    std::vector<int> order(m), at(m);
+    for (int t = 0; t < m; ++t) order[t] = t;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+        return tab[x].K != tab[y].K ? tab[x].K < tab[y].K : tab[x].kind < tab[y].kind;
+    });
+    std::vector<RunBuild> rj(m);
+    for (int p = 0; p < m; ++p) {
+        at[order[p]] = p;
+        rj[p] = byt[order[p]];
+    }
+    for (int p = 0; p < m; ++p) rows[p] = rj[p].rows;
     size_t bytes = jb + cls_words * 8;
     for (int p = 0; p < m; ++p) {
         if (rows[p] > MEMO_MAX_ROWS)
             return set_error(FZ_EINVAL, "batch run-order memo too large");
-        rj[p].rows = rows[p];
         bytes += a256((size_t)rows[p] * 4 * run_stride(tab[order[p]].K + 1) + 16);
     }
     rc = b->runs.alloc(bytes);
@@ -586,10 +626,11 @@ int batch_create_runs(fz_batch_s *b, uint64_t *tb, cudaStream_t s) {
     rc = device_props(&dp);
     if (rc != FZ_OK) return rc;
     for (int p = 0; p < m;) {
-        const int K = tab[order[p]].K;
+        const int K = tab[order[p]].K, kind = tab[order[p]].kind;
         int e = p;
         uint64_t cost = 0;
-        for (; e < m && tab[order[e]].K == K; ++e) cost += run_build_cost(rj[e], false);
+        for (; e < m && tab[order[e]].K == K && tab[order[e]].kind == kind; ++e)
+            cost += run_build_cost(rj[e], false);
         const uint32_t share = run_build_share(cost, dp.sms);
         uint64_t blocks = 0;
         for (int q = p; q < e; ++q) {
@@ -603,7 +644,7 @@ int batch_create_runs(fz_batch_s *b, uint64_t *tb, cudaStream_t s) {
             }
             R.per_warp = share;
             R.blk0 = (uint32_t)blocks;
-            const uint32_t nb = run_build_blocks(R, K, false);
+            const uint32_t nb = run_build_blocks(R, kind, false);
             blocks += nb;
             if (nb > 1) ++b->run_wide;
             if (tab[order[q]].final) {
@@ -614,7 +655,7 @@ int batch_create_runs(fz_batch_s *b, uint64_t *tb, cudaStream_t s) {
         }
         if (blocks > 0x7fffffffull)
             return set_error(FZ_EINVAL, "batch run-order memos too large");
-        b->run_levels.push_back({K, p, e - p, (uint32_t)blocks});
+        b->run_levels.push_back({kind, p, e - p, (uint32_t)blocks});
         p = e;
     }
     b->run_jobs_dev = reinterpret_cast<RunBuild *>(base);
@@ -656,6 +697,10 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
         int &m = n_set[key];
         m = std::max(m, inst[i].n);
     }
+    double est_rows = 0;
+    for (int i = 0; i < count; ++i)
+        if (inst[i].g && inst[i].d >= 1 && inst[i].d <= FZ_MAX_D && validate_gens(inst[i].g, inst[i].d) == FZ_OK)
+            est_rows += lattice_volume(inst[i].g, inst[i].d, inst[i].n, false);
     for (int i = 0; i < count; ++i) {
         const fz_instance_t &x = inst[i];
         int rc = validate_gens(x.g, x.d);
@@ -669,7 +714,7 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
         const bool runs = run_memo_enabled() && pol.run_order[I.d];
         const bool part = opt && opt->top != FZ_AUTO && opt->top <= I.n;  // a partial memo
         if (runs && !part && walk_progression_enabled() && I.d >= 3 && I.d <= 8)
-            choose_batch_run(I, ns, pol.cap_rows[x.d]);
+            choose_batch_run(I, ns, pol.cap_rows[x.d], est_rows < BATCH_FEW_ROWS);
         else
             choose_batch_memo(I, ns, pol.cap_rows[x.d]);
         if (opt && opt->k != FZ_AUTO) {
@@ -699,8 +744,13 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
         I.off_RT = (size_t)-1;
         if (I.d >= 2) {
             balance_level(I.d, I.K, I.top, I.n, I.run, I.pair, &I.lam_r, &I.W, &I.clamp_row);
-            I.off_RT = words;
-            words += (size_t)(I.lam_r + 1) * len;
+            I.flat = I.d <= 8 &&
+                     (I.run ? flat_serves(I.d, lam, SRC_RUN)
+                            : (I.pair || (I.K == 0 && walk_progression_enabled())) &&
+                                  flat_serves(I.d, I.d - 2, SRC_PAIR));
+            const int rt_rows = I.flat ? I.lam_r - 1 : I.lam_r + 1;
+            if (rt_rows > 0) I.off_RT = words;
+            words += (size_t)rt_rows * len;
         } else {
             I.lam_r = -1;
         }
@@ -797,10 +847,8 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
         FZ_CUDA_TRY(cudaMemcpyAsync(b->tasks_dev, tasks.data(), tasks.size() * sizeof(ScanTask),
                                     cudaMemcpyHostToDevice, s));
     // count and runs tables
-    for (const auto &L : b->scan_launches) {
-        rc = launch_scan_tasks(b->jobs_dev, b->tasks_dev + L.first, L.second, s);
-        if (rc != FZ_OK) return fail(rc);
-    }
+    rc = batch_enqueue_scans(b, s);
+    if (rc != FZ_OK) return fail(rc);
     // memo sizes, then allocation and build
     std::vector<uint64_t> mrows(b->nmemo, 0);
     if (b->nmemo) {
@@ -862,6 +910,10 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
     rc = gather(pc, cnt, s);
     if (rc == FZ_OK) rc = gather(pr, runs, s);
     if (rc != FZ_OK) return fail(rc);
+    for (int i = 0; i < count; ++i) {
+        const Inst &I = b->inst[i];
+        if (I.flat && I.lam_r == 1) runs[i] = (uint64_t)(I.n / I.g[0]) + 1;
+    }
     int hstatus = 0;
     FZ_CUDA_TRY(cudaMemcpyAsync(&hstatus, b->status_dev, 4, cudaMemcpyDeviceToHost, s));
     FZ_CUDA_TRY(cudaStreamSynchronize(s));
@@ -913,11 +965,10 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
             L.cls_beg = I.cls_beg;
             L.memo_rows = I.run_rows;
         }
-        if (I.off_RT != (size_t)-1) {
-            L.RT = tb + I.off_RT;
-            L.W = I.W;
-            L.lam_r = I.lam_r;
-        }
+        if (I.off_RT != (size_t)-1) L.RT = tb + I.off_RT;
+        L.W = I.W;
+        L.lam_r = I.lam_r;
+        L.by_cost = I.flat || L.RT != nullptr;
         // out holds the word offset; the kernel adds the output base
         fill_batch_params(L, reinterpret_cast<int32_t *>(I.word_off * 4), I.count,
                           images.data() + (size_t)i * pbytes);

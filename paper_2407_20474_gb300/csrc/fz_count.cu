@@ -10,7 +10,8 @@
 //
 // Each row is a strided inclusive prefix sum of the row below it (stride
 // g_{j+1}): for every residue class rho mod g the entries rho, rho + g, ...
-// are summed in order.  Short chains are scanned by one warp each; long
+// are summed in order.  Short chains are scanned by a warp or a lane each or tile
+// by tile; long
 // chains are cut into blocks of RB entries, the block sums are scanned by the
 // same routine (they form a strided array of the same shape), and the blocks
 // are then re-walked with their carries.  All sums saturate at 2^64 - 1.
@@ -24,8 +25,9 @@ namespace fz {
 namespace {
 
 constexpr int64_t DIRECT_T = 4096;  // chains up to this length: one warp each
-constexpr int64_t LANE_T = 1024;    // chains up to this length, 32 or more: one lane each
+constexpr int64_t LANE_T = 256;     // chains up to this length, 32 or more: one lane each
 constexpr int LANE_ILP = 8;
+constexpr int64_t TILE_MAX_T = 16384;  // fewer than 8 chains up to this length: a tile each
 constexpr int RB = 32;              // entries per block in the blocked scan
 constexpr int THREADS = 256;
 
@@ -33,6 +35,71 @@ __global__ void row_delta_kernel(uint64_t *__restrict__ row, int64_t len) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (; i < len; i += stride) row[i] = (i == 0) ? 1ull : 0ull;
+}
+
+// ---------------------------------------------------------------------------
+// Tile scan: a block scans `width` (1, 8 or 32) neighbouring residue chains, its
+// threads cut into 256 / width segments of TILE_U consecutive chain entries (16
+// for a row on its own, 8 in the batched scans' 64 registers), so that loads
+// cover neighbouring entries of the row, all of a chunk's entries are in
+// flight at once, and each is read once.
+// The segments' sums meet by shuffles and in shared memory.  For chains longer
+// than 256 entries, where a warp or a lane a chain takes dozens of dependent
+// rounds of loads (six rows of 39065 entries, chains of 200 to 600: 47 us by a
+// warp a chain, 34 by tiles of 8; twelve rows of 1106 entries, chains of 25 to
+// 70: 44 and 57).  Entry r of the chains is entry off + r es of the row.
+// ---------------------------------------------------------------------------
+template <int TILE_U, class In>
+__device__ __forceinline__ void tile_scan(In input, uint64_t *__restrict__ out, int64_t len,
+                                          int64_t g, int64_t first, int width,
+                                          int64_t ones_below, int64_t off = 0, int64_t es = 1) {
+    __shared__ uint64_t part[2][8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int cls = threadIdx.x & (width - 1), seg = threadIdx.x / width;
+    const int nseg = THREADS / width;
+    const int64_t rho = first + cls;
+    const int64_t chains = g < len ? g : len;
+    const int64_t T = rho < chains ? (len - rho + g - 1) / g : 0;
+    const int64_t Tmax = (len - first + g - 1) / g;  // the tile's longest chain
+    uint64_t carry = 0;
+    int buf = 0;
+    for (int64_t t0 = 0; t0 < Tmax; t0 += (int64_t)nseg * TILE_U, buf ^= 1) {
+        const int64_t tb = t0 + (int64_t)seg * TILE_U;
+        uint64_t v[TILE_U];
+#pragma unroll
+        for (int u = 0; u < TILE_U; ++u)
+            v[u] = tb + u < T ? input(off + (rho + (tb + u) * g) * es) : 0ull;
+#pragma unroll
+        for (int u = 1; u < TILE_U; ++u) v[u] = sat_add(v[u], v[u - 1]);
+        uint64_t x = v[TILE_U - 1];  // inclusive over the warp's segments of the class
+        for (int o = width; o < 32; o <<= 1) {
+            const uint64_t y = __shfl_up_sync(FULL, x, o);
+            if (lane >= o) x = sat_add(x, y);
+        }
+        if (lane >= 32 - width) part[buf][warp][cls] = x;
+        uint64_t before = __shfl_up_sync(FULL, x, width & 31);
+        if (lane < width) before = 0;
+        __syncthreads();
+        before = sat_add(before, carry);
+#pragma unroll
+        for (int w = 0; w < THREADS / 32; ++w) {
+            const uint64_t y = part[buf][w][cls];
+            if (w < warp) before = sat_add(before, y);
+            carry = sat_add(carry, y);
+        }
+#pragma unroll
+        for (int u = 0; u < TILE_U; ++u) {
+            const int64_t x = off + (rho + (tb + u) * g) * es;
+            if (tb + u < T) out[x] = x < ones_below ? 1ull : sat_add(before, v[u]);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(THREADS, 4)
+row_tile_kernel(const uint64_t *__restrict__ in, uint64_t *__restrict__ out, int64_t len, int64_t g,
+                int width) {
+    tile_scan<16>([&](int64_t r) { return __ldg(in + r); }, out, len, g,
+              (int64_t)blockIdx.x * width, width, 0);
 }
 
 // One warp per residue chain; 4 x 32 entries loaded ahead of the scan.
@@ -129,6 +196,13 @@ int strided_scan(const uint64_t *in, uint64_t *out, int64_t len, int64_t g, uint
     const int64_t T = (len + g - 1) / g;
     if (T <= DIRECT_T) {
         int64_t chains = g < len ? g : len;
+        if (chains >= 8 && T > LANE_T) {
+            // 8 chains a block: a single row has few, and latency bounds it
+            row_tile_kernel<<<grid_for(chains, 8), THREADS, 0, s>>>(in, out, len, g, 8);
+            note_launch();
+            FZ_CUDA_TRY(cudaGetLastError());
+            return FZ_OK;
+        }
         int blocks = grid_for(chains * 32, THREADS);
         chain_scan_direct_kernel<<<blocks, THREADS, 0, s>>>(in, out, len, g);
         note_launch();
@@ -216,8 +290,15 @@ int launch_runs_table(const int32_t *g, int lam, int32_t n, uint64_t *RT, uint64
 // Logical entry r of a job's rows is entry off + r * es of the table row
 // (es = 1, off = 0: the whole row; es = g_1, off = n mod g_1: the one chain
 // of row 0 that is ever read).
-__device__ __forceinline__ void chain_scan_warp(const uint64_t *__restrict__ in,
-                                                uint64_t *__restrict__ out, int64_t len,
+__device__ __forceinline__ uint64_t scan_input(const ScanJob &J, const uint64_t *in, int64_t x) {
+    if (J.input == SCAN_LOAD) return __ldg(in + x);
+    if (J.input == SCAN_PAIR) return pair_form_count(J.pair, (uint32_t)x);
+    return (uint64_t)fd_div((uint32_t)x, J.lin) + 1ull;
+}
+
+// One chain by a warp, input(x) -> out (or S -> Sincl with a plain view).
+template <class In>
+__device__ __forceinline__ void chain_scan_warp(In input, uint64_t *__restrict__ out, int64_t len,
                                                 int64_t g, int64_t rho, int lane,
                                                 int64_t ones_below = 0, int64_t off = 0,
                                                 int64_t es = 1) {
@@ -228,7 +309,7 @@ __device__ __forceinline__ void chain_scan_warp(const uint64_t *__restrict__ in,
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             int64_t t = t0 + u * 32 + lane;
-            v[u] = t < T ? __ldg(in + off + (rho + t * g) * es) : 0ull;
+            v[u] = t < T ? input(off + (rho + t * g) * es) : 0ull;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -255,9 +336,9 @@ __global__ void __launch_bounds__(THREADS, MINB) scan_tasks_kernel(const ScanJob
     const int nwarps = blockDim.x >> 5;
     const int64_t es = J.es ? J.es : 1, off = J.off;
     switch (t.kind) {
-        case TK_DIRECT:
-            for (int64_t rho = t.begin + warp; rho < t.end; rho += nwarps)
-                chain_scan_warp(J.in, J.out, J.len, J.g, rho, lane, J.ones_below, off, es);
+        case TK_TILE:  // t.end: chains of the tile
+            tile_scan<8>([&](int64_t x) { return scan_input(J, J.in, x); }, J.out, J.len, J.g, t.begin,
+                      (int)t.end, J.ones_below, off, es);
             break;
         case TK_LANES: {
             // lane l of warp w: chain rho = begin + 32 w + l, walked down with
@@ -273,7 +354,7 @@ __global__ void __launch_bounds__(THREADS, MINB) scan_tasks_kernel(const ScanJob
                 uint64_t v[LANE_ILP];
 #pragma unroll
                 for (int u = 0; u < LANE_ILP; ++u)
-                    v[u] = t0 + u < T ? __ldg(in + off + (rho + (t0 + u) * J.g) * es) : 0ull;
+                    v[u] = t0 + u < T ? scan_input(J, in, off + (rho + (t0 + u) * J.g) * es) : 0ull;
 #pragma unroll
                 for (int u = 0; u < LANE_ILP; ++u) {
                     if (t0 + u < T) {
@@ -287,7 +368,8 @@ __global__ void __launch_bounds__(THREADS, MINB) scan_tasks_kernel(const ScanJob
         }
         case TK_SSCAN:
             for (int64_t rho = t.begin + warp; rho < t.end; rho += nwarps)
-                chain_scan_warp(J.S, J.Sincl, J.slen, J.g, rho, lane);
+                chain_scan_warp([&](int64_t x) { return __ldg(J.S + x); }, J.Sincl, J.slen, J.g, rho,
+                                lane);
             break;
         case TK_BSUM: {
             const int64_t rb = J.rb > 0 ? J.rb : RB;
@@ -300,7 +382,7 @@ __global__ void __launch_bounds__(THREADS, MINB) scan_tasks_kernel(const ScanJob
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
                         const int64_t r = r0 + (u0 + u) * J.g;
-                        v[u] = (u0 + u < rb && r < J.len) ? __ldg(J.in + off + r * es) : 0ull;
+                        v[u] = (u0 + u < rb && r < J.len) ? scan_input(J, J.in, off + r * es) : 0ull;
                     }
 #pragma unroll
                     for (int u = 0; u < 8; ++u) acc = sat_add(acc, v[u]);
@@ -320,7 +402,7 @@ __global__ void __launch_bounds__(THREADS, MINB) scan_tasks_kernel(const ScanJob
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
                         const int64_t r = r0 + (u0 + u) * J.g;
-                        v[u] = (u0 + u < rb && r < J.len) ? __ldg(J.in + off + r * es) : 0ull;
+                        v[u] = (u0 + u < rb && r < J.len) ? scan_input(J, J.in, off + r * es) : 0ull;
                     }
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
@@ -344,29 +426,13 @@ __global__ void __launch_bounds__(THREADS, MINB) scan_tasks_kernel(const ScanJob
                 J.out[off + i * es] = 1ull;
             break;
         case TK_PAIR:
-            // |Z(r, (g, h))|: the a with g a = r (mod h) in [0, r / g] are
-            // a = a* (mod h1), a* = (r / e) inv (mod h1), when e divides r
-            // (row d-1 is written only for whole rows: es == 1)
-            // (32-bit: entries, generators and their quotients are below
-            // 2^31; the product (re mod h1) inv needs 64 bits when h1 >= 2^16)
-            {
-                const uint32_t e = (uint32_t)J.e, h1 = (uint32_t)J.h1, g1 = (uint32_t)J.g1;
-                const uint32_t h = (uint32_t)J.h, inv = (uint32_t)J.inv;
-                const bool small = h1 < 65536u;
-                for (int64_t i = t.begin + threadIdx.x; i < t.end; i += blockDim.x) {
-                    const uint32_t r = (uint32_t)(off + i * es);
-                    uint64_t c = 0;
-                    if (r % e == 0) {
-                        const uint32_t re = r / e;
-                        const uint32_t astar =
-                            small ? (re % h1) * inv % h1
-                                  : (uint32_t)((uint64_t)(re % h1) * inv % h1);
-                        const uint32_t q = re / g1;
-                        c = q >= astar ? (uint64_t)((q - astar) / h1 + 1) : 0ull;
-                    }
-                    J.out[r] = c;
-                    if (J.ones_below && es == 1) J.out[J.len + r] = (r % h == 0) ? 1ull : 0ull;
-                }
+            // row d-2 in closed form, and row d-1 when a memo is built from it
+            // (whole rows only: es == 1)
+            for (int64_t i = t.begin + threadIdx.x; i < t.end; i += blockDim.x) {
+                const uint32_t r = (uint32_t)(off + i * es);
+                J.out[r] = pair_form_count(J.pair, r);
+                if (J.ones_below && es == 1)
+                    J.out[J.len + r] = fd_mod(r, J.pair.fh) == 0 ? 1ull : 0ull;
             }
             break;
         case TK_LINEAR:
@@ -402,6 +468,14 @@ int launch_scan_tasks(const ScanJob *jobs, const ScanTask *tasks, int ntasks, cu
     return FZ_OK;
 }
 
+// How the chains of a row (`chains` of them, the longest T entries) are
+// scanned: 0 = a lane each, else tiles of that width; -1 = blocked.
+int scan_plan(int64_t chains, int64_t T) {
+    if (chains < 8) return T <= TILE_MAX_T ? 1 : -1;
+    if (T > DIRECT_T) return -1;
+    if (chains >= 32 && T <= LANE_T) return 0;
+    return chains >= 32 && T <= 512 ? 32 : 8;
+}
 int64_t scan_direct_limit() { return DIRECT_T; }
 // Block sums a task of a blocked scan covers: one a thread (256).
 // FZ_SCAN_BS_TASK=2048 gives a thread eight (tuning only).
@@ -414,14 +488,6 @@ int64_t scan_blocks_per_task() {
     return v;
 }
 
-// FZ_SCAN_LANES=0 scans every short chain with a warp (tuning only).
-int64_t scan_lane_limit() {
-    static const int64_t v = [] {
-        const char *e = getenv("FZ_SCAN_LANES");
-        return (e && strcmp(e, "0") == 0) ? (int64_t)0 : LANE_T;
-    }();
-    return v;
-}
 int scan_block_rows() { return RB; }
 
 int launch_count_rolling(const int32_t *g, int d, int32_t n, uint64_t *a, uint64_t *b,

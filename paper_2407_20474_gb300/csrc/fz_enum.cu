@@ -1139,6 +1139,7 @@ static EnumParams make_params(const EnumLaunch &L) {
         P.flat_src = SRC_PAIR;
     }
     if (!flat_serves(L.d, P.flat_np, P.flat_src)) P.flat_np = 0;
+    P.by_cost = L.by_cost && (!P.flat_np || P.lam_r == P.flat_np);
     // the run walk's candidates are the prefixes of its LAMF = d - K - 1
     // leading coordinates; a table counted at another level cannot balance it
     if (runs && P.lam_r != L.d - L.K - 1) P.RT = nullptr;

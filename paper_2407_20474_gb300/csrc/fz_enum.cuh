@@ -28,6 +28,7 @@ struct EnumParams {
     uint64_t slice_rows;   // S (multiple of 4), used when RT is null
     uint64_t nslices;
     const uint64_t *RT;    // candidates table rows 0..lam_r (stride cs), or null
+    int by_cost;           // batch items by cost (see EnumLaunch)
     uint64_t W;            // cost of one unit of walk work (a prefix of length lam_r), in rows
     uint64_t slice_cost;   // cost units per work item when RT is set
     int lam_r;             // one past the leaf coordinate (RT[lam_r] = 1)
@@ -520,18 +521,27 @@ __device__ __forceinline__ bool flat_slice(const PA &pa, unsigned char *mem, uin
                                          (uint32_t)(row1 - row0), desc, ring, B, pol, lane);
 }
 
+// The flat walk's costs: the candidates table's row NP - 1 is x / g + 1, computed.
+template <int NP>
+__device__ __forceinline__ uint64_t flat_total_cost(const EnumParams &P) {
+    const uint64_t runs =
+        NP == 1 ? (uint64_t)fd_div((uint32_t)P.n, P.fdg[0]) + 1ull : __ldg(P.RT + P.n);
+    return __ldg(P.C + P.n) + P.W * runs;
+}
+
 // Ranks at which the cumulative costs t0 <= t1 are reached (cost_to_rank for a
 // candidates table counted at level NP), both searches' loads in flight
 // together.
 template <int NP>
 __device__ __forceinline__ void flat_cost_to_ranks(const EnumParams &P, uint64_t t0, uint64_t t1,
                                                    int lane, uint64_t &rank0, uint64_t &rank1) {
-    uint64_t tgt[2] = {t0, t1}, rank[2] = {0, 0};
+    uint64_t tgt[2] = {t0, t1}, rank[2] = {0, 0}, rows[2] = {0, 0};
     uint32_t rem[2] = {(uint32_t)P.n, (uint32_t)P.n};
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
         const uint32_t g = (uint32_t)P.g[j];
-        const uint64_t *C = P.C + (int64_t)j * P.cs, *T = P.RT + (int64_t)j * P.cs;
+        const uint64_t *C = P.C + (int64_t)j * P.cs;
+        const uint64_t *T = j < NP - 1 ? P.RT + (int64_t)j * P.cs : nullptr;
         uint32_t lo[2] = {0, 0}, hi[2], um[2];
         uint64_t flo[2] = {0, 0}, clo[2] = {0, 0};
 #pragma unroll
@@ -551,7 +561,7 @@ __device__ __forceinline__ void flat_cost_to_ranks(const EnumParams &P, uint64_t
                 if (in[k]) {
                     const uint32_t x = rem[k] - (um[k] + 1u - (uint32_t)u) * g;
                     cu[k] = __ldg(C + x);
-                    fu[k] = __ldg(T + x);
+                    fu[k] = j < NP - 1 ? __ldg(T + x) : (uint64_t)fd_div(x, P.fdg[j]) + 1ull;
                 }
             }
 #pragma unroll
@@ -574,14 +584,15 @@ __device__ __forceinline__ void flat_cost_to_ranks(const EnumParams &P, uint64_t
         for (int k = 0; k < 2; ++k) {
             rank[k] += clo[k];
             tgt[k] -= flo[k];
+            // the leaf's rows: the count row there less the children above it
+            if (j == NP - 1) rows[k] = __ldg(C + (rem[k] - (um[k] - lo[k]) * g)) - clo[k];
             rem[k] -= (um[k] - lo[k]) * g;
         }
     }
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        const uint64_t rows = __ldg(P.C + (int64_t)NP * P.cs + rem[k]);
         const uint64_t t = tgt[k] > P.W ? tgt[k] - P.W : 0ull;
-        rank[k] += t < rows ? t : rows;
+        rank[k] += t < rows[k] ? t : rows[k];
     }
     rank0 = rank[0];
     rank1 = rank[1];

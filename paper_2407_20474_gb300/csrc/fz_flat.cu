@@ -206,8 +206,8 @@ __global__ void __launch_bounds__(ENUM_THREADS, 3)
         const uint64_t s = batch_locate(BP, ep, cur, item, lane);
         const EnumParams &P = params();
         uint64_t row0, row1;
-        if (P.RT) {
-            const uint64_t cost_hi = cost_at(P, 0, P.n);
+        if (P.by_cost) {
+            const uint64_t cost_hi = flat_total_cost<NP>(P);
             const uint64_t c0 = s * P.slice_cost, c1 = c0 + P.slice_cost;
             if (c0 >= cost_hi) continue;
             row0 = 0;

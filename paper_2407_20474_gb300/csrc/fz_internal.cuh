@@ -68,6 +68,73 @@ __device__ __forceinline__ uint64_t warp_incl_scan(uint64_t v, int lane) {
     return v;
 }
 
+// Division and remainder of a 32-bit value by a fixed divisor via one
+// precomputed 64-bit multiplier (Lemire, Kaser and Kurz, "Faster remainder by
+// direct computation", 2019): M = floor((2^64 - 1) / g) + 1, a / g =
+// hi64(M * a), a % g = hi64(lo64(M * a) * g), exact for all a, g < 2^32, g > 1.
+struct FastDiv {
+    uint64_t M;
+    uint32_t g;
+};
+__host__ __device__ inline FastDiv make_fastdiv(uint32_t g) {
+    FastDiv f;
+    f.g = g;
+    f.M = g > 1 ? ~0ull / g + 1 : 0ull;
+    return f;
+}
+__device__ __forceinline__ uint32_t fd_div(uint32_t a, FastDiv f) {
+    return f.g > 1 ? (uint32_t)__umul64hi(f.M, a) : a;
+}
+__device__ __forceinline__ uint32_t fd_mod(uint32_t a, FastDiv f) {
+    return a - fd_div(a, f) * f.g;
+}
+
+// The pair (g, h) of the last two generators as a closed form: with e =
+// gcd(g, h), h1 = h / e, g1 = g / e, inv = g1^-1 mod h1, row o of
+// Z(p, (g, h)) is (a_top - o h1, b_0 + o g1), a_top the largest valid first
+// coordinate and b_0 = (p - a_top g) / h.
+struct PairForm {
+    FastDiv fe, fh1, fg, fh;
+    uint32_t inv, h1, g1, g;
+};
+
+__host__ inline PairForm make_pair_form(int32_t g, int32_t h) {
+    int64_t e, h1, g1, inv;
+    pair_params(g, h, &e, &h1, &g1, &inv);
+    PairForm F;
+    F.fe = make_fastdiv((uint32_t)e);
+    F.fh1 = make_fastdiv((uint32_t)h1);
+    F.fg = make_fastdiv((uint32_t)g);
+    F.fh = make_fastdiv((uint32_t)h);
+    F.inv = (uint32_t)inv;
+    F.h1 = (uint32_t)h1;
+    F.g1 = (uint32_t)g1;
+    F.g = (uint32_t)g;
+    return F;
+}
+
+// a_top of element p (meaningful when Z(p, (g, h)) is not empty): the
+// product (p / e mod h1) inv fits 32 bits when h1 < 2^16, else it takes a
+// 64-bit remainder.
+__device__ __forceinline__ uint32_t pair_form_top(const PairForm &F, uint32_t p) {
+    const uint32_t xr = fd_mod(fd_div(p, F.fe), F.fh1);
+    const uint32_t astar = F.h1 < 65536u ? fd_mod(xr * F.inv, F.fh1)
+                                         : (uint32_t)((uint64_t)xr * F.inv % F.h1);
+    const uint32_t q = fd_div(p, F.fg);
+    return q >= astar ? q - fd_mod(q - astar, F.fh1) : 0u;
+}
+
+// |Z(p, (g, h))|.
+__device__ __forceinline__ uint32_t pair_form_count(const PairForm &F, uint32_t p) {
+    const uint32_t re = fd_div(p, F.fe);
+    if (re * F.fe.g != p) return 0u;
+    const uint32_t xr = fd_mod(re, F.fh1);
+    const uint32_t astar = F.h1 < 65536u ? fd_mod(xr * F.inv, F.fh1)
+                                         : (uint32_t)((uint64_t)xr * F.inv % F.h1);
+    const uint32_t q = fd_div(p, F.fg);
+    return q >= astar ? fd_div(q - astar, F.fh1) + 1u : 0u;
+}
+
 // ---------------------------------------------------------------------------
 // Memory-model helpers.
 // ---------------------------------------------------------------------------
@@ -279,21 +346,24 @@ struct ScanJob {
     uint64_t *Sincl;     // their strided inclusive scan
     int64_t slen;        // entries of S
     int64_t ones_below;  // entries r < ones_below of out are written as 1
+    // TK_PAIR: out = row d-2 of a count table, out + len = row d-1 (written
+    // only when ones_below != 0), for the last two generators (pair)
+    PairForm pair;
+    // scan input: SCAN_LOAD reads `in`; SCAN_PAIR computes the pair's count
+    // and SCAN_LINEAR x / lin + 1 at entry x, so those rows need no memory
+    int input;
+    FastDiv lin;
     // strided view: logical entry r of in/out is entry off + r * es (es = 0
     // means 1); the one chain of a row that is ever read
-    // TK_PAIR: out = row d-2 of a count table, out + len = row d-1 (written
-    // only when ones_below != 0), for the last two generators g (= this g)
-    // and h, e = gcd(g, h), h1 = h / e, g1 = g / e, inv = g1^-1 mod h1 (0 when
-    // h1 = 1)
-    int64_t h, e, h1, g1, inv;
     int64_t off, es;
     // entries per block of a blocked scan (0: scan_block_rows()); long
     // chains take larger blocks so their chains of block sums stay within
     // the direct-scan limit
     int64_t rb;
 };
+enum ScanInput : int { SCAN_LOAD = 0, SCAN_PAIR = 1, SCAN_LINEAR = 2 };
 enum ScanTaskKind : int {
-    TK_DIRECT = 0,  // chains [begin, end) of in -> out, one warp each
+    TK_TILE = 0,    // chains [begin, begin + end) of in -> out, a tile scan
     TK_BSUM = 1,    // block sums S[begin..end)
     TK_SSCAN = 2,   // chains [begin, end) of S -> Sincl
     TK_APPLY = 3,   // blocks [begin, end): out = carry + running sum
@@ -310,7 +380,7 @@ struct ScanTask {
 };
 int launch_scan_tasks(const ScanJob *jobs, const ScanTask *tasks, int ntasks, cudaStream_t s);
 int64_t scan_direct_limit();  // chains up to this length are scanned directly
-int64_t scan_lane_limit();    // chains up to this length, 32 or more of them: a lane each
+int scan_plan(int64_t chains, int64_t T);  // 0: a lane a chain, w: tiles of w chains, -1: blocked
 int64_t scan_blocks_per_task();  // block sums a TK_BSUM / TK_APPLY task covers
 int scan_block_rows();        // entries per block of a blocked scan
 
@@ -400,6 +470,9 @@ struct EnumLaunch {
     const uint64_t *RT = nullptr;
     uint64_t W = 0;
     int lam_r = 0;
+    // items by cost (RT may then lack the rows from lam_r - 1 on, and be null
+    // for lam_r = 1: the flat walk's batch kernels compute them)
+    bool by_cost = false;
     uint64_t total_cost = 0, total_rows = 0;
     // the output is host memory reached over the host link: flush rows with
     // plain coalesced stores instead of bulk (TMA) stores

@@ -220,6 +220,46 @@ __global__ void __launch_bounds__(BT)
     reinterpret_cast<int4 *>(J.dst)[row] = make_int4((int)q, (int)m, 0, 0);
 }
 
+// Tables of depth 2 with fewer rows than elements: a thread per lattice point
+// (x, y), element p = x t0 + y t1 <= n, writes its one row.  The points of the
+// columns x and X - x (X = n div t0) share one line of `wide` threads, about as
+// many as both hold.  The row's place inside its element counts the points
+// with a greater x; all rows of an element below p are its class's count.
+//
+// 4096 instances of widths 3..8 (4.1e7 elements, 1.1e7 rows): 270 us
+// with the dense tables' flat walk, against 613 us by the flat walk alone, which reads a count for every element.
+__global__ void __launch_bounds__(BT)
+    run_build2_kernel(const RunBuild *__restrict__ jobs, int njobs, int *status) {
+    __shared__ RunBuild sj;
+    load_job(jobs, njobs, sj);
+    const RunBuild &J = sj;
+    const PairForm &F = J.src.pair;
+    const uint32_t t0 = F.g, t1 = F.fh.g, n = (uint32_t)J.n;
+    const uint32_t wide = (n + t0) / t1 + 2u, X = fd_div(n, F.fg);
+    const uint64_t i = (uint64_t)(blockIdx.x - J.blk0) * BT + threadIdx.x;
+    uint32_t x = (uint32_t)(i / wide);
+    uint32_t y = (uint32_t)(i - (uint64_t)x * wide);
+    if (x > X / 2u) return;
+    const uint32_t len = fd_div(n - x * t0, F.fh) + 1u;
+    if (y >= len) {
+        y -= len;
+        const uint32_t other = X - x;
+        if (other == x || y > fd_div(n - other * t0, F.fh)) return;
+        x = other;
+    }
+    const uint32_t p = x * t0 + y * t1;
+    const uint32_t top = pair_form_top(F, p);
+    const uint32_t cnt = fd_div(top, F.fh1) + 1u;  // rows of the element
+    const uint32_t q = p / (uint32_t)J.g;
+    const uint64_t row = __ldg(J.cls + (p - q * (uint32_t)J.g)) + __ldg(J.F + p) - cnt +
+                         fd_div(top - x, F.fh1);
+    if (row >= J.rows) {
+        atomicExch(status, (int)DEV_INTERNAL);
+        return;
+    }
+    reinterpret_cast<int4 *>(J.dst)[row] = make_int4((int)q, (int)x, (int)y, 0);
+}
+
 // Class starts of each job's table: cls[c] = rows of the classes below c (a
 // class's rows are the count row at its last element).  One block a job.
 __global__ void __launch_bounds__(BT)
@@ -346,6 +386,11 @@ int launch_run_build(const RunBuild *jobs_dev, int njobs, int K, bool csr, uint3
             note_launch();
             FZ_CUDA_TRY(cudaGetLastError());
             return FZ_OK;
+        case RUN_LATTICE:
+            run_build2_kernel<<<blocks, BT, 0, s>>>(jobs_dev, njobs, status);
+            note_launch();
+            FZ_CUDA_TRY(cudaGetLastError());
+            return FZ_OK;
         case 2: return launch_level<2, SRC_PAIR, false>(jobs_dev, njobs, blocks, status, s);
         case 3: return launch_level<3, SRC_RUN, false>(jobs_dev, njobs, blocks, status, s);
         case 4: return launch_level<4, SRC_RUN, false>(jobs_dev, njobs, blocks, status, s);
@@ -387,9 +432,18 @@ uint32_t run_build_share(uint64_t total, int sms) {
     return (uint32_t)((per + 31) & ~31ull);
 }
 
+int run_build_kind(const RunBuild &R, int K) {
+    return K == 2 && R.rows < (uint64_t)R.n ? RUN_LATTICE : K;
+}
+
 uint32_t run_build_blocks(const RunBuild &R, int K, bool csr) {
     if (R.rows == 0) return 0;
     if (K == 1) return (uint32_t)(((uint64_t)R.n / R.src.fg.g + 1 + BT - 1) / BT);
+    if (K == RUN_LATTICE) {
+        const uint64_t t0 = R.src.pair.g, t1 = R.src.pair.fh.g;
+        const uint64_t wide = ((uint64_t)R.n + t0) / t1 + 2, lines = (uint64_t)R.n / t0 / 2 + 1;
+        return (uint32_t)((lines * wide + BT - 1) / BT);
+    }
     const uint64_t items = (run_build_cost(R, csr) + R.per_warp - 1) / R.per_warp;
     return (uint32_t)((items + BW - 1) / BW);
 }
@@ -465,7 +519,7 @@ int run_levels_init(const int32_t *t, int k, int32_t n, const uint64_t *sums, bo
         R.dst = rows[j];
         fill_run_build(t, k, n, j, false, &R);
         R.per_warp = run_build_share(run_build_cost(R, false), dp.sms);
-        L->K[L->n] = k - 1 - j;
+        L->K[L->n] = run_build_kind(R, k - 1 - j);
         if (j < last) {
             R.src.rows = rows[j + 1];
             R.src.cls = cls[j + 1];

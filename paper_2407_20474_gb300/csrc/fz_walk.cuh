@@ -7,62 +7,6 @@
 
 namespace fz {
 
-// Division and remainder of a 32-bit value by a fixed divisor via one
-// precomputed 64-bit multiplier (Lemire, Kaser and Kurz, "Faster remainder by
-// direct computation", 2019): M = floor((2^64 - 1) / g) + 1, a / g =
-// hi64(M * a), a % g = hi64(lo64(M * a) * g), exact for all a, g < 2^32, g > 1.
-struct FastDiv {
-    uint64_t M;
-    uint32_t g;
-};
-__host__ __device__ inline FastDiv make_fastdiv(uint32_t g) {
-    FastDiv f;
-    f.g = g;
-    f.M = g > 1 ? ~0ull / g + 1 : 0ull;
-    return f;
-}
-__device__ __forceinline__ uint32_t fd_div(uint32_t a, FastDiv f) {
-    return f.g > 1 ? (uint32_t)__umul64hi(f.M, a) : a;
-}
-__device__ __forceinline__ uint32_t fd_mod(uint32_t a, FastDiv f) {
-    return a - fd_div(a, f) * f.g;
-}
-
-// The pair (g, h) of the last two generators as a closed form: with e =
-// gcd(g, h), h1 = h / e, g1 = g / e, inv = g1^-1 mod h1, row o of
-// Z(p, (g, h)) is (a_top - o h1, b_0 + o g1), a_top the largest valid first
-// coordinate and b_0 = (p - a_top g) / h.
-struct PairForm {
-    FastDiv fe, fh1, fg, fh;
-    uint32_t inv, h1, g1, g;
-};
-
-__host__ inline PairForm make_pair_form(int32_t g, int32_t h) {
-    int64_t e, h1, g1, inv;
-    pair_params(g, h, &e, &h1, &g1, &inv);
-    PairForm F;
-    F.fe = make_fastdiv((uint32_t)e);
-    F.fh1 = make_fastdiv((uint32_t)h1);
-    F.fg = make_fastdiv((uint32_t)g);
-    F.fh = make_fastdiv((uint32_t)h);
-    F.inv = (uint32_t)inv;
-    F.h1 = (uint32_t)h1;
-    F.g1 = (uint32_t)g1;
-    F.g = (uint32_t)g;
-    return F;
-}
-
-// a_top of element p (meaningful when Z(p, (g, h)) is not empty): the
-// product (p / e mod h1) inv fits 32 bits when h1 < 2^16, else it takes a
-// 64-bit remainder.
-__device__ __forceinline__ uint32_t pair_form_top(const PairForm &F, uint32_t p) {
-    const uint32_t xr = fd_mod(fd_div(p, F.fe), F.fh1);
-    const uint32_t astar = F.h1 < 65536u ? fd_mod(xr * F.inv, F.fh1)
-                                         : (uint32_t)((uint64_t)xr * F.inv % F.h1);
-    const uint32_t q = fd_div(p, F.fg);
-    return q >= astar ? q - fd_mod(q - astar, F.fh1) : 0u;
-}
-
 // ---------------------------------------------------------------------------
 // Staged rows.  A warp assembles rows in a shared-memory ring of two halves
 // of B rows and sends every full half to global memory with one bulk (TMA)
@@ -200,6 +144,10 @@ int launch_run_levels(const RunLevels &L, int *status, cudaStream_t s);
 void fill_run_build(const int32_t *t, int k, int32_t n, int j, bool csr, RunBuild *out);
 uint64_t run_build_cost(const RunBuild &R, bool csr);
 uint32_t run_build_share(uint64_t total, int sms);
+// How a table of depth K is built: K, or RUN_LATTICE for depth 2 with fewer
+// rows than elements (rows and n set).
+constexpr int RUN_LATTICE = -2;
+int run_build_kind(const RunBuild &R, int K);
 uint32_t run_build_blocks(const RunBuild &R, int K, bool csr);
 int launch_run_totals(const RunBuild *jobs_dev, int njobs, uint64_t *totals, cudaStream_t s);
 int launch_run_classes(const RunBuild *jobs_dev, int njobs, int *status, cudaStream_t s);

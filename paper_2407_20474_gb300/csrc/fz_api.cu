@@ -68,10 +68,46 @@ int validate_gens(const int32_t *g, int d) {
 
 namespace {
 
-// RAII device buffer (cudaMalloc / cudaFree).
+// Device memory that lives no longer than one call comes from a stream-ordered
+// pool of the library's own, one per device: allocating and freeing then costs
+// microseconds and no device synchronisation (cudaMalloc and cudaFree took
+// most of a small call: 324 us for 3.8e3 rows, 154 with the pool).  The
+// pool keeps at most POOL_KEEP_BYTES between calls; what lies above goes back
+// to the device at the next synchronisation.  Allocation and release are
+// ordered on the call's stream, so any number of threads and streams share it.
+// Handles (plans, memos, batches, servers) own cudaMalloc memory.
+constexpr uint64_t POOL_KEEP_BYTES = 64ull << 20;
+
+cudaMemPool_t call_pool() {
+    static std::mutex mu;
+    static cudaMemPool_t pools[64];
+    static bool tried[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!tried[dev]) {
+        tried[dev] = true;
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        uint64_t keep = POOL_KEEP_BYTES;
+        if (cudaMemPoolCreate(&pool, &props) == cudaSuccess &&
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+            pools[dev] = pool;
+        cudaGetLastError();
+    }
+    return pools[dev];
+}
+
+// RAII device buffer: cudaMalloc / cudaFree, or the call pool on a stream.
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
+    bool pooled = false;
+    cudaStream_t stream = nullptr;
     DevBuf() = default;
     DevBuf(const DevBuf &) = delete;
     DevBuf &operator=(const DevBuf &) = delete;
@@ -87,10 +123,30 @@ struct DevBuf {
         bytes = b;
         return FZ_OK;
     }
+    // For memory whose every use is on stream s and which is released before
+    // the call returns.  Without a pool (or when it fails) as alloc.
+    int alloc_call(size_t b, cudaStream_t s) {
+        release();
+        if (b == 0) b = 16;
+        cudaMemPool_t pool = call_pool();
+        if (pool && cudaMallocFromPoolAsync(&p, b, pool, s) == cudaSuccess) {
+            bytes = b;
+            pooled = true;
+            stream = s;
+            return FZ_OK;
+        }
+        if (pool) cudaGetLastError();
+        p = nullptr;
+        return alloc(b);
+    }
     void release() {
-        if (p) cudaFree(p);
+        if (p && pooled)
+            cudaFreeAsync(p, stream);
+        else if (p)
+            cudaFree(p);
         p = nullptr;
         bytes = 0;
+        pooled = false;
     }
     template <class T>
     T *as() const {
@@ -150,6 +206,12 @@ struct fz_plan_s {
     int *status = nullptr;
     unsigned *bar = nullptr;
     unsigned long long *counter = nullptr;
+    // a plan that lives inside one call takes its memory from the call pool
+    bool one_call = false;
+    cudaStream_t call_stream = nullptr;
+    int alloc(DevBuf &b, size_t bytes) {
+        return one_call ? b.alloc_call(bytes, call_stream) : b.alloc(bytes);
+    }
 };
 
 struct fz_memo_s {
@@ -363,7 +425,7 @@ int plan_alloc_memo(fz_plan_s *p, const uint64_t *sums, cudaStream_t s) {
     const int lam = d - k - 1;
     if (p->top > p->n && lam >= 0 && (k <= 3 || flat_serves(d, lam, SRC_RUN)) &&
         run_memo_enabled()) {
-        if (p->lvbuf.alloc(run_levels_bytes(p->g + lam, k + 1, p->n, sums + lam, false)) ==
+        if (p->alloc(p->lvbuf, run_levels_bytes(p->g + lam, k + 1, p->n, sums + lam, false)) ==
             FZ_OK) {
             const int rc = run_levels_init(p->g + lam, k + 1, p->n, sums + lam, false,
                                            p->C + (int64_t)lam * cs, cs, nullptr, nullptr,
@@ -379,7 +441,7 @@ int plan_alloc_memo(fz_plan_s *p, const uint64_t *sums, cudaStream_t s) {
     const size_t rows_bytes = align256(p->memo_rows * (size_t)k * 4 + 16);
     if (csr && p->memo_rows > 0) {
         const size_t b = run_levels_bytes(p->g + (d - k), k, p->top - 1, sums + (d - k), true);
-        if (p->lvbuf.alloc(b) == FZ_OK && p->memo.alloc(rows_bytes) == FZ_OK) {
+        if (p->alloc(p->lvbuf, b) == FZ_OK && p->alloc(p->memo, rows_bytes) == FZ_OK) {
             p->rows = p->memo.as<int32_t>();
             return run_levels_init(p->g + (d - k), k, p->top - 1, sums + (d - k), true,
                                    p->C + (int64_t)(d - k) * cs, cs, p->O, p->rows, p->lvbuf.p,
@@ -389,7 +451,7 @@ int plan_alloc_memo(fz_plan_s *p, const uint64_t *sums, cudaStream_t s) {
         p->lvbuf.release();
     }
     const size_t off_rows = k <= 2 ? 0 : align256(p->memo_rows * 8);
-    int rc = p->memo.alloc(off_rows + rows_bytes);
+    int rc = p->alloc(p->memo, off_rows + rows_bytes);
     if (rc != FZ_OK) return rc;
     p->map = k <= 2 ? nullptr : p->memo.as<uint64_t>();
     p->rows = reinterpret_cast<int32_t *>(p->memo.as<char>() + off_rows);
@@ -422,7 +484,7 @@ int plan_create_impl(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, f
     const size_t off_bar = off_status + 256;
     const size_t off_counter = off_bar + 256;
     const size_t total = off_counter + 256;
-    rc = p->base.alloc(total);
+    rc = p->alloc(p->base, total);
     if (rc != FZ_OK) return rc;
     char *b = p->base.as<char>();
     p->C = reinterpret_cast<uint64_t *>(b + off_C);
@@ -478,8 +540,6 @@ int plan_create_impl(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, f
         if (rc != FZ_OK) return rc;
         rc = plan_enqueue_memo(p, s);
         if (rc != FZ_OK) return rc;
-        rc = read_status(p->status, s);
-        if (rc != FZ_OK) return rc;
     }
     // runs table for work-balanced slicing (not needed when the output is a
     // single block: d == 1 or k == d with a full memo)
@@ -487,13 +547,17 @@ int plan_create_impl(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, f
     if (!single_block && p->count > 0) {
         balance_level(d, p->K, p->top, n, p->run_memo != nullptr, false, &p->lam_r, &p->W,
                       &p->clamp_row);
-        rc = p->runs.alloc((size_t)(p->lam_r + 1) * cs * 8);
+        rc = p->alloc(p->runs, (size_t)(p->lam_r + 1) * cs * 8);
         if (rc != FZ_OK) return rc;
         p->RT = p->runs.as<uint64_t>();
         rc = launch_runs_table(p->g, p->lam_r, n, p->RT, p->tmp, p->clamp_row, p->top, s);
         if (rc != FZ_OK) return rc;
         FZ_CUDA_TRY(cudaMemcpyAsync(&p->total_runs, p->RT + n, 8, cudaMemcpyDeviceToHost, s));
-        FZ_CUDA_TRY(cudaStreamSynchronize(s));
+    }
+    // one read back: the memo build's status and the run total
+    rc = read_status(p->status, s);
+    if (rc != FZ_OK) return rc;
+    if (p->RT) {
         uint64_t wr = 0;
         if (mul_overflows(p->W, p->total_runs, &wr) || p->count + wr < p->count) {
             p->RT = nullptr;  // costs would not fit in 64 bits: slice by rows
@@ -864,7 +928,7 @@ int fz_count_upto(const int32_t *g, int d, int32_t n_max, uint64_t *counts, void
     const int64_t len = (int64_t)n_max + 1;
     int64_t tmpw = count_table_tmp_words(g, d, n_max);
     DevBuf buf;
-    rc = buf.alloc((size_t)(2 * len + tmpw) * 8);
+    rc = buf.alloc_call((size_t)(2 * len + tmpw) * 8, s);
     if (rc != FZ_OK) return rc;
     uint64_t *a = buf.as<uint64_t>(), *b = a + len, *tmp = b + len, *res = nullptr;
     rc = launch_count_rolling(g, d, n_max, a, b, tmp, &res, s);
@@ -883,7 +947,7 @@ int fz_count(const int32_t *g, int d, int32_t n, uint64_t *count, void *stream) 
     const int64_t len = (int64_t)n + 1;
     int64_t tmpw = count_table_tmp_words(g, d, n);
     DevBuf buf;
-    rc = buf.alloc((size_t)(2 * len + tmpw) * 8);
+    rc = buf.alloc_call((size_t)(2 * len + tmpw) * 8, s);
     if (rc != FZ_OK) return rc;
     uint64_t *a = buf.as<uint64_t>(), *b = a + len, *tmp = b + len, *res = nullptr;
     rc = launch_count_rolling(g, d, n, a, b, tmp, &res, s);
@@ -904,7 +968,16 @@ int fz_count_table(const int32_t *g, int d, int32_t n, uint64_t *table_dev, void
     cudaStream_t s = as_stream(stream);
     int64_t tmpw = count_table_tmp_words(g, d, n);
     uint64_t *tmp = nullptr;
-    if (tmpw > 0) FZ_CUDA_TRY(cudaMallocAsync((void **)&tmp, (size_t)tmpw * 8, s));
+    // (a stream under capture takes its graph's own memory)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    FZ_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+    cudaMemPool_t pool = cap == cudaStreamCaptureStatusNone ? call_pool() : nullptr;
+    if (tmpw > 0 && pool &&
+        cudaMallocFromPoolAsync((void **)&tmp, (size_t)tmpw * 8, pool, s) != cudaSuccess) {
+        cudaGetLastError();
+        tmp = nullptr;
+    }
+    if (tmpw > 0 && !tmp) FZ_CUDA_TRY(cudaMallocAsync((void **)&tmp, (size_t)tmpw * 8, s));
     rc = launch_count_table_tmp(g, d, n, table_dev, tmp, s);
     if (tmp) cudaFreeAsync(tmp, s);
     return rc;
@@ -919,7 +992,7 @@ static int memo_common(const int32_t *tail, int k, int32_t top, cudaStream_t s, 
     const int32_t n = top > 0 ? top - 1 : 0;
     const int64_t cs = (int64_t)n + 1;
     int64_t tmpw = std::max(count_table_tmp_words(tail, k, n), exclusive_scan_tmp_words(cs));
-    rc = table.alloc((size_t)((k + 1) * cs + tmpw + 64) * 8);
+    rc = table.alloc_call((size_t)((k + 1) * cs + tmpw + 64) * 8, s);
     if (rc != FZ_OK) return rc;
     *C = table.as<uint64_t>();
     *tmpw_out = tmpw;
@@ -940,7 +1013,7 @@ int fz_memo_rows(const int32_t *tail, int k, int32_t top, uint64_t *rows, void *
     int64_t tmpw = 0;
     int rc = memo_common(tail, k, top, s, table, &C, &tmpw);
     if (rc != FZ_OK) return rc;
-    rc = off.alloc((size_t)(top + 1) * 8);
+    rc = off.alloc_call((size_t)(top + 1) * 8, s);
     if (rc != FZ_OK) return rc;
     const int64_t cs = (int64_t)top;
     rc = launch_exclusive_scan_tmp(C, off.as<uint64_t>(), top, C + (k + 1) * cs, s);
@@ -965,9 +1038,15 @@ static int build_memo_to(const int32_t *tail, int k, int32_t top, uint64_t *O, i
     uint64_t *tmp = C + (k + 1) * cs;
     rc = launch_exclusive_scan_tmp(C, O, top, tmp, s);
     if (rc != FZ_OK) return rc;
-    uint64_t rows = 0;
+    uint64_t rows = 0, sums[FZ_MAX_D + 1] = {};
+    const bool levels = schedule == MEMO_LEVELS && !memo_fill_forced() && k <= CSR_MAX_K;
     FZ_CUDA_TRY(cudaMemcpyAsync(&rows, O + top, 8, cudaMemcpyDeviceToHost, s));
-    FZ_CUDA_TRY(cudaStreamSynchronize(s));
+    if (levels && k > 2) {  // the rows of every level, read together with the memo's
+        rc = row_sums(C, cs, k, top, C + (k + 1) * cs + tmpw, sums, s);
+        if (rc != FZ_OK) return rc;
+    } else {
+        FZ_CUDA_TRY(cudaStreamSynchronize(s));
+    }
     if (rows_needed) *rows_needed = rows;
     if (rows == ~0ull) return set_error(FZ_EOVERFLOW, "memo rows do not fit in 64 bits");
     if (own_rows) {
@@ -982,19 +1061,15 @@ static int build_memo_to(const int32_t *tail, int k, int32_t top, uint64_t *O, i
         // depth 1 and 2: the closed form; deeper: the run-order levels while
         // they apply and their scratch fits; else the dynamic pass
         schedule = FZ_MEMO_BATCHED;
-        if (!memo_fill_forced() && k <= CSR_MAX_K) {
-            uint64_t sums[FZ_MAX_D + 1];
+        if (levels) {
             size_t bytes = 256;
             bool fits = true;
-            uint64_t *small = C + (k + 1) * cs + tmpw;  // 64 words past the scan scratch
             if (k > 2) {
-                rc = row_sums(C, cs, k, top, small, sums, s);
-                if (rc != FZ_OK) return rc;
                 sums[0] = rows;
                 fits = sums[1] < (1ull << 32) && rows / 256 < (1ull << 31);
                 if (fits) bytes += run_levels_bytes(tail, k, top - 1, sums, true);
             }
-            if (fits && work.alloc(bytes) == FZ_OK) {
+            if (fits && work.alloc_call(bytes, s) == FZ_OK) {
                 int *status = work.as<int>();
                 FZ_CUDA_TRY(cudaMemsetAsync(status, 0, 256, s));
                 if (k <= 2) {
@@ -1013,7 +1088,7 @@ static int build_memo_to(const int32_t *tail, int k, int32_t top, uint64_t *O, i
     }
     // gather map + status + barrier words
     const size_t map_bytes = align256(rows * 8);
-    rc = work.alloc(map_bytes + 512);
+    rc = work.alloc_call(map_bytes + 512, s);
     if (rc != FZ_OK) return rc;
     MemoBuffers mb;
     mb.Ct = C;
@@ -1254,11 +1329,13 @@ int fz_autotune(const int32_t *g, int d, int32_t n, fz_opts_t *best, double *bes
 }
 
 // -------------------------------------------------------------------- plans
-int fz_plan_create(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, fz_plan_t *plan,
-                   void *stream) {
+static int plan_create(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, bool one_call,
+                       fz_plan_t *plan, void *stream) {
     if (!plan) return set_error(FZ_EINVAL, "plan: null pointer");
     fz_plan_s *p = new (std::nothrow) fz_plan_s;
     if (!p) return set_error(FZ_ENOMEM, "host allocation");
+    p->one_call = one_call;
+    p->call_stream = as_stream(stream);
     int rc = plan_create_impl(g, d, n, opt, p, as_stream(stream));
     if (rc != FZ_OK) {
         cudaStreamSynchronize(as_stream(stream));
@@ -1267,6 +1344,11 @@ int fz_plan_create(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, fz_
     }
     *plan = p;
     return FZ_OK;
+}
+
+int fz_plan_create(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, fz_plan_t *plan,
+                   void *stream) {
+    return plan_create(g, d, n, opt, false, plan, stream);
 }
 
 int fz_plan_info(fz_plan_t p, fz_plan_info_t *info) {
@@ -1325,9 +1407,7 @@ int fz_plan_unrank(fz_plan_t p, const uint64_t *ranks_dev, uint64_t m, int32_t *
 
 int fz_plan_sync(fz_plan_t p, void *stream) {
     if (!p) return set_error(FZ_EINVAL, "plan: null pointer");
-    cudaStream_t s = as_stream(stream);
-    FZ_CUDA_TRY(cudaStreamSynchronize(s));
-    return read_status(p->status, s);
+    return read_status(p->status, as_stream(stream));
 }
 
 int fz_plan_destroy(fz_plan_t p) {
@@ -1341,7 +1421,7 @@ int fz_enumerate(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, uint6
                  uint64_t rank_end, int32_t *out_dev, uint64_t out_capacity_rows,
                  uint64_t *written, void *stream) {
     fz_plan_t p = nullptr;
-    int rc = fz_plan_create(g, d, n, opt, &p, stream);
+    int rc = plan_create(g, d, n, opt, true, &p, stream);
     if (rc != FZ_OK) return rc;
     rc = fz_plan_enumerate(p, rank_begin, rank_end, out_dev, out_capacity_rows, written, stream);
     if (rc == FZ_OK) rc = fz_plan_sync(p, stream);
@@ -1361,7 +1441,7 @@ int fz_enumerate_host_chunks(const int32_t *g, int d, int32_t n, const fz_opts_t
                              uint64_t out_capacity_rows, uint64_t chunk_rows,
                              uint64_t *written, void *stream) {
     fz_plan_t p = nullptr;
-    int rc = fz_plan_create(g, d, n, opt, &p, stream);
+    int rc = plan_create(g, d, n, opt, true, &p, stream);
     if (rc != FZ_OK) return rc;
     const uint64_t rows = rows_in(p, rank_begin, rank_end);
     if (written) *written = rows;

@@ -495,14 +495,19 @@ int plan_create_impl(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, f
     p->counter = reinterpret_cast<unsigned long long *>(b + off_counter);
     FZ_CUDA_TRY(cudaMemsetAsync(b + off_status, 0, 768, s));
 
-    rc = launch_count_table_tmp(g, d, n, p->C, p->tmp, s);
-    if (rc != FZ_OK) return rc;
     // the count, and the memo rows of every depth (one read)
     uint64_t sums[FZ_MAX_D + 1] = {};
     uint64_t *sums_dev = reinterpret_cast<uint64_t *>(p->status + 16);
+    const bool small = small_tables(n);
+    rc = small ? launch_tables_small(g, d, n, p->C, nullptr, 0, -1, 0, sums_dev, s)
+               : launch_count_table_tmp(g, d, n, p->C, p->tmp, s);
+    if (rc != FZ_OK) return rc;
     FZ_CUDA_TRY(cudaMemcpyAsync(&p->count, p->C + n, sizeof(uint64_t), cudaMemcpyDeviceToHost,
                                 s));
-    if (!opt || opt->k != 0) {
+    if (small) {
+        FZ_CUDA_TRY(cudaMemcpyAsync(sums, sums_dev, (size_t)(d + 1) * 8, cudaMemcpyDeviceToHost, s));
+        FZ_CUDA_TRY(cudaStreamSynchronize(s));
+    } else if (!opt || opt->k != 0) {
         rc = row_sums(p->C, cs, d + 1, cs, sums_dev, sums, s);
         if (rc != FZ_OK) return rc;
     } else {
@@ -1270,7 +1275,7 @@ int fz_autotune_report(const int32_t *g, int d, int32_t n, fz_tune_entry_t *entr
         }
         const uint64_t base_slice = p->slice_rows;
         for (uint64_t sl : {base_slice, base_slice / 2, base_slice * 2}) {
-            if (sl < 1024) continue;
+            if (sl < 128) continue;
             p->slice_rows = (sl + 31) & ~31ull;
             // screening pass (also the warm-up): one window, scaled to the set
             double b_ms = 0, e_ms = 0;
@@ -1375,6 +1380,12 @@ int fz_plan_set_enum_ctas_per_sm(fz_plan_t p, int32_t ctas) {
 int fz_plan_rebuild(fz_plan_t p, void *stream) {
     if (!p) return set_error(FZ_EINVAL, "plan: null pointer");
     cudaStream_t s = as_stream(stream);
+    if (small_tables(p->n)) {
+        const int rc = launch_tables_small(p->g, p->d, p->n, p->C, p->RT, p->lam_r, p->clamp_row,
+                                           p->top, nullptr, s);
+        if (rc != FZ_OK) return rc;
+        return plan_enqueue_memo(p, s);
+    }
     int rc = launch_count_table_tmp(p->g, p->d, p->n, p->C, p->tmp, s);
     if (rc != FZ_OK) return rc;
     if (p->RT) {

@@ -173,6 +173,89 @@ block_apply_kernel(const uint64_t *__restrict__ in, uint64_t *__restrict__ out,
     }
 }
 
+// ---------------------------------------------------------------------------
+// Short tables (n <= SMALL_N): all rows of a table in one launch, one block,
+// the row in hand in shared memory.  A row is scanned by doubling: log2(n / g)
+// steps add the entry s = g, 2 g, 4 g, ... below.  Block 0: the count table
+// (or its row 0 only), block 1: the candidates table.  Row by row these are a
+// launch each of which the GPU runs in 3 us, 12 launches for a set of width 9.
+// ---------------------------------------------------------------------------
+constexpr int SMALL_N = 12000;
+constexpr int SMALL_THREADS = 1024;
+struct SmallTables {
+    uint64_t *C;      // rows 0..d, or null
+    uint64_t *C0;     // row 0 only, or null
+    uint64_t *RT;     // rows 0..lam, or null
+    uint64_t *sums;   // sums[j] of row j's entries (each clamped to 2^32), or null
+    int d, n, lam, clamp_row, clamp_top;
+    int g[FZ_MAX_D];
+};
+
+__global__ void __launch_bounds__(SMALL_THREADS) small_tables_kernel(const __grid_constant__ SmallTables P) {
+    extern __shared__ __align__(16) uint64_t small_smem[];
+    __shared__ uint64_t part[SMALL_THREADS / 32];
+    const bool runs = P.C == nullptr && P.C0 == nullptr ? true : blockIdx.x == 1;
+    const int len = P.n + 1, rows = runs ? P.lam : P.d;
+    uint64_t *a = small_smem, *b = small_smem + len;
+    uint64_t *out = runs ? P.RT : P.C;
+    for (int r = threadIdx.x; r < len; r += SMALL_THREADS) {
+        const uint64_t v = runs || r == 0 ? 1ull : 0ull;
+        a[r] = v;
+        if (out) out[(int64_t)rows * len + r] = v;
+    }
+    __syncthreads();
+    for (int j = rows - 1;; --j) {
+        if (!runs && P.sums) {  // of row j + 1, in hand
+            uint64_t acc = 0;
+            for (int r = threadIdx.x; r < len; r += SMALL_THREADS)
+                acc += a[r] < (1ull << 32) ? a[r] : (1ull << 32);
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+            if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                for (int w = 1; w < SMALL_THREADS / 32; ++w) acc += part[w];
+                P.sums[j + 1] = acc;
+            }
+            __syncthreads();
+        }
+        if (j < 0) break;
+        for (int64_t s = P.g[j]; s < len; s *= 2) {
+            for (int r = threadIdx.x; r < len; r += SMALL_THREADS)
+                b[r] = r >= s ? sat_add(a[r], a[r - s]) : a[r];
+            __syncthreads();
+            uint64_t *t = a;
+            a = b;
+            b = t;
+        }
+        if (runs && j == P.clamp_row) {
+            for (int r = threadIdx.x; r < len && r < P.clamp_top; r += SMALL_THREADS) a[r] = 1ull;
+            __syncthreads();
+        }
+        if (out)
+            for (int r = threadIdx.x; r < len; r += SMALL_THREADS) out[(int64_t)j * len + r] = a[r];
+    }
+    if (!runs && P.C0)
+        for (int r = threadIdx.x; r < len; r += SMALL_THREADS) P.C0[r] = a[r];
+}
+
+int launch_small_tables(const SmallTables &P, cudaStream_t s) {
+    static DeviceOnce attr_set;
+    int dev = 0;
+    FZ_CUDA_TRY(cudaGetDevice(&dev));
+    if (!attr_set.is_set(dev)) {
+        FZ_CUDA_TRY(cudaFuncSetAttribute(small_tables_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         2 * (SMALL_N + 1) * 8));
+        attr_set.set(dev);
+    }
+    const int blocks = (P.C || P.C0 ? 1 : 0) + (P.RT ? 1 : 0);
+    small_tables_kernel<<<blocks, SMALL_THREADS, 2 * ((size_t)P.n + 1) * 8, s>>>(P);
+    note_launch();
+    FZ_CUDA_TRY(cudaGetLastError());
+    return FZ_OK;
+}
+
 int grid_for(int64_t work, int per_block) {
     int64_t b = (work + per_block - 1) / per_block;
     if (b < 1) b = 1;
@@ -236,8 +319,26 @@ int64_t count_table_tmp_words(const int32_t *g, int d, int32_t n) {
 
 int64_t exclusive_scan_tmp_words(int64_t len) { return scan_tmp_words(len, 1); }
 
+bool small_tables(int32_t n) { return n <= SMALL_N; }
+
+int launch_tables_small(const int32_t *g, int d, int32_t n, uint64_t *C, uint64_t *RT, int lam,
+                        int clamp_row, int64_t clamp_top, uint64_t *sums, cudaStream_t s) {
+    SmallTables P{};
+    P.C = C;
+    P.RT = RT;
+    P.sums = sums;
+    P.d = d;
+    P.n = n;
+    P.lam = lam;
+    P.clamp_row = clamp_top > 0 ? clamp_row : -1;
+    P.clamp_top = (int)(clamp_top < (int64_t)n + 1 ? clamp_top : (int64_t)n + 1);
+    for (int i = 0; i < d; ++i) P.g[i] = g[i];
+    return launch_small_tables(P, s);
+}
+
 int launch_count_table_tmp(const int32_t *g, int d, int32_t n, uint64_t *table, uint64_t *tmp,
                            cudaStream_t s) {
+    if (small_tables(n)) return launch_tables_small(g, d, n, table, nullptr, 0, -1, 0, nullptr, s);
     const int64_t len = (int64_t)n + 1;
     uint64_t *last = table + (int64_t)d * len;
     row_delta_kernel<<<grid_for(len, THREADS), THREADS, 0, s>>>(last, len);
@@ -262,6 +363,8 @@ __global__ void row_ones_kernel(uint64_t *__restrict__ row, int64_t len) {
 // stride g_j -- the count-table recurrence over the leading generators.
 int launch_runs_table(const int32_t *g, int lam, int32_t n, uint64_t *RT, uint64_t *tmp,
                       int clamp_row, int64_t clamp_top, cudaStream_t s) {
+    if (small_tables(n))
+        return launch_tables_small(g, lam, n, nullptr, RT, lam, clamp_row, clamp_top, nullptr, s);
     const int64_t len = (int64_t)n + 1;
     row_ones_kernel<<<grid_for(len, THREADS), THREADS, 0, s>>>(RT + (int64_t)lam * len, len);
     note_launch();
@@ -493,6 +596,15 @@ int scan_block_rows() { return RB; }
 int launch_count_rolling(const int32_t *g, int d, int32_t n, uint64_t *a, uint64_t *b,
                          uint64_t *tmp, uint64_t **result, cudaStream_t s) {
     const int64_t len = (int64_t)n + 1;
+    if (small_tables(n)) {
+        SmallTables P{};
+        P.C0 = a;
+        P.d = d;
+        P.n = n;
+        for (int i = 0; i < d; ++i) P.g[i] = g[i];
+        *result = a;
+        return launch_small_tables(P, s);
+    }
     row_delta_kernel<<<grid_for(len, THREADS), THREADS, 0, s>>>(a, len);
     note_launch();
     FZ_CUDA_TRY(cudaGetLastError());

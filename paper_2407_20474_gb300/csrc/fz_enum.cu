@@ -1179,6 +1179,7 @@ int launch_enumerate(const EnumLaunch &L, uint64_t rank_begin, uint64_t nrows, i
     P.rank_begin = rank_begin;
     P.nrows = nrows;
     P.aligned = ((uintptr_t)out & 15u) == 0 && !L.plain_stores;
+    P.whole = rank_begin == 0 && L.total_rows == nrows;
     if (L.d == 1 || (L.K == L.d && L.top > L.n)) {
         const int mode = (L.d == 1 && !(L.K == 1 && L.top > L.n)) ? 2 : 1;
         uint64_t words = nrows * (uint64_t)L.d;
@@ -1361,11 +1362,15 @@ int launch_enumerate_batch(const void *params_dev, const uint64_t *item0_dev,
 }
 
 uint64_t default_slice_rows(uint64_t nrows, int sms) {
-    // about eight work items per resident warp, between 1024 and 65536 rows
-    uint64_t warps = (uint64_t)sms * 2 * ENUM_WARPS;
-    uint64_t s = nrows / (warps * 8 + 1);
-    if (s < 1024) s = 1024;
-    if (s > 65536) s = 65536;
+    // about 2.5 items a resident warp, between 128 and 24576 rows: an item
+    // starts with a dozen dependent loads, long ones leave a tail and write
+    // too far apart (kernel us at 1024 / 4096 / 16384 / 65536 rows an item:
+    // 5e8 rows of width 6 2660 / 1914 / 1830 / 2456, 1e8 558 / 401 / 516 / -,
+    // 1.4e7 of width 9 128 / 152 / 314 / -)
+    uint64_t s = nrows * 2 / ((uint64_t)sms * 4 * ENUM_WARPS * 5);
+    const uint64_t least = nrows / 64 < 128 ? 128 : nrows / 64 > 512 ? 512 : nrows / 64;
+    if (s < least) s = least;
+    if (s > 24576) s = 24576;
     return (s + 31) & ~31ull;
 }
 

@@ -28,7 +28,8 @@ struct EnumParams {
     uint64_t slice_rows;   // S (multiple of 4), used when RT is null
     uint64_t nslices;
     const uint64_t *RT;    // candidates table rows 0..lam_r (stride cs), or null
-    int by_cost;           // batch items by cost (see EnumLaunch)
+    int by_cost;           // items by cost (see EnumLaunch)
+    int whole;             // all rows of the set are asked for
     uint64_t W;            // cost of one unit of walk work (a prefix of length lam_r), in rows
     uint64_t slice_cost;   // cost units per work item when RT is set
     int lam_r;             // one past the leaf coordinate (RT[lam_r] = 1)

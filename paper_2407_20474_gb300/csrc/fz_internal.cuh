@@ -331,6 +331,12 @@ int validate_gens(const int32_t *g, int d);
 int64_t count_table_tmp_words(const int32_t *g, int d, int32_t n);
 int launch_count_table_tmp(const int32_t *g, int d, int32_t n, uint64_t *table, uint64_t *tmp,
                            cudaStream_t s);
+// Short tables (small_tables(n)): count table C and candidates table RT (rows
+// 0..lam, clamped as launch_runs_table; either may be null) in one launch, with
+// the rows' sums (d + 1, entries clamped to 2^32) if asked for.
+bool small_tables(int32_t n);
+int launch_tables_small(const int32_t *g, int d, int32_t n, uint64_t *C, uint64_t *RT, int lam,
+                        int clamp_row, int64_t clamp_top, uint64_t *sums, cudaStream_t s);
 // Only row 0 (|Z(r, g)|, r = 0..n) with two rolling rows a, b (n + 1 words
 // each); returns which of them holds the result.
 int launch_count_rolling(const int32_t *g, int d, int32_t n, uint64_t *a, uint64_t *b,

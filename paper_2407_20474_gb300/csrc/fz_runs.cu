@@ -177,17 +177,22 @@ __global__ void __launch_bounds__(BT, 4)
         flat_rows<NP, W, DS, SRC>(wk, base, (uint32_t)(row0 - base), job, row0, left, desc, ring,
                                   B, pol, lane);
     } else {
-        // equal cost; a table's rows are whole 16-byte vectors, so a warp may
-        // start at any row
+        // equal cost; a warp starts at any row of a table whose rows are whole
+        // 16-byte vectors, at an even one of 24-byte rows (bulk stores)
         __shared__ uint64_t s_row[BW + 1];
         const uint64_t total = J.rows + FLAT_LEAF_COST * ((uint64_t)J.n + 1u);
         const uint64_t x = item * J.per_warp;
         TablePlace pl{0, 0, J.rows};
+        auto even = [&](uint64_t r) {
+            if (DS % 4 != 0) r = (r + 1) & ~1ull;
+            return r < J.rows ? r : J.rows;
+        };
         if (x < total) pl = table_place(J, x, lane);
+        pl.row = even(pl.row);
         if (lane == 0) s_row[wid] = pl.row;
         if (wid == 0) {
             const uint64_t xe = (item + BW) * J.per_warp;
-            const uint64_t re = xe < total ? table_place(J, xe, lane).row : J.rows;
+            const uint64_t re = xe < total ? even(table_place(J, xe, lane).row) : J.rows;
             if (lane == 0) s_row[BW] = re;
         }
         __syncthreads();

@@ -70,8 +70,32 @@ __device__ __forceinline__ void store_row(int32_t *dst, const int (&w)[DS], int 
 }
 
 // Words between the rows of a run-order table whose rows hold W words (the
-// quotient and W - 1 coordinates): whole 16-byte vectors.
-__host__ __device__ constexpr int run_stride(int W) { return (W + 3) & ~3; }
+// quotient and W - 1 coordinates): whole 16-byte vectors, or 24 bytes for 5
+// and 6 words (a memo of 3.6e7 rows copied from rows of 32 bytes was bound by
+// L2: 197 us, 171 us with 24).
+__host__ __device__ constexpr int run_stride(int W) {
+    return W == 5 || W == 6 ? 6 : (W + 3) & ~3;
+}
+template <int SS>
+__device__ __forceinline__ void load_run_row(const int32_t *p, int (&x)[SS]) {
+    if constexpr (SS % 4 == 0) {
+#pragma unroll
+        for (int v = 0; v < SS / 4; ++v) {
+            const int4 y = __ldg(reinterpret_cast<const int4 *>(p) + v);
+            x[4 * v] = y.x;
+            x[4 * v + 1] = y.y;
+            x[4 * v + 2] = y.z;
+            x[4 * v + 3] = y.w;
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < SS / 2; ++v) {
+            const int2 y = __ldg(reinterpret_cast<const int2 *>(p) + v);
+            x[2 * v] = y.x;
+            x[2 * v + 1] = y.y;
+        }
+    }
+}
 
 // Where the rows of a leaf (an element p) come from.
 //   SRC_RUN:  the run-order table of (gen; tail): the rows of Z(p, (gen,
@@ -215,7 +239,7 @@ __device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip
     bool ok = true;
 
     struct Frag {
-        int4 v[RPL][SRC == SRC_RUN ? SS / 4 : 1];
+        int x[RPL][SRC == SRC_RUN ? SS : 1];
         int l[RPL];
     };
 
@@ -253,13 +277,12 @@ __device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip
         const uint32_t e = E - base < 0xffffffffull ? (uint32_t)(E - base) : 0xffffffffu;
         const uint32_t s = Eprev - base < 0xffffffffull ? (uint32_t)(Eprev - base) : 0xffffffffu;
         const uint32_t e_all = __shfl_sync(FULL, e, 31);
-        // the end of this batch's rows (skip lies in leaf 0, so only an
-        // inconsistent table has e_all below it)
+        // the end of this batch's rows (skip may lie a row past leaf 0)
         const uint32_t q_end = e_all <= skip ? skip : e_all - skip < left ? e_all : skip + left;
         // leaves with rows in the window, in order
         const bool used = live && e > s && e > skip && s < q_end;
         const uint32_t rank = __popc(__ballot_sync(FULL, used) & (le >> 1));
-        bool bad = E < Eprev || e_all < skip;
+        bool bad = E < Eprev;
         __syncwarp();  // the previous batch's descriptors have been read
         if (used) {
             int d[DV * 4];
@@ -309,10 +332,7 @@ __device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip
                     if ((uint32_t)lane + 32u * u < cnt) {
                         const uint32_t row =
                             reinterpret_cast<const uint32_t *>(desc + F.l[u])[0] + qh + lane;
-                        const int4 *src =
-                            reinterpret_cast<const int4 *>(K.src().rows) + (size_t)row * (SS / 4);
-#pragma unroll
-                        for (int v = 0; v < SS / 4; ++v) F.v[u][v] = __ldg(src + v);
+                        load_run_row<SS>(K.src().rows + (size_t)row * SS, F.x[u]);
                     }
                 }
             }
@@ -344,17 +364,9 @@ __device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip
 #pragma unroll
                     for (int c = 0; c < NP; ++c) w[c] = d[H + c];
                     if constexpr (SRC == SRC_RUN) {
-                        int x[SS];
+                        w[NP] = d[1] - F.x[u][0];
 #pragma unroll
-                        for (int v = 0; v < SS / 4; ++v) {
-                            x[4 * v] = F.v[u][v].x;
-                            x[4 * v + 1] = F.v[u][v].y;
-                            x[4 * v + 2] = F.v[u][v].z;
-                            x[4 * v + 3] = F.v[u][v].w;
-                        }
-                        w[NP] = d[1] - x[0];
-#pragma unroll
-                        for (int c = 1; c < W; ++c) w[NP + c] = x[c];
+                        for (int c = 1; c < W; ++c) w[NP + c] = F.x[u][c];
                     } else {
                         const uint32_t o = q0 + 32u * u + lane - (uint32_t)d[0];
                         w[NP] = d[1] - (int)(o * K.src().pair.h1);
@@ -414,7 +426,7 @@ __device__ __forceinline__ bool flat_rows(Walk &wk, uint64_t base, uint32_t skip
             }
         }
         left -= rows;
-        skip = 0;
+        skip = skip > e_all ? skip - e_all : 0u;
         base = Elast;
     }
     if (hpos > 0)

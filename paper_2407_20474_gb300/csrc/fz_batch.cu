@@ -969,6 +969,8 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
         L.W = I.W;
         L.lam_r = I.lam_r;
         L.by_cost = I.flat || L.RT != nullptr;
+        L.total_rows = I.count;
+        L.total_cost = costs[i];
         // out holds the word offset; the kernel adds the output base
         fill_batch_params(L, reinterpret_cast<int32_t *>(I.word_off * 4), I.count,
                           images.data() + (size_t)i * pbytes);

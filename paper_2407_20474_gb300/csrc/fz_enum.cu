@@ -1166,6 +1166,17 @@ static EnumParams make_params(const EnumLaunch &L) {
         default: return set_error(FZ_EINVAL, "d out of range"); \
     }
 
+// More than `least` prefixes a row: by rank.  The flat walk visits every prefix
+// (12 us a million), the rank walk searches every row (41 us a million; 1e7
+// rows of width 6 under 8.6e7 prefixes: 1054 against 409 us): 3 for one set.
+// In a batch the searches of many sets miss L2 (4096 sets of 1e2..1e6 rows:
+// 4557 us without, 4672 with 3, 4557 with 10; 96 sets of 1e2..1e4 rows 218,
+// 210, 209): 10.
+static bool by_rank(const EnumLaunch &L, const EnumParams &P, uint64_t least) {
+    return P.flat_np > 0 && P.flat_src == SRC_PAIR && rank_walk_serves(L.d) && L.RT &&
+           L.total_cost > L.total_rows + least * L.W * L.total_rows;
+}
+
 // Enumerate ranks [rank_begin, rank_begin + nrows) into out.  Asynchronous.
 int launch_enumerate(const EnumLaunch &L, uint64_t rank_begin, uint64_t nrows, int32_t *out,
                      uint64_t slice_rows, cudaStream_t s) {
@@ -1206,10 +1217,7 @@ int launch_enumerate(const EnumLaunch &L, uint64_t rank_begin, uint64_t nrows, i
         uint64_t sc = (uint64_t)((double)slice_rows * per_row);
         P.slice_cost = sc < 64 ? 64 : sc;
     }
-    // more prefixes than rows: by rank (the flat walk visits every prefix)
-    if (P.flat_np > 0 && P.flat_src == SRC_PAIR && rank_walk_serves(L.d) && L.RT &&
-        L.total_cost > L.total_rows + L.W * L.total_rows)
-        return launch_rank_walk(P, ring_bytes_for(L.ctas_per_sm), s, dp.sms);
+    if (by_rank(L, P, 3)) return launch_rank_walk(P, ring_bytes_for(L.ctas_per_sm), s, dp.sms);
     if (P.flat_np > 0) return launch_enum_flat(P, ring_bytes_for(L.ctas_per_sm), s, dp.sms);
     P.half_rows = half_rows_for(L.d, ring_bytes_for(L.ctas_per_sm));
     FZ_DISPATCH_D(L.d, launch_enum_d, P, s, dp.sms);
@@ -1240,13 +1248,14 @@ void fill_batch_params(const EnumLaunch &L, int32_t *out, uint64_t count, void *
     P.aligned = ((uintptr_t)out & 15u) == 0;
     P.half_rows = half_rows_for(L.d);
     if (L.d > 8) P.flat_np = 0;  // the batch kernel's flat walk: widths 3..8
+    if (by_rank(L, P, 10)) P.flat_src = SRC_RANK;
     memcpy(dst, &P, sizeof(P));
 }
 
 uint32_t enum_params_shape(const void *image) {
     EnumParams P;
     memcpy(&P, image, sizeof(P));
-    return P.flat_np ? (uint32_t)(P.d << 8 | P.flat_np << 1 | P.flat_src) : 0u;
+    return P.flat_np ? (uint32_t)(P.d << 8 | P.flat_np << 2 | P.flat_src) : 0u;
 }
 
 void batch_order(const unsigned char *images, size_t pb, const uint64_t *cost, int count,
@@ -1282,9 +1291,15 @@ void batch_order(const unsigned char *images, size_t pb, const uint64_t *cost, i
 // 1900), although an item starts with a dozen dependent loads (about 10 us).
 void batch_items(unsigned char *params, size_t pb, const uint64_t *cost, const int *order,
                  std::vector<BatchGroup> *groups, int sms, uint64_t *item0) {
+    // by rank a row costs about four rows of the flat walk, a prefix nothing
+    auto cost_of = [&](int p) {
+        EnumParams P;
+        memcpy(&P, params + (size_t)p * pb, sizeof(P));
+        return P.flat_src == SRC_RANK ? 4 * P.nrows : cost[order[p]];
+    };
     uint64_t total = 0;
     for (const BatchGroup &G : *groups)
-        for (int p = G.first; p < G.last; ++p) total += cost[order[p]];
+        for (int p = G.first; p < G.last; ++p) total += cost_of(p);
     uint64_t target = total / ((uint64_t)sms * 24 * 8 + 1);
     target = target < 512 ? 512 : target > 2048 ? 2048 : target;
     item0[0] = 0;
@@ -1293,7 +1308,7 @@ void batch_items(unsigned char *params, size_t pb, const uint64_t *cost, const i
         for (int p = G.first; p < G.last; ++p) {
             EnumParams P;
             memcpy(&P, params + (size_t)p * pb, sizeof(P));
-            const uint64_t c = cost[order[p]];
+            const uint64_t c = cost_of(p);
             const uint64_t items = P.nrows == 0 || c == 0 ? 0 : (c + target - 1) / target;
             if (items) {
                 P.slice_cost = (c + items - 1) / items;
@@ -1331,8 +1346,8 @@ int launch_enumerate_batch(const void *params_dev, const uint64_t *item0_dev,
         BP.item_counter = counters + i;
         BP.chained = chained ? 1 : 0;
         if (G.shape) {
-            rc = launch_flat_batch(BP, (int)(G.shape >> 8), (int)(G.shape >> 1 & 127),
-                                   (int)(G.shape & 1), s, dp.sms, ctas_per_sm);
+            rc = launch_flat_batch(BP, (int)(G.shape >> 8), (int)(G.shape >> 2 & 63),
+                                   (int)(G.shape & 3), s, dp.sms, ctas_per_sm);
             if (rc != FZ_OK) return rc;
             chained = true;
             continue;

@@ -57,7 +57,7 @@ struct EnumParams {
     // is a_{d-2} = a_top - o h1, a_{d-1} = (p - a_{d-2} g_{d-2}) / g_{d-1}.
     int pair_memo;
     int flat_np;           // > 0: the flat walk, leaves are prefixes of this length
-    int flat_src;          // SRC_RUN or SRC_PAIR
+    int flat_src;          // SRC_RUN, SRC_PAIR or (batches) SRC_RANK
 };
 
 struct WarpPath {

@@ -93,18 +93,95 @@ int launch_one(EnumParams P, int warp_bytes, cudaStream_t s, int sms) {
 // Bound by the latency of the searches' dependent loads.  The case above: 1054
 // us by the flat walk, 409 by the rank walk.
 // ---------------------------------------------------------------------------
+// Rows [row0, row0 + rows) of the set.  Returns false if the tables disagree.
+template <int D, class PA>
+__device__ __forceinline__ bool rank_rows(const PA &params, int32_t *ring, uint32_t B,
+                                          uint64_t row0, uint32_t rows, uint64_t pol, int lane) {
+    constexpr int NP = D - 2;
+    bool ok = true;
+    // a[j], remainders, and the ranks where the subtree of (a_0..a_{j-1})
+    // begins and that of (a_0..a_j) ends
+    uint32_t a[NP], r[NP + 1];
+    uint64_t beg[NP + 1], end[NP];
+    r[0] = (uint32_t)params().n;
+    beg[0] = 0;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+        a[j] = 0;
+        end[j] = 0;
+    }
+    uint32_t at = 0, b0 = 0, hpos = 0, half = 0, nfull = 0;
+    for (uint32_t q = 0; q < rows;) {
+        uint32_t cnt = rows - q;
+        if (cnt > 32u) cnt = 32u;
+        if (cnt > B - hpos) cnt = B - hpos;
+        const bool act = (uint32_t)lane < cnt;
+        const uint64_t R = params().rank_begin + row0 + q + lane;
+        if (act && R >= end[NP - 1]) {
+            bool fresh = false;  // the parent changed
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+                if (!fresh && R < end[j]) continue;
+                const uint32_t g = (uint32_t)params().g[j];
+                const uint64_t *row = params().C + (int64_t)j * params().cs;
+                const uint32_t vmax = fd_div(r[j], params().fdg[j]);
+                const bool again = !fresh && end[j] > 0;  // same parent, a later child
+                const uint64_t all = again ? 0ull : __ldg(row + r[j]);
+                uint64_t before;
+                if (again)
+                    a[j] = thread_child_from(row, r[j], g, vmax, R - beg[j],
+                                             a[j] > 0 ? a[j] - 1u : 0u, &before);
+                else
+                    a[j] = thread_child(row, r[j], g, vmax, R - beg[j], all, D - 1 - j, &before);
+                r[j + 1] = r[j] - a[j] * g;
+                end[j] = beg[j] + __ldg(row + r[j + 1]);
+                beg[j + 1] = beg[j] + before;
+                fresh = true;
+            }
+            at = pair_form_top(params().leaf.pair, r[NP]);
+            b0 = fd_div(r[NP] - at * params().leaf.pair.g, params().leaf.pair.fh);
+            if (R >= end[NP - 1]) ok = false;  // the tables disagree
+        }
+        if (hpos == 0 && nfull >= 2) {
+            if (lane == 0) bulk_wait_read<1>();
+            __syncwarp();
+        }
+        if (act) {
+            const uint32_t o = (uint32_t)(R - beg[NP]);
+            int w[D];
+#pragma unroll
+            for (int j = 0; j < NP; ++j) w[j] = (int)a[j];
+            w[NP] = (int)(at - o * params().leaf.pair.h1);
+            w[NP + 1] = (int)(b0 + o * params().leaf.pair.g1);
+            store_row<D>(ring + (size_t)(half * B + hpos + lane) * D, w, lane);
+        }
+        q += cnt;
+        hpos += cnt;
+        if (hpos == B) {
+            flush_words(params().out + (row0 + (uint64_t)nfull * B) * D, params().aligned != 0,
+                        ring + (size_t)half * B * D, B * D, lane, pol);
+            ++nfull;
+            half ^= 1u;
+            hpos = 0;
+        }
+    }
+    if (hpos > 0)
+        flush_words(params().out + (row0 + (uint64_t)nfull * B) * D, params().aligned != 0,
+                    ring + (size_t)half * B * D, hpos * D, lane, pol);
+    if (lane == 0) bulk_wait_read_all();
+    ok = __all_sync(FULL, ok);
+    if (!ok && lane == 0) atomicExch(params().status, (int)DEV_INTERNAL);
+    return ok;
+}
+
 template <int D>
 __global__ void __launch_bounds__(ENUM_THREADS, 4)
     fz_enum_rank_kernel(const __grid_constant__ EnumParams P, int warp_bytes) {
-    constexpr int NP = D - 2;
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
     int32_t *ring = reinterpret_cast<int32_t *>(enum_smem + (size_t)wid * warp_bytes);
-    const uint32_t B = (uint32_t)P.half_rows;
     const uint64_t pol = policy_evict_first();
-    const PairForm &F = P.leaf.pair;
-    bool ok = true;
-    while (ok) {
+    for (;;) {
         unsigned long long s = 0;
         if (lane == 0) s = atomicAdd(P.slice_counter, 1ull);
         s = __shfl_sync(FULL, s, 0);
@@ -112,78 +189,7 @@ __global__ void __launch_bounds__(ENUM_THREADS, 4)
         const uint64_t row0 = s * P.slice_rows;
         const uint64_t rest = P.nrows - row0;
         const uint32_t rows = rest < P.slice_rows ? (uint32_t)rest : (uint32_t)P.slice_rows;
-        // a[j], remainders, and the ranks where the subtree of (a_0..a_{j-1})
-        // begins and that of (a_0..a_j) ends
-        uint32_t a[NP], r[NP + 1];
-        uint64_t beg[NP + 1], end[NP];
-        r[0] = (uint32_t)P.n;
-        beg[0] = 0;
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            a[j] = 0;
-            end[j] = 0;
-        }
-        uint32_t at = 0, b0 = 0, hpos = 0, half = 0, nfull = 0;
-        for (uint32_t q = 0; q < rows;) {
-            uint32_t cnt = rows - q;
-            if (cnt > 32u) cnt = 32u;
-            if (cnt > B - hpos) cnt = B - hpos;
-            const bool act = (uint32_t)lane < cnt;
-            const uint64_t R = P.rank_begin + row0 + q + lane;
-            if (act && R >= end[NP - 1]) {
-                bool fresh = false;  // the parent changed
-#pragma unroll
-                for (int j = 0; j < NP; ++j) {
-                    if (!fresh && R < end[j]) continue;
-                    const uint32_t g = (uint32_t)P.g[j];
-                    const uint64_t *row = P.C + (int64_t)j * P.cs;
-                    const uint32_t vmax = fd_div(r[j], P.fdg[j]);
-                    const bool again = !fresh && end[j] > 0;  // same parent, a later child
-                    const uint64_t all = again ? 0ull : __ldg(row + r[j]);
-                    uint64_t before;
-                    if (again)
-                        a[j] = thread_child_from(row, r[j], g, vmax, R - beg[j],
-                                                 a[j] > 0 ? a[j] - 1u : 0u, &before);
-                    else
-                        a[j] = thread_child(row, r[j], g, vmax, R - beg[j], all, D - 1 - j, &before);
-                    r[j + 1] = r[j] - a[j] * g;
-                    end[j] = beg[j] + __ldg(row + r[j + 1]);
-                    beg[j + 1] = beg[j] + before;
-                    fresh = true;
-                }
-                at = pair_form_top(F, r[NP]);
-                b0 = fd_div(r[NP] - at * F.g, F.fh);
-                if (R >= end[NP - 1]) ok = false;  // the tables disagree
-            }
-            if (hpos == 0 && nfull >= 2) {
-                if (lane == 0) bulk_wait_read<1>();
-                __syncwarp();
-            }
-            if (act) {
-                const uint32_t o = (uint32_t)(R - beg[NP]);
-                int w[D];
-#pragma unroll
-                for (int j = 0; j < NP; ++j) w[j] = (int)a[j];
-                w[NP] = (int)(at - o * F.h1);
-                w[NP + 1] = (int)(b0 + o * F.g1);
-                store_row<D>(ring + (size_t)(half * B + hpos + lane) * D, w, lane);
-            }
-            q += cnt;
-            hpos += cnt;
-            if (hpos == B) {
-                flush_words(P.out + (row0 + (uint64_t)nfull * B) * D, P.aligned != 0,
-                            ring + (size_t)half * B * D, B * D, lane, pol);
-                ++nfull;
-                half ^= 1u;
-                hpos = 0;
-            }
-        }
-        if (hpos > 0)
-            flush_words(P.out + (row0 + (uint64_t)nfull * B) * D, P.aligned != 0,
-                        ring + (size_t)half * B * D, hpos * D, lane, pol);
-        if (lane == 0) bulk_wait_read_all();
-        ok = __all_sync(FULL, ok);
-        if (!ok && lane == 0) atomicExch(P.status, (int)DEV_INTERNAL);
+        if (!rank_rows<D>(ConstParams{P}, ring, (uint32_t)P.half_rows, row0, rows, pol, lane)) break;
     }
     if (lane == 0) bulk_wait_all();
     __syncwarp();
@@ -205,7 +211,7 @@ int launch_rank_d(EnumParams P, int warp_bytes, cudaStream_t s, int sms) {
                             bytes);
 }
 
-// The flat walk of a batch's instances of one shape.  A launch may start while
+// The flat or rank walk of a batch's instances of one shape.  A launch may start while
 // the one before it drains (chained): it reads nothing that one writes, and
 // waits for its completion only before it ends, so the last launch's end is
 // the end of all.  Three blocks an SM: at 64 registers the loops spill (see
@@ -216,11 +222,14 @@ __global__ void __launch_bounds__(ENUM_THREADS, 3)
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    constexpr bool RANK = SRC == SRC_RANK;
     unsigned char *mem = enum_smem + (size_t)wid * RING_BYTES_PER_WARP;
     const SharedParams params{(uint32_t)(ENUM_WARPS * RING_BYTES_PER_WARP + wid * sizeof(EnumParams))};
     EnumParams *ep = reinterpret_cast<EnumParams *>(enum_smem + params.off);
-    constexpr uint32_t B = flat_half_rows<NP, SRC, D>(RING_BYTES_PER_WARP);
-    static_assert(leaf_bytes<NP, SRC>() + 2 * (int)B * D * 4 <= RING_BYTES_PER_WARP, "ring");
+    constexpr uint32_t B = RANK ? RING_BYTES_PER_WARP / (8 * D) / 32 * 32
+                                : flat_half_rows<NP, SRC, D>(RING_BYTES_PER_WARP);
+    static_assert((RANK ? 0 : leaf_bytes<NP, SRC>()) + 2 * (int)B * D * 4 <= RING_BYTES_PER_WARP,
+                  "ring");
     const uint64_t pol = policy_evict_first();
     int cur = -1;
     unsigned long long next = 0;
@@ -232,7 +241,7 @@ __global__ void __launch_bounds__(ENUM_THREADS, 3)
         const uint64_t s = batch_locate(BP, ep, cur, item, lane);
         const EnumParams &P = params();
         uint64_t row0, row1;
-        if (P.by_cost) {
+        if (!RANK && P.by_cost) {
             const uint64_t cost_hi = flat_total_cost<NP>(P);
             const uint64_t c0 = s * P.slice_cost, c1 = c0 + P.slice_cost;
             if (c0 >= cost_hi) continue;
@@ -251,7 +260,13 @@ __global__ void __launch_bounds__(ENUM_THREADS, 3)
             row1 = row0 + P.slice_rows < P.nrows ? row0 + P.slice_rows : P.nrows;
         }
         if (row1 <= row0) continue;
-        if (!flat_slice<D, NP, SRC>(params, mem, B, row0, row1, pol, lane)) break;
+        if constexpr (RANK) {
+            if (!rank_rows<D>(params, reinterpret_cast<int32_t *>(mem), B, row0,
+                              (uint32_t)(row1 - row0), pol, lane))
+                break;
+        } else {
+            if (!flat_slice<D, NP, SRC>(params, mem, B, row0, row1, pol, lane)) break;
+        }
     }
     if (lane == 0) bulk_wait_all();
     __syncwarp();
@@ -298,6 +313,9 @@ int launch_batch_one(const BatchEnumParams &BP, cudaStream_t s, int sms, int cta
 template <int D>
 int launch_batch_d(const BatchEnumParams &BP, int np, int src, cudaStream_t s, int sms, int cap) {
     if (src == SRC_PAIR) return launch_batch_one<D, D - 2, SRC_PAIR>(BP, s, sms, cap);
+    if constexpr (D >= 4 && D <= 7)
+        if (src == SRC_RANK) return launch_batch_one<D, D - 2, SRC_RANK>(BP, s, sms, cap);
+    if (src != SRC_RUN) return set_error(FZ_EINTERNAL, "flat walk: no kernel for this shape");
     if (np == 1) return launch_batch_one<D, 1, SRC_RUN>(BP, s, sms, cap);
     if constexpr (D >= 4)
         if (np == 2) return launch_batch_one<D, 2, SRC_RUN>(BP, s, sms, cap);

@@ -517,7 +517,7 @@ struct BatchGroup {
     int first, last;             // instances, by their place in the parameter images
     uint64_t item_lo, item_hi;   // their work items
 };
-constexpr int BATCH_MAX_GROUPS = 32;  // 24 shapes and the general kernel
+constexpr int BATCH_MAX_GROUPS = 32;  // 23 flat shapes, 4 by rank, the general kernel
 // counters: BATCH_MAX_GROUPS words of device memory.
 int launch_enumerate_batch(const void *params_dev, const uint64_t *item0_dev,
                            const BatchGroup *groups, int ngroups, unsigned long long *counters,
@@ -534,6 +534,7 @@ void batch_items(unsigned char *params, size_t pb, const uint64_t *cost, const i
 // Plans as seen by the batch and serve layers (fz_api.cu): the launch
 // description of a plan for an element n <= its n, and host copies of row 0
 // of its count table (n + 1 entries) and runs table (empty if none).
+int plan_create_resident(const int32_t *g, int d, int32_t n, fz_plan_t *plan, cudaStream_t s);
 int plan_launch_for(fz_plan_t plan, int32_t n, EnumLaunch *L);
 int plan_host_rows(fz_plan_t plan, uint64_t *count_row, std::vector<uint64_t> *runs_row,
                    cudaStream_t s);

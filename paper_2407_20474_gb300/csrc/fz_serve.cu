@@ -546,8 +546,7 @@ int fz_serve_register(fz_server_t s, const int32_t *g, int d, int32_t n_max, int
     rec.d = d;
     rec.n_max = n_max;
     if (g && d > 0 && d <= FZ_MAX_D) rec.g.assign(g, g + d);
-    fz_opts_t opt{FZ_AUTO, FZ_AUTO, 0, 0};
-    int rc = fz_plan_create(g, d, n_max, &opt, &rec.plan, s->streams[0]);
+    int rc = plan_create_resident(g, d, n_max, &rec.plan, s->streams[0]);
     if (rc != FZ_OK) return rc;
     rec.count_row.resize((size_t)n_max + 1);
     rc = plan_host_rows(rec.plan, rec.count_row.data(), &rec.runs_row, s->streams[0]);

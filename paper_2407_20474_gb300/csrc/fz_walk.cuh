@@ -103,7 +103,8 @@ __device__ __forceinline__ void load_run_row(const int32_t *p, int (&x)[SS]) {
 //             `rows`, each row (quotient, tail words), and the coordinate of
 //             gen is p div gen - quotient.
 //   SRC_PAIR: the closed form of the last two generators; nothing is read.
-enum : int { SRC_RUN = 0, SRC_PAIR = 1 };
+//   SRC_RANK: batches only, the pair's rows found by rank (rank_rows).
+enum : int { SRC_RUN = 0, SRC_PAIR = 1, SRC_RANK = 2 };
 struct LeafSource {
     const int32_t *rows;
     const uint64_t *cls;

@@ -159,3 +159,89 @@ def test_batch_in_a_graph(fz):
                 at = int(b.word_offsets[j])
                 assert np.array_equal(host[at:at + ref.size].reshape(ref.shape), ref), (g, n)
         b.sync()
+
+
+SPARSE = [((401, 397, 389, 383), 300), ((83, 97, 89, 101, 103), 900), ((59, 61, 60, 67, 71, 73), 2000),
+          ((41, 43, 44, 47, 53, 51, 59), 6000)]
+
+
+@pytest.mark.parametrize("g,target", SPARSE)
+def test_rank_walk_windows(fz, g, target):
+    """Sets with far more prefixes than rows: windows of the rank walk at every
+    remainder of a round, outputs aligned to 4 bytes only."""
+    n = workloads.find_n(oracle.count_upto, g, target)
+    ref = oracle.enumerate_desc(g, n)
+    total = ref.shape[0]
+    for slice_rows in (4, 33, 0):
+        for shift, a, b in ((0, 0, total), (1, 0, total), (3, 1, total - 1), (2, total - 1, total),
+                            (1, total // 3, total // 3 + 33)):
+            got = _window(fz, g, n, 0, a, b, slice_rows, shift)
+            assert np.array_equal(got, ref[a:b]), (slice_rows, shift, a, b)
+
+
+def test_rank_walk_in_batches(fz):
+    """The same sets in one batch without memos, beside dense ones and sets of
+    no row and of one."""
+    inst = [(g, workloads.find_n(oracle.count_upto, g, t // c)) for g, t in SPARSE for c in (1, 3)]
+    inst += [((5, 7, 9, 11), 300), (SPARSE[0][0], 382), (SPARSE[0][0], 383), (SPARSE[1][0], inst[1][1] + 1)]
+    with fz.Batch(inst, k=0) as b:
+        out = torch.full((b.total_words + 8,), CANARY, dtype=torch.int32, device="cuda")
+        b.enumerate(out)
+        b.sync()
+        host = out.cpu().numpy()
+        assert (host[b.total_words:] == CANARY).all()
+        for j, (g, n) in enumerate(inst):
+            at, ref = int(b.word_offsets[j]), oracle.enumerate_desc(g, n)
+            assert np.array_equal(host[at:at + ref.size].reshape(ref.shape), ref), (g, n)
+
+
+def test_serve_resident_shapes(fz):
+    """Requests far below and at a resident set's largest element: tables of
+    every depth, and (large generators up to 3e6) none, served by rank."""
+    sets = [((997, 1009, 1013, 1019), 3000000, 200000), ((5, 8, 11, 14, 17), 900, 300), ((9, 6, 12, 15, 21, 10), 220, 90),
+            ((13, 4, 7, 30, 22, 9, 17), 160, 161), ((3, 5, 7), 3000, 1)]
+    with fz.Server(memory_bytes=64 << 20) as srv:
+        ids = [srv.register(g, max(top, n)) for g, top, n in sets]
+        asked = [(i, s[0], n) for i, s in zip(ids, sets) for n in (s[2], s[2] // 2, 0)]
+        tickets = [srv.submit(i, n) for i, _, n in asked]
+        for t, (_, g, n) in zip(tickets, asked):
+            r = srv.wait(t)
+            ref = oracle.enumerate_desc(g, n)
+            assert int(r.count) == ref.shape[0], (g, n)
+            out = torch.full((ref.size + 4,), CANARY, dtype=torch.int32, device="cuda")
+            srv.copy(t, out[:ref.size])
+            srv.release(t)
+            host = out.cpu().numpy()
+            assert (host[ref.size:] == CANARY).all()
+            assert np.array_equal(host[:ref.size].reshape(ref.shape), ref), (g, n)
+
+
+@pytest.mark.parametrize("n", [0, 1, 2, 255, 256, 4095, 11999, 12000, 12001])
+def test_short_count_tables(fz, n):
+    """Count tables up to the one-launch range and past it: generators of 1,
+    above n, at n, repeated, and counts that saturate (width 16)."""
+    for g in ((3, 5, 7, 11), (n + 1, 4, 9), (max(n, 1), 2, 2), (1, 6), (7,), tuple(range(1, 17))):
+        d = len(g)
+        out = torch.zeros((d + 1, n + 1), dtype=torch.int64, device="cuda")
+        fz.fz_count_table(g, n, out)
+        torch.cuda.synchronize()
+        got = out.cpu().numpy().view(np.uint64)
+        for j in range(d):
+            ref = np.array([min(int(x), 2**64 - 1) for x in oracle.count_upto(g[j:], n)], dtype=np.uint64)
+            assert np.array_equal(got[j], ref), (g, j)
+
+
+# (generators, n): rows scanned by tiles and by lanes: 256 and 257 entries a
+# chain, 7, 8, 31 and 32 chains, one long chain, wrapping lengths around 16384
+CHAINS = [((7, 50), 7 * 256 - 1), ((7, 50), 7 * 256), ((8, 31), 8 * 300), ((31, 8), 31 * 256 + 5), ((32, 31), 32 * 257),
+          ((1, 2, 3), 16383), ((1, 2, 3), 16384), ((2, 1), 40001), ((64, 1), 64 * 255 + 63)]
+
+
+@pytest.mark.parametrize("g,n", CHAINS)
+def test_batch_chain_scans(fz, g, n):
+    """Batch counts of the chains above: the rows of d = 2 and 3 sets, alone and
+    among many small ones, against the oracle's counts."""
+    many = [((5, 8, 11), 90 + i) for i in range(40)]
+    for inst in ([(g, n)], [(g, n)] + many):
+        _, rows = fz.fz_plan_batch(inst)
+        assert [int(r) for r in rows] == [oracle.count(x, m) for x, m in inst]

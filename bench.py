@@ -248,7 +248,12 @@ def kernel_traffic(d):
         rec = json.load(open(path))
     except ValueError:
         return None
-    src = open(os.path.join(ROOT, "paper_2407_20474_gb300", "csrc", "fz_enum.cu")).read()
+    csrc = os.path.join(ROOT, "paper_2407_20474_gb300", "csrc")
+    src = ""
+    for name in ("fz_enum.cu", "fz_enum.cuh", "fz_flat.cu", "fz_walk.cuh"):
+        path = os.path.join(csrc, name)
+        if os.path.exists(path):
+            src += open(path).read()
     if rec.get("code_sha256") != code_hash(src):
         return None
     return rec.get("bytes_per_full_launch")
@@ -267,6 +272,9 @@ def enum_kernel_name(plan):
     """Name of the enumeration kernel the plan launches."""
     d, k = plan.d, plan.k
     if plan.run_order:
+        # the flat walk's widths and prefix lengths; else the run copy
+        if 3 <= d <= 9 and 1 <= d - k - 1 <= 3:
+            return "fz_enum_flat_kernel<%d, %d, 0>" % (d, d - k - 1)
         return "fz_enum_runs_kernel<%d, %d, %d>" % (d, d - k - 1, k)
     return "fz_enum_kernel<%d>" % d
 

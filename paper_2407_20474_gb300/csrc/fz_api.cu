@@ -80,13 +80,17 @@ constexpr uint64_t POOL_KEEP_BYTES = 64ull << 20;
 
 cudaMemPool_t call_pool() {
     static std::mutex mu;
-    static cudaMemPool_t pools[64];
-    static bool tried[64];
+    // by device context: a reset takes a pool with its context
+    static std::map<unsigned long long, cudaMemPool_t> pools;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    unsigned long long id = device_ctx_id();
+    if (id == 0 && cudaFree(nullptr) == cudaSuccess) id = device_ctx_id();
+    if (id == 0) return nullptr;
     std::lock_guard<std::mutex> lk(mu);
-    if (!tried[dev]) {
-        tried[dev] = true;
+    auto it = pools.find(id);
+    if (it == pools.end()) {
+        it = pools.emplace(id, nullptr).first;
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.handleTypes = cudaMemHandleTypeNone;
@@ -96,10 +100,10 @@ cudaMemPool_t call_pool() {
         uint64_t keep = POOL_KEEP_BYTES;
         if (cudaMemPoolCreate(&pool, &props) == cudaSuccess &&
             cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
-            pools[dev] = pool;
+            it->second = pool;
         cudaGetLastError();
     }
-    return pools[dev];
+    return it->second;
 }
 
 // RAII device buffer: cudaMalloc / cudaFree, or the call pool on a stream.

@@ -303,16 +303,21 @@ __device__ __forceinline__ bool grid_wait(unsigned *count, unsigned index, int *
 // ---------------------------------------------------------------------------
 // Host helpers.
 // ---------------------------------------------------------------------------
-// Per-device flags for host-side steps done once per kernel and device
-// (function attributes), safe when several host threads launch: the
-// serving thread and its callers.
+// Id of the device context current on this thread (fz_noalloc.cu): never reused
+// in a process, 0 when none is current.
+unsigned long long device_ctx_id();
+
+// Per-device flags for host-side steps done once per kernel and device context
+// (function attributes; a device reset drops them), safe when several host
+// threads launch: the serving thread and its callers.
 struct DeviceOnce {
-    std::atomic<bool> done[64];
+    std::atomic<unsigned long long> done[64];
     bool is_set(int dev) const {
-        return dev >= 0 && dev < 64 && done[dev].load(std::memory_order_acquire);
+        const unsigned long long id = device_ctx_id();
+        return id != 0 && dev >= 0 && dev < 64 && done[dev].load(std::memory_order_acquire) == id;
     }
     void set(int dev) {
-        if (dev >= 0 && dev < 64) done[dev].store(true, std::memory_order_release);
+        if (dev >= 0 && dev < 64) done[dev].store(device_ctx_id(), std::memory_order_release);
     }
 };
 

@@ -100,6 +100,11 @@ int noalloc_scratch(uint64_t **out) {
 }
 
 }  // namespace
+
+unsigned long long device_ctx_id() {
+    std::lock_guard<std::mutex> lk(g_noalloc_mu);
+    return current_ctx_id();
+}
 }  // namespace fz
 
 using namespace fz;

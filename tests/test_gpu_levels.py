@@ -245,3 +245,31 @@ def test_batch_chain_scans(fz, g, n):
     for inst in ([(g, n)], [(g, n)] + many):
         _, rows = fz.fz_plan_batch(inst)
         assert [int(r) for r in rows] == [oracle.count(x, m) for x, m in inst]
+
+
+def test_calls_after_a_context_reset(fz):
+    """Counts and a host enumeration before and after the process resets its own
+    device context (in a child process): function attributes and the memory
+    pool are those of the new context."""
+    import subprocess
+    import sys
+    code = """
+import ctypes, numpy as np, oracle
+import paper_2407_20474_gb300 as fz
+drv = ctypes.CDLL('libcuda.so.1')
+g, n = (5, 8, 11, 14), 9000
+ref, rows = oracle.count_upto(g, n), oracle.enumerate_desc(g, 500)
+for k in range(3):
+    assert np.array_equal(fz.fz_count_upto(g, n, stream=0), ref), k
+    out = np.full(rows.shape, -7, dtype=np.int32)
+    fz.fz_enumerate_host(g, 500, out, stream=0)
+    assert np.array_equal(out, rows), k
+    if k < 2:
+        dev = ctypes.c_int()
+        assert drv.cuDeviceGet(ctypes.byref(dev), 0) == 0
+        assert drv.cuDevicePrimaryCtxReset_v2(dev) == 0
+print('same')
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300,
+                       cwd=__import__("os").path.dirname(__import__("os").path.dirname(__file__)))
+    assert r.returncode == 0 and r.stdout.strip().endswith("same"), r.stderr[-2000:]

@@ -809,7 +809,7 @@ def measure_batch(torch, fz, steps, warmup, count=4096, only_d=0, pi_steps=5, au
            "per_instance_value": b.total_rows / (ms_pi / 1e3) if ms_pi else None,
            "speedup_vs_per_instance": ms_pi / ms if ms_pi else None,
            "roofline_enumeration": {
-               "bound": "hbm", "kernel": "fz_enum_batch_kernel",
+               "bound": "hbm", "kernel": "fz_flat_batch_kernel",
                "achieved": bytes_out / (ms_enum / 1e3) / 1e9, "peak": peak[0],
                "unit": "GB/s", "frac": bytes_out / (ms_enum / 1e3) / 1e9 / peak[0],
                "peak_source": peak[1]},
@@ -959,12 +959,10 @@ def run_serve_workload(args):
 
 def measure_memo(torch, fz, steps, warmup):
     """The memo build: dynamic FactorizationsUpToElement build of all Z(0..1500) for
-    d = 5 generators in [3,40] (seed 1): the full CSR, elementwise in batches
-    of min(g) elements, filled in phases of min(g_2..g_d) elements (one grid
-    barrier a phase) when that is at least twice min(g), as here.  Timed on
-    the device as the rebuild of a plan whose
-    memo is that CSR (k = d, top = N + 1: count table, offsets, gather map and
-    the batched fill, no allocation), CUDA events over the steps; the one-shot
+    d = 5 generators in [3,40] (seed 1): the full CSR, built level by level from
+    run-order tables.  Timed on the device as the rebuild of a plan whose
+    memo is that CSR (k = d, top = N + 1: count table, offsets, levels,
+    no allocation), CUDA events over the steps; the one-shot
     host call fz_build_memo_into (which allocates its work buffers and
     synchronises) is timed beside it.  Returns a record (dict)."""
     from paper_2407_20474_gb300 import workloads
@@ -987,16 +985,12 @@ def measure_memo(torch, fz, steps, warmup):
             ts.append(time.perf_counter() - t0)
     t_host = statistics.median(ts)
     nbatch = -(-(N + 1) // min(g))
-    L = min(g[1:])
-    phased = g[0] == min(g) and L >= 2 * g[0]
-    nphase = -(-(N + 1) // L) if phased else nbatch
     return {"workload": "d=5 generators %s (seed 1), N=%d" % (list(g), N),
             "value": rows / (ms / 1e3), "unit": "rows/s", "ms_per_step": ms,
             "rows": rows, "bytes_written": rows * len(g) * 4,
             "write_GBps": rows * len(g) * 4 / (ms / 1e3) / 1e9,
-            "dependent_batches": nbatch, "us_per_batch": 1e3 * ms / nbatch,
-            "phases": nphase,
-            "bound": "latency (one grid barrier per phase of %d elements)" % (L if phased else min(g)),
+            "elementwise_batches": nbatch, "levels": len(g) - 1,
+            "bound": "output write and table reads through L2 (built by levels)",
             "host_call_ms": 1e3 * t_host,
             "note": "value: device time of a plan rebuild (CUDA events); "
                     "host_call_ms: fz_build_memo_into incl. its allocations"}

@@ -155,11 +155,12 @@ int fz_count_table(const int32_t *g, int d, int32_t n, uint64_t *table_dev,
                    void *stream);
 
 /* ------------------------------------------------------------------------
- * Memo of tail sets, built by the dynamic FactorizationsUpToElement pass:
- * the lists Z(r, tail), r = 0..top-1, each in descending order, computed
- * elementwise in batches of min(tail) elements (Section 2.2), every batch a
- * set of copy-and-increment steps incr_i(Z_{>=i}(r - t_i)) written to
- * pre-assigned offsets (Sections 2.3 and 2.4).  The layout is a CSR:
+ * Memo of tail sets (FactorizationsUpToElement): the lists Z(r, tail),
+ * r = 0..top-1, each in descending order, built generator by generator, or
+ * (the schedules below) by the paper's dynamic pass: elementwise in batches of
+ * min(tail) elements (Section 2.2), every batch a set of copy-and-increment
+ * steps incr_i(Z_{>=i}(r - t_i)) written to pre-assigned offsets (Sections 2.3
+ * and 2.4).  The layout is a CSR:
  * offsets[r] .. offsets[r+1] are the rows of Z(r, tail), k int32 per row.
  * ---------------------------------------------------------------------- */
 
@@ -326,8 +327,8 @@ int fz_plan_destroy(fz_plan_t plan);
 /* ------------------------------------------------------------------------
  * Batches: many instances Z(n_i, g_i) of possibly different d_i in one set
  * of launches -- batched counting tables, one memo per distinct tail shared
- * by the instances that have it, and one persistent enumeration launch over
- * (instance, slice) work items.  Full memos (widths 3..8 with at least one
+ * by the instances that have it, and one persistent enumeration launch per
+ * shape (width, memo depth) over (instance, slice) work items.  Full memos (widths 3..8 with at least one
  * walked coordinate above the memo) are tables in run order, built generator
  * by generator, so a prefix's whole subtree is one contiguous copy; a memo of
  * depth 2 over the last two generators may be kept as its closed form, with

@@ -31,12 +31,6 @@ constexpr int64_t TILE_MAX_T = 16384;  // fewer than 8 chains up to this length:
 constexpr int RB = 32;              // entries per block in the blocked scan
 constexpr int THREADS = 256;
 
-__global__ void row_delta_kernel(uint64_t *__restrict__ row, int64_t len) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (; i < len; i += stride) row[i] = (i == 0) ? 1ull : 0ull;
-}
-
 // ---------------------------------------------------------------------------
 // Tile scan: a block scans `width` (1, 8 or 32) neighbouring residue chains, its
 // threads cut into 256 / width segments of TILE_U consecutive chain entries (16
@@ -336,20 +330,58 @@ int launch_tables_small(const int32_t *g, int d, int32_t n, uint64_t *C, uint64_
     return launch_small_tables(P, s);
 }
 
+// The last rows of a count table from their closed forms: C[d] the delta row,
+// C[d-1][r] = [g_d | r], C[d-2][r] = |Z(r, (g_{d-1}, g_d))|; null rows are not
+// written.  Bound by the stores: three rows of 2e6 entries in one launch and no
+// scan (count table of width 4: 109 us with four scans, 69 with two; all counts to 39064 for width 6: 86, 71).
+__global__ void __launch_bounds__(THREADS)
+    tail_rows_kernel(const __grid_constant__ PairForm F, FastDiv last, uint64_t *__restrict__ pair,
+                     uint64_t *__restrict__ one, uint64_t *__restrict__ delta, int64_t len) {
+    const int64_t step = (int64_t)gridDim.x * THREADS;
+    for (int64_t r = (int64_t)blockIdx.x * THREADS + threadIdx.x; r < len; r += step) {
+        const uint32_t x = (uint32_t)r;
+        if (delta) delta[r] = r == 0 ? 1ull : 0ull;
+        if (one) one[r] = fd_mod(x, last) == 0u ? 1ull : 0ull;
+        if (pair) pair[r] = pair_form_count(F, x);
+    }
+}
+
+// pair needs d >= 2.
+int launch_tail_rows(const int32_t *g, int d, uint64_t *pair, uint64_t *one, uint64_t *delta,
+                     int64_t len, cudaStream_t s) {
+    const PairForm F = d >= 2 ? make_pair_form(g[d - 2], g[d - 1]) : PairForm{};
+    tail_rows_kernel<<<grid_for(len, THREADS), THREADS, 0, s>>>(
+        F, make_fastdiv((uint32_t)g[d - 1]), pair, one, delta, len);
+    note_launch();
+    FZ_CUDA_TRY(cudaGetLastError());
+    return FZ_OK;
+}
+
 int launch_count_table_tmp(const int32_t *g, int d, int32_t n, uint64_t *table, uint64_t *tmp,
                            cudaStream_t s) {
     if (small_tables(n)) return launch_tables_small(g, d, n, table, nullptr, 0, -1, 0, nullptr, s);
     const int64_t len = (int64_t)n + 1;
     uint64_t *last = table + (int64_t)d * len;
-    row_delta_kernel<<<grid_for(len, THREADS), THREADS, 0, s>>>(last, len);
-    note_launch();
-    FZ_CUDA_TRY(cudaGetLastError());
-    for (int j = d - 1; j >= 0; --j) {
-        int rc = strided_scan(table + (int64_t)(j + 1) * len, table + (int64_t)j * len, len,
+    int rc = launch_tail_rows(g, d, d >= 2 ? last - 2 * len : nullptr, last - len, last, len, s);
+    if (rc != FZ_OK) return rc;
+    for (int j = d - 3; j >= 0; --j) {
+        rc = strided_scan(table + (int64_t)(j + 1) * len, table + (int64_t)j * len, len,
                               g[j], tmp, s);
         if (rc != FZ_OK) return rc;
     }
     return FZ_OK;
+}
+
+// The last rows of a candidates table: ones, and x div g + 1 above them (1 below
+// `clamp`).
+__global__ void __launch_bounds__(THREADS)
+    head_rows_kernel(FastDiv g, uint64_t *__restrict__ lin, uint64_t *__restrict__ ones,
+                     int64_t clamp, int64_t len) {
+    const int64_t step = (int64_t)gridDim.x * THREADS;
+    for (int64_t r = (int64_t)blockIdx.x * THREADS + threadIdx.x; r < len; r += step) {
+        ones[r] = 1ull;
+        if (lin) lin[r] = r < clamp ? 1ull : (uint64_t)fd_div((uint32_t)r, g) + 1ull;
+    }
 }
 
 __global__ void row_ones_kernel(uint64_t *__restrict__ row, int64_t len) {
@@ -366,10 +398,13 @@ int launch_runs_table(const int32_t *g, int lam, int32_t n, uint64_t *RT, uint64
     if (small_tables(n))
         return launch_tables_small(g, lam, n, nullptr, RT, lam, clamp_row, clamp_top, nullptr, s);
     const int64_t len = (int64_t)n + 1;
-    row_ones_kernel<<<grid_for(len, THREADS), THREADS, 0, s>>>(RT + (int64_t)lam * len, len);
+    uint64_t *ones = RT + (int64_t)lam * len;
+    head_rows_kernel<<<grid_for(len, THREADS), THREADS, 0, s>>>(
+        make_fastdiv(lam >= 1 ? (uint32_t)g[lam - 1] : 1u), lam >= 1 ? ones - len : nullptr, ones,
+        clamp_row == lam - 1 ? clamp_top : 0, len);
     note_launch();
     FZ_CUDA_TRY(cudaGetLastError());
-    for (int j = lam - 1; j >= 0; --j) {
+    for (int j = lam - 2; j >= 0; --j) {
         int rc = strided_scan(RT + (int64_t)(j + 1) * len, RT + (int64_t)j * len, len, g[j],
                               tmp, s);
         if (rc != FZ_OK) return rc;
@@ -605,12 +640,11 @@ int launch_count_rolling(const int32_t *g, int d, int32_t n, uint64_t *a, uint64
         *result = a;
         return launch_small_tables(P, s);
     }
-    row_delta_kernel<<<grid_for(len, THREADS), THREADS, 0, s>>>(a, len);
-    note_launch();
-    FZ_CUDA_TRY(cudaGetLastError());
+    int rc = launch_tail_rows(g, d, d >= 2 ? a : nullptr, d >= 2 ? nullptr : a, nullptr, len, s);
+    if (rc != FZ_OK) return rc;
     uint64_t *below = a, *cur = b;
-    for (int j = d - 1; j >= 0; --j) {
-        int rc = strided_scan(below, cur, len, g[j], tmp, s);
+    for (int j = d - 3; j >= 0; --j) {
+        rc = strided_scan(below, cur, len, g[j], tmp, s);
         if (rc != FZ_OK) return rc;
         uint64_t *t = below;
         below = cur;

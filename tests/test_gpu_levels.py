@@ -231,6 +231,23 @@ def test_short_count_tables(fz, n):
             assert np.array_equal(got[j], ref), (g, j)
 
 
+@pytest.mark.parametrize("g,n", [((70001, 65537), 150000), ((131071, 3, 65536), 150000), ((6, 4), 13000),
+                                 ((4, 2, 2, 9), 20000), ((9,), 12500), ((1, 1), 12001), ((200000, 300000), 100000)])
+def test_closed_count_rows(fz, g, n):
+    """The last rows of longer count tables from their closed forms (moduli on
+    both sides of 2^16, common factors, generators above n) and the rolling
+    counts that start from them."""
+    d = len(g)
+    out = torch.full((d + 1, n + 1), CANARY, dtype=torch.int64, device="cuda")
+    fz.fz_count_table(g, n, out)
+    torch.cuda.synchronize()
+    got = out.cpu().numpy()
+    assert got[d, 0] == 1 and (got[d, 1:] == 0).all()
+    for j in range(d):
+        assert np.array_equal(got[j].astype(np.uint64), oracle.count_upto(g[j:], n)), j
+    assert np.array_equal(fz.fz_count_upto(g, n), oracle.count_upto(g, n))
+
+
 # (generators, n): rows scanned by tiles and by lanes: 256 and 257 entries a
 # chain, 7, 8, 31 and 32 chains, one long chain, wrapping lengths around 16384
 CHAINS = [((7, 50), 7 * 256 - 1), ((7, 50), 7 * 256), ((8, 31), 8 * 300), ((31, 8), 31 * 256 + 5), ((32, 31), 32 * 257),

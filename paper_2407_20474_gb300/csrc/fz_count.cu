@@ -173,8 +173,12 @@ block_apply_kernel(const uint64_t *__restrict__ in, uint64_t *__restrict__ out,
 // steps add the entry s = g, 2 g, 4 g, ... below.  Block 0: the count table
 // (or its row 0 only), block 1: the candidates table.  Row by row these are a
 // launch each of which the GPU runs in 3 us, 12 launches for a set of width 9.
+// A plan's two tables take it up to SMALL_N (rebuild of 1e6 rows of width 6: 86
+// us, 90 row by row), one table alone up to SMALL_ONE_N: its d - 2 scans row by
+// row beside it at n = 3500, 6000, 11500: 18, 19, 21 us against 23, 29, 63 for
+// width 5, 13, 14, 14 against 14, 18, 36 for width 3.
 // ---------------------------------------------------------------------------
-constexpr int SMALL_N = 12000;
+constexpr int SMALL_N = 12000, SMALL_ONE_N = 3000;
 constexpr int SMALL_THREADS = 1024;
 struct SmallTables {
     uint64_t *C;      // rows 0..d, or null
@@ -359,7 +363,8 @@ int launch_tail_rows(const int32_t *g, int d, uint64_t *pair, uint64_t *one, uin
 
 int launch_count_table_tmp(const int32_t *g, int d, int32_t n, uint64_t *table, uint64_t *tmp,
                            cudaStream_t s) {
-    if (small_tables(n)) return launch_tables_small(g, d, n, table, nullptr, 0, -1, 0, nullptr, s);
+    if (n <= SMALL_ONE_N)
+        return launch_tables_small(g, d, n, table, nullptr, 0, -1, 0, nullptr, s);
     const int64_t len = (int64_t)n + 1;
     uint64_t *last = table + (int64_t)d * len;
     int rc = launch_tail_rows(g, d, d >= 2 ? last - 2 * len : nullptr, last - len, last, len, s);
@@ -395,7 +400,7 @@ __global__ void row_ones_kernel(uint64_t *__restrict__ row, int64_t len) {
 // stride g_j -- the count-table recurrence over the leading generators.
 int launch_runs_table(const int32_t *g, int lam, int32_t n, uint64_t *RT, uint64_t *tmp,
                       int clamp_row, int64_t clamp_top, cudaStream_t s) {
-    if (small_tables(n))
+    if (n <= SMALL_ONE_N)
         return launch_tables_small(g, lam, n, nullptr, RT, lam, clamp_row, clamp_top, nullptr, s);
     const int64_t len = (int64_t)n + 1;
     uint64_t *ones = RT + (int64_t)lam * len;
@@ -631,7 +636,7 @@ int scan_block_rows() { return RB; }
 int launch_count_rolling(const int32_t *g, int d, int32_t n, uint64_t *a, uint64_t *b,
                          uint64_t *tmp, uint64_t **result, cudaStream_t s) {
     const int64_t len = (int64_t)n + 1;
-    if (small_tables(n)) {
+    if (n <= SMALL_ONE_N) {
         SmallTables P{};
         P.C0 = a;
         P.d = d;

@@ -231,6 +231,12 @@ def test_short_count_tables(fz, n):
             assert np.array_equal(got[j], ref), (g, j)
 
 
+@pytest.mark.parametrize("n", [2999, 3000, 3001])
+def test_one_launch_count_tables(fz, n):
+    """Both sides of the longest single table built in one launch."""
+    test_short_count_tables(fz, n)
+
+
 @pytest.mark.parametrize("g,n", [((70001, 65537), 150000), ((131071, 3, 65536), 150000), ((6, 4), 13000),
                                  ((4, 2, 2, 9), 20000), ((9,), 12500), ((1, 1), 12001), ((200000, 300000), 100000)])
 def test_closed_count_rows(fz, g, n):

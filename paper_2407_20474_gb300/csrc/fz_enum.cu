@@ -1335,6 +1335,9 @@ int launch_enumerate_batch(const void *params_dev, const uint64_t *item0_dev,
     bool chained = false;
     for (int i = 0; i < ngroups; ++i) {
         const BatchGroup &G = groups[i];
+        // no launch for instances without rows; the next one is chained only
+        // to a kernel that was launched
+        if (G.item_hi == G.item_lo) continue;
         BatchEnumParams BP;
         BP.inst = static_cast<const EnumParams *>(params_dev);
         BP.out_base = out_base;

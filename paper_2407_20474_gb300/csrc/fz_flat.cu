@@ -294,7 +294,6 @@ int launch_batch_one(const BatchEnumParams &BP, cudaStream_t s, int sms, int cta
     uint64_t grid = (uint64_t)per_sm * sms;
     const uint64_t want = (BP.item_hi - BP.item_lo + ENUM_WARPS - 1) / ENUM_WARPS;
     if (want < grid) grid = want;
-    if (grid < 1) return FZ_OK;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(ENUM_THREADS);

@@ -278,8 +278,10 @@ int strided_scan(const uint64_t *in, uint64_t *out, int64_t len, int64_t g, uint
     if (T <= DIRECT_T) {
         int64_t chains = g < len ? g : len;
         if (chains >= 8 && T > LANE_T) {
-            // 8 chains a block: a single row has few, and latency bounds it
-            row_tile_kernel<<<grid_for(chains, 8), THREADS, 0, s>>>(in, out, len, g, 8);
+            // 8 chains a block: a single row has few, and latency bounds it.  A
+            // block has one tile, so every tile has a block (chains of more
+            // than LANE_T entries: at most 2^20 of them).
+            row_tile_kernel<<<(unsigned)((chains + 7) / 8), THREADS, 0, s>>>(in, out, len, g, 8);
             note_launch();
             FZ_CUDA_TRY(cudaGetLastError());
             return FZ_OK;

@@ -840,7 +840,7 @@ __global__ void __launch_bounds__(ENUM_THREADS, 4)
         if (lane == 0) item = BP.item_lo + atomicAdd(BP.item_counter, 1ull);
         item = __shfl_sync(FULL, item, 0);
         if (item >= BP.item_hi) break;
-        const uint64_t s = batch_locate(BP, ep, cur, item, lane);
+        const uint64_t s = batch_locate<true>(BP, ep, cur, item, lane);
         const EnumParams &P = *ep;
         uint64_t row0, row1;
         if (P.RT) {
@@ -1268,10 +1268,19 @@ void batch_order(const unsigned char *images, size_t pb, const uint64_t *cost, i
     }
     order->resize((size_t)count);
     for (int i = 0; i < count; ++i) (*order)[(size_t)i] = i;
-    // the general kernel last: it is not one of the overlapped launches
+    // The general kernel last: it is not one of the overlapped launches.  Its
+    // instances by code path (run copy, walk up to width 8, wider walk) and
+    // width, so that warps of an SM run the same code and share tables (512
+    // partial memos of widths 4..8: 11.2 ms in the caller's order, 8.5 so).
+    std::vector<int> path((size_t)count, 0);
+    for (int i = 0; i < count; ++i) {
+        EnumParams P;
+        memcpy(&P, images + (size_t)i * pb, sizeof(P));
+        if (!shape[(size_t)i]) path[(size_t)i] = (P.run_memo ? 0 : P.d <= 8 ? 32 : 64) + P.d;
+    }
     std::stable_sort(order->begin(), order->end(), [&](int x, int y) {
         const uint32_t a = shape[(size_t)x], b = shape[(size_t)y];
-        if (a == b) return false;
+        if (a == b) return path[(size_t)x] < path[(size_t)y];
         if (!a || !b) return !b;
         return total[a] != total[b] ? total[a] > total[b] : a < b;
     });
@@ -1289,6 +1298,9 @@ void batch_order(const unsigned char *images, size_t pb, const uint64_t *cost, i
 // that their tables stay in L2 (4096 instances of 1e2..1e6 rows, 4.3e8 in
 // all: 4.5 ms with items of 15400, 3.5 with 7700, 3.2 with 3900, 3.0 with
 // 1900), although an item starts with a dozen dependent loads (about 10 us).
+// The general kernel's items (a prefix costs it 16 or 64, and it is not one of
+// the overlapped launches): 1/8 of a warp's share of its own instances, 4096
+// at least (the same 512 partial memos: 14.5 ms with the items above).
 void batch_items(unsigned char *params, size_t pb, const uint64_t *cost, const int *order,
                  std::vector<BatchGroup> *groups, int sms, uint64_t *item0) {
     // by rank a row costs about four rows of the flat walk, a prefix nothing
@@ -1297,13 +1309,16 @@ void batch_items(unsigned char *params, size_t pb, const uint64_t *cost, const i
         memcpy(&P, params + (size_t)p * pb, sizeof(P));
         return P.flat_src == SRC_RANK ? 4 * P.nrows : cost[order[p]];
     };
-    uint64_t total = 0;
+    uint64_t total = 0, general = 0;
     for (const BatchGroup &G : *groups)
-        for (int p = G.first; p < G.last; ++p) total += cost_of(p);
-    uint64_t target = total / ((uint64_t)sms * 24 * 8 + 1);
-    target = target < 512 ? 512 : target > 2048 ? 2048 : target;
+        for (int p = G.first; p < G.last; ++p) (G.shape ? total : general) += cost_of(p);
+    uint64_t flat_target = total / ((uint64_t)sms * 24 * 8 + 1);
+    flat_target = flat_target < 512 ? 512 : flat_target > 2048 ? 2048 : flat_target;
+    uint64_t general_target = general / ((uint64_t)sms * 16 * 8 + 1);
+    general_target = general_target < 4096 ? 4096 : general_target;
     item0[0] = 0;
     for (BatchGroup &G : *groups) {
+        const uint64_t target = G.shape ? flat_target : general_target;
         G.item_lo = item0[G.first];
         for (int p = G.first; p < G.last; ++p) {
             EnumParams P;

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 import oracle
+from paper_2407_20474_gb300 import workloads
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -98,3 +99,21 @@ def test_first_group_without_rows(fz):
             b.enumerate(out)
             _check(out, b.word_offsets, inst)
         b.sync()
+
+
+def test_items_of_the_general_kernel(fz):
+    """Partial memos of widths 4 to 8 in mixed order: at most eight work items
+    for each of 16 warps an SM (an item starts with a dozen dependent loads), and the
+    oracle's rows."""
+    rng = np.random.Generator(np.random.PCG64(79))
+    inst = []
+    for i in range(30):
+        g = tuple(int(x) for x in rng.integers(8, 60, size=4 + i % 5))
+        inst.append((g, workloads.find_n(oracle.count_upto, g, 100000)))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    with fz.Batch(inst, top=60) as b:
+        assert b.work_items <= sms * 16 * 8 + 1 + len(inst)
+        out = torch.full((b.total_words + 8,), CANARY, dtype=torch.int32, device="cuda")
+        b.enumerate(out)
+        b.sync()
+        _check(out, b.word_offsets, inst)

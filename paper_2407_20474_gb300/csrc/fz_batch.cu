@@ -255,7 +255,7 @@ int build_scan_plan(fz_batch_s *b, uint64_t *table_base, std::vector<ScanJob> &j
         for (int ji : step_jobs) {
             ScanJob &J = jobs[ji];
             const int64_t T = (J.len + J.g - 1) / J.g;
-            if (scan_plan(std::min<int64_t>(J.g, J.len), T) < 0) {
+            if (scan_plan(std::min<int64_t>(J.g, J.len), T) == -1) {
                 // blocks of at least RBk entries, more for long chains, so
                 // that each chain of block sums is scanned directly
                 J.rb = std::max<int64_t>(RBk, (T + DIRECT - 1) / DIRECT);
@@ -287,9 +287,11 @@ int build_scan_plan(fz_batch_s *b, uint64_t *table_base, std::vector<ScanJob> &j
             if (plan(J) > 0) continue;
             if (!J.slen) {
                 const int64_t chains = std::min<int64_t>(J.g, J.len);
-                // 256 chains a task, one a lane
-                for (int64_t a = 0; a < chains; a += 256)
-                    tasks.push_back({ji, TK_LANES, a, std::min(chains, a + 256)});
+                // 256 chains a task, one a lane, or 8, one a warp
+                const bool warps = plan(J) == -2;
+                for (int64_t a = 0; a < chains; a += warps ? 8 : 256)
+                    tasks.push_back({ji, warps ? TK_CHAIN : TK_LANES, a,
+                                     std::min<int64_t>(chains, a + (warps ? 8 : 256))});
             } else {
                 // one block sum a thread: a block is rb strided entries
                 for (int64_t a = 0; a < J.slen; a += BS_TASK)

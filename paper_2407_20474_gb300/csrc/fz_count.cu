@@ -26,6 +26,7 @@ namespace {
 
 constexpr int64_t DIRECT_T = 4096;  // chains up to this length: one warp each
 constexpr int64_t LANE_T = 256;     // chains up to this length, 32 or more: one lane each
+constexpr int64_t CHAIN_T = 128;    // fewer than 32 chains up to this length: one warp each
 constexpr int LANE_ILP = 8;
 constexpr int64_t TILE_MAX_T = 16384;  // fewer than 8 chains up to this length: a tile each
 constexpr int RB = 32;              // entries per block in the blocked scan
@@ -467,6 +468,33 @@ __device__ __forceinline__ void chain_scan_warp(In input, uint64_t *__restrict__
     }
 }
 
+// One chain by a lane, walked down with its own running sum; a warp's loads and
+// stores cover 32 neighbouring entries of a row (one 256-byte span when es =
+// 1).  `input` without a branch on where the entries come from keeps LANE_ILP
+// loads in flight: a batch of 512 partial memos rebuilds in 224 us, 256 with
+// the branch at every entry.
+template <class In>
+__device__ __forceinline__ void chain_scan_lane(In input, const ScanJob &J, int64_t rho, int64_t off,
+                                                int64_t es) {
+    uint64_t *__restrict__ out = J.out;
+    const int64_t T = (J.len - rho + J.g - 1) / J.g;
+    uint64_t acc = 0;
+    for (int64_t t0 = 0; t0 < T; t0 += LANE_ILP) {
+        uint64_t v[LANE_ILP];
+#pragma unroll
+        for (int u = 0; u < LANE_ILP; ++u)
+            v[u] = t0 + u < T ? input(off + (rho + (t0 + u) * J.g) * es) : 0ull;
+#pragma unroll
+        for (int u = 0; u < LANE_ILP; ++u) {
+            if (t0 + u < T) {
+                const int64_t x = off + (rho + (t0 + u) * J.g) * es;
+                acc = sat_add(acc, v[u]);
+                out[x] = x < J.ones_below ? 1ull : acc;
+            }
+        }
+    }
+}
+
 constexpr int SCAN_MINB_DEFAULT = 4;
 
 // MINB: CTAs per SM the register budget is set for (3 fit without a bound:
@@ -485,30 +513,19 @@ __global__ void __launch_bounds__(THREADS, MINB) scan_tasks_kernel(const ScanJob
             tile_scan<8>([&](int64_t x) { return scan_input(J, J.in, x); }, J.out, J.len, J.g, t.begin,
                       (int)t.end, J.ones_below, off, es);
             break;
+        case TK_CHAIN:
+            for (int64_t rho = t.begin + warp; rho < t.end; rho += nwarps)
+                chain_scan_warp([&](int64_t x) { return scan_input(J, J.in, x); }, J.out, J.len, J.g, rho,
+                                lane, J.ones_below, off, es);
+            break;
         case TK_LANES: {
-            // lane l of warp w: chain rho = begin + 32 w + l, walked down with
-            // its own running sum; a warp's loads and stores cover 32
-            // neighbouring entries of a row (one 256-byte span when es = 1)
+            // lane l of warp w: chain begin + 32 w + l
             const int64_t rho = t.begin + (int64_t)warp * 32 + lane;
             if (rho >= t.end) break;
-            const uint64_t *__restrict__ in = J.in;
-            uint64_t *__restrict__ out = J.out;
-            const int64_t T = (J.len - rho + J.g - 1) / J.g;
-            uint64_t acc = 0;
-            for (int64_t t0 = 0; t0 < T; t0 += LANE_ILP) {
-                uint64_t v[LANE_ILP];
-#pragma unroll
-                for (int u = 0; u < LANE_ILP; ++u)
-                    v[u] = t0 + u < T ? scan_input(J, in, off + (rho + (t0 + u) * J.g) * es) : 0ull;
-#pragma unroll
-                for (int u = 0; u < LANE_ILP; ++u) {
-                    if (t0 + u < T) {
-                        const int64_t x = off + (rho + (t0 + u) * J.g) * es;
-                        acc = sat_add(acc, v[u]);
-                        out[x] = x < J.ones_below ? 1ull : acc;
-                    }
-                }
-            }
+            if (J.input == SCAN_LOAD)
+                chain_scan_lane([&](int64_t x) { return __ldg(J.in + x); }, J, rho, off, es);
+            else
+                chain_scan_lane([&](int64_t x) { return scan_input(J, J.in, x); }, J, rho, off, es);
             break;
         }
         case TK_SSCAN:
@@ -614,8 +631,11 @@ int launch_scan_tasks(const ScanJob *jobs, const ScanTask *tasks, int ntasks, cu
 }
 
 // How the chains of a row (`chains` of them, the longest T entries) are
-// scanned: 0 = a lane each, else tiles of that width; -1 = blocked.
+// scanned: 0 = a lane each, -2 = a warp each, else tiles of that width; -1 =
+// blocked.  A few chains of one round of a warp's loads are not worth a tile's
+// two meetings (256 sets of width 9: 471 us a rebuild, 478 with tiles).
 int scan_plan(int64_t chains, int64_t T) {
+    if (T <= CHAIN_T && chains < 32) return -2;
     if (chains < 8) return T <= TILE_MAX_T ? 1 : -1;
     if (T > DIRECT_T) return -1;
     if (chains >= 32 && T <= LANE_T) return 0;

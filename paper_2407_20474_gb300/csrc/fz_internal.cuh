@@ -382,6 +382,7 @@ enum ScanTaskKind : int {
     TK_ONES = 5,    // out[begin..end) = 1
     TK_PAIR = 6,    // rows d-2 and d-1 of a count table in closed form
     TK_LINEAR = 7,  // out[x] = x / g + 1 (a runs-table row above the ones row)
+    TK_CHAIN = 9,   // chains [begin, end) of in -> out, a warp each
     TK_LANES = 8    // chains [begin, end) of in -> out, 32 neighbouring chains a warp
 };
 struct ScanTask {
@@ -391,7 +392,7 @@ struct ScanTask {
 };
 int launch_scan_tasks(const ScanJob *jobs, const ScanTask *tasks, int ntasks, cudaStream_t s);
 int64_t scan_direct_limit();  // chains up to this length are scanned directly
-int scan_plan(int64_t chains, int64_t T);  // 0: a lane a chain, w: tiles of w chains, -1: blocked
+int scan_plan(int64_t chains, int64_t T);  // 0, -2: a lane, a warp a chain, w: tiles of w, -1: blocked
 int64_t scan_blocks_per_task();  // block sums a TK_BSUM / TK_APPLY task covers
 int scan_block_rows();        // entries per block of a blocked scan
 

@@ -972,6 +972,59 @@ __global__ void __launch_bounds__(UNRANK_THREADS)
     }
 }
 
+// The same for few ranks, a warp per rank: the 32-probe searches take two rounds
+// of independent loads a coordinate where a thread's gallop takes three to
+// five dependent ones, and a rank does not wait for the longest gallop of
+// 32.  A memo in element order ends the searches where it applies, too.
+constexpr int UNRANK_WARP_THREADS = 64;
+
+template <int D>
+__global__ void __launch_bounds__(UNRANK_WARP_THREADS)
+    fz_unrank_warp_kernel(const __grid_constant__ EnumParams P, const uint64_t *ranks, uint64_t m) {
+    constexpr int WARPS = UNRANK_WARP_THREADS / 32;
+    const int lane = threadIdx.x & 31;
+    const int levels = P.run_memo ? D - P.K - 1 : D - 1;
+    const uint64_t total = __ldg(P.C + P.n);
+    for (uint64_t i = (uint64_t)blockIdx.x * WARPS + (threadIdx.x >> 5); i < m;
+         i += (uint64_t)gridDim.x * WARPS) {
+        uint64_t R = __ldg(ranks + i);
+        bool good = R < total, leaf = false;
+        int rem = P.n, word = 0;  // word: a_lane
+        for (int j = 0; j < levels; ++j) {
+            int v;
+            uint64_t before;
+            find_child(P, j, rem, R, lane, v, before);
+            if (lane == j) word = v;
+            R -= before;
+            rem -= v * P.g[j];
+            leaf = j == P.lam_m && rem < P.top && !P.run_memo;
+            if (leaf) break;
+            if (j + 1 < levels) good = good && R < __ldg(P.C + (int64_t)(j + 1) * P.cs + rem);
+        }
+        if (leaf) {
+            const uint64_t at = __ldg(P.O + rem) + R;
+            good = good && at < P.memo_rows;  // bounds guard
+            if (good && lane > P.lam_m && lane < D)
+                word = __ldg(P.memo + (size_t)at * P.K + (lane - P.lam_m - 1));
+        } else if (P.run_memo) {
+            const uint32_t q = fd_div((uint32_t)rem, P.leaf.fg);
+            const uint64_t at = __ldg(P.cls_beg + ((uint32_t)rem - q * P.leaf.fg.g)) + R;
+            good = good && at < P.memo_rows;  // bounds guard
+            if (good && lane >= levels && lane < D) {
+                const int x = __ldg(reinterpret_cast<const int32_t *>(P.run_memo) +
+                                    (size_t)at * run_stride(P.K + 1) + (lane - levels));
+                word = lane == levels ? (int)q - x : x;
+            }
+        } else {
+            const uint32_t q = fd_div((uint32_t)rem, P.leaf.pair.fh);
+            good = good && q * P.leaf.pair.fh.g == (uint32_t)rem;
+            if (lane == D - 1) word = (int)q;
+        }
+        if (lane < D) P.out[i * D + lane] = good ? word : -1;
+        if (!good && lane == 0) atomicExch(P.status, (int)DEV_INTERNAL);
+    }
+}
+
 // Whole output taken from one place: d == 1 (one candidate) or k == d (the
 // output is Memo[n] itself).  mode 1: copy memo rows; mode 2: single row.
 __global__ void fz_direct_kernel(const EnumParams P, int mode) {
@@ -1052,9 +1105,24 @@ static int launch_enum_d(const EnumParams &P, cudaStream_t s, int sms) {
     return launch_enum_dl<D, -1>(P, s, sms);
 }
 
+// Up to how many ranks a warp takes each (us a launch by warps / by threads of
+// a width-6 set at 1000, 6000, 8000, 12000 ranks: with a depth-3 table 3.8 /
+// 5.8, 5.2 / 6.1, 5.8 / 6.1, 7.7 / 6.1; searched to the end 6.5 / 14.7, 8.2 /
+// 14.7, 10.1 / 14.8, 14.1 / 14.8; width 4 with a depth-2 table 3.3 / 4.4, 4.4 /
+// 4.4, 4.9 / 4.3).
+constexpr uint64_t UNRANK_WARP_RUN = 6144, UNRANK_WARP_MAX = 8192;
+
 template <int D>
 static int launch_unrank_d(const EnumParams &P, const uint64_t *ranks, uint64_t m,
                            cudaStream_t s) {
+    if (m <= (P.run_memo ? UNRANK_WARP_RUN : UNRANK_WARP_MAX)) {
+        constexpr int WARPS = UNRANK_WARP_THREADS / 32;
+        fz_unrank_warp_kernel<D>
+            <<<(unsigned)((m + WARPS - 1) / WARPS), UNRANK_WARP_THREADS, 0, s>>>(P, ranks, m);
+        note_launch();
+        FZ_CUDA_TRY(cudaGetLastError());
+        return FZ_OK;
+    }
     uint64_t blocks = (m + UNRANK_THREADS - 1) / UNRANK_THREADS;
     if (blocks > 65536) blocks = 65536;
     fz_unrank_kernel<D><<<(unsigned)blocks, UNRANK_THREADS, 0, s>>>(P, ranks, m);

@@ -260,8 +260,10 @@ int fz_plan_create(const int32_t *g, int d, int32_t n, const fz_opts_t *opt,
 int fz_plan_info(fz_plan_t plan, fz_plan_info_t *info);
 
 /* Cap the enumeration kernel of this plan at `ctas` blocks per SM (0 = as
- * many as fit; the kernel fits 4).  Leaving room lets other kernels run
- * beside it, e.g. another plan's rebuild overlapping this enumeration.
+ * many as fit; the kernel fits 4).  A cap of 1 to 3 leaves room for other
+ * kernels beside it, e.g. another plan's rebuild overlapping this enumeration;
+ * that plan is to have such a cap too, which also keeps the blocks of its
+ * rebuild small.
  * Errors: FZ_EINVAL. */
 int fz_plan_set_enum_ctas_per_sm(fz_plan_t plan, int32_t ctas);
 
@@ -378,9 +380,10 @@ int fz_batch_layout(fz_batch_t batch, uint64_t *rows, uint64_t *word_offsets,
                     int32_t *k, int32_t *top);
 /* Recompute every table and memo in place.  Asynchronous (capturable). */
 int fz_batch_rebuild(fz_batch_t batch, void *stream);
-/* Cap the batch's enumeration kernel at `ctas` blocks per SM (0 = as many
- * as fit; it fits 4), leaving room for other kernels beside it, e.g. the
- * rebuild of another batch overlapping this enumeration.
+/* Cap the batch's enumeration kernels at `ctas` blocks per SM (0 = as many
+ * as fit: 3, or 4 of the general kernel).  A cap of 1 to 3 takes one less than
+ * fit at most, leaving room for other kernels beside it, e.g. the rebuild of
+ * another batch overlapping this enumeration.
  * Errors: FZ_EINVAL. */
 int fz_batch_set_enum_ctas_per_sm(fz_batch_t batch, int32_t ctas);
 /* All instances' rows into out_dev (capacity in int32 words).  Asynchronous,

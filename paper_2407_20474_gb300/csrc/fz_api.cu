@@ -306,7 +306,7 @@ int plan_enqueue_memo(fz_plan_s *p, cudaStream_t s) {
     mb.status = p->status;
     mb.bar = p->bar;
     // an enumeration capped below full occupancy leaves room for a small build
-    mb.small_ctas = p->ctas_per_sm > 0 && p->ctas_per_sm <= 3;
+    mb.small_ctas = leaves_room(p->ctas_per_sm);
     return launch_memo_build(tail, p->K, p->top, p->memo_rows, mb, s);
 }
 
@@ -1394,16 +1394,20 @@ int fz_plan_set_enum_ctas_per_sm(fz_plan_t p, int32_t ctas) {
 int fz_plan_rebuild(fz_plan_t p, void *stream) {
     if (!p) return set_error(FZ_EINVAL, "plan: null pointer");
     cudaStream_t s = as_stream(stream);
-    if (small_tables(p->n)) {
+    // (a block of 1024 threads and up to 192 KB does not fit beside another
+    // plan's enumeration)
+    const bool one_block = !leaves_room(p->ctas_per_sm);
+    if (one_block && small_tables(p->n)) {
         const int rc = launch_tables_small(p->g, p->d, p->n, p->C, p->RT, p->lam_r, p->clamp_row,
                                            p->top, nullptr, s);
         if (rc != FZ_OK) return rc;
         return plan_enqueue_memo(p, s);
     }
-    int rc = launch_count_table_tmp(p->g, p->d, p->n, p->C, p->tmp, s);
+    int rc = launch_count_table_tmp(p->g, p->d, p->n, p->C, p->tmp, s, one_block);
     if (rc != FZ_OK) return rc;
     if (p->RT) {
-        rc = launch_runs_table(p->g, p->lam_r, p->n, p->RT, p->tmp, p->clamp_row, p->top, s);
+        rc = launch_runs_table(p->g, p->lam_r, p->n, p->RT, p->tmp, p->clamp_row, p->top, s,
+                               one_block);
         if (rc != FZ_OK) return rc;
     }
     return plan_enqueue_memo(p, s);

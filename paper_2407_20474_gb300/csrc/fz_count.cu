@@ -365,8 +365,8 @@ int launch_tail_rows(const int32_t *g, int d, uint64_t *pair, uint64_t *one, uin
 }
 
 int launch_count_table_tmp(const int32_t *g, int d, int32_t n, uint64_t *table, uint64_t *tmp,
-                           cudaStream_t s) {
-    if (n <= SMALL_ONE_N)
+                           cudaStream_t s, bool one_block) {
+    if (one_block && n <= SMALL_ONE_N)
         return launch_tables_small(g, d, n, table, nullptr, 0, -1, 0, nullptr, s);
     const int64_t len = (int64_t)n + 1;
     uint64_t *last = table + (int64_t)d * len;
@@ -402,8 +402,8 @@ __global__ void row_ones_kernel(uint64_t *__restrict__ row, int64_t len) {
 // with remainder x: RT[lam][x] = 1 and RT[j] = RT[j+1] strided-summed with
 // stride g_j -- the count-table recurrence over the leading generators.
 int launch_runs_table(const int32_t *g, int lam, int32_t n, uint64_t *RT, uint64_t *tmp,
-                      int clamp_row, int64_t clamp_top, cudaStream_t s) {
-    if (n <= SMALL_ONE_N)
+                      int clamp_row, int64_t clamp_top, cudaStream_t s, bool one_block) {
+    if (one_block && n <= SMALL_ONE_N)
         return launch_tables_small(g, lam, n, nullptr, RT, lam, clamp_row, clamp_top, nullptr, s);
     const int64_t len = (int64_t)n + 1;
     uint64_t *ones = RT + (int64_t)lam * len;

@@ -1053,7 +1053,10 @@ static int half_rows_for(int d, int ring_bytes = RING_BYTES_PER_WARP) {
 }
 
 // Ring bytes per warp for an occupancy cap: fewer resident warps get larger
-// rings, so the bytes in flight per SM stay about the same.
+// rings, so the bytes in flight per SM stay about the same.  A cap leaves 52 KB
+// of an SM's 228 and a quarter of its registers: one block of any kernel of a
+// rebuild (run_build_kernel has 45 KB; with rings of 192 KB together it waited
+// for the end of the enumeration).
 // FZ_ENUM_RING_KB overrides (tuning only).
 static int ring_bytes_for(int ctas_per_sm) {
     static const int forced = [] {
@@ -1062,8 +1065,8 @@ static int ring_bytes_for(int ctas_per_sm) {
         return (kb >= 4 && kb <= 24) ? kb * 1024 : 0;
     }();
     if (forced) return forced;
-    if (ctas_per_sm <= 0 || ctas_per_sm >= 4) return RING_BYTES_PER_WARP;
-    const int b = (192 * 1024) / (ctas_per_sm * ENUM_WARPS);
+    if (!leaves_room(ctas_per_sm)) return RING_BYTES_PER_WARP;
+    const int b = (176 * 1024) / (ctas_per_sm * ENUM_WARPS);
     return b > 16 * 1024 ? 16 * 1024 : (b / 1024) * 1024;
 }
 
@@ -1450,14 +1453,11 @@ int launch_enumerate_batch(const void *params_dev, const uint64_t *item0_dev,
         int per_sm = 0;
         FZ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fz_enum_batch_kernel,
                                                                   ENUM_THREADS, smem));
-        if (per_sm < 1) per_sm = 1;
-        if (ctas_per_sm > 0 && ctas_per_sm < per_sm) per_sm = ctas_per_sm;
-        uint64_t grid = (uint64_t)per_sm * dp.sms;
+        uint64_t grid = (uint64_t)batch_blocks_for(per_sm, ctas_per_sm) * dp.sms;
         const uint64_t want = (G.item_hi - G.item_lo + ENUM_WARPS - 1) / ENUM_WARPS;
         if (want < grid) grid = want;
-        fz_enum_batch_kernel<<<(unsigned)grid, ENUM_THREADS, smem, s>>>(BP);
-        note_launch();
-        FZ_CUDA_TRY(cudaGetLastError());
+        rc = launch_capped(fz_enum_batch_kernel, (unsigned)grid, smem, s, ctas_per_sm, false, BP);
+        if (rc != FZ_OK) return rc;
     }
     return FZ_OK;
 }

@@ -665,6 +665,41 @@ int launch_flat_batch(const BatchEnumParams &BP, int d, int np, int src, cudaStr
                       int ctas_per_sm);
 // fz_enum.cu: grid and launch of a persistent enumeration kernel.
 constexpr int ENUM_MAX_SMEM = 200 * 1024;
+// Blocks an SM takes when `fit` do.
+inline int blocks_for(int fit, int ctas_per_sm) {
+    if (ctas_per_sm > 0 && ctas_per_sm < fit) fit = ctas_per_sm;
+    return fit < 1 ? 1 : fit;
+}
+// Batches: three blocks of the flat walk's kernels fill an SM's registers, so a
+// cap that is to leave room takes one less than fit.
+inline int batch_blocks_for(int fit, int ctas_per_sm) {
+    return blocks_for(leaves_room(ctas_per_sm) ? fit - 1 : fit, ctas_per_sm);
+}
+// A launch of ENUM_THREADS threads a block.  Under a cap the SM is asked for
+// all its shared memory, so that other kernels' blocks find some; chained: it
+// may start while the launch before it drains.
+template <typename Kern, typename... Args>
+int launch_capped(Kern kern, unsigned grid, size_t smem, cudaStream_t s, int ctas_per_sm,
+                  bool chained, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(ENUM_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    if (chained) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (leaves_room(ctas_per_sm)) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[cfg.numAttrs++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+    }
+    FZ_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
+    note_launch();
+    return FZ_OK;
+}
 template <typename Kern, typename... Args>
 int launch_enum_grid(Kern kern, const EnumParams &P, size_t smem, cudaStream_t s, int sms,
                      DeviceOnce &attr_set, Args... args) {
@@ -678,17 +713,12 @@ int launch_enum_grid(Kern kern, const EnumParams &P, size_t smem, cudaStream_t s
     }
     int per_sm = 0;
     FZ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, ENUM_THREADS, smem));
-    if (P.ctas_per_sm > 0 && per_sm > P.ctas_per_sm) per_sm = P.ctas_per_sm;
-    if (per_sm < 1) per_sm = 1;
     uint64_t want = (P.nslices + ENUM_WARPS - 1) / ENUM_WARPS;
-    uint64_t grid = (uint64_t)per_sm * sms;
+    uint64_t grid = (uint64_t)blocks_for(per_sm, P.ctas_per_sm) * sms;
     if (want < grid) grid = want;
     if (grid < 1) grid = 1;
     FZ_CUDA_TRY(cudaMemsetAsync(P.slice_counter, 0, sizeof(unsigned long long), s));
-    kern<<<(unsigned)grid, ENUM_THREADS, smem, s>>>(P, args...);
-    note_launch();
-    FZ_CUDA_TRY(cudaGetLastError());
-    return FZ_OK;
+    return launch_capped(kern, (unsigned)grid, smem, s, P.ctas_per_sm, false, P, args...);
 }
 
 }  // namespace fz

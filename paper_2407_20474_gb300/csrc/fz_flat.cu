@@ -289,24 +289,10 @@ int launch_batch_one(const BatchEnumParams &BP, cudaStream_t s, int sms, int cta
                                                                   ENUM_THREADS, smem));
         attr_set.set(dev);
     }
-    int per_sm = occupancy[dev] < 1 ? 1 : occupancy[dev];
-    if (ctas_per_sm > 0 && ctas_per_sm < per_sm) per_sm = ctas_per_sm;
-    uint64_t grid = (uint64_t)per_sm * sms;
+    uint64_t grid = (uint64_t)batch_blocks_for(occupancy[dev], ctas_per_sm) * sms;
     const uint64_t want = (BP.item_hi - BP.item_lo + ENUM_WARPS - 1) / ENUM_WARPS;
     if (want < grid) grid = want;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(ENUM_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = BP.chained ? 1 : 0;
-    FZ_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, BP));
-    note_launch();
-    return FZ_OK;
+    return launch_capped(kern, (unsigned)grid, smem, s, ctas_per_sm, BP.chained != 0, BP);
 }
 
 template <int D>

@@ -334,8 +334,9 @@ int validate_gens(const int32_t *g, int d);
 // n + 1, into table (device), using `tmp` (count_table_tmp_words words) as
 // scratch.  Asynchronous; saturates at 2^64 - 1.
 int64_t count_table_tmp_words(const int32_t *g, int d, int32_t n);
+// one_block: short tables may take the one-block kernel below.
 int launch_count_table_tmp(const int32_t *g, int d, int32_t n, uint64_t *table, uint64_t *tmp,
-                           cudaStream_t s);
+                           cudaStream_t s, bool one_block = true);
 // Short tables (small_tables(n)): count table C and candidates table RT (rows
 // 0..lam, clamped as launch_runs_table; either may be null) in one launch, with
 // the rows' sums (d + 1, entries clamped to 2^32) if asked for.
@@ -504,12 +505,16 @@ struct EnumLaunch {
 // (before the rows above it are summed).
 int launch_runs_table(const int32_t *g, int lam, int32_t n, uint64_t *RT, uint64_t *tmp,
                       int clamp_row, int64_t clamp_top,
-                      cudaStream_t s);
+                      cudaStream_t s, bool one_block = true);
 int launch_enumerate(const EnumLaunch &L, uint64_t rank_begin, uint64_t nrows, int32_t *out,
                      uint64_t slice_rows, cudaStream_t s);
 int launch_unrank(const EnumLaunch &L, const uint64_t *ranks, uint64_t m, int32_t *out,
                   cudaStream_t s);
 uint64_t default_slice_rows(uint64_t nrows, int sms);
+// Whether an occupancy cap (ctas_per_sm) is to leave room beside the
+// enumeration (4 blocks of the plans' kernels fit an SM), and whether a plan so
+// capped, one of several that take turns, is to be rebuilt by small blocks.
+inline bool leaves_room(int ctas_per_sm) { return ctas_per_sm > 0 && ctas_per_sm <= 3; }
 // Batched enumeration (fz_enum.cu): per-instance parameter images, then one
 // persistent launch per group of instances of one shape (the flat walk's
 // kernels are compiled per width, leaf length and source; shape 0: the

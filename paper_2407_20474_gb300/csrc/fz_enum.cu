@@ -1245,7 +1245,7 @@ static EnumParams make_params(const EnumLaunch &L) {
 // 210, 209): 10.
 static bool by_rank(const EnumLaunch &L, const EnumParams &P, uint64_t least) {
     return P.flat_np > 0 && P.flat_src == SRC_PAIR && rank_walk_serves(L.d) && L.RT &&
-           L.total_cost > L.total_rows + least * L.W * L.total_rows;
+           prefixes_exceed(L.total_cost, L.total_rows, L.W, least);
 }
 
 // Enumerate ranks [rank_begin, rank_begin + nrows) into out.  Asynchronous.

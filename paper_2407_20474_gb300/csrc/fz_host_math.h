@@ -69,4 +69,12 @@ inline uint64_t pair_rows_upto(int64_t n, int64_t t0, int64_t t1) {
     return s > (unsigned __int128)~0ull ? ~0ull : (uint64_t)s;
 }
 
+// Whether a set of `rows` rows and total cost rows + W prefixes (W >= 1) has more
+// than `least` prefixes a row.  Divides: least W rows would wrap for the counts
+// next to 2^64 that windows are enumerated of.
+inline bool prefixes_exceed(uint64_t cost, uint64_t rows, uint64_t W, uint64_t least) {
+    const uint64_t prefixes = cost > rows ? (cost - rows) / W : 0;
+    return prefixes > 0 && (prefixes - 1) / least >= rows;
+}
+
 }  // namespace fz

@@ -1082,18 +1082,19 @@ static int build_memo_to(const int32_t *tail, int k, int32_t top, uint64_t *O, i
                 if (fits) bytes += run_levels_bytes(tail, k, top - 1, sums, true);
             }
             if (fits && work.alloc_call(bytes, s) == FZ_OK) {
+                RunLevels lv;
                 int *status = work.as<int>();
                 FZ_CUDA_TRY(cudaMemsetAsync(status, 0, 256, s));
                 if (k <= 2) {
                     rc = launch_memo_closed(tail, k, top, O, *R, status, s);
                 } else {
-                    RunLevels lv;
                     rc = run_levels_init(tail, k, top - 1, sums, true, C, cs, O, *R,
                                          work.as<char>() + 256, &lv, s);
                     if (rc == FZ_OK) rc = launch_run_levels(lv, status, s);
                 }
-                if (rc != FZ_OK) return rc;
-                return read_status(status, s);
+                if (rc == FZ_OK) return read_status(status, s);
+                cudaStreamSynchronize(s);
+                return rc;
             }
             cudaGetLastError();
         }

@@ -45,6 +45,13 @@ struct DevArena {
     }
 };
 
+// Synchronises at the end of a scope whose host memory is the source of copies
+// (declared after it, so destroyed before it).
+struct SyncAtEnd {
+    cudaStream_t s;
+    ~SyncAtEnd() { cudaStreamSynchronize(s); }
+};
+
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // Elementwise batches a batch memo may take (its top is cut to this many
@@ -575,7 +582,8 @@ int batch_create_runs(fz_batch_s *b, uint64_t *tb, cudaStream_t s) {
     if (rc != FZ_OK) return rc;
     RunBuild *tj = static_cast<RunBuild *>(sizes.p);
     uint64_t *td = reinterpret_cast<uint64_t *>(static_cast<char *>(sizes.p) + jb);
-    std::vector<RunBuild> byt(m);
+    std::vector<RunBuild> byt(m), rj(m);
+    SyncAtEnd sync{s};
     size_t cls_words = 0;
     for (int t = 0; t < m; ++t) {
         const std::vector<int32_t> &g = gens[t];
@@ -600,7 +608,6 @@ int batch_create_runs(fz_batch_s *b, uint64_t *tb, cudaStream_t s) {
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
         return tab[x].K != tab[y].K ? tab[x].K < tab[y].K : tab[x].kind < tab[y].kind;
     });
-    std::vector<RunBuild> rj(m);
     for (int p = 0; p < m; ++p) {
         at[order[p]] = p;
         rj[p] = byt[order[p]];
@@ -665,7 +672,6 @@ int batch_create_runs(fz_batch_s *b, uint64_t *tb, cudaStream_t s) {
                                 cudaMemcpyHostToDevice, s));
     rc = batch_enqueue_runs(b, s);
     if (rc != FZ_OK) return rc;
-    FZ_CUDA_TRY(cudaStreamSynchronize(s));  // rj is a host temporary
     for (Inst &I : b->inst) {
         if (!I.run) continue;
         const RunBuild &R = rj[at[I.run_job]];

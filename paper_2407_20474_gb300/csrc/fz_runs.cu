@@ -495,7 +495,7 @@ int run_levels_init(const int32_t *t, int k, int32_t n, const uint64_t *sums, bo
     L->jobs_dev = reinterpret_cast<RunBuild *>(m);
     m += up256((size_t)FZ_MAX_D * sizeof(RunBuild));
     const int last = k - 3 > 0 ? k - 3 : 0;
-    RunBuild h[FZ_MAX_D] = {};
+    RunBuild *h = L->jobs;
     size_t size[FZ_MAX_D], buf[2] = {0, 0};
     uint64_t *cls[FZ_MAX_D];
     int32_t *rows[FZ_MAX_D];
@@ -552,8 +552,6 @@ int run_levels_init(const int32_t *t, int k, int32_t n, const uint64_t *sums, bo
         L->blocks[L->n] = run_build_blocks(R, k, true);
         ++L->n;
     }
-    // the jobs are a host temporary: the copy from pageable memory returns
-    // once it has been read
     FZ_CUDA_TRY(cudaMemcpyAsync(L->jobs_dev, h, (size_t)L->n * sizeof(RunBuild),
                                 cudaMemcpyHostToDevice, s));
     return FZ_OK;

@@ -132,6 +132,9 @@ struct RunBuild {
 // The levels of one chain (fz_runs.cu): tables[, the memo in element order].
 struct RunLevels {
     RunBuild *jobs_dev = nullptr;
+    // source of the copy to jobs_dev, which need not have been read when the
+    // call that enqueued it returns: stays until the stream is synchronised
+    RunBuild jobs[FZ_MAX_D] = {};
     int n = 0, tables = 0;
     bool csr = false;
     int K[FZ_MAX_D] = {};

@@ -72,10 +72,11 @@ namespace {
 // pool of the library's own, one per device: allocating and freeing then costs
 // microseconds and no device synchronisation (cudaMalloc and cudaFree took
 // most of a small call: 324 us for 3.8e3 rows, 154 with the pool).  The
-// pool keeps at most POOL_KEEP_BYTES between calls; what lies above goes back
-// to the device at the next synchronisation.  Allocation and release are
-// ordered on the call's stream, so any number of threads and streams share it.
-// Handles (plans, memos, batches, servers) own cudaMalloc memory.
+// pool keeps at most POOL_KEEP_BYTES between calls (CallMemory): cudaMalloc does
+// not take what a pool holds, not even when it would fail.  Allocation and
+// release are ordered on the call's stream, so any number of threads and
+// streams share it.  Handles (plans, memos, batches, servers) own cudaMalloc
+// memory.
 constexpr uint64_t POOL_KEEP_BYTES = 64ull << 20;
 
 cudaMemPool_t call_pool() {
@@ -155,6 +156,25 @@ struct DevBuf {
     template <class T>
     T *as() const {
         return static_cast<T *>(p);
+    }
+};
+
+// Declared before a call's pool buffers: at the end of the call, when they have
+// been released, what the pool holds above POOL_KEEP_BYTES (and no other call
+// uses) goes back to the device.
+struct CallMemory {
+    cudaStream_t s;
+    ~CallMemory() {
+        cudaMemPool_t pool = call_pool();
+        uint64_t held = 0;
+        if (pool &&
+            cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+            held > POOL_KEEP_BYTES) {
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+                cudaStreamSynchronize(s);  // (a call on a captured stream has been refused)
+            cudaMemPoolTrimTo(pool, POOL_KEEP_BYTES);
+        }
     }
 };
 
@@ -939,6 +959,7 @@ int fz_count_upto(const int32_t *g, int d, int32_t n_max, uint64_t *counts, void
     cudaStream_t s = as_stream(stream);
     const int64_t len = (int64_t)n_max + 1;
     int64_t tmpw = count_table_tmp_words(g, d, n_max);
+    CallMemory mem{s};
     DevBuf buf;
     rc = buf.alloc_call((size_t)(2 * len + tmpw) * 8, s);
     if (rc != FZ_OK) return rc;
@@ -958,6 +979,7 @@ int fz_count(const int32_t *g, int d, int32_t n, uint64_t *count, void *stream) 
     cudaStream_t s = as_stream(stream);
     const int64_t len = (int64_t)n + 1;
     int64_t tmpw = count_table_tmp_words(g, d, n);
+    CallMemory mem{s};
     DevBuf buf;
     rc = buf.alloc_call((size_t)(2 * len + tmpw) * 8, s);
     if (rc != FZ_OK) return rc;
@@ -1020,6 +1042,7 @@ int fz_memo_rows(const int32_t *tail, int k, int32_t top, uint64_t *rows, void *
         if (rc == FZ_OK) *rows = 0;
         return rc;
     }
+    CallMemory mem{s};
     DevBuf table, off;
     uint64_t *C = nullptr;
     int64_t tmpw = 0;
@@ -1041,6 +1064,7 @@ int fz_memo_rows(const int32_t *tail, int k, int32_t top, uint64_t *rows, void *
 static int build_memo_to(const int32_t *tail, int k, int32_t top, uint64_t *O, int32_t **R,
                          uint64_t rows_capacity, uint64_t *rows_needed, DevBuf *own_rows,
                          cudaStream_t s, int schedule = MEMO_LEVELS) {
+    CallMemory mem{s};
     DevBuf table, work;
     uint64_t *C = nullptr;
     int64_t tmpw = 0;
@@ -1450,6 +1474,7 @@ int fz_plan_destroy(fz_plan_t p) {
 int fz_enumerate(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, uint64_t rank_begin,
                  uint64_t rank_end, int32_t *out_dev, uint64_t out_capacity_rows,
                  uint64_t *written, void *stream) {
+    CallMemory mem{as_stream(stream)};
     fz_plan_t p = nullptr;
     int rc = plan_create(g, d, n, opt, true, &p, stream);
     if (rc != FZ_OK) return rc;
@@ -1470,6 +1495,7 @@ int fz_enumerate_host_chunks(const int32_t *g, int d, int32_t n, const fz_opts_t
                              uint64_t rank_begin, uint64_t rank_end, int32_t *out_host,
                              uint64_t out_capacity_rows, uint64_t chunk_rows,
                              uint64_t *written, void *stream) {
+    CallMemory mem{as_stream(stream)};
     fz_plan_t p = nullptr;
     int rc = plan_create(g, d, n, opt, true, &p, stream);
     if (rc != FZ_OK) return rc;

@@ -257,13 +257,14 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 }  // namespace
 
 // FZ_RUN_COST overrides W (tuning only).
-void balance_level(int d, int K, int top, int n, bool run_order, bool pair, int *lam_r,
+void balance_level(int d, int K, int top, int n, bool run_order, bool pair, bool batch, int *lam_r,
                    uint64_t *W, int *clamp_row) {
     static const long long forced = [] {
         const char *e = getenv("FZ_RUN_COST");
         return e ? atoll(e) : 0ll;
     }();
     const bool memo = K >= 1 && K <= d - 1 && top > 0;
+    const bool flat_pair = flat_serves(d, d - 2, SRC_PAIR) && !(batch && d > BATCH_FLAT_MAX_D);
     *clamp_row = -1;
     if (run_order) {
         // the run-order walk visits every prefix of the leading d - K - 1
@@ -273,7 +274,7 @@ void balance_level(int d, int K, int top, int n, bool run_order, bool pair, int 
     } else if (memo && top > n) {
         // full memo: the leaves are the memo leaves, evaluated 32 at a time
         *lam_r = d - K;
-        *W = pair && flat_serves(d, d - 2, SRC_PAIR) ? FLAT_LEAF_COST : 16;
+        *W = pair && flat_pair ? FLAT_LEAF_COST : 16;
     } else if (K == 1 || !walk_progression_enabled()) {
         // walk leaves evaluated candidate by candidate: count the candidates
         *lam_r = d - 1;
@@ -283,7 +284,7 @@ void balance_level(int d, int K, int top, int n, bool run_order, bool pair, int 
         // prefix plus a progression; a memo leaf (a prefix of length d - K
         // with remainder below top) is one unit whatever lies under it
         *lam_r = d - 2;
-        *W = !memo && flat_serves(d, d - 2, SRC_PAIR) ? FLAT_LEAF_COST : 64;
+        *W = !memo && flat_pair ? FLAT_LEAF_COST : 64;
         if (memo && K > 2) *clamp_row = d - K;
     }
     if (*lam_r < 0) *lam_r = 0;
@@ -577,7 +578,7 @@ int plan_create_impl(const int32_t *g, int d, int32_t n, const fz_opts_t *opt, f
     // single block: d == 1 or k == d with a full memo)
     const bool single_block = d == 1 || (p->K == d && p->top > n);
     if (!single_block && p->count > 0) {
-        balance_level(d, p->K, p->top, n, p->run_memo != nullptr, false, &p->lam_r, &p->W,
+        balance_level(d, p->K, p->top, n, p->run_memo != nullptr, false, p->resident, &p->lam_r, &p->W,
                       &p->clamp_row);
         rc = p->alloc(p->runs, (size_t)(p->lam_r + 1) * cs * 8);
         if (rc != FZ_OK) return rc;

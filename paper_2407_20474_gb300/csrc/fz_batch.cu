@@ -751,7 +751,7 @@ int batch_create_impl(const fz_instance_t *inst, int count, const fz_opts_t *opt
         words += (size_t)(I.d + 1) * len;
         I.off_RT = (size_t)-1;
         if (I.d >= 2) {
-            balance_level(I.d, I.K, I.top, I.n, I.run, I.pair, &I.lam_r, &I.W, &I.clamp_row);
+            balance_level(I.d, I.K, I.top, I.n, I.run, I.pair, true, &I.lam_r, &I.W, &I.clamp_row);
             I.flat = I.d <= 8 &&
                      (I.run ? flat_serves(I.d, lam, SRC_RUN)
                             : (I.pair || (I.K == 0 && walk_progression_enabled())) &&

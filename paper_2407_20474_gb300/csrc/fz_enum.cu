@@ -1318,7 +1318,7 @@ void fill_batch_params(const EnumLaunch &L, int32_t *out, uint64_t count, void *
     P.nrows = count;
     P.aligned = ((uintptr_t)out & 15u) == 0;
     P.half_rows = half_rows_for(L.d);
-    if (L.d > 8) P.flat_np = 0;  // the batch kernel's flat walk: widths 3..8
+    if (L.d > BATCH_FLAT_MAX_D) P.flat_np = 0;
     if (by_rank(L, P, 10)) P.flat_src = SRC_RANK;
     memcpy(dst, &P, sizeof(P));
 }

@@ -461,11 +461,13 @@ bool walk_progression_enabled();
 // runs (the last two coordinates as a progression) and run-order runs walked
 // one at a time cost a chain of dependent loads each (W = 64); memo leaves
 // and candidates evaluated 32 at a time cost W = 16, leaves of the flat walk
-// FLAT_LEAF_COST.
+// FLAT_LEAF_COST.  batch: enumerated by the batch kernels, whose flat walk
+// takes widths up to BATCH_FLAT_MAX_D.
 // *clamp_row >= 0: the table row whose entries below top are set to 1 (a
 // memo leaf is one unit, whatever lies under it), else -1.
 bool run_memo_enabled();
-void balance_level(int d, int K, int top, int n, bool run_order, bool pair, int *lam_r,
+constexpr int BATCH_FLAT_MAX_D = 8;
+void balance_level(int d, int K, int top, int n, bool run_order, bool pair, bool batch, int *lam_r,
                    uint64_t *W, int *clamp_row);
 
 struct EnumLaunch {

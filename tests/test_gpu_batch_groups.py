@@ -117,3 +117,20 @@ def test_items_of_the_general_kernel(fz):
         b.enumerate(out)
         b.sync()
         _check(out, b.word_offsets, inst)
+
+
+@pytest.mark.parametrize("g", [(13, 17, 19, 23, 29, 31, 37, 41, 43), (13, 17, 19, 23, 29, 31, 37, 41, 43, 44)])
+def test_cost_of_a_wide_walk(fz, g):
+    """Widths above 8 without a memo are walked by the general kernel, where a
+    prefix of d - 2 coordinates costs as much as 64 rows: the work items."""
+    n = workloads.find_n(oracle.count_upto, g, 30000)
+    prefixes = oracle.count(g[:-2] + (1,), n)
+    cost = oracle.count(g, n) + 64 * prefixes
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    target = max(4096, cost // (sms * 16 * 8 + 1))
+    with fz.Batch([(g, n)], k=0) as b:
+        assert b.work_items == -(-cost // target)
+        out = torch.full((b.total_words + 8,), CANARY, dtype=torch.int32, device="cuda")
+        b.enumerate(out)
+        b.sync()
+        _check(out, b.word_offsets, [(g, n)])

@@ -79,6 +79,11 @@ namespace {
 // memory.
 constexpr uint64_t POOL_KEEP_BYTES = 64ull << 20;
 
+// Bytes of the calls' buffers, and whether they have been enough to take a pool
+// above POOL_KEEP_BYTES (a pool grows by blocks larger than what is asked for).
+std::atomic<uint64_t> g_pool_live{0};
+std::atomic<bool> g_pool_grown{false};
+
 cudaMemPool_t call_pool() {
     static std::mutex mu;
     // by device context: a reset takes a pool with its context
@@ -138,6 +143,7 @@ struct DevBuf {
             bytes = b;
             pooled = true;
             stream = s;
+            if (g_pool_live.fetch_add(b) + b > POOL_KEEP_BYTES / 4) g_pool_grown.store(true);
             return FZ_OK;
         }
         if (pool) cudaGetLastError();
@@ -145,9 +151,10 @@ struct DevBuf {
         return alloc(b);
     }
     void release() {
-        if (p && pooled)
+        if (p && pooled) {
+            g_pool_live.fetch_sub(bytes);
             cudaFreeAsync(p, stream);
-        else if (p)
+        } else if (p)
             cudaFree(p);
         p = nullptr;
         bytes = 0;
@@ -165,6 +172,8 @@ struct DevBuf {
 struct CallMemory {
     cudaStream_t s;
     ~CallMemory() {
+        if (!g_pool_grown.load() || !g_pool_grown.exchange(false)) return;
+        if (g_pool_live.load() > POOL_KEEP_BYTES / 4) g_pool_grown.store(true);  // others' buffers
         cudaMemPool_t pool = call_pool();
         uint64_t held = 0;
         if (pool &&

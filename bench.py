@@ -269,8 +269,12 @@ def code_hash(src):
 
 
 def enum_kernel_name(plan):
-    """Name of the enumeration kernel the plan launches."""
+    """Name of the enumeration kernel the plan launches (without a memo the rank
+    walk's, widths 4 to 7, when there are more than 3 prefixes a row)."""
     d, k = plan.d, plan.k
+    if k == 0 and 3 <= d <= 9:
+        flat = "fz_enum_flat_kernel<%d, %d, 1>" % (d, d - 2)
+        return flat + (" or fz_enum_rank_kernel<%d>" % d if 4 <= d <= 7 else "")
     if plan.run_order:
         # the flat walk's widths and prefix lengths; else the run copy
         if 3 <= d <= 9 and 1 <= d - k - 1 <= 3:

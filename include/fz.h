@@ -330,15 +330,15 @@ int fz_plan_destroy(fz_plan_t plan);
  * Batches: many instances Z(n_i, g_i) of possibly different d_i in one set
  * of launches -- batched counting tables, one memo per distinct tail shared
  * by the instances that have it, and one persistent enumeration launch per
- * shape (width, memo depth) over (instance, slice) work items.  Full memos (widths 3..8 with at least one
- * walked coordinate above the memo) are tables in run order, built generator
- * by generator, so a prefix's whole subtree is one contiguous copy; a memo of
- * depth 2 over the last two generators may be kept as its closed form, with
- * no table.  Memos in element order (partial memos, or where the policy turns
- * run order off) are built by the elementwise dynamic pass (Sections 2.2-2.4),
- * cut to at most 512 element batches; larger remainders take the ordinary
- * next-candidate step (Section 3.1).  The memo depth of each generator set is
- * chosen by the library unless opts.k is given.
+ * shape (width, memo depth) over (instance, slice) work items.  Full memos
+ * (widths 3..8 with at least one walked coordinate above the memo) are tables
+ * in run order, built generator by generator, so a prefix's whole subtree is
+ * one contiguous copy; a memo of depth 2 over the last two generators may be
+ * kept as its closed form, with no table.  Memos in element order (partial
+ * memos, or where the policy turns run order off) are built by the elementwise
+ * dynamic pass (Sections 2.2-2.4), cut to at most 512 element batches; larger
+ * remainders take the ordinary next-candidate step (Section 3.1).  The memo
+ * depth of each generator set is chosen by the library unless opts.k is given.
  * Output: instance i's rows (d_i int32 each, descending lexicographic order)
  * start at word word_offsets[i] of the output buffer (multiples of 32 words,
  * so 128-byte aligned when the buffer is); word_offsets[count] is the total.
@@ -387,7 +387,7 @@ int fz_batch_rebuild(fz_batch_t batch, void *stream);
  * Errors: FZ_EINVAL. */
 int fz_batch_set_enum_ctas_per_sm(fz_batch_t batch, int32_t ctas);
 /* All instances' rows into out_dev (capacity in int32 words).  Asynchronous,
- * one persistent kernel.  Errors: FZ_EINVAL, FZ_ENOSPC, FZ_ECUDA. */
+ * one persistent kernel per shape.  Errors: FZ_EINVAL, FZ_ENOSPC, FZ_ECUDA. */
 int fz_batch_enumerate(fz_batch_t batch, int32_t *out_dev,
                        uint64_t out_capacity_words, void *stream);
 /* Synchronise and report device-side errors (FZ_ETIMEOUT, FZ_EINTERNAL). */

@@ -289,7 +289,7 @@ int build_scan_plan(fz_batch_s *b, uint64_t *table_base, std::vector<ScanJob> &j
                          [&](const ScanTask &x, const ScanTask &y) {
                              return jobs[x.job].len / jobs[x.job].g > jobs[y.job].len / jobs[y.job].g;
                          });
-                for (int ji : step_jobs) {
+        for (int ji : step_jobs) {
             const ScanJob &J = jobs[ji];
             if (plan(J) > 0) continue;
             if (!J.slen) {

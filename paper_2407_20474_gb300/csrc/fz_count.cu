@@ -10,11 +10,11 @@
 //
 // Each row is a strided inclusive prefix sum of the row below it (stride
 // g_{j+1}): for every residue class rho mod g the entries rho, rho + g, ...
-// are summed in order.  Short chains are scanned by a warp or a lane each or tile
-// by tile; long
-// chains are cut into blocks of RB entries, the block sums are scanned by the
-// same routine (they form a strided array of the same shape), and the blocks
-// are then re-walked with their carries.  All sums saturate at 2^64 - 1.
+// are summed in order.  Short chains are scanned by a warp or a lane each or
+// tile by tile; long chains are cut into blocks of RB entries, the block sums
+// are scanned by the same routine (they form a strided array of the same
+// shape), and the blocks are then re-walked with their carries.  All sums
+// saturate at 2^64 - 1.
 #include <cstdlib>
 #include <cstring>
 
@@ -190,7 +190,8 @@ struct SmallTables {
     int g[FZ_MAX_D];
 };
 
-__global__ void __launch_bounds__(SMALL_THREADS) small_tables_kernel(const __grid_constant__ SmallTables P) {
+__global__ void __launch_bounds__(SMALL_THREADS)
+    small_tables_kernel(const __grid_constant__ SmallTables P) {
     extern __shared__ __align__(16) uint64_t small_smem[];
     __shared__ uint64_t part[SMALL_THREADS / 32];
     const bool runs = P.C == nullptr && P.C0 == nullptr ? true : blockIdx.x == 1;
@@ -340,7 +341,8 @@ int launch_tables_small(const int32_t *g, int d, int32_t n, uint64_t *C, uint64_
 // The last rows of a count table from their closed forms: C[d] the delta row,
 // C[d-1][r] = [g_d | r], C[d-2][r] = |Z(r, (g_{d-1}, g_d))|; null rows are not
 // written.  Bound by the stores: three rows of 2e6 entries in one launch and no
-// scan (count table of width 4: 109 us with four scans, 69 with two; all counts to 39064 for width 6: 86, 71).
+// scan (count table of width 4: 109 us with four scans, 69 with two; all counts
+// to 39064 for width 6: 86, 71).
 __global__ void __launch_bounds__(THREADS)
     tail_rows_kernel(const __grid_constant__ PairForm F, FastDiv last, uint64_t *__restrict__ pair,
                      uint64_t *__restrict__ one, uint64_t *__restrict__ delta, int64_t len) {

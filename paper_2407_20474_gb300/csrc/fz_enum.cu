@@ -890,10 +890,6 @@ __global__ void __launch_bounds__(ENUM_THREADS, 4)
     __syncwarp();
 }
 
-size_t enum_batch_smem_bytes() {
-    return (size_t)ENUM_WARPS * (BATCH_RING_BYTES + sizeof(EnumParams) + sizeof(WarpPath));
-}
-
 // Tuples of given ranks, a thread per rank.  Each leading coordinate is a
 // search in one count row: the rows of the children a_j >= v number
 // C[j][rem - v g_j], which grows about as the (d - 1 - j)-th power of its
@@ -1091,16 +1087,20 @@ static int launch_enum_runs(const EnumParams &P, cudaStream_t s, int sms) {
     return launch_enum_kernel(fz_enum_runs_kernel<D, LAMF, K>, P, D, s, sms, attr_set);
 }
 
-// Full memo of depth 2, 3 or 4: every run is a memo run at a fixed
-// coordinate; use the compile-time specialisation.  Otherwise generic.
+// Shapes the flat walk has no kernel for.  Full memo of depth 2, 3 or 4: every
+// run is a memo run at a fixed coordinate; use the compile-time
+// specialisation.  Otherwise generic.
 template <int D>
 static int launch_enum_d(const EnumParams &P, cudaStream_t s, int sms) {
     const bool full = P.lam_m >= 0 && P.top > P.n;
     const int K = P.K;
     if (full && P.run_memo && P.cls_beg) {
-        if (K == 1 && D >= 2) return launch_enum_runs<D, (D >= 2 ? D - 2 : 0), 1>(P, s, sms);
-        if (K == 2 && D >= 3) return launch_enum_runs<D, (D >= 3 ? D - 3 : 0), 2>(P, s, sms);
-        if (K == 3 && D >= 4) return launch_enum_runs<D, (D >= 4 ? D - 4 : 0), 3>(P, s, sms);
+        if constexpr (D >= 2 && !flat_serves(D, D - 2, SRC_RUN))
+            if (K == 1) return launch_enum_runs<D, D - 2, 1>(P, s, sms);
+        if constexpr (D >= 3 && !flat_serves(D, D - 3, SRC_RUN))
+            if (K == 2) return launch_enum_runs<D, D - 3, 2>(P, s, sms);
+        if constexpr (D >= 4 && !flat_serves(D, D - 4, SRC_RUN))
+            if (K == 3) return launch_enum_runs<D, D - 4, 3>(P, s, sms);
     }
     if (full && K == 2 && D >= 3) return launch_enum_dl<D, (D >= 3 ? D - 3 : 0)>(P, s, sms);
     if (full && K == 3 && D >= 4) return launch_enum_dl<D, (D >= 4 ? D - 4 : 0)>(P, s, sms);

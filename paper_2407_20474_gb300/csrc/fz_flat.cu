@@ -327,12 +327,6 @@ int launch_d(const EnumParams &P, int warp_bytes, cudaStream_t s, int sms) {
 
 }  // namespace
 
-bool flat_serves(int d, int np, int src) {
-    if (d < 3 || d > 9) return false;
-    if (src == SRC_PAIR) return np == d - 2;
-    return np >= 1 && np <= 3 && d - 1 - np >= 1 && d - 1 - np <= RUN_MAX_K;
-}
-
 int launch_enum_flat(const EnumParams &P, int warp_bytes, cudaStream_t s, int sms) {
     switch (P.d) {
         case 3: return launch_d<3>(P, warp_bytes, s, sms);

@@ -530,7 +530,7 @@ struct BatchGroup {
     int first, last;             // instances, by their place in the parameter images
     uint64_t item_lo, item_hi;   // their work items
 };
-constexpr int BATCH_MAX_GROUPS = 32;  // 23 flat shapes, 4 by rank, the general kernel
+constexpr int BATCH_MAX_GROUPS = 32;  // 21 flat shapes, 4 by rank, the general kernel
 // counters: BATCH_MAX_GROUPS words of device memory.
 int launch_enumerate_batch(const void *params_dev, const uint64_t *item0_dev,
                            const BatchGroup *groups, int ngroups, unsigned long long *counters,

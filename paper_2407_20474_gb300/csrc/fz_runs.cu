@@ -144,8 +144,9 @@ __device__ __forceinline__ TablePlace table_place(const RunBuild &J, uint64_t x,
     return pl;
 }
 
-// Rows of one level: a warp writes an even share (per_warp) of its job.  K: coordinates a row; CSR: the memo in element order (K packed
-// words a row), else a run-order table (quotient first).
+// Rows of one level: a warp writes an even share (per_warp) of its job.  K:
+// coordinates a row; CSR: the memo in element order (K packed words a row),
+// else a run-order table (quotient first).
 template <int K, int SRC, bool CSR>
 __global__ void __launch_bounds__(BT, 4)
     run_build_kernel(const RunBuild *__restrict__ jobs, int njobs, int *status) {
@@ -231,8 +232,9 @@ __global__ void __launch_bounds__(BT)
 // many as both hold.  The row's place inside its element counts the points
 // with a greater x; all rows of an element below p are its class's count.
 //
-// 4096 instances of widths 3..8 (4.1e7 elements, 1.1e7 rows): 270 us
-// with the dense tables' flat walk, against 613 us by the flat walk alone, which reads a count for every element.
+// 4096 instances of widths 3..8 (4.1e7 elements, 1.1e7 rows): 270 us with the
+// dense tables' flat walk, against 613 us by the flat walk alone, which reads a
+// count for every element.
 __global__ void __launch_bounds__(BT)
     run_build2_kernel(const RunBuild *__restrict__ jobs, int njobs, int *status) {
     __shared__ RunBuild sj;

@@ -312,9 +312,9 @@ int launch_group(fz_server_s *s, Group &G) {
             L.total_cost = r->count + L.W * S.runs_row[r->n];
             cost[j] = L.total_cost;
         }
-        // large requests take their plan's own kernel (its compiled-in walk
-        // or run copy writes faster than the batch kernel's generic one);
-        // so do those the batch kernel does not serve
+        // large requests take their plan's own kernel (its long items write
+        // faster than a batch's short ones); so do those the batch kernels do
+        // not serve
         direct[j] = (!batch_kernel_serves(L) || r->count >= serve_direct_rows()) ? 1 : 0;
     }
     std::vector<unsigned char> images((size_t)m * pb);

@@ -143,9 +143,6 @@ struct RunLevels {
     uint64_t *cls = nullptr;
 };
 
-// fz_flat.cu: true if the flat walk has a kernel for tuples of width d with
-// leaves of np prefix words.
-bool flat_serves(int d, int np, int src);
 // Cost of a leaf of the flat walk in rows (work-balanced slicing): 32 leaves
 // take about as many instructions as 100 rows.
 constexpr uint64_t FLAT_LEAF_COST = 4;
@@ -153,6 +150,14 @@ constexpr uint64_t FLAT_LEAF_COST = 4;
 // Deepest memo the levels build (rows of a table: quotient and coordinates).
 constexpr int RUN_MAX_K = 7;   // run-order tables
 constexpr int CSR_MAX_K = 8;   // memos in element order (from depth 3 on)
+
+// True if the flat walk has a kernel (fz_flat.cu) for tuples of width d with
+// leaves of np prefix words.
+constexpr bool flat_serves(int d, int np, int src) {
+    if (d < 3 || d > 9) return false;
+    if (src == SRC_PAIR) return np == d - 2;
+    return np >= 1 && np <= 3 && d - 1 - np >= 1 && d - 1 - np <= RUN_MAX_K;
+}
 
 // sums[j] (device) = sum over r < top of row j of C, exact when below 2^32.
 int launch_row_sums(const uint64_t *C, int64_t cs, int rows, int64_t top, uint64_t *sums,

@@ -32,6 +32,7 @@ int set_error(int status, const std::string &msg) {
 }
 
 int cuda_error(cudaError_t e, const char *what) {
+    cudaGetLastError();  // reported here, not by the next launch's check
     std::string m = std::string(what) + ": " + cudaGetErrorName(e) + " (" +
                     cudaGetErrorString(e) + ")";
     if (e == cudaErrorMemoryAllocation) return set_error(FZ_ENOMEM, m);

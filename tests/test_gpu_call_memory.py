@@ -47,3 +47,16 @@ def test_calls_give_their_memory_back(fz):
     for i, call in enumerate(calls):
         call()
         assert _free() >= start - KEPT, i
+
+
+def test_a_failed_allocation_is_reported_once(fz):
+    """Tables larger than the device: the call says so, and the next one works."""
+    g = tuple(range(1, 17))
+    for make in (lambda: fz.Plan(g, 2**31 - 2, k=0), lambda: fz.Batch([(g, 2**31 - 2)]),
+                 lambda: fz.Batch([((5, 8, 11, 14), 500), (g, 2**31 - 2)]),
+                 lambda: fz.Server(memory_bytes=1 << 42)):
+        with pytest.raises(fz.FzError, match="ENOMEM"):
+            make()
+        assert fz.fz_count((5, 8, 11, 14), 500) == 3783
+        with fz.Plan((5, 8, 11, 14), 500) as plan:
+            assert plan.count == 3783

@@ -2,14 +2,15 @@
 //
 // A batch keeps, for every instance, its count table and runs table (for
 // work-balanced slicing) and, per distinct tail, one memo shared by the
-// instances with that tail.  A rebuild is: one initialisation launch and
+// instances with that tail.  A rebuild is: one initialisation launch and up to
 // three launches per table level for all instances' tables together (the
-// batched strided scans of fz_count.cu), then the run-order tables of every
-// tail, one launch per depth (fz_runs.cu), and one launch for the memos kept
-// in element order, if any (one CTA per memo, the elementwise dynamic pass of
-// Section 2).  The enumeration is one persistent launch over (instance, slice)
-// work items (fz_enum.cu).  Everything after creation is asynchronous, so a rebuild plus
-// an enumeration can be captured in a CUDA graph.
+// batched strided scans of fz_count.cu), then one launch for the memos kept in
+// element order, if any (one CTA per memo, the elementwise dynamic pass of
+// Section 2), and the run-order tables of every tail, one launch per depth
+// (fz_runs.cu).  The enumeration is one persistent launch per shape over its
+// instances' (instance, slice) work items (fz_flat.cu, fz_enum.cu).
+// Everything after creation is asynchronous, so a rebuild plus an enumeration
+// can be captured in a CUDA graph.
 #include <cuda_runtime.h>
 
 #include <algorithm>

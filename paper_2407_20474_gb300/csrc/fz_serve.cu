@@ -8,20 +8,21 @@
 // A background thread admits queued requests in arrival order whenever a
 // slot and enough output memory (exact bytes, from a first-fit arena carved
 // out of one device allocation) are free.  By default every request admitted
-// in one pass of the loop is launched as one group: one persistent launch of
-// the batch enumeration kernel with a work-item range per request (its
-// parameters and item prefix staged in page-locked memory and copied in one
-// transfer), one copy back of the group's status words and one completion
+// in one pass of the loop is launched as one group: one persistent launch per
+// shape of the batch enumeration kernels with a work-item range per request
+// (its parameters and item prefix staged in page-locked memory and copied in
+// one transfer), one copy back of the group's status words and one completion
 // callback, on the next of several streams, so groups admitted while others
 // run overlap on the GPU.  With FZ_SERVE_PER_REQUEST every request is its
-// own launch of the single-instance kernel (and so is a request whose plan
-// the batch kernel does not serve: run order wider than 8).  Completion is recorded by a host callback on the
-// request's stream (cudaLaunchHostFunc), which frees the slot, stamps the
-// completion time and reads the request's own device status word (copied to
-// page-locked host memory just before the callback), so a device-side check
-// that failed marks that request, and only it, as failed.  The output stays
-// valid until the client releases it.  A queued request can be cancelled;
-// one already on the device runs to completion.
+// own launch of the single-instance kernel (and so is a large request, and one
+// whose plan the batch kernels do not serve: run order wider than 8).
+// Completion is recorded by a host callback on the request's stream
+// (cudaLaunchHostFunc), which frees the slot, stamps the completion time and
+// reads the request's own device status word (copied to page-locked host
+// memory just before the callback), so a device-side check that failed marks
+// that request, and only it, as failed.  The output stays valid until the
+// client releases it.  A queued request can be cancelled; one already on the
+// device runs to completion.
 #include <cuda_runtime.h>
 
 #include <atomic>

@@ -279,10 +279,10 @@ __global__ void __launch_bounds__(BT)
     const int32_t n = J.n, g = J.g, G = J.G;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint64_t carry = 0;
-    for (int base = 0; base < G; base += BT) {
-        const int c = base + (int)threadIdx.x;
+    for (int64_t base = 0; base < G; base += BT) {
+        const int64_t c = base + threadIdx.x;  // (past G near 2^31 on the way out)
         uint64_t v = 0;
-        if (c < G) v = __ldg(F + (c + (int64_t)((n - c) / g) * g));
+        if (c < G) v = __ldg(F + (c + (int64_t)((n - (int32_t)c) / g) * g));
         const uint64_t incl = warp_incl_scan(v, lane);
         if (lane == 31) warp_sum[wid] = incl;
         __syncthreads();
@@ -310,8 +310,8 @@ __global__ void __launch_bounds__(BT)
     const RunBuild &J = jobs[blockIdx.x];
     const int32_t n = J.n, g = J.g, G = J.G;
     uint64_t acc = 0;
-    for (int c = threadIdx.x; c < G; c += BT) {
-        const uint64_t v = __ldg(J.F + (c + (int64_t)((n - c) / g) * g));
+    for (int64_t c = threadIdx.x; c < G; c += BT) {
+        const uint64_t v = __ldg(J.F + (c + (int64_t)((n - (int32_t)c) / g) * g));
         acc += v < (1ull << 32) ? v : (1ull << 32);  // as row_sums_kernel
     }
 #pragma unroll

@@ -445,7 +445,7 @@ struct PrefixWalk {
         pb = 0;
 #pragma unroll
         for (int j = 0; j < NP - 1; ++j) {
-            const int idx = r[j] - (a[j] + 1) * P.g[j];
+            const int idx = r[j + 1] - P.g[j];  // r[j] - (a[j] + 1) g_j
             if (idx >= 0) pb += __ldg(P.C + (int64_t)j * P.cs + idx);
         }
     }
